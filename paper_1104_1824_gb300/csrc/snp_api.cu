@@ -87,8 +87,6 @@ int tc5_prepare(snp_system* h, uint64_t q) {
 
 namespace {
 
-size_t claim_smem(int m) { return (size_t)kWarpsPerBlock * 3 * m * sizeof(int32_t); }
-
 int check_device_errors(snp_system* h, cudaStream_t st, const char* where) {
   CK(cudaMemcpyAsync(h->pin.h, h->d_st.p, sizeof(ChunkState), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -460,36 +458,37 @@ int snp_step(snp_handle h, const int32_t* C, int64_t capacity, int32_t* out, uin
   if (!h || !C || !psi || capacity < 0 || (capacity > 0 && !out)) return fail(SNP_E_INVALID, "bad arguments");
   CK(cudaSetDevice(h->device));
   const int m = h->m;
-  std::vector<int32_t> c(m);
-  CK(cudaMemcpy(c.data(), C, sizeof(int32_t) * m, cudaMemcpyDefault));
+  // C twice: the second copy becomes the base child on the device
+  std::vector<int32_t> c(2 * (size_t)m);
+  if (is_device_ptr(C)) CK(cudaMemcpy(c.data(), C, sizeof(int32_t) * m, cudaMemcpyDefault));
+  else std::memcpy(c.data(), C, sizeof(int32_t) * m);
   for (int j = 0; j < m; ++j) {
     if (c[j] < 0) return fail(SNP_E_INVALID, "C[%d] = %d < 0", j, c[j]);
     if (c[j] > INT32_MAX - h->gain[j]) return fail(SNP_E_OVERFLOW, "C[%d] = %d: a child could leave int32", j, c[j]);
+    c[m + j] = c[j];
   }
-  TRY(h->d_tmp.reserve(sizeof(int32_t) * m + 64));
+  const size_t rows_bytes = (sizeof(int32_t) * 2 * m + 15) / 16 * 16;
+  TRY(h->d_tmp.reserve(rows_bytes + sizeof(StepPlan)));
   int32_t* dC = h->d_tmp.as<int32_t>();
-  uint64_t* dpsi = reinterpret_cast<uint64_t*>(h->d_tmp.as<char>() + ((sizeof(int32_t) * m + 15) / 16) * 16);
-  CK(cudaMemcpy(dC, c.data(), sizeof(int32_t) * m, cudaMemcpyHostToDevice));
-  CK(cudaMemset(h->d_st.p, 0, sizeof(ChunkState)));
-  launch_psi(h->dev(), dC, 4, nullptr, 1, -1, dpsi, nullptr, h->d_st.as<ChunkState>(), nullptr, sm_count(h->device));
+  StepPlan* plan = reinterpret_cast<StepPlan*>(h->d_tmp.as<char>() + rows_bytes);
+  const bool dev_out = capacity > 0 && is_device_ptr(out);
+  CK(cudaMemcpyAsync(dC, c.data(), sizeof(int32_t) * 2 * m, cudaMemcpyHostToDevice, nullptr));
+  launch_step_plan(h->dev(), dC, dC + m, plan, nullptr);
   CK(cudaGetLastError());
-  uint64_t ps = 0;
-  CK(cudaMemcpy(&ps, dpsi, sizeof ps, cudaMemcpyDeviceToHost));
-  *psi = ps;
-  const uint64_t n = std::min<uint64_t>(ps, (uint64_t)capacity);
-  if (n == 0) return SNP_OK;
-  int32_t* dst = out;
-  DevBuf tmp;
-  const bool dev_out = is_device_ptr(out);
-  if (!dev_out) {
-    TRY(tmp.reserve(sizeof(int32_t) * m * n));
-    dst = tmp.as<int32_t>();
+  CK(cudaMemcpyAsync(h->pin.u64, &plan->psi, sizeof(uint64_t), cudaMemcpyDeviceToHost, nullptr));
+  if (dev_out) {  // the kernel reads Psi itself: one wait for the whole call
+    launch_step_children(h->dev(), dC + m, plan, (uint64_t)capacity, out, nullptr, sm_count(h->device));
+    CK(cudaGetLastError());
   }
-  const int blocks = grid_for((int64_t)n, kWarpsPerBlock, sm_count(h->device) * 8);
-  k_step_children<<<blocks, kThreads, claim_smem(m)>>>(h->dev(), dC, n, dst);
+  CK(cudaStreamSynchronize(nullptr));
+  *psi = *h->pin.u64;
+  const uint64_t n = std::min<uint64_t>(*psi, (uint64_t)capacity);
+  if (n == 0 || dev_out) return SNP_OK;
+  DevBuf tmp;
+  TRY(tmp.reserve(sizeof(int32_t) * m * n));
+  launch_step_children(h->dev(), dC + m, plan, n, tmp.as<int32_t>(), nullptr, sm_count(h->device));
   CK(cudaGetLastError());
-  if (!dev_out) CK(cudaMemcpy(out, dst, sizeof(int32_t) * m * n, cudaMemcpyDeviceToHost));
-  CK(cudaDeviceSynchronize());
+  CK(cudaMemcpy(out, tmp.p, sizeof(int32_t) * m * n, cudaMemcpyDeviceToHost));
   return SNP_OK;
 }
 

@@ -397,36 +397,43 @@ __device__ __forceinline__ void load_parent(const DevSys& s, const int32_t* __re
   __syncwarp();
 }
 
-// Steps (b) and (c) for candidate t of the loaded parent: decode t in the
-// mixed radix of the choice counts (last neuron least significant), then
-// C' = C + sum of the chosen rules' rows of M_Pi, built in w.buf.
-__device__ __forceinline__ void build_child(const DevSys& s, WarpParent& w, uint64_t t, int lane) {
-  for (int n = lane; n < s.m; n += 32) w.buf[n] = w.par[n];
-  __syncwarp();
-  const int n0 = lane * s.K;
-  const int n1 = min(n0 + s.K, s.m);
-  if (n0 < n1) {
-    uint64_t q = (w.after > t) ? 0ull : t / w.after;
-    for (int n = n1 - 1; n >= n0; --n) {
-      const uint32_t mask = w.msk[n];
-      if (!mask) continue;  // the neuron cannot fire: one choice
-      const uint32_t radix = __popc(mask);
-      uint32_t d;
-      if ((q >> 32) == 0) {
-        uint32_t q32 = (uint32_t)q;
-        d = q32 % radix;
-        q = q32 / radix;
-      } else {
-        d = (uint32_t)(q % radix);
-        q /= radix;
-      }
-      const int r = __ldg(s.first_rule + n) + nth_set_bit(mask, (int)d);
-      const int e0 = __ldg(&s.rule[r].w), e1 = __ldg(&s.rule[r + 1].w);
-      for (int e = e0; e < e1; ++e) {
-        const int2 cv = __ldg(s.csr + e);
-        atomicAdd(&w.buf[cv.x], cv.y);
+// Mixed-radix digit of a neuron with `radix` choices; q moves to the next
+// more significant neuron.
+__device__ __forceinline__ uint32_t next_digit(uint64_t& q, uint32_t radix) {
+  if (radix <= 1) return 0;
+  if ((q >> 32) == 0) {
+    const uint32_t q32 = (uint32_t)q;
+    q = q32 / radix;
+    return q32 % radix;
+  }
+  const uint32_t d = (uint32_t)(q % radix);
+  q /= radix;
+  return d;
+}
+
+// row += M[rn] - M[ro] for two rules of one neuron, by the whole warp: the
+// columns of the neuron's support are distinct, so the lanes share them out.
+// A lane's loads for up to three support columns are all issued before its
+// updates, so that a support of up to 96 columns costs one round trip.
+__device__ __forceinline__ void warp_swap_rule(const DevSys& s, int32_t* row, int ro, int rn, int lane) {
+  const int4 dn = __ldg(s.rdesc + rn);
+  const int32_t* vn = s.rval + dn.z;
+  const int32_t* vo = s.rval + __ldg(&s.rdesc[ro].z);
+  const int32_t* col = s.scol + dn.x;
+  for (int i0 = 0; i0 < dn.y; i0 += 96) {
+    int c[3], v[3];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const int i = i0 + lane + 32 * u;
+      c[u] = -1;
+      if (i < dn.y) {
+        c[u] = __ldg(col + i);
+        v[u] = __ldg(vn + i) - __ldg(vo + i);
       }
     }
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (c[u] >= 0) row[c[u]] += v[u];
   }
   __syncwarp();
 }

@@ -496,20 +496,6 @@ __device__ __forceinline__ void resolve_warp(const ClaimArgs& a, const int32_t* 
     resolve_warp_body<RF>(a, row, key, lid, todo);
 }
 
-// Mixed-radix digit of a neuron with `radix` choices; q moves to the next
-// more significant neuron.
-__device__ __forceinline__ uint32_t next_digit(uint64_t& q, uint32_t radix) {
-  if (radix <= 1) return 0;
-  if ((q >> 32) == 0) {
-    const uint32_t q32 = (uint32_t)q;
-    q = q32 / radix;
-    return q32 % radix;
-  }
-  const uint32_t d = (uint32_t)(q % radix);
-  q /= radix;
-  return d;
-}
-
 // Four counts of a row in global memory, from count 4 * j on (VEC rows).
 template <class RF>
 __device__ __forceinline__ int4 load4(const typename RF::T* row, int j) {
@@ -696,33 +682,6 @@ __device__ __forceinline__ void warp_copy_row(const int32_t* src, int32_t* dst, 
   } else {
     for (int j = lane; j < m; j += 32) dst[j] = src[j];
   }
-}
-
-// row += M[rn] - M[ro] for two rules of one neuron, by the whole warp: the
-// columns of the neuron's support are distinct, so the lanes share them out.
-// A lane's loads for up to three support columns are all issued before its
-// updates, so that a support of up to 96 columns costs one round trip.
-__device__ __forceinline__ void warp_swap_rule(const DevSys& s, int32_t* row, int ro, int rn, int lane) {
-  const int4 dn = __ldg(s.rdesc + rn);
-  const int32_t* vn = s.rval + dn.z;
-  const int32_t* vo = s.rval + __ldg(&s.rdesc[ro].z);
-  const int32_t* col = s.scol + dn.x;
-  for (int i0 = 0; i0 < dn.y; i0 += 96) {
-    int c[3], v[3];
-#pragma unroll
-    for (int u = 0; u < 3; ++u) {
-      const int i = i0 + lane + 32 * u;
-      c[u] = -1;
-      if (i < dn.y) {
-        c[u] = __ldg(col + i);
-        v[u] = __ldg(vn + i) - __ldg(vo + i);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 3; ++u)
-      if (c[u] >= 0) row[c[u]] += v[u];
-  }
-  __syncwarp();
 }
 
 // Row of candidate L of the current block in the scratch row: the block base

@@ -512,24 +512,6 @@ void launch_insert_rows(DevSys s, const int32_t* pool, int w, const uint32_t* pe
   fn<<<blocks, kWarpsPerBlock * 32, 0, stream>>>(s, pool, perm, r0, r1, t, st);
 }
 
-// All children of one configuration C in canonical order (no deduplication).
-__global__ void __launch_bounds__(kWarpsPerBlock * 32) k_step_children(DevSys s, const int32_t* C, uint64_t n,
-                                                                       int32_t* out) {
-  extern __shared__ int32_t smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int m = s.m;
-  WarpParent w;
-  w.par = smem + (size_t)wib * 3 * m;
-  w.msk = reinterpret_cast<uint32_t*>(w.par + m);
-  w.buf = w.par + 2 * m;
-  load_parent(s, C, w, lane);
-  const uint64_t nw = (uint64_t)gridDim.x * kWarpsPerBlock;
-  for (uint64_t t = (uint64_t)blockIdx.x * kWarpsPerBlock + wib; t < n; t += nw) {
-    build_child(s, w, t, lane);
-    for (int j = lane; j < m; j += 32) out[t * m + j] = w.buf[j];
-  }
-}
-
 __global__ void k_fill_u64(unsigned long long* p, uint64_t n, unsigned long long v) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
     p[i] = v;

@@ -209,7 +209,21 @@ void launch_pack_rows(const int32_t* src, int64_t n, int m, int w, int32_t* dst,
 // (blocks CTAs of kWarpsPerBlock warps).
 void launch_insert_rows(DevSys s, const int32_t* pool, int w, const uint32_t* perm, int64_t r0, int64_t r1,
                         DevTable t, ChunkState* st, int blocks, cudaStream_t stream);
-__global__ void k_step_children(DevSys s, const int32_t* C, uint64_t n, int32_t* out);
+// All children of one configuration (snp_step.cu).  Plan of a step: Psi(C) and
+// the multi-choice neurons, least significant first, as far as the first
+// `capacity` children reach (each has two or more choices: at most 64).
+constexpr int kStepList = 64;
+struct StepPlan {
+  unsigned long long psi;
+  int32_t len;
+  int32_t neuron[kStepList];
+  uint32_t mask[kStepList];
+};
+// Reads C, turns base (C on entry) into the base child and fills *plan.
+void launch_step_plan(DevSys s, const int32_t* C, int32_t* base, StepPlan* plan, cudaStream_t st);
+// Children 0 .. min(Psi, capacity) - 1, canonical order, to out (no deduplication).
+void launch_step_children(DevSys s, const int32_t* base, const StepPlan* plan, uint64_t capacity, int32_t* out,
+                          cudaStream_t st, int nsm);
 __global__ void k_fill_u64(unsigned long long* p, uint64_t n, unsigned long long v);
 
 // Device-wide exclusive scans (n elements, in -> out; "total" gets the sum).
