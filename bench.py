@@ -79,7 +79,7 @@ WORKLOADS = {
     "batch4096": dict(n=4096, base_seed=1000, depth=6, cap=1 << 12, budget=1 << 16,
                       desc="4096 independent random SNP systems (system s: seed 1000+s; m U[16,256], 1-4 rules/neuron, "
                            "out-degree U[2,8], otherwise as random64), each explored to depth 6 with cap 2^12 and "
-                           "budget 2^16; one launch per depth for all systems (batch engine, CUDA graph)",
+                           "budget 2^16; all systems advance together (batch engine)",
                       cpu_sample=dict(systems=2, depth=6, cap=1 << 12, budget=1 << 16),
                       ref_sample=dict(systems=1, depth=4, cap=1 << 12, budget=1 << 16)),
 }
@@ -455,7 +455,7 @@ def bench_ours(args):
 
 
 def time_batch(args, w, systems, handles, snp, torch, dist, dev, world, local, form: str, steps: int, warmup: int):
-    """Times `steps` batch explorations (one launch per depth for all systems)
+    """Times `steps` batch explorations
     in one transition form; returns the timing, plan and per-step counts."""
     import numpy as np
     hs = [h.h for h in handles]

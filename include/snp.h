@@ -291,12 +291,14 @@ int snp_row_width(snp_handle h, int32_t* bytes_per_count);
 /* Breadth-first exploration of n independent systems at once (the batch
  * engine): every system runs exactly what snp_explore would run on it with
  * the same options, and afterwards each handle answers snp_reachable,
- * snp_depth_stats and friends for its own exploration.  All systems advance
- * together, one device launch per depth (captured in a CUDA graph); a CTA
- * takes one system at a time and runs its whole depth.
+ * snp_depth_stats and friends for its own exploration.  Sparse form: all
+ * systems' passes share every launch, each system in its own depth and pass.
+ * Tensor-core form: one device launch per depth (captured in a CUDA graph); a
+ * CTA takes one system at a time and runs its whole depth.
  *  hs        [n] host array of handles, all on the current device, distinct.
  *  opts      depth, frontier_cap (required: 1 <= cap <= 2^20), candidate_budget,
- *            max_expand_value, chunk (candidates per pass, <= 0: 2048),
+ *            max_expand_value, chunk (candidates per pass and system, <= 0:
+ *            by the cap, or 2048 in the tensor-core form),
  *            tile, warps, stream; transition must be SNP_T_SPARSE_I32 and
  *            record_parents 0.
  *  statuses  (host, [n], may be NULL) per system: SNP_OK, SNP_E_OVERFLOW,
@@ -318,15 +320,15 @@ int snp_batch_autotune(snp_handle* hs, int32_t n, const snp_explore_opts* opts, 
  * The paper's simulator runs one system at a time; this loop serves many.  A
  * server thread admits pending requests while its device memory allows (each
  * request needs its pool, 4m (1 + depth * cap) bytes, and its hash table),
- * then advances every admitted request by one depth per launch of the batch
- * engine, so requests that arrive while others run join at the next launch
- * (continuous batching).  A finished request's configurations are copied
+ * then advances every admitted request by a few passes at a time (a tick)
+ * with the batch engine's kernels, so requests that arrive while others run
+ * join at the next tick (continuous batching).  A finished request's configurations are copied
  * into its handle, which then answers snp_reachable and snp_depth_stats
  * exactly as after snp_explore; its memory goes back to the server. */
 typedef struct {
   int64_t submitted, completed, active, pending;
   int64_t new_configs;  /* new configurations of the completed requests */
-  int64_t ticks;        /* batch launches */
+  int64_t ticks;        /* times the admitted requests were advanced */
   double busy_ms;       /* host time spent running launches */
   double span_ms;       /* first submit to last completion */
   double p50_ms, p99_ms, max_ms;  /* latency: submit to result ready */

@@ -310,7 +310,7 @@ def _handle_array(handles):
 
 
 def snp_explore_batch(handles, opts: snp_explore_opts, statuses: Optional[np.ndarray] = None) -> None:
-    """Explores the systems of `handles` together (one launch per depth)."""
+    """Explores the systems of `handles` together."""
     arr = _handle_array(handles)
     _check(load_library().snp_explore_batch(arr, len(handles), ctypes.byref(opts), _ptr(statuses)))
 

@@ -1,6 +1,8 @@
 // Batch engine, host side (snp_explore_batch, snp_batch_autotune): packs many
-// loaded systems into one device arena and advances them all one depth per
-// launch of k_batch_depth, the depth launches captured in one CUDA graph.
+// loaded systems into one device arena and advances them together.  Sparse
+// form: iterations of snp_many.cu until no system is left, the next one
+// enqueued before the last one's count is read back.  Tensor-core form: one
+// depth per launch of k_batch_depth_tc, captured in one CUDA graph.
 #include <algorithm>
 #include <chrono>
 #include <cstring>
@@ -14,12 +16,12 @@ namespace snp {
 
 // Device memory of one batch; shared by its handles until they move on.
 struct BatchArena {
-  DevBuf sys, stats, pools, slots, scratch, queue, c0, c0_off;
+  DevBuf sys, stats, pools, slots, scratch, queue, items, c0, c0_off;
   int32_t n = 0, depth = 0;
   // shape the buffers and the captured graph were made for
   std::vector<snp_system*> handles;
   int64_t cap = 0, budget = 0;
-  int32_t max_expand = 0, blocks = 0, warps = 0, B = 0, tc = 0;
+  int32_t max_expand = 0, blocks = 0, tc = 0;
   uint32_t qc = 0;
   uint64_t nslots = 0;
   size_t scratch_stride = 0, pool_bytes = 0;
@@ -34,9 +36,62 @@ struct BatchArena {
 namespace {
 
 struct BatchPlan {
-  uint32_t qc = 2048;
-  int tile = 0, warps = 8;
+  uint32_t qc = 0;         // candidates per pass (0: chosen by the cap)
+  int tile = 0, warps = 0;  // rows of an expand tile, warps per CTA (0: automatic)
 };
+
+// Scratch the systems of one group share the device with.
+constexpr size_t kGroupScratch = (size_t)12 << 30;
+
+// Runs systems [lo, hi) of the arena (sparse form) to their end on st.
+int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_off, int32_t lo, int32_t hi,
+               const BatchPlan& plan, uint32_t qc, PinnedState& pin, cudaEvent_t* evs, cudaStream_t st, int nsm) {
+  const int32_t n = hi - lo;
+  std::vector<int> ms(n);
+  for (int32_t i = 0; i < n; ++i) ms[i] = sys[lo + i].sys.m;
+  const ManyPlan mp = many_plan(ms.data(), n, plan.tile, plan.warps);
+  // runs of about a quarter of a warp's share of a full pass
+  const uint64_t warps = (uint64_t)nsm * mp.ctas_per_sm * mp.warps;
+  const uint32_t run = (uint32_t)std::min<uint64_t>(512, std::max<uint64_t>(64, ((uint64_t)n * qc / (4 * warps) + 31) / 32 * 32));
+  size_t at = 0;
+  int64_t items = 0;
+  for (int32_t i = lo; i < hi; ++i) {
+    BatchSys& b = sys[i];
+    many_carve(b, arena->scratch.as<unsigned char>() + at, qc, run);
+    at += many_scratch_bytes(b.cap, qc, b.sys.m);
+    b.tile = many_tile(mp, b.sys.m, plan.tile);
+    b.fixed_q = plan.qc > 0 ? 1 : 0;
+    items += many_items(b.cap, qc, run);
+  }
+  TRY(arena->items.reserve(sizeof(int2) * (2 * kMqForms + 2) * items));
+  TRY(arena->queue.reserve(sizeof(uint32_t) * kMqCounters));
+  ManyQueue q;
+  q.expand[0] = arena->items.as<int2>();
+  q.expand[1] = q.expand[0] + kMqForms * items;
+  q.copy = q.expand[1] + kMqForms * items;
+  q.psi = q.copy + items;
+  q.ctr = arena->queue.as<uint32_t>();
+  q.cap = items;
+  BatchSys* dsys = arena->sys.as<BatchSys>() + lo;
+  CK(cudaMemcpyAsync(dsys, sys.data() + lo, sizeof(BatchSys) * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemsetAsync(q.ctr, 0, sizeof(uint32_t) * kMqCounters, st));
+  launch_many_init(dsys, nullptr, arena->c0.as<int32_t>(), arena->c0_off.as<int64_t>() + lo, n, q, st);
+  CK(cudaGetLastError());
+  // two iterations in flight: the count read back is the one before last
+  uint32_t* active[2] = {reinterpret_cast<uint32_t*>(pin.slot[0]), reinterpret_cast<uint32_t*>(pin.slot[1])};
+  for (int it = 0;; ++it) {
+    if (it >= 2) {
+      CK(cudaEventSynchronize(evs[it & 1]));
+      if (*active[it & 1] == 0) break;
+    }
+    launch_many_iteration(dsys, n, q, it & 1, mp, st, nsm);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(active[it & 1], q.ctr + kMqActive, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    CK(cudaEventRecord(evs[it & 1], st));
+  }
+  CK(cudaStreamSynchronize(st));
+  return SNP_OK;
+}
 
 int batch_setup(snp_handle* hs, int32_t n, const snp_explore_opts* o) {
   if (!hs || n < 1 || !o) return fail(SNP_E_INVALID, "bad arguments");
@@ -63,6 +118,41 @@ int batch_setup(snp_handle* hs, int32_t n, const snp_explore_opts* o) {
   return SNP_OK;
 }
 
+// Tensor-core form: depth launches, captured once per arena and replayed as one graph.
+int run_tc_depths(BatchArena* arena, const std::vector<BatchSys>& sys, const BatchArgs& args, int blocks, int depth,
+                  bool fresh, size_t scratch_stride, cudaStream_t st, int nsm) {
+  const int32_t n = (int32_t)sys.size();
+  CK(cudaMemcpyAsync(arena->sys.p, sys.data(), sizeof(BatchSys) * n, cudaMemcpyHostToDevice, st));
+  CK(cudaMemsetAsync(arena->queue.p, 0, sizeof(unsigned int) * (depth + 1), st));
+  if (fresh) CK(cudaMemsetAsync(arena->scratch.p, 0, scratch_stride * blocks, st));  // bitmaps start (and stay) clear
+  k_batch_init<<<grid_for(n, 8, nsm * 16), 256, 0, st>>>(arena->sys.as<BatchSys>(), arena->c0.as<int32_t>(),
+                                                          arena->c0_off.as<int64_t>(), n);
+  CK(cudaGetLastError());
+  if (!arena->exec) {
+    BatchArgs a = args;
+    cudaStream_t cap_st = nullptr;
+    CK(cudaStreamCreateWithFlags(&cap_st, cudaStreamNonBlocking));
+    cudaGraph_t graph = nullptr;
+    CK(cudaStreamBeginCapture(cap_st, cudaStreamCaptureModeThreadLocal));
+    for (int d = 1; d <= depth; ++d) {
+      a.launch = d;
+      launch_batch_depth_tc(a, blocks, cap_st);
+    }
+    cudaError_t ce = cudaStreamEndCapture(cap_st, &graph);
+    if (ce == cudaSuccess) ce = cudaGraphInstantiate(&arena->exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    cudaStreamDestroy(cap_st);
+    if (ce != cudaSuccess) {
+      arena->exec = nullptr;
+      return fail(SNP_E_CUDA, "batch graph: %s", cudaGetErrorString(ce));
+    }
+  }
+  cudaError_t ce = cudaGraphLaunch(arena->exec, st);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+  if (ce != cudaSuccess) return fail(SNP_E_CUDA, "batch run: %s", cudaGetErrorString(ce));
+  return SNP_OK;
+}
+
 // Runs depths 1..depth of the batch (all handles) with the given plan; fills
 // the handles' results.  ms (optional) receives the device time of the depths.
 int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchPlan& plan, int32_t* statuses,
@@ -77,31 +167,14 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
   int m_max = 1;
   for (int32_t i = 0; i < n; ++i) m_max = std::max(m_max, hs[i]->m);
   const int64_t rows_per = 1 + (int64_t)depth * cap;
-  const uint64_t want_slots = (uint64_t)((long double)(rows_per + (int64_t)depth * plan.qc) * 4.0L / 3.0L) + kBucket;
+  // passes: the caller's size, else up to 2048 in the tensor-core form and by the cap in the sparse form
+  const uint32_t qs = plan.qc > 0 ? plan.qc : 2048;  // claims past the cap the table has room for, per depth
+  const uint32_t qc = plan.qc > 0 ? plan.qc : tc ? 2048 : many_default_qc(cap);
+  const uint64_t want_slots = (uint64_t)((long double)(rows_per + (int64_t)depth * qs) * 4.0L / 3.0L) + kBucket;
   const uint64_t nslots = std::max<uint64_t>(pow2_at_least(want_slots), kBucket);
-  // tile rows and warps
-  int ts = 0;
-  int B = plan.tile > 0 ? plan.tile : 32;  // shrunk below to what the shared memory holds
-  const int warps = (tc || plan.warps == 4) ? 4 : 8;
-  size_t warp_smem = expand_smem_bytes(m_max, B, &ts);
-  while (B > 1 && warp_smem * warps > (200u << 10)) warp_smem = expand_smem_bytes(m_max, --B, &ts);
-  if (plan.tile <= 0 && B > 16 && B < 32) {  // measured: 16 rows beat 17 (-3%) and 18 (-17%) on the batch workload
-    B = 16;
-    warp_smem = expand_smem_bytes(m_max, B, &ts);
-  }
-  if (!tc && warp_smem * warps > (220u << 10))
-    return fail(SNP_E_INVALID, "rows of %d neurons do not fit the batch tile", m_max);
-  int blocks_per_sm = 1;
-  {
-    int nb = 0;
-    // one CTA per SM is always resident; two when registers and shared memory allow (the
-    // tensor-core form: two CTAs of 128 TMEM columns each)
-    nb = tc ? 2 : (warps == 4 && warp_smem * warps * 2 <= (200u << 10)) ? 2 : 1;
-    blocks_per_sm = nb;
-  }
-  if (tc) B = 0;
-  const int blocks = std::max(1, std::min<int>(nsm * blocks_per_sm, n));
-  const size_t scratch_stride = (batch_scratch_bytes(cap, plan.qc, m_max) + 255) & ~size_t(255);
+  // tensor-core form: two CTAs of 128 TMEM columns per SM
+  const int blocks = std::max(1, std::min<int>(nsm * 2, n));
+  const size_t scratch_stride = tc ? (batch_scratch_bytes(cap, qc, m_max) + 255) & ~size_t(255) : 0;
 
   size_t pool_bytes = 0;
   std::vector<size_t> pool_off(n);
@@ -113,8 +186,8 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
   std::shared_ptr<BatchArena> arena = hs[0]->batch;
   bool same = arena && arena->n == n && arena->depth == depth && arena->cap == cap &&
               arena->budget == (o->candidate_budget > 0 ? o->candidate_budget : 0) &&
-              arena->max_expand == o->max_expand_value && arena->blocks == blocks && arena->warps == warps &&
-              arena->B == B && arena->qc == plan.qc && arena->nslots == nslots && arena->pool_bytes == pool_bytes &&
+              arena->max_expand == o->max_expand_value && arena->blocks == blocks && arena->qc == qc &&
+              arena->nslots == nslots && arena->pool_bytes == pool_bytes &&
               arena->scratch_stride == scratch_stride && arena->tc == (tc ? 1 : 0);
   for (int32_t i = 0; same && i < n; ++i) same = arena->handles[i] == hs[i] && hs[i]->batch == arena;
   if (!same) {
@@ -126,9 +199,7 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
     arena->budget = o->candidate_budget > 0 ? o->candidate_budget : 0;
     arena->max_expand = o->max_expand_value;
     arena->blocks = blocks;
-    arena->warps = warps;
-    arena->B = B;
-    arena->qc = plan.qc;
+    arena->qc = qc;
     arena->nslots = nslots;
     arena->pool_bytes = pool_bytes;
     arena->scratch_stride = scratch_stride;
@@ -144,8 +215,10 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
   TRY(arena->stats.reserve(sizeof(BatchDepthStat) * n * (depth + 1)));
   TRY(arena->pools.reserve(pool_bytes));
   TRY(arena->slots.reserve(sizeof(unsigned long long) * nslots * n));
-  TRY(arena->scratch.reserve(scratch_stride * blocks));
-  TRY(arena->queue.reserve(sizeof(unsigned int) * (depth + 1)));
+  if (tc) {
+    TRY(arena->scratch.reserve(scratch_stride * blocks));
+    TRY(arena->queue.reserve(sizeof(unsigned int) * (depth + 1)));
+  }
   std::vector<int32_t> c0;
   std::vector<int64_t> c0_off(n);
   std::vector<BatchSys> sys(n);
@@ -172,72 +245,68 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
     b.MB = tc ? h->d_MB.as<uint8_t>() : nullptr;
     b.np = h->t5_np;
     b.nblocks = h->t5_nblocks;
+    b.overshoot = qs;
   }
   TRY(arena->c0.reserve(sizeof(int32_t) * c0.size()));
   TRY(arena->c0_off.reserve(sizeof(int64_t) * n));
-  CK(cudaMemcpyAsync(arena->sys.p, sys.data(), sizeof(BatchSys) * n, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(arena->c0.p, c0.data(), sizeof(int32_t) * c0.size(), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(arena->c0_off.p, c0_off.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
   CK(cudaMemsetAsync(arena->stats.p, 0, sizeof(BatchDepthStat) * n * (depth + 1), st));
-  CK(cudaMemsetAsync(arena->queue.p, 0, sizeof(unsigned int) * (depth + 1), st));
-  if (!same) CK(cudaMemsetAsync(arena->scratch.p, 0, scratch_stride * blocks, st));  // bitmaps start (and stay) clear
   k_fill_u64<<<grid_for((int64_t)(nslots * n), 256, nsm * 32), 256, 0, st>>>(arena->slots.as<unsigned long long>(),
                                                                              nslots * n, kEmpty);
   CK(cudaGetLastError());
-  k_batch_init<<<grid_for(n, 8, nsm * 16), 256, 0, st>>>(arena->sys.as<BatchSys>(), arena->c0.as<int32_t>(),
-                                                          arena->c0_off.as<int64_t>(), n);
-  CK(cudaGetLastError());
-
-  BatchArgs a;
+  BatchArgs a;  // tensor-core form
   std::memset(&a, 0, sizeof a);
   a.sys = arena->sys.as<BatchSys>();
   a.n = n;
-  a.qc = plan.qc;
-  a.B = B;
-  a.ts = ts;
-  a.run = 4 * B;
-  a.warp_smem = warp_smem;
+  a.qc = qc;
   a.queue = arena->queue.as<unsigned int>();
   a.scratch = arena->scratch.as<unsigned char>();
   a.scratch_stride = scratch_stride;
   a.pmax = cap;
   a.m_max = m_max;
-  a.tc = tc ? 1 : 0;
-
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (ms) {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
   }
-  // depth launches, captured once per arena and replayed as one graph
-  if (!arena->exec) {
-    cudaStream_t cap_st = nullptr;
-    CK(cudaStreamCreateWithFlags(&cap_st, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    CK(cudaStreamBeginCapture(cap_st, cudaStreamCaptureModeThreadLocal));
-    for (int d = 1; d <= depth; ++d) {
-      a.launch = d;
-      launch_batch_depth(a, blocks, warps, cap_st);
-    }
-    cudaError_t ce = cudaStreamEndCapture(cap_st, &graph);
-    if (ce == cudaSuccess) ce = cudaGraphInstantiate(&arena->exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    cudaStreamDestroy(cap_st);
-    if (ce != cudaSuccess) {
-      arena->exec = nullptr;
-      return fail(SNP_E_CUDA, "batch graph: %s", cudaGetErrorString(ce));
-    }
-  }
+  int rc = SNP_OK;
   if (ms) CK(cudaEventRecord(e0, st));
-  cudaError_t ce = cudaGraphLaunch(arena->exec, st);
-  if (ms && ce == cudaSuccess) ce = cudaEventRecord(e1, st);
-  if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-  if (ce != cudaSuccess) return fail(SNP_E_CUDA, "batch run: %s", cudaGetErrorString(ce));
-  if (ms) {
-    CK(cudaEventElapsedTime(ms, e0, e1));
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+  if (tc) {
+    rc = run_tc_depths(arena.get(), sys, a, blocks, depth, !same, scratch_stride, st, nsm);
+  } else {
+    // groups of systems whose scratch fits kGroupScratch; with little memory
+    // left, smaller groups (down to one system) and passes of 2048
+    size_t limit = kGroupScratch;
+    uint32_t q = qc;
+    for (int32_t lo = 0; lo < n && rc == SNP_OK;) {
+      int32_t hi = lo;
+      size_t need = 0;
+      while (hi < n) {
+        const size_t one = many_scratch_bytes(cap, q, hs[hi]->m);
+        if (hi > lo && need + one > limit) break;
+        need += one;
+        ++hi;
+      }
+      rc = arena->scratch.reserve(need);
+      if (rc == SNP_E_NOMEM && (hi > lo + 1 || q > qs)) {
+        limit = std::min(limit, need) / 4;
+        q = std::min(q, std::max<uint32_t>(qs, 1));
+        rc = SNP_OK;
+        continue;
+      }
+      if (rc == SNP_OK) rc = many_group(arena.get(), sys, c0_off.data(), lo, hi, plan, q, hs[0]->pin, hs[0]->evs, st, nsm);
+      lo = hi;
+    }
   }
+  if (ms && rc == SNP_OK) {
+    CK(cudaEventRecord(e1, st));
+    CK(cudaEventSynchronize(e1));
+    CK(cudaEventElapsedTime(ms, e0, e1));
+  }
+  if (e0) cudaEventDestroy(e0);
+  if (e1) cudaEventDestroy(e1);
+  if (rc != SNP_OK) return rc;
   // results
   std::vector<BatchDepthStat> stats((size_t)n * (depth + 1));
   CK(cudaMemcpy(sys.data(), arena->sys.p, sizeof(BatchSys) * n, cudaMemcpyDeviceToHost));

@@ -1,16 +1,15 @@
-// Kernels of the batch engine and the serving loop.
+// The batch engine's tensor-core form (the sparse form: snp_many.cu).
 #include <algorithm>
 
 #include "snp_expand.cuh"
 #include "snp_tcgen05.cuh"
 
-// ---------------------------------------------------------------------------
-// Batch engine: one launch runs depth d of every system of a batch.  A CTA
-// takes systems from a work queue; for each it runs the whole depth with block
-// barriers in place of the host: Psi of its frontier (Eq. psi), the saturating
-// scan, then passes of up to qc candidates -- expand (the same warp code as
-// k_expand), first-occurrence marks, ranks, commit -- until the frontier cap,
-// the candidate budget or the candidates run out.
+// One launch runs depth d of every system of a batch.  A CTA takes systems
+// from a work queue; for each it runs the whole depth with block barriers in
+// place of the host: Psi of its frontier (Eq. psi), the saturating scan, then
+// passes of up to qc candidates -- rows by tensor core, resolve,
+// first-occurrence marks, ranks, commit -- until the frontier cap, the
+// candidate budget or the candidates run out.
 
 namespace snp {
 
@@ -48,40 +47,6 @@ __device__ __forceinline__ BatchScratch batch_scratch(unsigned char* base, int64
   b.hash = reinterpret_cast<unsigned long long*>(take((size_t)qc * 8));
   b.red = reinterpret_cast<uint8_t*>(take(qc));
   return b;
-}
-
-// Block-wide exclusive scan of v[0..n) in place (saturating u64), in tiles of blockDim.x.
-__device__ void block_scan_sat(uint64_t* v, int64_t n, uint64_t* wsum) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  uint64_t carry = 0;
-  for (int64_t t0 = 0; t0 < n; t0 += blockDim.x) {
-    const int64_t i = t0 + tid;
-    uint64_t inc = i < n ? v[i] : 0ull;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc = sat_add(y, inc);
-    }
-    if (lane == 31) wsum[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-      uint64_t ws = lane < nw ? wsum[lane] : 0ull;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(0xffffffffu, ws, o);
-        if (lane >= o) ws = sat_add(y, ws);
-      }
-      if (lane < nw) wsum[lane] = ws;
-    }
-    __syncthreads();
-    const uint64_t before = sat_add(carry, warp > 0 ? wsum[warp - 1] : 0ull);
-    uint64_t ex = __shfl_up_sync(0xffffffffu, inc, 1);
-    if (lane == 0) ex = 0;
-    if (i < n) v[i] = sat_add(before, ex);
-    const uint64_t tile_total = wsum[nw - 1];
-    __syncthreads();
-    carry = sat_add(carry, tile_total);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -303,8 +268,11 @@ __global__ void k_batch_init(BatchSys* sys, const int32_t* c0, const int64_t* c0
   }
 }
 
-template <int kThreads, bool TC>
-__global__ void __launch_bounds__(kThreads) k_batch_depth(BatchArgs ba) {
+// Tensor-core form: one depth of every system, a system's whole depth by one
+// CTA of four warps (the 128 TMEM lanes of a tile).
+constexpr int kTcThreads = 128;
+__global__ void __launch_bounds__(kTcThreads) k_batch_depth_tc(BatchArgs ba) {
+  constexpr int kThreads = kTcThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned int s_next;
   __shared__ uint64_t s_wsum[kThreads / 32];
@@ -312,35 +280,30 @@ __global__ void __launch_bounds__(kThreads) k_batch_depth(BatchArgs ba) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kThreads / 32;
   BatchScratch sc = batch_scratch(ba.scratch + (size_t)blockIdx.x * ba.scratch_stride, ba.pmax, ba.qc, ba.m_max);
   // tensor-core form: operands in shared memory, 128 TMEM columns, two mbarriers
-  BatchTcSmem tw{};
-  uint32_t tmem = 0, ph_b = 0, ph_m = 0;
-  if constexpr (TC) {
-    tw = batch_tc_smem(smem_raw);
-    if (tid == 0) {
-      t5::bar_init(t5::saddr(tw.bars), 1);
-      t5::bar_init(t5::saddr(tw.bars + 1), 1);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      s_broken = 0;
-    }
-    if (warp == 0) {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t5::saddr(tw.tmem_slot)),
-                   "r"((uint32_t)t5::kT5NC));
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    t5::fence_before_sync();
-    __syncthreads();
-    t5::fence_after_sync();
-    tmem = *tw.tmem_slot;
+  uint32_t ph_b = 0, ph_m = 0;
+  BatchTcSmem tw = batch_tc_smem(smem_raw);
+  if (tid == 0) {
+    t5::bar_init(t5::saddr(tw.bars), 1);
+    t5::bar_init(t5::saddr(tw.bars + 1), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_broken = 0;
   }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t5::saddr(tw.tmem_slot)),
+                 "r"((uint32_t)t5::kT5NC));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  t5::fence_before_sync();
+  __syncthreads();
+  t5::fence_after_sync();
+  const uint32_t tmem = *tw.tmem_slot;
   for (;;) {
     if (tid == 0) s_next = atomicAdd(ba.queue + ba.launch, 1u);
     __syncthreads();
     const int32_t si = (int32_t)s_next;
     __syncthreads();
     if (si >= ba.n) break;
-    if constexpr (TC) {
-      if (s_broken) break;
-    }
+    if (s_broken) break;
     BatchSys* bs = ba.sys + si;
     const int32_t d = bs->cur_depth + 1;
     if (bs->done || d > bs->target_depth) continue;
@@ -386,7 +349,6 @@ __global__ void __launch_bounds__(kThreads) k_batch_depth(BatchArgs ba) {
     int64_t nnew = 0, n_rows = bs->n_rows;
     int32_t chunks = 0;
     bool capped = false;
-    ExpandSmem w = expand_smem(smem_raw + (size_t)warp * ba.warp_smem, m, ba.B, ba.ts);
     if (tid == 0) s_stop = bs->error ? 1u : 0u;
     __syncthreads();
     while (g0 < T && !capped && !s_stop) {
@@ -398,7 +360,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_depth(BatchArgs ba) {
       a.P = P;
       a.g0 = g0;
       a.Q = Q;
-      a.run = (uint32_t)ba.run;
+      a.run = 0;
       a.table = DevTable{bs->slots, bs->bmask};
       a.pool = bs->pool;
       a.staging = sc.staging;
@@ -412,33 +374,26 @@ __global__ void __launch_bounds__(kThreads) k_batch_depth(BatchArgs ba) {
       a.sidx_of = nullptr;
       a.store_cap = 0;
       a.st = sc.st;
-      if constexpr (TC) {
-        if (!batch_tc_rows(a, bs, tw, tmem, sc.hash, sc.red, ph_b, ph_m)) {
-          if (tid == 0) {
-            s_broken = 1;
-            atomicOr(&bs->error, kErrTimeout);
-          }
-          __syncthreads();
-          break;
+      if (!batch_tc_rows(a, bs, tw, tmem, sc.hash, sc.red, ph_b, ph_m)) {
+        if (tid == 0) {
+          s_broken = 1;
+          atomicOr(&bs->error, kErrTimeout);
         }
-        __threadfence();
         __syncthreads();
-        // step (d) for the pass's rows, 32 candidates per warp at a time
-        for (uint32_t b0 = (uint32_t)warp * 32u; b0 < Q; b0 += (uint32_t)nwarps * 32u) {
-          const uint32_t lid = b0 + (uint32_t)lane;
-          const bool todo = lid < Q && !sc.red[lid];
-          const uint64_t key = todo ? mix64(sc.hash[lid]) : 0ull;
-          const int32_t* row = sc.staging + (size_t)(lid < Q ? lid : 0) * m;
-          if ((m & 3) == 0)
-            resolve_warp<RowI32V, 1>(a, row, key, lid, todo);
-          else
-            resolve_warp<RowI32, 1>(a, row, key, lid, todo);
-        }
-      } else {
+        break;
+      }
+      __threadfence();
+      __syncthreads();
+      // step (d) for the pass's rows, 32 candidates per warp at a time
+      for (uint32_t b0 = (uint32_t)warp * 32u; b0 < Q; b0 += (uint32_t)nwarps * 32u) {
+        const uint32_t lid = b0 + (uint32_t)lane;
+        const bool todo = lid < Q && !sc.red[lid];
+        const uint64_t key = todo ? mix64(sc.hash[lid]) : 0ull;
+        const int32_t* row = sc.staging + (size_t)(lid < Q ? lid : 0) * m;
         if ((m & 3) == 0)
-          expand_warp<RowI32V, 1>(a, ba.B, ba.ts, w, warp, nwarps, lane);
+          resolve_warp<RowI32V, 1>(a, row, key, lid, todo);
         else
-          expand_warp<RowI32, 1>(a, ba.B, ba.ts, w, warp, nwarps, lane);
+          resolve_warp<RowI32, 1>(a, row, key, lid, todo);
       }
       __threadfence();
       __syncthreads();
@@ -538,17 +493,13 @@ __global__ void __launch_bounds__(kThreads) k_batch_depth(BatchArgs ba) {
     }
     __syncthreads();
   }
-  if constexpr (TC) {
-    // products of a pass whose wait ran out may still be in flight
-    if (s_broken && tid == 0) (void)t5::bar_wait(t5::saddr(tw.bars + 1), ph_m ^ 1u);
-    t5::fence_before_sync();
-    __syncthreads();
-    if (warp == 0)
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)t5::kT5NC));
-  }
+  // products of a pass whose wait ran out may still be in flight
+  if (s_broken && tid == 0) (void)t5::bar_wait(t5::saddr(tw.bars + 1), ph_m ^ 1u);
+  t5::fence_before_sync();
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)t5::kT5NC));
 }
-
-size_t batch_tc_smem_bytes_host() { return batch_tc_smem_bytes() + 1024; }
 
 size_t batch_scratch_bytes(int64_t pmax, uint32_t qc, int m_max) {
   auto r = [](size_t b) { return (b + 255) & ~size_t(255); };
@@ -557,26 +508,10 @@ size_t batch_scratch_bytes(int64_t pmax, uint32_t qc, int m_max) {
          r(sizeof(ChunkState)) + r((size_t)qc * 8) + r(qc);
 }
 
-size_t expand_smem_bytes(int m_max, int B, int* ts) {
-  *ts = round4(m_max) + 4;
-  return expand_warp_bytes(m_max, B, *ts);
-}
-
-void launch_batch_depth(const BatchArgs& a, int blocks, int warps, cudaStream_t st) {
-  if (a.tc) {  // four warps: the 128 TMEM lanes of a tile
-    const size_t smem = batch_tc_smem_bytes_host();
-    cudaFuncSetAttribute(k_batch_depth<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_batch_depth<128, true><<<blocks, 128, smem, st>>>(a);
-    return;
-  }
-  const size_t smem = a.warp_smem * warps;
-  if (warps == 4) {
-    cudaFuncSetAttribute(k_batch_depth<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_batch_depth<128, false><<<blocks, 128, smem, st>>>(a);
-  } else {
-    cudaFuncSetAttribute(k_batch_depth<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_batch_depth<256, false><<<blocks, 256, smem, st>>>(a);
-  }
+void launch_batch_depth_tc(const BatchArgs& a, int blocks, cudaStream_t st) {
+  const size_t smem = batch_tc_smem_bytes() + 1024;
+  cudaFuncSetAttribute(k_batch_depth_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_batch_depth_tc<<<blocks, kTcThreads, smem, st>>>(a);
 }
 
 }  // namespace snp

@@ -323,8 +323,18 @@ __device__ __forceinline__ uint64_t appl(const DevSys& s, int n, int32_t x) {
   return (uint64_t)e.mask | ((uint64_t)e.keep << 32);
 }
 
+static __device__ __noinline__ uint64_t appl_folded(const DevSys& s, int n, int32_t x) { return appl(s, n, x); }
+
+// Applicable rules of neuron n with x spikes: one lookup in the direct table,
+// counts beyond it (rare) out of line.
+__device__ __forceinline__ uint32_t appl_mask(const DevSys& s, int n, int32_t x) {
+  if ((uint32_t)x < (uint32_t)kDirect) return __ldg(s.dmask + (size_t)n * kDirect + (uint32_t)x);
+  return (uint32_t)appl_folded(s, n, x);
+}
+
 // Position of the d-th set bit (0-based) of mask.
 __device__ __forceinline__ int nth_set_bit(uint32_t mask, int d) {
+#pragma unroll 1
   for (int k = 0; k < d; ++k) mask &= mask - 1;
   return __ffs(mask) - 1;
 }
@@ -397,18 +407,17 @@ __device__ __forceinline__ void load_parent(const DevSys& s, const int32_t* __re
   __syncwarp();
 }
 
+// q / radix; the remainder is the digit (out of line: indices beyond 32 bits
+// are rare, and the 64-bit division is long).
+static __device__ __noinline__ uint64_t next_digit_wide(uint64_t q, uint32_t radix) { return q / radix; }
+
 // Mixed-radix digit of a neuron with `radix` choices; q moves to the next
 // more significant neuron.
 __device__ __forceinline__ uint32_t next_digit(uint64_t& q, uint32_t radix) {
   if (radix <= 1) return 0;
-  if ((q >> 32) == 0) {
-    const uint32_t q32 = (uint32_t)q;
-    q = q32 / radix;
-    return q32 % radix;
-  }
-  const uint32_t d = (uint32_t)(q % radix);
-  q /= radix;
-  return d;
+  const uint64_t q0 = q;
+  q = (q >> 32) == 0 ? (uint64_t)((uint32_t)q / radix) : next_digit_wide(q, radix);
+  return (uint32_t)q0 - (uint32_t)q * radix;
 }
 
 // row += M[rn] - M[ro] for two rules of one neuron, by the whole warp: the
@@ -485,6 +494,140 @@ __device__ __forceinline__ bool rows_equal(const int32_t* buf, const int32_t* ot
   bool ok = true;
   for (int n = lane; n < m; n += 32) ok &= (__ldcg(other + n) == buf[n]);
   return __all_sync(0xffffffffu, ok);
+}
+
+// Step (a) for one configuration, neuron by neuron: Psi = prod max(1, omega)
+// (saturating; four counts are multiplied in 32 bits, at most 2^20, and a
+// product below 2^43 cannot overflow by such a factor), whether
+// a child could leave int32, whether the row is past max_expand, and its
+// ParentRec (base-child hash, multi-choice neurons in neuron order).
+struct PsiAcc {
+  uint64_t prod = 1, hb = 0;
+  uint32_t nnt = 0, part = 1;
+  int parts = 0;
+  bool ov = false, skip = false;
+
+  // prod *= part (saturating; part <= 2^20)
+  __device__ __forceinline__ void flush() {
+    if (part > 1) prod = (prod >> 43) ? (__umul64hi(prod, part) ? kSat : prod * part) : prod * part;
+    part = 1;
+    parts = 0;
+  }
+
+  // One neuron: its applicable mask and, with records, its share of the base
+  // child's hash.
+  template <bool REC>
+  __device__ __forceinline__ void add(int n, int32_t x, uint32_t mask, uint64_t hx, int32_t max_expand,
+                                      ParentRec* rec) {
+    const uint32_t cnt = __popc(mask);
+    part *= cnt > 1 ? cnt : 1u;  // four counts of at most 32 fit 32 bits
+    if (++parts == 4) flush();
+    skip |= max_expand >= 0 && x > max_expand;
+    if (REC) {
+      hb += hx;
+      if (cnt > 1) {
+        const bool fits = nnt < (uint32_t)kRecNt && n < 65536 && mask < 65536u;
+        if (fits) rec->nt[nnt] = ((uint32_t)n << 16) | mask;
+        nnt = fits ? nnt + 1 : kRecFull;
+      }
+    }
+  }
+
+  template <bool REC>
+  __device__ __forceinline__ void visit(const DevSys& s, int n, int32_t x, int32_t max_expand, ParentRec* rec) {
+    uint32_t mask;
+    uint64_t hx = 0;
+    if ((uint32_t)x < (uint32_t)kDirect) {  // small count: one entry of the direct table
+      const size_t k = (size_t)n * kDirect + (uint32_t)x;
+      mask = __ldg(s.dmask + k);
+      if (REC) hx = __ldg(s.dhx + k);
+      if (!s.gain_small) ov |= x > INT32_MAX - __ldg(s.gain + n);
+    } else {
+      const NeuronInfo ni = neuron_info(s, n);
+      const ApplEntry e = appl_entry(s, ni, n, x);
+      mask = e.mask;
+      if (REC) hx = (uint64_t)(uint32_t)x * ni.colkey + e.hfirst;
+      ov |= x > INT32_MAX - ni.gain;
+    }
+    add<REC>(n, x, mask, hx, max_expand, rec);
+  }
+
+  // Neurons n .. n + w - 1 holding x[0 .. w): eight lookups in flight where
+  // their counts are in the direct table (a lookup at a time, each visit
+  // waited out an L2 round trip).
+  template <bool REC>
+  __device__ __forceinline__ void visit_run(const DevSys& s, int n, const int32_t* x, int w, int32_t max_expand,
+                                            ParentRec* rec) {
+    constexpr int U = 8;
+    int j = 0;
+#pragma unroll 1
+    for (; j + U <= w; j += U) {
+      int32_t v[U];
+      uint32_t any = 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        v[u] = x[j + u];
+        any |= (uint32_t)v[u];
+      }
+      if (any < (uint32_t)kDirect && s.gain_small) {
+        uint32_t mask[U];
+        uint64_t hx[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const size_t k = (size_t)(n + j + u) * kDirect + (uint32_t)v[u];
+          mask[u] = __ldg(s.dmask + k);
+          hx[u] = REC ? __ldg(s.dhx + k) : 0ull;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) add<REC>(n + j + u, v[u], mask[u], hx[u], max_expand, rec);
+      } else {
+#pragma unroll 1
+        for (int u = 0; u < U; ++u) visit<REC>(s, n + j + u, x[j + u], max_expand, rec);
+      }
+    }
+#pragma unroll 1
+    for (; j < w; ++j) visit<REC>(s, n + j, x[j], max_expand, rec);
+  }
+
+  __device__ __forceinline__ uint64_t psi() {
+    flush();
+    return skip ? 0ull : prod;
+  }
+  __device__ __forceinline__ bool overflow() const { return ov && !skip; }
+};
+
+// Block-wide exclusive scan of v[0..n) in place (saturating u64), in tiles of blockDim.x.
+static __device__ void block_scan_sat(uint64_t* v, int64_t n, uint64_t* wsum) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  uint64_t carry = 0;
+  for (int64_t t0 = 0; t0 < n; t0 += blockDim.x) {
+    const int64_t i = t0 + tid;
+    uint64_t inc = i < n ? v[i] : 0ull;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc = sat_add(y, inc);
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+      uint64_t ws = lane < nw ? wsum[lane] : 0ull;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xffffffffu, ws, o);
+        if (lane >= o) ws = sat_add(y, ws);
+      }
+      if (lane < nw) wsum[lane] = ws;
+    }
+    __syncthreads();
+    const uint64_t before = sat_add(carry, warp > 0 ? wsum[warp - 1] : 0ull);
+    uint64_t ex = __shfl_up_sync(0xffffffffu, inc, 1);
+    if (lane == 0) ex = 0;
+    if (i < n) v[i] = sat_add(before, ex);
+    const uint64_t tile_total = wsum[nw - 1];
+    __syncthreads();
+    carry = sat_add(carry, tile_total);
+  }
 }
 
 }  // namespace snp

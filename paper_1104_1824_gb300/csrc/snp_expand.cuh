@@ -164,8 +164,9 @@ __device__ __forceinline__ uint64_t parent_state(const DevSys& s, const T* __res
   __syncwarp();
   uint64_t prod = 1;
   const int n0 = lane * s.K, n1 = min(n0 + s.K, s.m);
+#pragma unroll 1
   for (int n = n0; n < n1; ++n) {
-    const uint32_t mask = (uint32_t)appl(s, n, w.par ? w.par[n] : (int32_t)row[n]);
+    const uint32_t mask = appl_mask(s, n, w.par ? w.par[n] : (int32_t)row[n]);
     w.msk[n] = mask;
     prod = sat_mul(prod, mask ? (uint64_t)__popc(mask) : 1ull);
   }
@@ -178,6 +179,7 @@ __device__ __forceinline__ uint64_t parent_state(const DevSys& s, const T* __res
   const uint64_t a = __shfl_down_sync(0xffffffffu, v, 1);
   __syncwarp();
   int count = 0;
+#pragma unroll 1
   for (int top = s.m - 1; top >= 0; top -= 32) {
     const int n = top - lane;
     const bool nt = n >= 0 && __popc(w.msk[n]) > 1;
@@ -215,22 +217,14 @@ __device__ __forceinline__ void decode_full(const DevSys& s, ExpandSmem& w, uint
   const int n0 = lane * s.K, n1 = min(n0 + s.K, s.m);
   uint64_t q = (after > t) ? 0ull : t / after;
   int red = 0;
+#pragma unroll 1
   for (int n = n1 - 1; n >= n0; --n) {
     const uint32_t mask = w.msk[n];
     if (!mask) {
       w.dig[n] = 0;
       continue;
     }
-    const uint32_t radix = __popc(mask);
-    uint32_t d;
-    if ((q >> 32) == 0) {
-      const uint32_t q32 = (uint32_t)q;
-      d = q32 % radix;
-      q = q32 / radix;
-    } else {
-      d = (uint32_t)(q % radix);
-      q /= radix;
-    }
+    const uint32_t d = next_digit(q, __popc(mask));
     w.dig[n] = (uint8_t)d;
     const int r = __ldg(s.first_rule + n) + nth_set_bit(mask, (int)d);
     if (WIDE) {  // long rows of M_Pi: eight loads in flight before their adds
@@ -514,14 +508,14 @@ __device__ __forceinline__ int4 load4(const typename RF::T* row, int j) {
 template <class RF, typename F>
 __device__ __forceinline__ void for_each_neuron_desc(const typename RF::T* row, int m, F&& f) {
   if constexpr (RF::VEC) {
+#pragma unroll 1
     for (int n4 = (m >> 2) - 1; n4 >= 0; --n4) {
       const int4 v = load4<RF>(row, n4);
-      f(4 * n4 + 3, v.w);
-      f(4 * n4 + 2, v.z);
-      f(4 * n4 + 1, v.y);
-      f(4 * n4, v.x);
+#pragma unroll 1
+      for (int k = 3; k >= 0; --k) f(4 * n4 + k, k == 3 ? v.w : k == 2 ? v.z : k == 1 ? v.y : v.x);
     }
   } else {
+#pragma unroll 1
     for (int n = m - 1; n >= 0; --n) f(n, (int32_t)row[n]);
   }
 }
@@ -587,6 +581,7 @@ __device__ __forceinline__ int flat_decode(const ClaimArgs& a, uint64_t g, int n
   }
   if (nnt != kRecFull) {
     uint64_t h = f.h;
+#pragma unroll 1
     for (int i = (int)nnt - 1; i >= 0; --i) {
       const uint32_t e = __ldcg(rec->nt + i);
       const uint32_t mask = e & 0xFFFFu;
@@ -602,7 +597,7 @@ __device__ __forceinline__ int flat_decode(const ClaimArgs& a, uint64_t g, int n
     uint64_t h = 0;
     for_each_neuron_desc<RF>(parent_row<RF>(a, f.pc), s.m, [&](int n, int32_t x) {
       h += col_hash(s, n, x);
-      const uint64_t am = appl(s, n, x);
+      const uint64_t am = appl_folded(s, n, x);
       const uint32_t mask = (uint32_t)am;
       if (!mask) return;
       const int kb = nth_set_bit(mask, (int)next_digit(q, __popc(mask)));
@@ -624,7 +619,7 @@ __device__ __forceinline__ void flat_build(const ClaimArgs& a, int64_t pc, uint6
   load_row<RF>(prow, trow, s.m);
   uint64_t q = t;
   for_each_neuron_desc<RF>(prow, s.m, [&](int n, int32_t x) {
-    const uint32_t mask = (uint32_t)appl(s, n, x);
+    const uint32_t mask = appl_mask(s, n, x);
     if (!mask) return;
     const int kb = nth_set_bit(mask, (int)next_digit(q, __popc(mask)));
     add_rule<KIND>(s, trow, __ldg(s.first_rule + n) + kb);
@@ -706,6 +701,7 @@ __device__ __forceinline__ void build_block_row(const DevSys& s, ExpandSmem& w, 
   }
   cur = pk;
   const bool tab = w.hdr[kLowOk] != 0;
+#pragma unroll 1
   for (int i = 0; i < nlow; ++i) {
     const uint32_t d0 = (from >> (5 * i)) & 31u, d = (pk >> (5 * i)) & 31u;
     if (d == d0) continue;
@@ -744,6 +740,7 @@ __device__ __forceinline__ void build_low_table(const DevSys& s, ExpandSmem& w, 
   const int nlow = w.hdr[kNlow];
   if (lane < w.hdr[kRL]) {  // RL <= 32 with every radix >= 2: at most 5 low neurons, digits < 32
     uint32_t q = (uint32_t)lane, pk = 0;
+#pragma unroll 1
     for (int i = 0; i < nlow; ++i) {
       const uint32_t radix = __popc(w.msk[w.ntl[i]]);
       pk |= (q % radix) << (5 * i);
@@ -753,6 +750,7 @@ __device__ __forceinline__ void build_low_table(const DevSys& s, ExpandSmem& w, 
   }
   int at = 0;
   bool fits = true;
+#pragma unroll 1
   for (int i = 0; fits && i < nlow; ++i) {
     const int n = w.ntl[i];
     const int radix = __popc(w.msk[n]);
@@ -764,6 +762,7 @@ __device__ __forceinline__ void build_low_table(const DevSys& s, ExpandSmem& w, 
     }
     int32_t* t = w.low + kLowHdr + at;
     for (int k = lane; k < len; k += 32) t[k] = __ldg(s.scol + d0.x + k);
+#pragma unroll 1
     for (int d = 1; d < radix; ++d) {
       const int vz = __ldg(&s.rdesc[rule_of(s, w, n, d)].z);
       for (int k = lane; k < len; k += 32) t[d * len + k] = __ldg(s.rval + vz + k) - __ldg(s.rval + d0.z + k);
@@ -784,15 +783,16 @@ __device__ __forceinline__ void build_low_table(const DevSys& s, ExpandSmem& w, 
 // place value is the product of the choice counts of the later lanes' neurons
 // (last neuron least significant), and adds its chosen rules' rows.
 template <class RF>
-__device__ __forceinline__ void build_flat_row(const ClaimArgs& a, int32_t* row, int64_t pc, uint64_t t, int lane) {
+__device__ __noinline__ void build_flat_row(const ClaimArgs& a, int32_t* row, int64_t pc, uint64_t t, int lane) {
   const DevSys& s = a.sys;
   const typename RF::T* prow = parent_row<RF>(a, pc);
   __syncwarp();
   for (int n = lane; n < s.m; n += 32) row[n] = prow[n];
   const int n0 = lane * s.K, n1 = min(n0 + s.K, s.m);
   uint64_t prod = 1;
+#pragma unroll 1
   for (int n = n0; n < n1; ++n) {
-    const uint32_t mask = (uint32_t)appl(s, n, prow[n]);
+    const uint32_t mask = appl_mask(s, n, prow[n]);
     prod = sat_mul(prod, mask ? (uint64_t)__popc(mask) : 1ull);
   }
   uint64_t v = prod;
@@ -805,8 +805,9 @@ __device__ __forceinline__ void build_flat_row(const ClaimArgs& a, int32_t* row,
   const uint64_t after = lane == 31 ? 1ull : nxt;
   __syncwarp();
   uint64_t q = (after > t) ? 0ull : t / after;
+#pragma unroll 1
   for (int n = n1 - 1; n >= n0; --n) {
-    const uint32_t mask = (uint32_t)appl(s, n, prow[n]);
+    const uint32_t mask = appl_mask(s, n, prow[n]);
     if (!mask) continue;
     const int kb = nth_set_bit(mask, (int)next_digit(q, __popc(mask)));
     add_row_shared(s, row, __ldg(s.first_rule + n) + kb, 1);
@@ -1058,10 +1059,13 @@ __device__ __forceinline__ void resolve_warp_wide(const ClaimArgs& a, int32_t* s
 
 // Resolves the queued crossing-batch candidates in the wide mode.
 template <class RF>
-__device__ __forceinline__ void flush_queue_wide(const ClaimArgs& a, ExpandSmem& w, int fill, int lane) {
+__device__ __noinline__ void flush_queue_wide(const ClaimArgs& a, int32_t* scratch, const unsigned long long* keys,
+                                              const long long* dpc, const unsigned long long* dt,
+                                              const uint32_t* lids, int fill) {
+  const int lane = threadIdx.x & 31;
   const bool mine = lane < fill;
-  resolve_warp_wide<RF>(a, w.tile, mine ? w.keys[lane] : 0ull, mine ? w.lids[lane] : 0u, mine, lane,
-                        [&](int L) { build_flat_row<RF>(a, w.tile, w.dpc[L], w.dt[L], lane); });
+  resolve_warp_wide<RF>(a, scratch, mine ? keys[lane] : 0ull, mine ? lids[lane] : 0u, mine, lane,
+                        [&](int L) { build_flat_row<RF>(a, scratch, dpc[L], dt[L], lane); });
 }
 
 // Base children (every firing neuron on its first applicable rule) of the
@@ -1092,6 +1096,7 @@ __device__ __forceinline__ void decode_from_base(const DevSys& s, ExpandSmem& w,
   uint64_t h = hbase, q = t;
   int red = 0;
   const int nnt = w.hdr[kNnt];
+#pragma unroll 1
   for (int i = 0; i < nnt && q != 0; ++i) {
     const int n = w.ntl[i];
     const uint32_t mask = w.msk[n];
@@ -1146,6 +1151,7 @@ __device__ __forceinline__ uint64_t block_run_wide(const ClaimArgs& a, ExpandSme
   if (lane < RL) {
     redk = false;
     uint32_t q = (uint32_t)lane;
+#pragma unroll 1
     for (int i = 0; i < nlow; ++i) {
       const int n = w.ntl[i];
       const uint32_t mask = w.msk[n];
@@ -1170,6 +1176,7 @@ __device__ __forceinline__ uint64_t block_run_wide(const ClaimArgs& a, ExpandSme
     // next block: the odometer, every lane following the same digits
     uint64_t h = hbase_of(w);
     int red = w.hdr[kNred];
+#pragma unroll 1
     for (int i = nlow; i < nnt; ++i) {
       const int n = w.ntl[i];
       const uint32_t mask = w.msk[n];
@@ -1192,13 +1199,19 @@ __device__ __forceinline__ uint64_t block_run_wide(const ClaimArgs& a, ExpandSme
   return gend - a.g0;
 }
 
-// Resolves the queued rows of crossing batches (building them first).
+// Resolves the queued rows of crossing batches (building them first).  Out of
+// line, as flush_queue_wide: the expand loop has two places that flush, and
+// a copy of the row builder in each made the kernel outgrow the instruction
+// cache.
 template <class RF, int KIND>
-__device__ __forceinline__ void flush_queue(const ClaimArgs& a, ExpandSmem& w, int ts, int fill, int lane) {
+__device__ __noinline__ void flush_queue(const ClaimArgs& a, int32_t* tile, const unsigned long long* keys,
+                                         const long long* dpc, const unsigned long long* dt, const uint32_t* lids,
+                                         int ts, int fill) {
+  const int lane = threadIdx.x & 31;
   const bool mine = lane < fill;
-  if (mine && w.dpc[lane] >= 0) flat_build<RF, KIND>(a, w.dpc[lane], w.dt[lane], w.tile + lane * ts);
+  if (mine && dpc[lane] >= 0) flat_build<RF, KIND>(a, dpc[lane], dt[lane], tile + lane * ts);
   __syncwarp();
-  resolve_warp<RF, KIND>(a, w.tile + lane * ts, mine ? w.keys[lane] : 0ull, mine ? w.lids[lane] : 0u, mine);
+  resolve_warp<RF, KIND>(a, tile + lane * ts, mine ? keys[lane] : 0ull, mine ? lids[lane] : 0u, mine);
 }
 
 // Block mode for parent p from candidate a.g0 + l to the end of the parent or
@@ -1226,6 +1239,7 @@ __device__ __forceinline__ uint64_t block_run(const ClaimArgs& a, ExpandSmem& w,
     copy_row<RF::VEC>(w.buf, row, m);
     redk = false;
     uint32_t q = (uint32_t)lane;
+#pragma unroll 1
     for (int i = 0; i < nlow; ++i) {
       const int n = w.ntl[i];
       const uint32_t mask = w.msk[n];
@@ -1250,7 +1264,8 @@ __device__ __forceinline__ uint64_t block_run(const ClaimArgs& a, ExpandSmem& w,
     if (lane == 0) {
       uint64_t h = hbase_of(w);
       int red = w.hdr[kNred], nc = 0;
-      for (int i = nlow; i < nnt; ++i) {
+  #pragma unroll 1
+    for (int i = nlow; i < nnt; ++i) {
         const int n = w.ntl[i];
         const uint32_t mask = w.msk[n];
         const int d = w.dig[n];
@@ -1281,100 +1296,110 @@ __device__ __forceinline__ uint64_t block_run(const ClaimArgs& a, ExpandSmem& w,
 template <class RF, int KIND>
 __device__ __forceinline__ void flush_any(const ClaimArgs& a, ExpandSmem& w, int ts, int fill, int lane) {
   if constexpr (KIND == kWide)
-    flush_queue_wide<RF>(a, w, fill, lane);
+    flush_queue_wide<RF>(a, w.tile, w.keys, w.dpc, w.dt, w.lids, fill);
   else
-    flush_queue<RF, KIND>(a, w, ts, fill, lane);
+    flush_queue<RF, KIND>(a, w.tile, w.keys, w.dpc, w.dt, w.lids, ts, fill);
 }
 
-// Steps (b)-(d) for the tasks task0, task0 + tstride, ... of chunk a (a task
-// is a run of a.run consecutive candidates), by one warp: block mode while
-// the parent has 32 or more candidates left, else crossing batches.
-template <class RF, int KIND>
-__device__ __forceinline__ void expand_warp(const ClaimArgs& a, int B, int ts, ExpandSmem& w, uint64_t task0,
-                                            uint64_t tstride, int lane) {
-  const uint64_t ntasks = ((uint64_t)a.Q + a.run - 1) / a.run;
+// What a warp keeps from one task of a chunk to the next.
+struct WarpTask {
   int64_t p = -1;         // parent of the previous task's last candidate
   int64_t cached_p = -1;  // parent whose state the warp's shared memory holds
   uint64_t after = 0;     // its per-lane place values
-  for (uint64_t task = task0; task < ntasks; task += tstride) {
-    const uint64_t la = task * a.run;
-    const uint64_t lb = min(la + a.run, (uint64_t)a.Q);
-    {
-      // tasks come in increasing order: look among the 32 parents from the
-      // previous one first (off is sorted), else search all of them
-      const uint64_t g = a.g0 + la;
-      int k = 32;
-      if (p >= 0) {
-        const int64_t pj = p + 1 + lane;
-        k = __popc(__ballot_sync(0xffffffffu, pj <= a.P && __ldcg(a.off + pj) <= g));
-      }
-      p = k < 32 ? p + k : warp_find_parent(a.off, a.P, g, lane);
+};
+
+// Steps (b)-(d) for candidates [la, lb) of chunk a, by one warp: block mode
+// while the parent has 32 or more candidates left, else crossing batches.  A
+// warp takes the tasks of a chunk in increasing order.
+template <class RF, int KIND>
+__device__ __forceinline__ void expand_task(const ClaimArgs& a, int B, int ts, ExpandSmem& w, uint64_t la, uint64_t lb,
+                                            WarpTask& k, int lane) {
+  int64_t p = k.p;
+  {
+    // tasks come in increasing order: look among the 32 parents from the
+    // previous one first (off is sorted), else search all of them
+    const uint64_t g = a.g0 + la;
+    int n = 32;
+    if (p >= 0) {
+      const int64_t pj = p + 1 + lane;
+      n = __popc(__ballot_sync(0xffffffffu, pj <= a.P && __ldcg(a.off + pj) <= g));
     }
-    uint64_t p_lo = __ldcg(a.off + p), p_hi = __ldcg(a.off + p + 1);
-    if (task == 0 && lane == 0) a.st->p_first = (unsigned long long)p;
-    uint64_t l = la;
-    int fill = 0;  // rows queued by crossing batches
-    for (;;) {
-      const bool done = l >= lb;
-      const uint64_t g = a.g0 + l;
-      if (done || p_hi - g >= 32) {
-        if (fill > 0) {  // the tile is about to be reused, or the task ends
-          flush_any<RF, KIND>(a, w, ts, fill, lane);
-          fill = 0;
-        }
-        if (done) break;
-        if constexpr (KIND == kWide)
-          l = block_run_wide<RF>(a, w, p, p_lo, p_hi, l, lb, cached_p, after, lane);
-        else
-          l = block_run<RF, KIND>(a, w, B, ts, p, p_lo, p_hi, l, lb, cached_p, after, lane);
-        const uint64_t gn = a.g0 + l;
-        if (l < lb) {
-          do {
-            ++p;
-            p_lo = p_hi;
-            p_hi = __ldcg(a.off + p + 1);
-          } while (gn >= p_hi);
-        }
-        continue;
-      }
-      // crossing batch
-      FlatLane f;
-      bool keep = false;
-      const int nb = flat_decode<RF>(a, g, (int)min((uint64_t)B, lb - l), p, p_lo, lane, f, keep);
-      const uint32_t kept = __ballot_sync(0xffffffffu, keep);
-      if (fill + __popc(kept) > B) {
+    p = n < 32 ? p + n : warp_find_parent(a.off, a.P, g, lane);
+  }
+  uint64_t p_lo = __ldcg(a.off + p), p_hi = __ldcg(a.off + p + 1);
+  if (la == 0 && lane == 0) a.st->p_first = (unsigned long long)p;
+  uint64_t l = la;
+  int fill = 0;  // rows queued by crossing batches
+  for (;;) {
+    const bool done = l >= lb;
+    const uint64_t g = a.g0 + l;
+    if (done || p_hi - g >= 32) {
+      if (fill > 0) {  // the tile is about to be reused, or the task ends
         flush_any<RF, KIND>(a, w, ts, fill, lane);
         fill = 0;
       }
-      if (keep) {
-        const int slot = fill + __popc(kept & ((1u << lane) - 1u));
-        w.dpc[slot] = f.pc;
-        w.dt[slot] = f.t;
-        w.keys[slot] = mix64(f.h);
-        w.lids[slot] = (uint32_t)(l + lane);
-      }
-      fill += __popc(kept);
-      __syncwarp();
-      l += (uint64_t)nb;
-      if (l >= lb) {  // keep the parent of the task's last candidate
-        p = __shfl_sync(0xffffffffu, f.pc, nb - 1);
-        continue;
-      }
+      if (done) break;
+      if constexpr (KIND == kWide)
+        l = block_run_wide<RF>(a, w, p, p_lo, p_hi, l, lb, k.cached_p, k.after, lane);
+      else
+        l = block_run<RF, KIND>(a, w, B, ts, p, p_lo, p_hi, l, lb, k.cached_p, k.after, lane);
       const uint64_t gn = a.g0 + l;
-      const int kn = __popc(__ballot_sync(0xffffffffu, f.o <= gn));  // parents ending at or before gn
-      if (kn < 32) {
-        const uint64_t lo = __shfl_sync(0xffffffffu, f.o, kn > 0 ? kn - 1 : 0);
-        p_hi = __shfl_sync(0xffffffffu, f.o, kn);
-        if (kn > 0) p_lo = lo;
-        p += kn;
-      } else {
-        p = warp_find_parent(a.off, a.P, gn, lane);
-        p_lo = __ldcg(a.off + p);
-        p_hi = __ldcg(a.off + p + 1);
+      if (l < lb) {
+        do {
+          ++p;
+          p_lo = p_hi;
+          p_hi = __ldcg(a.off + p + 1);
+        } while (gn >= p_hi);
       }
+      continue;
     }
-    if (task + 1 == ntasks && lane == 0) a.st->p_last = (unsigned long long)p;
+    // crossing batch
+    FlatLane f;
+    bool keep = false;
+    const int nb = flat_decode<RF>(a, g, (int)min((uint64_t)B, lb - l), p, p_lo, lane, f, keep);
+    const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+    if (fill + __popc(kept) > B) {
+      flush_any<RF, KIND>(a, w, ts, fill, lane);
+      fill = 0;
+    }
+    if (keep) {
+      const int slot = fill + __popc(kept & ((1u << lane) - 1u));
+      w.dpc[slot] = f.pc;
+      w.dt[slot] = f.t;
+      w.keys[slot] = mix64(f.h);
+      w.lids[slot] = (uint32_t)(l + lane);
+    }
+    fill += __popc(kept);
+    __syncwarp();
+    l += (uint64_t)nb;
+    if (l >= lb) {  // keep the parent of the task's last candidate
+      p = __shfl_sync(0xffffffffu, f.pc, nb - 1);
+      continue;
+    }
+    const uint64_t gn = a.g0 + l;
+    const int kn = __popc(__ballot_sync(0xffffffffu, f.o <= gn));  // parents ending at or before gn
+    if (kn < 32) {
+      const uint64_t lo = __shfl_sync(0xffffffffu, f.o, kn > 0 ? kn - 1 : 0);
+      p_hi = __shfl_sync(0xffffffffu, f.o, kn);
+      if (kn > 0) p_lo = lo;
+      p += kn;
+    } else {
+      p = warp_find_parent(a.off, a.P, gn, lane);
+      p_lo = __ldcg(a.off + p);
+      p_hi = __ldcg(a.off + p + 1);
+    }
   }
+  if (lb == (uint64_t)a.Q && lane == 0) a.st->p_last = (unsigned long long)p;
+  k.p = p;
+}
+
+// The tasks task0, task0 + tstride, ... of chunk a (runs of a.run candidates).
+template <class RF, int KIND>
+__device__ __forceinline__ void expand_warp(const ClaimArgs& a, int B, int ts, ExpandSmem& w, uint64_t task0,
+                                            uint64_t tstride, int lane) {
+  WarpTask k;
+  for (uint64_t la = task0 * a.run; la < a.Q; la += tstride * a.run)
+    expand_task<RF, KIND>(a, B, ts, w, la, min(la + a.run, (uint64_t)a.Q), k, lane);
 }
 
 }  // namespace

@@ -34,60 +34,6 @@ __device__ __forceinline__ void set_error(ChunkState* st, uint32_t bits) { atomi
 
 }  // namespace
 
-// Step (a) for one configuration, neuron by neuron: Psi = prod max(1, omega)
-// (saturating; four counts are multiplied in 32 bits, at most 2^20, and a
-// product below 2^43 cannot overflow by such a factor), whether
-// a child could leave int32, whether the row is past max_expand, and its
-// ParentRec (base-child hash, multi-choice neurons in neuron order).
-struct PsiAcc {
-  uint64_t prod = 1, hb = 0;
-  uint32_t nnt = 0, part = 1;
-  int parts = 0;
-  bool ov = false, skip = false;
-
-  // prod *= part (saturating; part <= 2^20)
-  __device__ __forceinline__ void flush() {
-    if (part > 1) prod = (prod >> 43) ? (__umul64hi(prod, part) ? kSat : prod * part) : prod * part;
-    part = 1;
-    parts = 0;
-  }
-
-  template <bool REC>
-  __device__ __forceinline__ void visit(const DevSys& s, int n, int32_t x, int32_t max_expand, ParentRec* rec) {
-    uint32_t mask;
-    uint64_t hx = 0;
-    if ((uint32_t)x < (uint32_t)kDirect) {  // small count: one entry of the direct table
-      const size_t k = (size_t)n * kDirect + (uint32_t)x;
-      mask = __ldg(s.dmask + k);
-      if (REC) hx = __ldg(s.dhx + k);
-      if (!s.gain_small) ov |= x > INT32_MAX - __ldg(s.gain + n);
-    } else {
-      const NeuronInfo ni = neuron_info(s, n);
-      const ApplEntry e = appl_entry(s, ni, n, x);
-      mask = e.mask;
-      if (REC) hx = (uint64_t)(uint32_t)x * ni.colkey + e.hfirst;
-      ov |= x > INT32_MAX - ni.gain;
-    }
-    const uint32_t cnt = __popc(mask);
-    part *= cnt > 1 ? cnt : 1u;  // four counts of at most 32 fit 32 bits
-    if (++parts == 4) flush();
-    skip |= max_expand >= 0 && x > max_expand;
-    if (REC) {
-      hb += hx;
-      if (cnt > 1) {
-        const bool fits = nnt < (uint32_t)kRecNt && n < 65536 && mask < 65536u;
-        if (fits) rec->nt[nnt] = ((uint32_t)n << 16) | mask;
-        nnt = fits ? nnt + 1 : kRecFull;
-      }
-    }
-  }
-  __device__ __forceinline__ uint64_t psi() {
-    flush();
-    return skip ? 0ull : prod;
-  }
-  __device__ __forceinline__ bool overflow() const { return ov && !skip; }
-};
-
 // Step (a) and Eq. psi for every frontier row, one lane per row, with the
 // rows' ParentRecs when rec is given; rows not to be expanded (max_expand)
 // get Psi = 0, rows whose children could leave int32 raise kErrOverflow.

@@ -77,9 +77,12 @@ struct CommitArgs {
 };
 
 // ---------------------------------------------------------------------------
-// Batch engine: many independent systems advance one depth per launch.
+// Batch engine and serving loop: many independent systems advance together.
 
-// One system of a batch (device memory; updated by the batch kernel).
+// What a system of the sparse form does next (snp_many.cu).
+constexpr int32_t kPhaseIdle = 0, kPhasePsi = 1, kPhaseExpand = 2;
+
+// One system of a batch (device memory; updated by the batch kernels).
 struct BatchSys {
   DevSys sys;
   int32_t* pool;               // configurations, discovery order, pool_rows rows
@@ -99,7 +102,64 @@ struct BatchSys {
   // fp8 tensor-core form: M_Pi^T in e4m3 (tc5_pack_mt layout), columns rounded to 16, rule blocks
   const uint8_t* MB;
   int32_t np, nblocks;
+  // Sparse form (snp_many.cu): the pass's arguments for the expand code (its
+  // scratch among them), and where the depth stands.
+  ClaimArgs a;
+  uint64_t* off;               // [cap + 1] Psi, then its saturating exclusive scan
+  ParentRec* rec;              // [cap]
+  uint32_t* srow;              // [qc] owner of each first occurrence
+  uint32_t* order;             // [qc] owners in rank order
+  int32_t phase, tile;         // kPhase*; rows of the expand tile (narrow rows)
+  uint32_t qc;                 // largest pass the scratch holds
+  uint32_t overshoot;          // claims past the cap that the table has room for, per depth
+  int32_t fixed_q;             // 1: passes of qc candidates whatever the cap still takes (the caller's pass size)
+  int32_t chunks;
+  uint32_t copy_n, copy_acc;   // first occurrences of the last pass; the accepted ones (ranks 0 .. copy_acc - 1)
+  int64_t copy_row0;           // pool row of rank 0
+  uint64_t total, T;           // candidates of the depth; those within the budget
+  uint64_t remaining, examined, tombs;
+  int64_t nnew;
+  float rate;                  // first occurrences per candidate of the last pass
 };
+
+// Work items {system, first element} of one iteration of the sparse form.
+struct ManyQueue {
+  int2* expand[2];             // runs of a.run candidates: this iteration's and the next one's; kMqForms regions of `cap`
+  int2* copy;                  // 32 first occurrences each
+  int2* psi;                   // 32 frontier rows each
+  uint32_t* ctr;               // counters, kMq*
+  int64_t cap;                 // items of one region
+};
+// Systems by the form of the expand code they take (rows within or beyond
+// kWideM neurons, of whole 16-byte units or not): items of one form together.
+constexpr int kMqForms = 4;
+enum { kMqExpand = 0, kMqHead = 2 * kMqForms, kMqCopy = 4 * kMqForms, kMqPsi, kMqActive, kMqCounters = 20 };
+
+// Shape of the sparse form's expand launch.
+struct ManyPlan {
+  size_t warp_bytes = 0;       // shared memory per warp
+  int warps = 8, ctas_per_sm = 2;
+};
+// Plan for systems of these neuron counts; tile, warps: the caller's settings
+// (<= 0: automatic).  many_tile: rows of the expand tile for m neurons.
+ManyPlan many_plan(const int32_t* ms, int64_t n, int tile, int warps);
+int many_tile(const ManyPlan& p, int m, int tile);
+// Candidates per pass for a frontier cap when the caller sets none.
+uint32_t many_default_qc(int64_t cap);
+// Scratch of one system: size, and its pointers (and pass arguments) in b,
+// whose sys, pool, slots, bmask and cap are set.
+size_t many_scratch_bytes(int64_t cap, uint32_t qc, int m);
+void many_carve(BatchSys& b, unsigned char* base, uint32_t qc, uint32_t run);
+// Work items a system can have queued at once (expand, copy or psi).
+int64_t many_items(int64_t cap, uint32_t qc, uint32_t run);
+// C0 into pool and table, scratch bitmaps cleared, first frontier queued:
+// systems idx[i] (i without idx) for i < n.
+void launch_many_init(BatchSys* sys, const int32_t* idx, const int32_t* c0, const int64_t* c0_off, int32_t n,
+                      const ManyQueue& q, cudaStream_t st);
+// One iteration over the systems [0, n): each finishes the Psi scan of a new
+// frontier and at most one pass.  par alternates 0, 1.
+void launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par, const ManyPlan& p, cudaStream_t st,
+                           int nsm);
 
 struct BatchDepthStat {
   int64_t new_configs;
@@ -109,30 +169,23 @@ struct BatchDepthStat {
   int32_t chunks;
 };
 
-// One launch advances every system by one depth (cur_depth + 1), unless it
-// is finished or has run target_depth depths.
+// Tensor-core form: one launch advances every system by one depth (cur_depth
+// + 1), unless it is finished or has run target_depth depths.
 struct BatchArgs {
   BatchSys* sys;               // [n]
   int32_t n;
   int32_t launch;              // index of this launch (its work counter)
   uint32_t qc;                 // candidates per pass
-  int32_t B, ts, run;          // expand tile rows, tile row stride (words), candidates per warp task
-  size_t warp_smem;            // bytes of shared memory per warp
   unsigned int* queue;         // work counters, one per launch, zero before it
   unsigned char* scratch;      // per-CTA scratch
   size_t scratch_stride;
   int64_t pmax;                // largest frontier a system may have (largest cap)
   int32_t m_max;
-  int32_t tc;                  // 1: rows by the fp8 tensor-core form (four warps per CTA)
 };
 
 // Bytes of per-CTA scratch for frontiers of up to pmax rows and passes of qc candidates.
 size_t batch_scratch_bytes(int64_t pmax, uint32_t qc, int m_max);
-// Per-warp shared memory of the expand loop for rows of up to m_max neurons.
-size_t expand_smem_bytes(int m_max, int B, int* ts);
-void launch_batch_depth(const BatchArgs& a, int blocks, int warps, cudaStream_t st);
-// Dynamic shared memory of the batch kernel's tensor-core form.
-size_t batch_tc_smem_bytes_host();
+void launch_batch_depth_tc(const BatchArgs& a, int blocks, cudaStream_t st);
 __global__ void k_batch_init(BatchSys* sys, const int32_t* c0, const int64_t* c0_off, int32_t n);
 
 // Step (a) and Psi for P frontier rows; returns the launches made.

@@ -1,9 +1,9 @@
 // Serving loop (snp_server_*): explorations submitted at any time are admitted
-// while device memory allows and advanced together, one depth per tick, by
-// the batch kernel.  A request that arrives while others run joins at the
-// next tick (continuous batching); a finished request is copied into its
-// handle, its memory is returned, and its latency (submit to result ready) is
-// recorded.
+// while device memory allows and advanced together by the sparse batch form
+// (snp_many.cu), a few iterations per tick.  A request that arrives while
+// others run joins at the next tick (continuous batching); a finished request
+// is copied into its handle, its memory is returned, and its latency (submit
+// to result ready) is recorded.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -78,6 +78,9 @@ struct Request {
   size_t off = 0, bytes = 0;  // arena range: pool, table, stats
   int64_t rows = 0;
   uint64_t nslots = 0;
+  int32_t slot = -1;         // place in the device array of systems
+  std::unique_ptr<DevBuf> scratch;
+  int64_t items = 0;         // work items it can have queued
   BatchSys bs{};
   int status = SNP_OK;
 };
@@ -88,7 +91,12 @@ struct snp_server {
   int device = 0;
   size_t budget = 0;
   int32_t max_active = 0;
-  DevBuf arena, sys_dev, scratch, queue, c0_dev, c0_off_dev, fill_ptr, fill_cnt;
+  DevBuf arena, sys_dev, items, ctr, idx_dev, c0_dev, c0_off_dev, fill_ptr, fill_cnt;
+  std::vector<std::unique_ptr<DevBuf>> spare;  // scratch of finished requests, for the next ones (at most kSpare)
+  std::vector<Request*> slots;   // requests by their place in sys_dev (null: free)
+  std::vector<BatchSys> back;    // sys_dev as read back after a tick
+  int64_t item_cap = 0;          // items each queue holds
+  int par = 0;                   // parity of the next iteration
   RangeAlloc* alloc = nullptr;
   cudaStream_t st = nullptr;
   std::mutex mu;
@@ -106,14 +114,16 @@ struct snp_server {
   std::vector<double> lat_ms;
   Clock::time_point first_arrival, last_done;
   bool any = false;
-  size_t scratch_stride = 0;
   int loop_error = SNP_OK;
   std::string loop_msg;
 };
 
 namespace {
 
-constexpr uint32_t kServeQc = 2048;
+constexpr uint32_t kServeQc = 2048;    // claims past the cap a request's table has room for, per depth
+constexpr uint32_t kServeRun = 192;    // candidates per work item
+constexpr int kTickIterations = 8;
+constexpr size_t kSpare = 64;
 
 size_t request_bytes(const snp_system* h, const snp_explore_opts& o, int64_t* rows, uint64_t* nslots) {
   *rows = 1 + (int64_t)o.depth * o.frontier_cap;
@@ -123,42 +133,102 @@ size_t request_bytes(const snp_system* h, const snp_explore_opts& o, int64_t* ro
   return r((size_t)*rows * h->m * 4) + r(*nslots * 8) + r(sizeof(BatchDepthStat) * (o.depth + 1));
 }
 
+// Scratch for a request: the smallest spare buffer that holds it, else a new one.
+int take_scratch(snp_server* S, size_t bytes, std::unique_ptr<DevBuf>& out) {
+  size_t best = S->spare.size();
+  for (size_t i = 0; i < S->spare.size(); ++i)
+    if (S->spare[i]->bytes >= bytes && (best == S->spare.size() || S->spare[i]->bytes < S->spare[best]->bytes)) best = i;
+  if (best < S->spare.size()) {
+    out = std::move(S->spare[best]);
+    S->spare.erase(S->spare.begin() + best);
+    return SNP_OK;
+  }
+  out.reset(new DevBuf);
+  int rc = out->reserve(bytes);
+  if (rc == SNP_E_NOMEM && !S->spare.empty()) {  // the spare buffers are too small: give them back and try again
+    S->spare.clear();
+    rc = out->reserve(bytes);
+  }
+  if (rc != SNP_OK) out.reset();
+  return rc;
+}
+
+void return_scratch(snp_server* S, std::unique_ptr<DevBuf>& b) {
+  if (b && S->spare.size() < kSpare) S->spare.push_back(std::move(b));
+  b.reset();
+}
+
+ManyQueue queue_of(const snp_server* S) {
+  ManyQueue q;
+  q.expand[0] = S->items.as<int2>();
+  q.expand[1] = q.expand[0] + kMqForms * S->item_cap;
+  q.copy = q.expand[1] + kMqForms * S->item_cap;
+  q.psi = q.copy + S->item_cap;
+  q.ctr = S->ctr.as<uint32_t>();
+  q.cap = S->item_cap;
+  return q;
+}
+
+// Room in the queues for `items` work items (what is queued is kept).
+int ensure_items(snp_server* S, int64_t items) {
+  if (!S->ctr.p) {
+    TRY(S->ctr.reserve(sizeof(uint32_t) * kMqCounters));
+    CK(cudaMemsetAsync(S->ctr.p, 0, sizeof(uint32_t) * kMqCounters, S->st));
+  }
+  if (items <= S->item_cap) return SNP_OK;
+  const int64_t old = S->item_cap, want = std::max<int64_t>(items, 2 * old);
+  DevBuf grown;
+  TRY(grown.reserve(sizeof(int2) * (2 * kMqForms + 2) * want));
+  for (int k = 0; old > 0 && k < 2 * kMqForms + 2; ++k)
+    CK(cudaMemcpyAsync(grown.as<int2>() + k * want, S->items.as<int2>() + k * old, sizeof(int2) * old,
+                       cudaMemcpyDeviceToDevice, S->st));
+  CK(cudaStreamSynchronize(S->st));
+  std::swap(S->items.p, grown.p);
+  std::swap(S->items.bytes, grown.bytes);
+  S->item_cap = want;
+  return SNP_OK;
+}
+
 // Device state of newly admitted requests: empty tables, C0 in row 0 and in the table.
 int init_requests(snp_server* S, std::vector<Request*>& fresh) {
   if (fresh.empty()) return SNP_OK;
   const int n = (int)fresh.size();
   std::vector<unsigned long long*> ptr(n);
   std::vector<uint64_t> cnt(n);
-  std::vector<int32_t> c0;
+  std::vector<int32_t> c0, idx(n);
   std::vector<int64_t> c0_off(n);
-  std::vector<BatchSys> sys(n);
+  int64_t items = 0;
+  for (const Request* r : S->active) items += r->items;  // the new ones among them
+  TRY(ensure_items(S, items));
+  TRY(S->sys_dev.reserve(sizeof(BatchSys) * std::max<size_t>(64, S->slots.size() * 2), S->st, true));
   for (int i = 0; i < n; ++i) {
     Request* r = fresh[i];
     ptr[i] = r->bs.slots;
     cnt[i] = r->nslots;
+    idx[i] = r->slot;
     c0_off[i] = (int64_t)c0.size();
     c0.insert(c0.end(), r->h->c0.begin(), r->h->c0.end());
-    sys[i] = r->bs;
   }
   TRY(S->fill_ptr.reserve(sizeof(void*) * n));
   TRY(S->fill_cnt.reserve(sizeof(uint64_t) * n));
+  TRY(S->idx_dev.reserve(sizeof(int32_t) * n));
   TRY(S->c0_dev.reserve(sizeof(int32_t) * c0.size()));
   TRY(S->c0_off_dev.reserve(sizeof(int64_t) * n));
-  TRY(S->sys_dev.reserve(sizeof(BatchSys) * std::max<size_t>(n, S->active.size() + n)));
   CK(cudaMemcpyAsync(S->fill_ptr.p, ptr.data(), sizeof(void*) * n, cudaMemcpyHostToDevice, S->st));
   CK(cudaMemcpyAsync(S->fill_cnt.p, cnt.data(), sizeof(uint64_t) * n, cudaMemcpyHostToDevice, S->st));
+  CK(cudaMemcpyAsync(S->idx_dev.p, idx.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, S->st));
   CK(cudaMemcpyAsync(S->c0_dev.p, c0.data(), sizeof(int32_t) * c0.size(), cudaMemcpyHostToDevice, S->st));
   CK(cudaMemcpyAsync(S->c0_off_dev.p, c0_off.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, S->st));
-  CK(cudaMemcpyAsync(S->sys_dev.p, sys.data(), sizeof(BatchSys) * n, cudaMemcpyHostToDevice, S->st));
   dim3 grid(64, (unsigned)std::min(n, 1024));
   k_fill_ranges<<<grid, 256, 0, S->st>>>(S->fill_ptr.as<unsigned long long*>(), S->fill_cnt.as<uint64_t>(), n, kEmpty);
   CK(cudaGetLastError());
   for (int i = 0; i < n; ++i) {
     Request* r = fresh[i];
     CK(cudaMemsetAsync(r->bs.stats, 0, sizeof(BatchDepthStat) * (r->o.depth + 1), S->st));
+    CK(cudaMemcpyAsync(S->sys_dev.as<BatchSys>() + r->slot, &r->bs, sizeof(BatchSys), cudaMemcpyHostToDevice, S->st));
   }
-  k_batch_init<<<grid_for(n, 8, 152 * 16), 256, 0, S->st>>>(S->sys_dev.as<BatchSys>(), S->c0_dev.as<int32_t>(),
-                                                             S->c0_off_dev.as<int64_t>(), n);
+  launch_many_init(S->sys_dev.as<BatchSys>(), S->idx_dev.as<int32_t>(), S->c0_dev.as<int32_t>(),
+                   S->c0_off_dev.as<int64_t>(), n, queue_of(S), S->st);
   CK(cudaGetLastError());
   return SNP_OK;
 }
@@ -214,57 +284,24 @@ int retire(snp_server* S, Request* r) {
   return SNP_OK;
 }
 
+// A few iterations over every active request, then their state read back.
 int tick(snp_server* S) {
-  const int n = (int)S->active.size();
-  if (n == 0) return SNP_OK;
-  int m_max = 1;
-  int64_t pmax = 1;
-  std::vector<BatchSys> sys(n);
-  for (int i = 0; i < n; ++i) {
-    sys[i] = S->active[i]->bs;
-    m_max = std::max(m_max, sys[i].sys.m);
-    pmax = std::max<int64_t>(pmax, sys[i].cap);
+  if (S->active.empty()) return SNP_OK;
+  std::vector<int> ms;
+  for (const Request* r : S->active) ms.push_back(r->h->m);
+  const ManyPlan mp = many_plan(ms.data(), (int64_t)ms.size(), 0, 0);
+  // (a request's tile was chosen for its own rows alone: shared memory for all of them holds it)
+  const int n = (int)S->slots.size();
+  BatchSys* dsys = S->sys_dev.as<BatchSys>();
+  for (int k = 0; k < kTickIterations; ++k) {
+    launch_many_iteration(dsys, n, queue_of(S), S->par, mp, S->st, sm_count(S->device));
+    S->par ^= 1;
   }
-  const int nsm = sm_count(S->device);
-  const int warps = 8;
-  int ts = 0;
-  int B = 32;  // shrunk below to what the shared memory holds
-  size_t warp_smem = expand_smem_bytes(m_max, B, &ts);
-  while (B > 1 && warp_smem * warps > (200u << 10)) warp_smem = expand_smem_bytes(m_max, --B, &ts);
-  const int blocks = std::max(1, std::min(nsm, n));
-  const size_t stride = (batch_scratch_bytes(pmax, kServeQc, m_max) + 255) & ~size_t(255);
-  void* before = S->scratch.p;
-  TRY(S->scratch.reserve(stride * blocks));
-  // The bitmaps in the scratch must start cleared (the kernel leaves them
-  // cleared); a new buffer or a new layout (other stride) starts from zero.
-  if (S->scratch.p != before || stride != S->scratch_stride) {
-    CK(cudaMemsetAsync(S->scratch.p, 0, S->scratch.bytes, S->st));
-    S->scratch_stride = stride;
-  }
-  TRY(S->sys_dev.reserve(sizeof(BatchSys) * n));
-  TRY(S->queue.reserve(sizeof(unsigned int)));
-  CK(cudaMemcpyAsync(S->sys_dev.p, sys.data(), sizeof(BatchSys) * n, cudaMemcpyHostToDevice, S->st));
-  CK(cudaMemsetAsync(S->queue.p, 0, sizeof(unsigned int), S->st));
-  BatchArgs a;
-  std::memset(&a, 0, sizeof a);
-  a.sys = S->sys_dev.as<BatchSys>();
-  a.n = n;
-  a.launch = 0;
-  a.qc = kServeQc;
-  a.B = B;
-  a.ts = ts;
-  a.run = 4 * B;
-  a.warp_smem = warp_smem;
-  a.queue = S->queue.as<unsigned int>();
-  a.scratch = S->scratch.as<unsigned char>();
-  a.scratch_stride = stride;
-  a.pmax = pmax;
-  a.m_max = m_max;
-  launch_batch_depth(a, blocks, warps, S->st);
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(sys.data(), S->sys_dev.p, sizeof(BatchSys) * n, cudaMemcpyDeviceToHost, S->st));
+  S->back.resize(n);
+  CK(cudaMemcpyAsync(S->back.data(), dsys, sizeof(BatchSys) * n, cudaMemcpyDeviceToHost, S->st));
   CK(cudaStreamSynchronize(S->st));
-  for (int i = 0; i < n; ++i) S->active[i]->bs = sys[i];
+  for (Request* r : S->active) r->bs = S->back[r->slot];
   ++S->ticks;
   return SNP_OK;
 }
@@ -284,6 +321,18 @@ void server_loop(snp_server* S) {
         Request* r = S->pending.front();
         size_t off = 0;
         if (!S->alloc->alloc(r->bytes, &off)) break;  // admitted when memory frees up
+        const uint32_t qc = many_default_qc(r->o.frontier_cap);
+        const int rc = take_scratch(S, many_scratch_bytes(r->o.frontier_cap, qc, r->h->m), r->scratch);
+        if (rc != SNP_OK) {
+          S->alloc->release(off, r->bytes);
+          if (!S->active.empty()) break;  // admitted when running requests give theirs back
+          S->pending.pop_front();         // alone and it does not fit: this request fails
+          r->status = rc;
+          r->done = Clock::now();
+          S->finished.push_back(r);
+          S->cv_done.notify_all();
+          continue;
+        }
         S->pending.pop_front();
         r->off = off;
         auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
@@ -303,6 +352,15 @@ void server_loop(snp_server* S) {
         b.max_expand = r->o.max_expand_value;
         b.cap = r->o.frontier_cap;
         b.budget = r->o.candidate_budget > 0 ? r->o.candidate_budget : 0;
+        b.overshoot = kServeQc;
+        many_carve(b, r->scratch->as<unsigned char>(), qc, kServeRun);
+        const ManyPlan mine = many_plan(&r->h->m, 1, 0, 0);
+        b.tile = many_tile(mine, r->h->m, 0);
+        r->items = many_items(b.cap, qc, kServeRun);
+        r->slot = 0;
+        while (r->slot < (int32_t)S->slots.size() && S->slots[r->slot]) ++r->slot;
+        if (r->slot == (int32_t)S->slots.size()) S->slots.push_back(nullptr);
+        S->slots[r->slot] = r;
         S->active.push_back(r);
         fresh.push_back(r);
       }
@@ -318,6 +376,8 @@ void server_loop(snp_server* S) {
           rc = retire(S, r);
           if (rc != SNP_OK) break;
           r->done = Clock::now();
+          return_scratch(S, r->scratch);
+          S->slots[r->slot] = nullptr;
           done.push_back(r);
           S->active.erase(S->active.begin() + i);
         } else {
@@ -496,6 +556,7 @@ int snp_server_destroy(void* srv) {
   for (Request* r : S->finished) delete r;
   for (Request* r : S->pending) delete r;
   for (Request* r : S->active) delete r;
+  S->spare.clear();
   if (S->st) cudaStreamDestroy(S->st);
   delete S->alloc;
   delete S;
