@@ -143,9 +143,11 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
     const int wpb = (int)std::max<size_t>(1, std::min<size_t>(kWideWarps, (226u << 10) / per_warp));
     const size_t smem = per_warp * wpb;
     // one task per warp: a task's first block costs a full decode (C + S . M
-    // over every neuron), which wide rows make expensive
+    // over every neuron), which wide rows make expensive; at least 16
+    // candidates (919 neurons, passes of a few thousand: 1031 us per
+    // exploration with 256 or more, 552 with 32, 498 with 16, 502 with 8)
     const uint64_t warps = (uint64_t)nsm * wpb;
-    a.run = (uint32_t)std::max<uint64_t>(8ull * kWideB, ((uint64_t)a.Q + warps - 1) / warps);
+    a.run = (uint32_t)std::max<uint64_t>(16, ((uint64_t)a.Q + warps - 1) / warps);
     const uint64_t ntasks = ((uint64_t)a.Q + a.run - 1) / a.run;
     const int blocks = (int)std::min<uint64_t>((ntasks + wpb - 1) / wpb, (uint64_t)nsm);
     if (a.bcache) {  // base children of the pass's largest parents
@@ -166,11 +168,14 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
   const int wpb = (int)std::max<size_t>(1, std::min<size_t>(8, (100u << 10) / per_warp));
   const size_t smem = per_warp * wpb;
   const int per_sm = (int)std::max<size_t>(1, (220u << 10) / smem);
-  // a task (run of candidates) of at least 8 tiles, and about two per warp of
-  // the grid: each task pays one decode of its first block
+  // a task (run of candidates) pays one decode of its first block: in small
+  // passes every warp takes one task of at least 32 candidates (20 neurons,
+  // passes of at most 2^16: 404 us per exploration with 256 or more, 308 with
+  // 32); from 256 candidates per warp on, two tasks per warp (16 neurons,
+  // passes of half a million: two tasks of 103 each run 9% slower)
   {
-    const uint64_t two_per_warp = 2ull * nsm * per_sm * wpb;
-    a.run = (uint32_t)std::max<uint64_t>(8ull * B, ((uint64_t)a.Q + two_per_warp - 1) / two_per_warp);
+    const uint64_t warps = (uint64_t)nsm * per_sm * wpb, each = ((uint64_t)a.Q + warps - 1) / warps;
+    a.run = (uint32_t)std::max<uint64_t>(32, each <= 256 ? each : std::max<uint64_t>(256, (each + 1) / 2));
   }
   const uint64_t ntasks = ((uint64_t)a.Q + a.run - 1) / a.run;
   const int blocks = (int)std::min<uint64_t>((ntasks + wpb - 1) / wpb, (uint64_t)nsm * per_sm);
