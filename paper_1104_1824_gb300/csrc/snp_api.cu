@@ -109,9 +109,11 @@ int ensure_chunk_buffers(snp_system* h, uint64_t q, cudaStream_t st) {
   TRY(h->d_slot_of.reserve(sizeof(uint32_t) * q));
   TRY(h->d_srow.reserve(sizeof(uint32_t) * q));
   TRY(h->d_bits.reserve(sizeof(uint32_t) * words));
-  TRY(h->d_wbase.reserve(sizeof(uint32_t) * words));
   TRY(h->d_own.reserve(sizeof(uint32_t) * words));
-  TRY(h->d_scan_tmp.reserve(scan_temp_bytes((int64_t)words, 4)));
+  const size_t tiles = sizeof(unsigned long long) * (1 + (size_t)commit_tiles((uint32_t)words));  // two counters, words
+  TRY(h->d_tiles.reserve(tiles));
+  CK(cudaMemsetAsync(h->d_tiles.p, 0, h->d_tiles.bytes, st));
+  h->epoch = 0;
   CK(cudaMemsetAsync(h->d_bits.p, 0, sizeof(uint32_t) * words, st));
   CK(cudaMemsetAsync(h->d_own.p, 0, sizeof(uint32_t) * words, st));
   h->q_cap = q;
@@ -906,7 +908,6 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         TRY(ensure_chunk_buffers(h, Q, st));
         const int slot = next_slot;
         next_slot ^= 1;
-        CK(cudaMemsetAsync(h->d_st.p, 0, sizeof(ChunkState), st));
         {
           ClaimArgs a;
           a.sys = h->dev();
@@ -981,16 +982,18 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
           if (o->kernel_timing) CK(cudaEventRecord(h->evk[slot][1], st));
         }
         const uint32_t nwords = (uint32_t)((Q + 31) / 32);
-        k_mark<<<grid_for(nwords, 256, nsm * 8), 256, 0, st>>>(h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(),
-                                                                 h->d_bits.as<uint32_t>(), h->d_srow.as<uint32_t>(),
-                                                                 nwords, h->d_st.as<ChunkState>());
-        launch_popc(h->d_bits.as<uint32_t>(), h->d_wbase.as<uint32_t>(), nwords, st);
-        sd.launches += 2 + scan_u32(h->d_wbase.as<uint32_t>(), h->d_wbase.as<uint32_t>(), nwords, h->d_scan_tmp.p, st);
         CommitArgs c;
         c.sys = h->dev();
+        c.Q = (uint32_t)Q;
         c.nwords = nwords;
         c.bits = h->d_bits.as<uint32_t>();
-        c.wbase = h->d_wbase.as<uint32_t>();
+        c.ticket = h->d_tiles.as<uint32_t>();
+        c.tiles = h->d_tiles.as<unsigned long long>() + 1;
+        if (++h->epoch >> 30) {  // numbers used up: start over with clear words
+          CK(cudaMemsetAsync(h->d_tiles.p, 0, h->d_tiles.bytes, st));
+          h->epoch = 1;
+        }
+        c.epoch = h->epoch;
         c.srow = h->d_srow.as<uint32_t>();
         c.slot_of = h->d_slot_of.as<uint32_t>();
         c.staging = nullptr;
@@ -1008,14 +1011,10 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         c.parent_base = level_lo;
         c.g0 = g0;
         c.st = h->d_st.as<ChunkState>();
-        k_commit<<<grid_for(nwords, 8, nsm * 16), 256, 0, st>>>(c);
-        CK(cudaGetLastError());
-        k_clear_bits<<<grid_for(nwords, 256, nsm * 8), 256, 0, st>>>(h->d_bits.as<uint32_t>(), nwords,
-                                                                       h->d_ctr.as<unsigned long long>(),
-                                                                       h->d_st.as<ChunkState>());
+        c.host = h->pin.slot[slot];
+        launch_mark_commit(c, h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(), st, nsm);
         CK(cudaGetLastError());
         sd.launches += 2;
-        CK(cudaMemcpyAsync(h->pin.slot[slot], h->d_st.p, sizeof(ChunkState), cudaMemcpyDeviceToHost, st));
         CK(cudaEventRecord(h->evs[slot], st));
         fl[nfl++] = Flight{g0, Q, may_add, slot};
         pend_add += may_add;
@@ -1215,7 +1214,8 @@ struct StaticLayout {
   uint64_t* off;
   void* scan_tmp;
   int32_t* staging;
-  uint32_t *gmin, *slot_of, *srow, *bits, *wbase, *own;
+  uint32_t *gmin, *slot_of, *srow, *bits, *own;
+  unsigned long long* tiles;  // two counters, then look-back words
   uint64_t q;  // candidates per pass
 };
 
@@ -1234,13 +1234,13 @@ bool static_layout(unsigned char* base, int m, StaticLayout* L) {
   L->slots = reinterpret_cast<unsigned long long*>(take(kStaticSlots * sizeof(unsigned long long)));
   L->psi = reinterpret_cast<uint64_t*>(take((kStaticMaxRows + 1) * sizeof(uint64_t)));
   L->off = reinterpret_cast<uint64_t*>(take((kStaticMaxRows + 1) * sizeof(uint64_t)));
-  L->scan_tmp = take(std::max(scan_temp_bytes(kStaticMaxRows + 1, 8), scan_temp_bytes((int64_t)q / 32 + 1, 4)));
+  L->scan_tmp = take(scan_temp_bytes(kStaticMaxRows + 1, 8));
   L->staging = reinterpret_cast<int32_t*>(take(q * 4ull * m));
   L->gmin = reinterpret_cast<uint32_t*>(take(q * 4));
   L->slot_of = reinterpret_cast<uint32_t*>(take(q * 4));
   L->srow = reinterpret_cast<uint32_t*>(take(q * 4));
   L->bits = reinterpret_cast<uint32_t*>(take((q / 32 + 1) * 4));
-  L->wbase = reinterpret_cast<uint32_t*>(take((q / 32 + 1) * 4));
+  L->tiles = reinterpret_cast<unsigned long long*>(take((1 + (size_t)commit_tiles((uint32_t)(q / 32 + 1))) * 8));
   L->own = reinterpret_cast<uint32_t*>(take((q / 32 + 1) * 4));
   return at <= kStaticScratchBytes;
 }
@@ -1289,6 +1289,8 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
   CK(cudaMemsetAsync(L.st, 0, sizeof(ChunkState), st));
   CK(cudaMemsetAsync(L.bits, 0, sizeof(uint32_t) * (L.q / 32 + 1), st));
   CK(cudaMemsetAsync(L.own, 0, sizeof(uint32_t) * (L.q / 32 + 1), st));
+  CK(cudaMemsetAsync(L.tiles, 0, 8 * (1 + (size_t)commit_tiles((uint32_t)(L.q / 32 + 1))), st));
+  uint32_t epoch = 0;
   auto clear_and_insert = [&](int64_t rows) -> int {
     k_fill_u64<<<grid_for((int64_t)kStaticSlots, 256, nsm * 32), 256, 0, st>>>(L.slots, kStaticSlots, kEmpty);
     CK(cudaGetLastError());
@@ -1339,7 +1341,6 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
         TRY(clear_and_insert(n_rows));  // drops tombstones; n_rows + Q always fits
         tombs = 0;
       }
-      CK(cudaMemsetAsync(L.st, 0, sizeof(ChunkState), st));
       ClaimArgs a;
       a.sys = h->dev();
       a.parents = parents;
@@ -1365,14 +1366,15 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
       launch_expand(a, st, nsm);
       CK(cudaGetLastError());
       const uint32_t nwords = (uint32_t)((Q + 31) / 32);
-      k_mark<<<grid_for(nwords, 256, nsm * 8), 256, 0, st>>>(L.own, L.gmin, L.bits, L.srow, nwords, L.st);
-      launch_popc(L.bits, L.wbase, nwords, st);
-      scan_u32(L.wbase, L.wbase, nwords, L.scan_tmp, st);
       CommitArgs c;
       c.sys = h->dev();
+      c.Q = (uint32_t)Q;
       c.nwords = nwords;
       c.bits = L.bits;
-      c.wbase = L.wbase;
+      c.ticket = reinterpret_cast<uint32_t*>(L.tiles);
+      c.tiles = L.tiles + 1;
+      c.epoch = ++epoch;
+      c.host = h->pin.slot[0];
       c.srow = L.srow;
       c.slot_of = L.slot_of;
       c.staging = L.staging;
@@ -1390,12 +1392,10 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
       c.perm = nullptr;
       c.sidx_of = nullptr;
       c.st = L.st;
-      k_commit<<<grid_for(nwords, 8, nsm * 16), 256, 0, st>>>(c);
+      launch_mark_commit(c, L.own, L.gmin, st, nsm);
       CK(cudaGetLastError());
-      k_clear_bits<<<grid_for(nwords, 256, nsm * 8), 256, 0, st>>>(L.bits, nwords, nullptr, nullptr);
-      CK(cudaGetLastError());
-      CK(cudaMemcpyAsync(hst, L.st, sizeof(ChunkState), cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
+      *hst = *h->pin.slot[0];
       if (hst->error & kErrTimeout) return fail(SNP_E_TIMEOUT, "bounded wait for a hash slot ran out");
       if (hst->error) return fail(SNP_E_INTERNAL, "device consistency check failed (bits 0x%x)", hst->error);
       if (hst->n_alloc > room && room < remaining)

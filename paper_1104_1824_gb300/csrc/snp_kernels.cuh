@@ -51,9 +51,14 @@ size_t wide_base_bytes(int m);
 
 struct CommitArgs {
   DevSys sys;
+  uint32_t Q;                 // candidates in the chunk
   uint32_t nwords;            // ceil(Q / 32)
-  const uint32_t* bits;       // [nwords] first-occurrence bitmap over chunk-local indices
-  const uint32_t* wbase;      // [nwords] exclusive prefix of popcounts
+  uint32_t* bits;             // [nwords] first-occurrence bitmap over chunk-local indices; cleared on the way
+  // Look-back state: a word per tile (commit_tiles), two counters that start
+  // (and are left) at 0, and a number no earlier chunk of these words had.
+  unsigned long long* tiles;
+  uint32_t* ticket;
+  uint32_t epoch;
   const uint32_t* srow;       // [Q] owner (candidate that claimed the key) of each first occurrence
   const uint32_t* slot_of;
   const int32_t* staging;
@@ -65,7 +70,7 @@ struct CommitArgs {
   const uint32_t* sidx_of;
   int64_t row_base;           // pool row of rank 0
   uint64_t remaining;         // how many more configurations the depth may accept
-  const unsigned long long* ctr;  // or, when set, both from device counters {rows, still acceptable}
+  unsigned long long* ctr;    // or, when set, both from device counters {rows, still acceptable}, advanced at the end
   // parent records (optional)
   int64_t* rec_parent;        // [rows] or nullptr
   uint64_t* rec_index;
@@ -73,8 +78,15 @@ struct CommitArgs {
   int64_t P;
   int64_t parent_base;        // discovery index of frontier row 0
   uint64_t g0;
-  ChunkState* st;
+  ChunkState* st;             // the chunk's counters; with host, copied there and cleared at the end
+  ChunkState* host;           // pinned host copy, or nullptr
 };
+constexpr int kCommitWords = 64;  // bitmap words per commit tile
+constexpr int kMarkWords = 4;     // bitmap words per warp of the mark kernel
+uint32_t commit_tiles(uint32_t nwords);
+// First-occurrence marks of the chunk (ownbits cleared on the way), ranks and
+// commit: two launches.
+void launch_mark_commit(const CommitArgs& c, uint32_t* ownbits, const uint32_t* gmin, cudaStream_t st, int nsm);
 
 // ---------------------------------------------------------------------------
 // Batch engine and serving loop: many independent systems advance together.
@@ -243,16 +255,12 @@ int tc5_slots(int m, int nblocks);
 // driver entry point); rows are then stored by the threads.
 bool tc5_store_map(CUtensorMap* map, int32_t* pool, int m, uint64_t rows);
 void launch_tc5(const Tc5Args& a, const CUtensorMap& map, cudaStream_t st, int nsm);
-__global__ void k_mark(uint32_t* ownbits, const uint32_t* gmin, uint32_t* bits, uint32_t* srow, uint32_t nwords,
-                       ChunkState* st);
-__global__ void k_commit(CommitArgs a);
 void launch_iota_u32(uint32_t* out, int64_t n, cudaStream_t st);
 // out[k] = row perm[k] (row k without perm) of a pool of w bytes per count, as int32.
 void launch_gather_rows(const int32_t* pool, int w, const uint32_t* perm, int64_t n, int m, int32_t* out,
                         cudaStream_t st);
 // Testing hook: marks the slot holding store row `row` as being claimed.
 __global__ void k_hold_slot_of_row(unsigned long long* slots, uint64_t n, uint32_t row);
-__global__ void k_clear_bits(uint32_t* bits, uint32_t nwords, unsigned long long* ctr, const ChunkState* st);
 // *out = max(*out, x[0 .. n)) for counts x >= 0.
 void launch_count_max(const int32_t* x, int64_t n, int32_t* out, cudaStream_t st);
 // n int32 rows of m counts (m % 8 == 0, each count within the range of w
@@ -280,11 +288,9 @@ void launch_step_children(DevSys s, const int32_t* base, const StepPlan* plan, u
 __global__ void k_fill_u64(unsigned long long* p, uint64_t n, unsigned long long v);
 
 // Device-wide exclusive scans (n elements, in -> out; "total" gets the sum).
-// Saturating for u64 (sums of Psi), plain for u32.
+// Saturating (sums of Psi).
 size_t scan_temp_bytes(int64_t n, size_t elem);
-// Each returns the number of kernels it launched.
+// Returns the number of kernels it launched.
 int scan_u64_sat(const uint64_t* in, uint64_t* out, int64_t n, void* temp, cudaStream_t st);
-int scan_u32(const uint32_t* in, uint32_t* out, int64_t n, void* temp, cudaStream_t st);
-void launch_popc(const uint32_t* bits, uint32_t* cnt, uint32_t nwords, cudaStream_t st);
 
 }  // namespace snp
