@@ -87,16 +87,6 @@ int tc5_prepare(snp_system* h, uint64_t q) {
 
 namespace {
 
-int check_device_errors(snp_system* h, cudaStream_t st, const char* where) {
-  CK(cudaMemcpyAsync(h->pin.h, h->d_st.p, sizeof(ChunkState), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  const uint32_t e = h->pin.h->error;
-  if (!e) return SNP_OK;
-  if (e & kErrOverflow) return fail(SNP_E_OVERFLOW, "%s: a spike count could leave the int32 range", where);
-  if (e & kErrTimeout) return fail(SNP_E_TIMEOUT, "%s: bounded wait for a hash slot ran out", where);
-  return fail(SNP_E_INTERNAL, "%s: device consistency check failed (bits 0x%x)", where, e);
-}
-
 // Per-pass buffers for chunks of up to q candidates: owners' store rows and
 // the first-occurrence records (grow only; a fresh first-occurrence bitmap
 // starts cleared).
@@ -423,8 +413,8 @@ int snp_load_system(const snp_system_desc* d, snp_handle* out) {
     delete h;
     return fail(SNP_E_NOMEM, "pinned host allocation failed");
   }
-  CK(cudaEventCreate(&h->ev[0]));
-  CK(cudaEventCreate(&h->ev[1]));
+  for (auto& pair : h->ev)
+    for (auto& e : pair) CK(cudaEventCreate(&e));
   for (auto& pair : h->evk)
     for (auto& e : pair) CK(cudaEventCreate(&e));
   for (auto& e : h->evs) CK(cudaEventCreate(&e, cudaEventDisableTiming));
@@ -444,8 +434,9 @@ int snp_system_info(snp_handle h, int32_t* m, int32_t* R, int32_t* device) {
 int snp_free(snp_handle h) {
   if (!h) return SNP_OK;
   cudaSetDevice(h->device);
-  for (auto& e : h->ev)
-    if (e) cudaEventDestroy(e);
+  for (auto& pair : h->ev)
+    for (auto& e : pair)
+      if (e) cudaEventDestroy(e);
   for (auto& pair : h->evk)
     for (auto& e : pair)
       if (e) cudaEventDestroy(e);
@@ -729,6 +720,16 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
   }
   int64_t tombs = 0;
   double rate = 1.0;  // new configurations per candidate, for chunk sizing
+  bool few_before = true;  // the last depth had at most 256 candidates per parent
+  h->pin.ctr[0] = (unsigned long long)h->n_rows;
+  h->pin.ctr[1] = 0;  // set per depth by the Psi kernel
+  h->pin.ctr[2] = (unsigned long long)h->n_store;
+  CK(cudaMemcpyAsync(h->d_ctr.p, h->pin.ctr, 3 * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
+  int timed_depth = -1;  // depth whose events are still to be read
+  auto depth_ms = [&](int d) -> int {
+    CK(cudaEventElapsedTime(&h->stats[d].ms, h->ev[d & 1][0], h->ev[d & 1][1]));
+    return SNP_OK;
+  };
 
   for (int d = d_start; d <= o->depth; ++d) {
     if (cancelled()) {
@@ -739,61 +740,93 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     std::memset(&sd, 0, sizeof sd);
     const int64_t P = level_hi - level_lo;
     sd.parents = P;
-    CK(cudaEventRecord(h->ev[0], st));
-    if (h->psi_cap < P + 1) {
-      TRY(h->d_psi.reserve(sizeof(uint64_t) * (P + 1)));
-      TRY(h->d_prec.reserve(sizeof(ParentRec) * (P + 1)));
-      TRY(h->d_off.reserve(sizeof(uint64_t) * (P + 1)));
-      TRY(h->d_scan_tmp.reserve(scan_temp_bytes(P + 1, 8)));
-      h->psi_cap = P + 1;
+    CK(cudaEventRecord(h->ev[d & 1][0], st));
+    {  // buffers of the frontier: when capped, once for all depths
+      const int64_t want = cap > 0 ? std::max<int64_t>(P, std::min<int64_t>(cap, 1 << 22)) : P;
+      if (h->psi_cap < P) {
+        TRY(h->d_prec.reserve(sizeof(ParentRec) * want));
+        TRY(h->d_off.reserve(sizeof(uint64_t) * (want + 1)));
+        h->psi_cap = want;
+      }
+      const size_t tiles = sizeof(ScanTile) * (1 + psi_tiles(P, m, nsm));  // two counters, entries
+      if (h->d_scan.bytes < tiles) {
+        TRY(h->d_scan.reserve(std::max(tiles, sizeof(ScanTile) * 8192)));
+        h->scan_epoch = 0x3FFFFFFFu;  // clear it below
+      }
     }
     const int32_t* parents = h->d_pool.as<int32_t>();            // the store (W bytes per count)
     const uint32_t* pperm = h->d_perm.as<uint32_t>() + level_lo;  // its rows of this frontier
-    CK(cudaMemsetAsync(h->d_st.p, 0, sizeof(ChunkState), st));
-    uint64_t* psi = h->d_psi.as<uint64_t>();
-    CK(cudaMemsetAsync(psi + P, 0, sizeof(uint64_t), st));
+    // Parent records serve the batches that cross parents; they are worth their
+    // writing with few candidates per parent, as expected from the last depth.
+    bool with_records = !tc && !tc5 && few_before;
+    uint64_t remaining = cap > 0 ? (uint64_t)cap : ~0ull;  // as of the passes read back so far
+    PsiArgs pa;
+    std::memset(&pa, 0, sizeof pa);
+    pa.s = h->dev();
+    pa.rows = parents;
+    pa.max_expand = o->max_expand_value;
+    pa.ticket = h->d_scan.as<uint32_t>();
+    pa.tiles = h->d_scan.as<ScanTile>() + 1;
+    pa.st = h->d_st.as<ChunkState>();
+    auto psi_rows = [&](int64_t lo, int64_t hi) -> int {
+      if (++h->scan_epoch >> 30) {
+        CK(cudaMemsetAsync(h->d_scan.p, 0, h->d_scan.bytes, st));
+        h->scan_epoch = 1;
+      }
+      pa.perm = pperm + lo;
+      pa.P = hi - lo;
+      pa.off = h->d_off.as<uint64_t>() + lo;
+      pa.carry = lo > 0 ? pa.off : nullptr;
+      pa.rec = with_records ? h->d_prec.as<ParentRec>() + lo : nullptr;
+      pa.epoch = h->scan_epoch;
+      if (hi == P) {
+        pa.host_total = h->pin.u64;
+        pa.host = h->pin.h;
+        pa.ctr = h->d_ctr.as<unsigned long long>();
+        pa.remaining = remaining;
+      }
+      sd.launches += launch_psi(pa, W, st, nsm);
+      CK(cudaGetLastError());
+      return SNP_OK;
+    };
     // When the previous depth's Psi sum saturated, the first rows alone may
     // hold 2^64 - 1 candidates: they go first, and if they do, the rest are
     // not read (no candidate and no statistic depends on them).
     const int64_t P0 = psi_saturated_before && P > 2 * kPsiHead ? kPsiHead : P;
-    launch_psi(h->dev(), parents, W, pperm, P0, o->max_expand_value, psi, nullptr, h->d_st.as<ChunkState>(), st, nsm);
-    if (P0 < P) {
-      launch_psi_head_check(psi, P0, h->d_st.as<ChunkState>(), st);
-      launch_psi(h->dev(), parents, W, pperm + P0, P - P0, o->max_expand_value, psi + P0, nullptr,
-                 h->d_st.as<ChunkState>(), st, nsm);
-      sd.launches += 2;
+    TRY(psi_rows(0, P0));
+    if (P0 < P) TRY(psi_rows(P0, P));
+    CK(cudaEventRecord(h->evs[0], st));
+    CK(cudaEventSynchronize(h->evs[0]));
+    if (const uint32_t e = h->pin.h->error) {
+      if (e & kErrOverflow) return fail(SNP_E_OVERFLOW, "applicability scan: a spike count could leave the int32 range");
+      if (e & kErrTimeout) return fail(SNP_E_TIMEOUT, "applicability scan: bounded wait ran out");
+      return fail(SNP_E_INTERNAL, "applicability scan: device consistency check failed (bits 0x%x)", e);
     }
-    CK(cudaGetLastError());
-    sd.launches += 1 + scan_u64_sat(psi, h->d_off.as<uint64_t>(), P + 1, h->d_scan_tmp.p, st);
-    CK(cudaGetLastError());
-    uint64_t total = 0;
-    CK(cudaMemcpyAsync(h->pin.u64, h->d_off.as<uint64_t>() + P, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-    TRY(check_device_errors(h, st, "applicability scan"));
-    total = *h->pin.u64;
+    if (timed_depth >= 0) TRY(depth_ms(timed_depth));  // the last depth's events have passed
+    timed_depth = -1;
+    const uint64_t total = *h->pin.u64;
     sd.candidates = total;
     psi_saturated_before = total == ~0ull;
-    // Parent records serve the batches that cross parents; with few
-    // candidates per parent they are worth a second pass over the frontier.
-    const bool with_records = !tc && !tc5 && P > 0 && total <= 256ull * (uint64_t)P;
-    if (with_records) {
-      launch_psi(h->dev(), parents, W, pperm, P, o->max_expand_value, psi, h->d_prec.as<ParentRec>(),
-                 h->d_st.as<ChunkState>(), st, nsm);
+    few_before = total <= 256ull * (uint64_t)P;
+    if (!with_records && few_before && !tc && !tc5 && P > 0) {
+      with_records = true;
+      pa.perm = pperm;
+      pa.P = P;
+      pa.off = nullptr;
+      pa.carry = nullptr;
+      pa.rec = h->d_prec.as<ParentRec>();
+      pa.host_total = nullptr;
+      sd.launches += launch_psi(pa, W, st, nsm);
       CK(cudaGetLastError());
-      sd.launches += 1;
     }
     const uint64_t T = budget > 0 ? std::min<uint64_t>(total, (uint64_t)budget) : total;
-    uint64_t remaining = cap > 0 ? (uint64_t)cap : ~0ull;  // as of the passes read back so far
-    uint64_t g0 = 0, examined = 0;                         // g0: first candidate of the next pass
+    uint64_t g0 = 0, examined = 0;  // g0: first candidate of the next pass
     int64_t nnew = 0;
     bool capped = false;
-    // Device counters {rows, still acceptable}: the commit of a pass takes its
-    // row base and limit from them, so the next pass can be enqueued before
-    // this one is read back (at most two in flight; a pass that starts after
-    // the depth is full does nothing).
-    h->pin.ctr[0] = (unsigned long long)h->n_rows;
-    h->pin.ctr[1] = remaining;
-    h->pin.ctr[2] = (unsigned long long)h->n_store;
-    CK(cudaMemcpyAsync(h->d_ctr.p, h->pin.ctr, 3 * sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
+    // Device counters {rows, still acceptable, store rows}: the commit of a pass
+    // takes its row base and limit from them, so the next pass can be enqueued
+    // before this one is read back (at most two in flight; a pass that starts
+    // after the depth is full does nothing).
     struct Flight {
       uint64_t g0, Q, may_add;
       int slot;
@@ -1025,11 +1058,8 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
       if (nfl == 0) break;
       TRY(retire());
     }
-    CK(cudaEventRecord(h->ev[1], st));
-    CK(cudaEventSynchronize(h->ev[1]));
-    float ms = 0.f;
-    CK(cudaEventElapsedTime(&ms, h->ev[0], h->ev[1]));
-    sd.ms = ms;
+    CK(cudaEventRecord(h->ev[d & 1][1], st));
+    timed_depth = d;
     sd.new_configs = nnew;
     sd.examined = (int64_t)examined;
     sd.truncated = examined < total ? 1 : 0;
@@ -1038,6 +1068,10 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     h->depth_reached = d;
     level_lo = level_hi;
     level_hi = h->n_rows;
+  }
+  if (timed_depth >= 0) {
+    CK(cudaEventSynchronize(h->ev[timed_depth & 1][1]));
+    TRY(depth_ms(timed_depth));
   }
   h->explored = true;
   h->result_pool = h->d_pool.as<int32_t>();
@@ -1153,6 +1187,7 @@ constexpr size_t kStaticScratchBytes = 64ull << 20;    // 64 MiB
 constexpr uint64_t kStaticSlots = 1ull << 21;           // hash slots (16 MiB)
 constexpr int64_t kStaticMaxRows = 1ll << 20;           // configurations per call
 constexpr size_t kStaticStagingBytes = 24ull << 20;     // rows claimed per pass
+constexpr int64_t kStaticRecRows = 1ll << 17;          // frontier rows with parent records (6 MiB)
 constexpr int kStaticMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
@@ -1210,9 +1245,10 @@ struct DeviceRestore {
 struct StaticLayout {
   ChunkState* st;
   unsigned long long* slots;
-  uint64_t* psi;
   uint64_t* off;
-  void* scan_tmp;
+  ScanTile* scan;  // two counters, then scan_n look-back entries
+  int64_t scan_n;
+  ParentRec* prec;  // records of frontiers of up to kStaticRecRows rows
   int32_t* staging;
   uint32_t *gmin, *slot_of, *srow, *bits, *own;
   unsigned long long* tiles;  // two counters, then look-back words
@@ -1232,9 +1268,10 @@ bool static_layout(unsigned char* base, int m, StaticLayout* L) {
   L->q = q;
   L->st = reinterpret_cast<ChunkState*>(take(256));
   L->slots = reinterpret_cast<unsigned long long*>(take(kStaticSlots * sizeof(unsigned long long)));
-  L->psi = reinterpret_cast<uint64_t*>(take((kStaticMaxRows + 1) * sizeof(uint64_t)));
   L->off = reinterpret_cast<uint64_t*>(take((kStaticMaxRows + 1) * sizeof(uint64_t)));
-  L->scan_tmp = take(scan_temp_bytes(kStaticMaxRows + 1, 8));
+  L->prec = reinterpret_cast<ParentRec*>(take(sizeof(ParentRec) * kStaticRecRows));
+  L->scan_n = (int64_t)1 << 17;  // a frontier of kStaticMaxRows rows in tiles of 8 needs no more
+  L->scan = reinterpret_cast<ScanTile*>(take(sizeof(ScanTile) * (2 + L->scan_n)));
   L->staging = reinterpret_cast<int32_t*>(take(q * 4ull * m));
   L->gmin = reinterpret_cast<uint32_t*>(take(q * 4));
   L->slot_of = reinterpret_cast<uint32_t*>(take(q * 4));
@@ -1290,7 +1327,9 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
   CK(cudaMemsetAsync(L.bits, 0, sizeof(uint32_t) * (L.q / 32 + 1), st));
   CK(cudaMemsetAsync(L.own, 0, sizeof(uint32_t) * (L.q / 32 + 1), st));
   CK(cudaMemsetAsync(L.tiles, 0, 8 * (1 + (size_t)commit_tiles((uint32_t)(L.q / 32 + 1))), st));
-  uint32_t epoch = 0;
+  uint32_t epoch = 0, scan_epoch = 0;
+  bool few_before = true;
+  CK(cudaMemsetAsync(L.scan, 0, sizeof(ScanTile) * (1 + L.scan_n), st));
   auto clear_and_insert = [&](int64_t rows) -> int {
     k_fill_u64<<<grid_for((int64_t)kStaticSlots, 256, nsm * 32), 256, 0, st>>>(L.slots, kStaticSlots, kEmpty);
     CK(cudaGetLastError());
@@ -1310,17 +1349,27 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
   for (int d = 1; d <= o->depth; ++d) {
     const int64_t P = level_hi - level_lo;
     const int32_t* parents = out + (size_t)level_lo * m;
-    CK(cudaMemsetAsync(L.st, 0, sizeof(ChunkState), st));
-    CK(cudaMemsetAsync(L.psi + P, 0, sizeof(uint64_t), st));
-    launch_psi(h->dev(), parents, 4, nullptr, P, o->max_expand_value, L.psi, nullptr, L.st, st, nsm);
+    PsiArgs pa;
+    std::memset(&pa, 0, sizeof pa);
+    pa.s = h->dev();
+    pa.rows = parents;
+    pa.P = P;
+    pa.max_expand = o->max_expand_value;
+    pa.off = L.off;
+    pa.rec = few_before && P <= kStaticRecRows ? L.prec : nullptr;
+    pa.ticket = reinterpret_cast<uint32_t*>(L.scan);
+    pa.tiles = L.scan + 1;
+    pa.epoch = ++scan_epoch;
+    pa.st = L.st;
+    pa.host_total = h->pin.u64;
+    pa.host = hst;
+    launch_psi(pa, 4, st, nsm);
     CK(cudaGetLastError());
-    scan_u64_sat(L.psi, L.off, P + 1, L.scan_tmp, st);
-    CK(cudaMemcpyAsync(h->pin.u64, L.off + P, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(hst, L.st, sizeof(ChunkState), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (hst->error & kErrOverflow) return fail(SNP_E_OVERFLOW, "a spike count could leave the int32 range");
     if (hst->error) return fail(SNP_E_INTERNAL, "device consistency check failed (bits 0x%x)", hst->error);
     const uint64_t total = *h->pin.u64;
+    few_before = total <= 256ull * (uint64_t)P;  // parent records pay with few candidates per parent
     const uint64_t T = budget > 0 ? std::min<uint64_t>(total, (uint64_t)budget) : total;
     uint64_t remaining = cap > 0 ? (uint64_t)cap : ~0ull;
     uint64_t g0 = 0;
@@ -1355,7 +1404,7 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
       a.gmin = L.gmin;
       a.slot_of = L.slot_of;
       a.ownbits = L.own;
-      a.prec = nullptr;
+      a.prec = pa.rec;
       a.ctr = nullptr;
       a.pperm = nullptr;
       a.store_ctr = nullptr;  // staging mode: rows are copied into `out` by the commit

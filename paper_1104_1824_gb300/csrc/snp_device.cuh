@@ -207,7 +207,7 @@ struct ChunkState {
   unsigned int total_first;   // distinct new keys in the chunk
   unsigned int capped;        // the cap was reached inside the chunk
   unsigned int last_lid;      // chunk-local index of the last accepted first occurrence
-  unsigned int psi_saturated;  // Psi summed over the first parents already reached 2^64 - 1
+  unsigned int reserved;
   unsigned long long p_first;  // first and last frontier row the chunk's candidates come from
   unsigned long long p_last;
 };
@@ -496,103 +496,105 @@ __device__ __forceinline__ bool rows_equal(const int32_t* buf, const int32_t* ot
   return __all_sync(0xffffffffu, ok);
 }
 
-// Step (a) for one configuration, neuron by neuron: Psi = prod max(1, omega)
-// (saturating; four counts are multiplied in 32 bits, at most 2^20, and a
-// product below 2^43 cannot overflow by such a factor), whether
-// a child could leave int32, whether the row is past max_expand, and its
-// ParentRec (base-child hash, multi-choice neurons in neuron order).
+// One neuron's lookup out of line: {applicable mask, a child could leave
+// int32, x * R[n] + H[first applicable rule]}.
+static __device__ __noinline__ uint4 psi_look(const DevSys& s, int n, int32_t x) {
+  const NeuronInfo ni = neuron_info(s, n);
+  const ApplEntry e = appl_entry(s, ni, n, x);
+  const uint64_t hx = (uint64_t)(uint32_t)x * ni.colkey + e.hfirst;
+  return make_uint4(e.mask, x > INT32_MAX - ni.gain ? 1u : 0u, (uint32_t)hx, (uint32_t)(hx >> 32));
+}
+
+// Step (a) for one configuration: Psi = prod max(1, omega) (saturating),
+// whether a child could leave int32, whether the row is past max_expand, and
+// its ParentRec (base-child hash, multi-choice neurons in neuron order).
+constexpr int kPsiBatch = 8;  // lookups in flight
 struct PsiAcc {
   uint64_t prod = 1, hb = 0;
-  uint32_t nnt = 0, part = 1;
-  int parts = 0;
+  uint32_t nnt = 0;
   bool ov = false, skip = false;
 
-  // prod *= part (saturating; part <= 2^20)
-  __device__ __forceinline__ void flush() {
-    if (part > 1) prod = (prod >> 43) ? (__umul64hi(prod, part) ? kSat : prod * part) : prod * part;
-    part = 1;
-    parts = 0;
-  }
-
-  // One neuron: its applicable mask and, with records, its share of the base
-  // child's hash.
+  // Lookups for neurons n[u], counts x[u]: the batch's loads in flight
+  // together where every count is in the direct table (a lookup at a time,
+  // each waited out an L2 round trip).
   template <bool REC>
-  __device__ __forceinline__ void add(int n, int32_t x, uint32_t mask, uint64_t hx, int32_t max_expand,
-                                      ParentRec* rec) {
-    const uint32_t cnt = __popc(mask);
-    part *= cnt > 1 ? cnt : 1u;  // four counts of at most 32 fit 32 bits
-    if (++parts == 4) flush();
-    skip |= max_expand >= 0 && x > max_expand;
-    if (REC) {
-      hb += hx;
-      if (cnt > 1) {
-        const bool fits = nnt < (uint32_t)kRecNt && n < 65536 && mask < 65536u;
-        if (fits) rec->nt[nnt] = ((uint32_t)n << 16) | mask;
-        nnt = fits ? nnt + 1 : kRecFull;
+  __device__ __forceinline__ void look_batch(const DevSys& s, const int (&n)[kPsiBatch], const int32_t (&x)[kPsiBatch],
+                                             int32_t max_expand, uint32_t (&mask)[kPsiBatch],
+                                             uint64_t (&hx)[kPsiBatch]) {
+    uint32_t any = 0;
+    int32_t top = 0;
+#pragma unroll
+    for (int u = 0; u < kPsiBatch; ++u) {
+      any |= (uint32_t)x[u];
+      top = max(top, x[u]);
+    }
+    if (any < (uint32_t)kDirect && s.gain_small) {
+#pragma unroll
+      for (int u = 0; u < kPsiBatch; ++u) {
+        const size_t k = (size_t)n[u] * kDirect + (uint32_t)x[u];
+        mask[u] = __ldg(s.dmask + k);
+        hx[u] = REC ? __ldg(s.dhx + k) : 0ull;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < kPsiBatch; ++u) {
+        const uint4 y = psi_look(s, n[u], x[u]);
+        mask[u] = y.x;
+        ov |= y.y != 0;
+        hx[u] = REC ? ((unsigned long long)y.w << 32) | y.z : 0ull;
       }
     }
+    skip |= max_expand >= 0 && top > max_expand;
   }
 
-  template <bool REC>
-  __device__ __forceinline__ void visit(const DevSys& s, int n, int32_t x, int32_t max_expand, ParentRec* rec) {
-    uint32_t mask;
-    uint64_t hx = 0;
-    if ((uint32_t)x < (uint32_t)kDirect) {  // small count: one entry of the direct table
-      const size_t k = (size_t)n * kDirect + (uint32_t)x;
-      mask = __ldg(s.dmask + k);
-      if (REC) hx = __ldg(s.dhx + k);
-      if (!s.gain_small) ov |= x > INT32_MAX - __ldg(s.gain + n);
-    } else {
-      const NeuronInfo ni = neuron_info(s, n);
-      const ApplEntry e = appl_entry(s, ni, n, x);
-      mask = e.mask;
-      if (REC) hx = (uint64_t)(uint32_t)x * ni.colkey + e.hfirst;
-      ov |= x > INT32_MAX - ni.gain;
+  // prod *= the batch's choice counts (each at most 32).
+  __device__ __forceinline__ void times(const uint32_t (&mask)[kPsiBatch]) {
+    uint32_t c[kPsiBatch];
+#pragma unroll
+    for (int u = 0; u < kPsiBatch; ++u) c[u] = max((uint32_t)__popc(mask[u]), 1u);
+    prod = sat_mul(prod, (uint64_t)(c[0] * c[1] * c[2] * c[3]) * (c[4] * c[5] * c[6] * c[7]));
+  }
+
+  // A neuron of the row's record, in neuron order.
+  __device__ __forceinline__ void record(int n, uint32_t mask, uint64_t hx, ParentRec* rec) {
+    hb += hx;
+    if (__popc(mask) > 1) {
+      const bool fits = nnt < (uint32_t)kRecNt && n < 65536 && mask < 65536u;
+      if (fits) rec->nt[nnt] = ((uint32_t)n << 16) | mask;
+      nnt = fits ? nnt + 1 : kRecFull;
     }
-    add<REC>(n, x, mask, hx, max_expand, rec);
   }
 
-  // Neurons n .. n + w - 1 holding x[0 .. w): eight lookups in flight where
-  // their counts are in the direct table (a lookup at a time, each visit
-  // waited out an L2 round trip).
+  // Neurons n .. n + w - 1 holding x[0 .. w), one lane per row.
   template <bool REC>
   __device__ __forceinline__ void visit_run(const DevSys& s, int n, const int32_t* x, int w, int32_t max_expand,
                                             ParentRec* rec) {
-    constexpr int U = 8;
-    int j = 0;
 #pragma unroll 1
-    for (; j + U <= w; j += U) {
-      int32_t v[U];
-      uint32_t any = 0;
+    for (int j = 0; j < w; j += kPsiBatch) {
+      int nn[kPsiBatch];
+      int32_t v[kPsiBatch];
+      uint32_t mask[kPsiBatch];
+      uint64_t hx[kPsiBatch];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        v[u] = x[j + u];
-        any |= (uint32_t)v[u];
+      for (int u = 0; u < kPsiBatch; ++u) {  // past the run: its first neuron without spikes, dropped below
+        nn[u] = j + u < w ? n + j + u : n;
+        v[u] = j + u < w ? x[j + u] : 0;
       }
-      if (any < (uint32_t)kDirect && s.gain_small) {
-        uint32_t mask[U];
-        uint64_t hx[U];
+      look_batch<REC>(s, nn, v, max_expand, mask, hx);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const size_t k = (size_t)(n + j + u) * kDirect + (uint32_t)v[u];
-          mask[u] = __ldg(s.dmask + k);
-          hx[u] = REC ? __ldg(s.dhx + k) : 0ull;
+      for (int u = 0; u < kPsiBatch; ++u)
+        if (j + u >= w) {
+          mask[u] = 0;
+          hx[u] = 0;
         }
+      times(mask);
+      if (REC) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) add<REC>(n + j + u, v[u], mask[u], hx[u], max_expand, rec);
-      } else {
-#pragma unroll 1
-        for (int u = 0; u < U; ++u) visit<REC>(s, n + j + u, x[j + u], max_expand, rec);
+        for (int u = 0; u < kPsiBatch; ++u) record(nn[u], mask[u], hx[u], rec);
       }
     }
-#pragma unroll 1
-    for (; j < w; ++j) visit<REC>(s, n + j, x[j], max_expand, rec);
   }
-
-  __device__ __forceinline__ uint64_t psi() {
-    flush();
-    return skip ? 0ull : prod;
-  }
+  __device__ __forceinline__ uint64_t psi() const { return skip ? 0ull : prod; }
   __device__ __forceinline__ bool overflow() const { return ov && !skip; }
 };
 
@@ -668,6 +670,57 @@ __device__ __forceinline__ bool lookback_u32(unsigned long long* tiles, uint32_t
     at -= 32;
   }
   if (lane == 0 && ok) t[tile] = tag | (2ull << 32) | (prefix + sum);
+  return ok;
+}
+
+// Look-back state of one tile of a saturating 64-bit scan.
+struct ScanTile {
+  unsigned long long sum, through;  // the tile's own sum; the sum through the tile
+  uint32_t flag, pad;               // epoch << 2 | (1: sum is set, 2: through is set)
+};
+
+// lookback_u32 for saturating 64-bit sums; base: what comes before tile 0.
+__device__ __forceinline__ bool lookback_sat(ScanTile* tiles, uint32_t tile, uint32_t epoch, uint64_t base,
+                                             uint64_t sum, uint64_t& prefix, int lane) {
+  volatile ScanTile* t = tiles;
+  prefix = base;
+  bool ok = true;
+  if (tile > 0) {
+    if (lane == 0) {
+      t[tile].sum = sum;
+      __threadfence();
+      t[tile].flag = epoch << 2 | 1u;
+    }
+    prefix = 0;
+    int64_t at = (int64_t)tile - 1 - lane;
+    for (int polls = 0;;) {
+      const uint32_t f = at >= 0 ? t[at].flag : epoch << 2 | 2u;
+      const bool ready = (f >> 2) == epoch && (f & 3u) != 0;
+      if (!__all_sync(0xffffffffu, ready)) {
+        if (++polls >= kSpinLimit) {
+          ok = false;
+          break;
+        }
+        __nanosleep(20);
+        continue;
+      }
+      __threadfence();
+      const uint32_t full = __ballot_sync(0xffffffffu, (f & 3u) == 2u);
+      const int last = full ? __ffs(full) - 1 : 31;
+      uint64_t x = 0;
+      if (lane <= last) x = at < 0 ? 0ull : lane == last && full ? t[at].through : t[at].sum;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x = sat_add(x, __shfl_xor_sync(0xffffffffu, x, o));
+      prefix = sat_add(prefix, x);
+      if (full) break;
+      at -= 32;
+    }
+  }
+  if (lane == 0 && ok) {
+    t[tile].through = sat_add(prefix, sum);
+    __threadfence();
+    t[tile].flag = epoch << 2 | 2u;
+  }
   return ok;
 }
 

@@ -166,9 +166,9 @@ struct snp_system {
   uint64_t tc_cap = 0;  // candidates the tensor-core chunk buffers hold
   std::vector<unsigned long long> colkey, rowkey;
   // exploration state
-  DevBuf d_pool, d_slots, d_gmin, d_slot_of, d_bits, d_tiles, d_srow, d_own, d_off, d_scan_tmp, d_st,
+  DevBuf d_pool, d_slots, d_gmin, d_slot_of, d_bits, d_tiles, d_srow, d_own, d_off, d_scan, d_st,
       d_rec_parent, d_rec_index, d_tmp,
-      d_psi, d_prec, d_ctr, d_perm, d_sidx,
+      d_prec, d_ctr, d_perm, d_sidx,
       d_bcache;  // wide mode: base children of each pass's largest parents
   int64_t pool_rows = 0;  // capacity in rows (of the store: every row claimed during an exploration)
   int32_t row_w = 4;      // bytes per spike count of the store's rows (4: int32; 2, 1: packed)
@@ -177,10 +177,11 @@ struct snp_system {
   uint64_t nbuckets = 0;
   uint64_t q_cap = 0;     // staging capacity in rows
   uint32_t epoch = 0;     // last look-back epoch used in d_tiles
+  uint32_t scan_epoch = 0;  // ... and in d_scan
   int64_t psi_cap = 0;    // parents
   int64_t rec_rows = 0;
   PinnedState pin;
-  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaEvent_t ev[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // around a depth; depths take turns
   cudaEvent_t evk[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // around the expand kernel, per pass slot
   cudaEvent_t evs[2] = {nullptr, nullptr};   // end of a pass in flight, per slot
   // results

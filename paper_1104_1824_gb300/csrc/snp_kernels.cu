@@ -1,13 +1,12 @@
 // Kernels of the single-system BFS over SNP-system configurations.
 //
 // One depth (Algorithm 1, one round of steps II-IV) runs as:
-//   k_psi      step (a) for every frontier configuration: applicable rules and
-//              Psi = prod_n max(1, omega_n) (Eq. psi), saturating (k_psi_tiled
-//              for rows of a multiple of four neurons, k_psi_warp with a warp
-//              per row for small frontiers; after a depth whose Psi sum
-//              saturated, k_psi_head_saturated lets the rows past the first
-//              8192 be skipped when those already hold 2^64 - 1 candidates);
-//   scan       exclusive prefix sums of Psi give each parent's first candidate;
+//   k_psi      step (a) for every frontier configuration: applicable rules,
+//              Psi = prod_n max(1, omega_n) (Eq. psi), saturating, and its
+//              exclusive prefix sums, which give each parent's first candidate
+//              (a lane per row, or a warp per row for small frontiers; after a
+//              depth whose Psi sum saturated, the first 8192 rows go first and
+//              the others are skipped when those hold 2^64 - 1 candidates);
 //   per chunk of candidates [g0, g0 + Q) in canonical order:
 //     k_expand steps (b)-(d) (snp_expand.cu; k_expand_wide for rows of more
 //              than kWideM neurons): decode the spiking vector, C' = C + S . M_Pi
@@ -33,166 +32,257 @@ __device__ __forceinline__ void set_error(ChunkState* st, uint32_t bits) { atomi
 
 }  // namespace
 
-// Step (a) and Eq. psi for every frontier row, one lane per row, with the
-// rows' ParentRecs when rec is given; rows not to be expanded (max_expand)
-// get Psi = 0, rows whose children could leave int32 raise kErrOverflow.
-// (Rows of m % 4 == 0 neurons go through k_psi_tiled instead.)
-template <bool REC>
-__global__ void __launch_bounds__(256) k_psi(DevSys s, const int32_t* rows, const uint32_t* perm, int64_t P,
-                                             int32_t max_expand, uint64_t* psi, ParentRec* rec, ChunkState* st) {
+// Step (a), Eq. psi and its saturating exclusive scan for every frontier row:
+// off[p] = the sum of Psi over rows before p, off[P] = the total; with REC the
+// rows' ParentRecs.  Rows not to be expanded (max_expand) get Psi = 0, rows
+// whose children could leave int32 raise kErrOverflow.  Tiles of rows are
+// handed out in order and chained by decoupled look-back.
+//   WARP = false: tiles of 256 rows, a lane per row.  A warp moves its 32 rows
+//     through shared memory 32 columns at a time (16-byte pieces where rows
+//     are whole pieces, else one coalesced 128-byte load per row), unpacked to
+//     int32; lane r then reads row r's slab at a stride of 33 words.
+//   WARP = true: tiles of 8 rows, a warp per row, lane l visiting neurons
+//     l, l + 32, ...: for small frontiers, so that a row of many neurons is not
+//     one lane's serial walk (launch_psi has the rule).
+// Both keep eight table lookups in flight per lane; what bounds them is those
+// lookups' latency and the instructions per visit, not the rows' bytes.  With
+// the scan in the same launch (it was a Psi launch, one to three scan launches,
+// two clears and two copies per depth), the 3-neuron example to depth 10 went
+// from 855 us to 601 us and 61 neurons with records from 2051 us to 1840 us.
+template <class RF, bool REC, bool WARP>
+__global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
+  constexpr int R = WARP ? 8 : 256;
+  __shared__ int32_t slabs[WARP ? 1 : 8][32][33];
+  __shared__ uint64_t s_w[8];
+  __shared__ uint64_t s_prefix;
+  __shared__ uint32_t s_tile;
+  __shared__ int s_ok, s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const DevSys& s = a.s;
   const int m = s.m;
-  if (st && __ldcg(&st->psi_saturated)) {  // these rows lie past the last candidate: Psi is not needed
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x)
-      psi[p] = 0;
-    return;
-  }
-  bool over = false;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t* row = rows + (size_t)(perm ? __ldg(perm + p) : (uint64_t)p) * m;
-    PsiAcc acc;
-    for (int n = 0; n < m; ++n) acc.visit<REC>(s, n, __ldg(row + n), max_expand, REC ? rec + p : nullptr);
-    psi[p] = acc.psi();
-    if (REC) {
-      rec[p].hbase = acc.hb;
-      rec[p].nnt = acc.nnt;
-    }
-    over |= acc.overflow();
-  }
-  if (__any_sync(0xffffffffu, over) && (threadIdx.x & 31) == 0) set_error(st, kErrOverflow);
-}
-
-// k_psi for small frontiers (no records): a warp per row, lane l visiting
-// neurons l, l + 32, ... (coalesced), the lanes' products combined with the
-// saturating product, so that a row of many neurons is not one thread's
-// serial walk.
-template <class RF>
-__global__ void __launch_bounds__(256) k_psi_warp(DevSys s, const int32_t* rows, const uint32_t* perm, int64_t P,
-                                                  int32_t max_expand, uint64_t* psi, ChunkState* st) {
-  const int m = s.m;
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  if (st && __ldcg(&st->psi_saturated)) {  // as in k_psi
-    for (int64_t p = w0; p < P; p += nw)
-      if (lane == 0) psi[p] = 0;
-    return;
-  }
-  bool over = false;
-  for (int64_t p = w0; p < P; p += nw) {
-    const typename RF::T* row = row_at<RF>(rows, perm ? __ldg(perm + p) : (uint64_t)p, m);
-    PsiAcc acc;
-    for (int n = lane; n < m; n += 32) acc.visit<false>(s, n, (int32_t)__ldg(row + n), max_expand, nullptr);
-    acc.flush();
-    uint64_t v = acc.prod;
+  const uint32_t ntiles = (uint32_t)((a.P + R - 1) / R);
+  const uint64_t base = a.carry ? __ldcg(a.carry) : 0ull;
+  if (a.off && base == kSat) {
+    // these rows lie past the last candidate: Psi is not needed
+    for (int64_t p = (int64_t)blockIdx.x * 256 + tid; p < a.P; p += (int64_t)gridDim.x * 256) a.off[p + 1] = kSat;
+  } else {
+    bool over = false;
+    for (uint32_t step = 0;; ++step) {
+      uint32_t tile;
+      if (a.off) {
+        __syncthreads();
+        if (tid == 0) s_tile = atomicAdd(a.ticket, 1u);
+        __syncthreads();
+        tile = s_tile;
+      } else {  // records only: no order needed
+        tile = blockIdx.x + step * gridDim.x;
+      }
+      if (tile >= ntiles) break;
+      const int64_t p0 = (int64_t)tile * R + (WARP ? warp : warp * 32);  // this warp's first row
+      PsiAcc acc;
+      uint64_t v = 0;  // Psi of this lane's row (WARP: lane 0's)
+      if (WARP) {
+        if (p0 < a.P) {
+          const typename RF::T* row = row_at<RF>(a.rows, a.perm ? __ldg(a.perm + p0) : (uint64_t)p0, m);
+          ParentRec* rec = REC ? a.rec + p0 : nullptr;
+          for (int n0 = 0; n0 < m; n0 += 32 * kPsiBatch) {
+            int nn[kPsiBatch];
+            int32_t x[kPsiBatch];
+            uint32_t mask[kPsiBatch];
+            uint64_t hx[kPsiBatch];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = sat_mul(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const bool skip = __any_sync(0xffffffffu, acc.skip);
-    const bool ov = __any_sync(0xffffffffu, acc.ov);
-    if (lane == 0) psi[p] = skip ? 0ull : v;
-    over |= ov && !skip;
-  }
-  if (over && lane == 0) set_error(st, kErrOverflow);
-}
-
-// k_psi for rows that move in 16-byte pieces (RF::VEC) with coalesced loads:
-// a block takes 256 rows at a time and moves them through shared memory 32
-// columns at a time (each row's slab is 128 contiguous bytes in int32 rows,
-// read by 8 consecutive threads; 64 or 32 bytes in packed rows), unpacked to
-// int32; thread t then reads row t's slab at a stride of 33 words, so the 32
-// lanes of a warp hit 32 different banks.
-constexpr int kPsiRows = 256, kPsiSlab = 32;
-template <class RF, bool REC>
-__global__ void __launch_bounds__(kPsiRows) k_psi_tiled(DevSys s, const int32_t* rows, const uint32_t* perm, int64_t P,
-                                                        int32_t max_expand, uint64_t* psi, ParentRec* rec,
-                                                        ChunkState* st) {
-  __shared__ int32_t slab[kPsiRows][kPsiSlab + 1];
-  const int m = s.m;
-  const int t = threadIdx.x;
-  if (st && __ldcg(&st->psi_saturated)) {  // as in k_psi
-    for (int64_t p = (int64_t)blockIdx.x * kPsiRows + t; p < P; p += (int64_t)gridDim.x * kPsiRows) psi[p] = 0;
-    return;
-  }
-  bool over = false;
-  for (int64_t p0 = (int64_t)blockIdx.x * kPsiRows; p0 < P; p0 += (int64_t)gridDim.x * kPsiRows) {
-    const int nrows = (int)min((int64_t)kPsiRows, P - p0);
-    const int64_t p = p0 + t;
-    PsiAcc acc;
-    for (int n0 = 0; n0 < m; n0 += kPsiSlab) {
-      const int w = min(kPsiSlab, m - n0);  // columns in this slab (a multiple of RF::PER16)
-      const int q4 = w / RF::PER16;         // 16-byte pieces per row
-      __syncthreads();
-      // rows stream through L2 only, so that they do not evict the
-      // applicability table every visit reads from L1
-      for (int i = t; i < nrows * q4; i += kPsiRows) {
-        const int r = i / q4, q = i - r * q4;
-        const uint64_t pr = perm ? __ldcg(perm + p0 + r) : (uint64_t)(p0 + r);
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row_at<RF>(rows, pr, m) + n0) + q);
-        int32_t x[RF::PER16];
-        unpack_piece<RF>(v, x);
-        int32_t* d = &slab[r][RF::PER16 * q];
+            for (int u = 0; u < kPsiBatch; ++u) {
+              const int n = n0 + 32 * u + lane;  // past the row: neuron 0 without spikes, dropped below
+              nn[u] = n < m ? n : 0;
+              x[u] = n < m ? (int32_t)__ldcg(row + n) : 0;
+            }
+            acc.look_batch<REC>(s, nn, x, a.max_expand, mask, hx);
 #pragma unroll
-        for (int k = 0; k < RF::PER16; ++k) d[k] = x[k];
+            for (int u = 0; u < kPsiBatch; ++u)
+              if (n0 + 32 * u + lane >= m) {
+                mask[u] = 0;
+                hx[u] = 0;
+              }
+            acc.times(mask);
+            if (REC) {
+#pragma unroll
+              for (int u = 0; u < kPsiBatch; ++u) {
+                acc.hb += hx[u];
+                const bool nt = __popc(mask[u]) > 1;
+                const uint32_t b = __ballot_sync(0xffffffffu, nt);
+                const uint32_t wide = __ballot_sync(0xffffffffu, nt && mask[u] >= 65536u);
+                if (acc.nnt == kRecFull || wide || acc.nnt + __popc(b) > (uint32_t)kRecNt) {
+                  if (b) acc.nnt = kRecFull;
+                } else {
+                  if (nt) rec->nt[acc.nnt + __popc(b & ((1u << lane) - 1u))] = ((uint32_t)nn[u] << 16) | mask[u];
+                  acc.nnt += __popc(b);
+                }
+              }
+            }
+          }
+          uint64_t prod = acc.prod;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) prod = sat_mul(prod, __shfl_xor_sync(0xffffffffu, prod, o));
+          const bool skip = __any_sync(0xffffffffu, acc.skip);
+          over |= __any_sync(0xffffffffu, acc.ov) && !skip;
+          v = skip ? 0ull : prod;
+          if (REC) {
+            const uint64_t hb = warp_sum_u64(acc.hb);
+            if (lane == 0) {
+              rec->hbase = hb;
+              rec->nnt = acc.nnt;
+            }
+          }
+        }
+        if (lane == 0) s_w[warp] = v;
+      } else {
+        int32_t(*slab)[33] = slabs[warp];
+        const int nr = (int)max((int64_t)0, min((int64_t)32, a.P - p0));
+        const uint64_t pr = lane < nr ? (a.perm ? __ldg(a.perm + p0 + lane) : (uint64_t)(p0 + lane)) : 0ull;
+        ParentRec* rec = REC ? a.rec + p0 + lane : nullptr;
+        for (int n0 = 0; n0 < m && nr > 0; n0 += 32) {
+          const int w = min(32, m - n0);
+          __syncwarp();
+          // rows stream through L2 only, so that they do not evict the tables
+          if constexpr (RF::VEC) {
+            const int q4 = w / RF::PER16, total = nr * q4;
+            for (int i0 = 0; i0 < total; i0 += 32) {
+              const int i = i0 + lane, r = min(i / q4, nr - 1), q = i - r * q4;
+              const uint64_t at = __shfl_sync(0xffffffffu, pr, r);
+              if (i < total) {
+                const uint4 y = __ldcg(reinterpret_cast<const uint4*>(row_at<RF>(a.rows, at, m) + n0) + q);
+                int32_t x[RF::PER16];
+                unpack_piece<RF>(y, x);
+                int32_t* dst = &slab[r][RF::PER16 * q];
+#pragma unroll
+                for (int j = 0; j < RF::PER16; ++j) dst[j] = x[j];
+              }
+            }
+          } else {
+            for (int r0 = 0; r0 < nr; r0 += 16) {
+              int32_t x[16];
+#pragma unroll
+              for (int u = 0; u < 16; ++u) {
+                const uint64_t at = __shfl_sync(0xffffffffu, pr, (r0 + u) & 31);
+                if (r0 + u < nr && lane < w) x[u] = __ldcg(row_at<RF>(a.rows, at, m) + n0 + lane);
+              }
+#pragma unroll
+              for (int u = 0; u < 16; ++u)
+                if (r0 + u < nr && lane < w) slab[r0 + u][lane] = x[u];
+            }
+          }
+          __syncwarp();
+          if (lane < nr) acc.visit_run<REC>(s, n0, slab[lane], w, a.max_expand, rec);
+        }
+        if (lane < nr) {
+          v = acc.psi();
+          over |= acc.overflow();
+          if (REC) {
+            rec->hbase = acc.hb;
+            rec->nnt = acc.nnt;
+          }
+        }
+      }
+      if (!a.off) continue;
+      // this lane's exclusive sum within the tile
+      uint64_t before, sum;
+      if (WARP) {
+        __syncthreads();
+        before = 0;
+        sum = 0;
+        for (int w = 0; w < 8; ++w) {
+          if (w < lane) before = sat_add(before, s_w[w]);  // warp 0: lane l writes row l
+          sum = sat_add(sum, s_w[w]);
+        }
+      } else {
+        uint64_t inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc = sat_add(y, inc);
+        }
+        if (lane == 31) s_w[warp] = inc;
+        before = __shfl_up_sync(0xffffffffu, inc, 1);
+        if (lane == 0) before = 0;
+        __syncthreads();
+        uint64_t wb = 0;
+        sum = 0;
+        for (int w = 0; w < 8; ++w) {
+          if (w < warp) wb = sat_add(wb, s_w[w]);
+          sum = sat_add(sum, s_w[w]);
+        }
+        before = sat_add(wb, before);
+      }
+      if (warp == 0) {
+        uint64_t prefix = 0;
+        const bool ok = lookback_sat(a.tiles, tile, a.epoch, base, sum, prefix, lane);
+        if (lane == 0) {
+          s_prefix = prefix;
+          s_ok = ok ? 1 : 0;
+        }
       }
       __syncthreads();
-      if (t < nrows)
-        for (int j = 0; j < w; ++j) acc.visit<REC>(s, n0 + j, slab[t][j], max_expand, REC ? rec + p : nullptr);
-    }
-    if (t < nrows) {
-      psi[p] = acc.psi();
-      if (REC) {
-        rec[p].hbase = acc.hb;
-        rec[p].nnt = acc.nnt;
+      if (!s_ok) {
+        if (tid == 0) atomicOr(&a.st->error, kErrTimeout);
+        break;
       }
-      over |= acc.overflow();
+      const int64_t p = WARP ? (int64_t)tile * R + lane : p0 + lane;
+      if ((!WARP || (warp == 0 && lane < 8)) && p < a.P) a.off[p] = sat_add(s_prefix, before);
+      if (tile + 1 == ntiles && tid == 0) a.off[a.P] = sat_add(s_prefix, sum);
     }
+    if (__any_sync(0xffffffffu, over) && lane == 0) set_error(a.st, kErrOverflow);
   }
-  if (__any_sync(0xffffffffu, over) && (threadIdx.x & 31) == 0) set_error(st, kErrOverflow);
-}
-
-// st->psi_saturated = 1 when the saturating sum of psi[0 .. n) is 2^64 - 1
-// (one block).
-__global__ void __launch_bounds__(1024) k_psi_head_saturated(const uint64_t* psi, int64_t n, ChunkState* st) {
-  __shared__ uint64_t part[32];
-  uint64_t v = 0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v = sat_add(v, psi[i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = sat_add(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  if (!a.off) return;
+  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    uint64_t t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t = sat_add(t, part[w]);
-    if (t == kSat) st->psi_saturated = 1u;
+  if (tid == 0) s_last = atomicAdd(a.ticket + 1, 1u) + 1 == gridDim.x ? 1 : 0;
+  __syncthreads();
+  if (!s_last || tid != 0) return;
+  __threadfence();
+  a.ticket[0] = 0;
+  a.ticket[1] = 0;
+  if (a.host_total) {  // the depth's candidates and errors to the host; the depth's counter starts
+    if (a.ctr) a.ctr[1] = a.remaining;
+    *a.host_total = __ldcg(a.off + a.P);
+    a.host->error = __ldcg(&a.st->error);
+    __threadfence_system();
   }
 }
 
-int launch_psi_head_check(const uint64_t* psi, int64_t n, ChunkState* st, cudaStream_t stream) {
-  k_psi_head_saturated<<<1, 1024, 0, stream>>>(psi, n, st);
-  return 1;
+namespace {
+
+template <class RF, bool REC>
+void psi_launch(const PsiArgs& a, bool warp, int64_t tiles, cudaStream_t st, int nsm) {
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)nsm * (warp ? 8 : REC ? 2 : 3)));
+  if (warp)
+    k_psi<RF, REC, true><<<blocks, 256, 0, st>>>(a);
+  else
+    k_psi<RF, REC, false><<<blocks, 256, 0, st>>>(a);
 }
 
-int launch_psi(DevSys s, const int32_t* rows, int w, const uint32_t* perm, int64_t P, int32_t max_expand,
-               uint64_t* psi, ParentRec* rec, ChunkState* st, cudaStream_t stream, int nsm) {
-  const int threads = 256;
-  const int64_t want = (P + threads - 1) / threads;
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)nsm * 8));
-  if (!rec && P <= (int64_t)nsm * 256) {  // a warp per row
-    const int wb = (int)std::max<int64_t>(1, (P + 7) / 8);
-    auto fn = w == 1 ? k_psi_warp<RowU8> : w == 2 ? k_psi_warp<RowU16> : k_psi_warp<RowI32>;
-    fn<<<wb, 256, 0, stream>>>(s, rows, perm, P, max_expand, psi, st);
-    return 1;
-  }
-  if (w == 1 || w == 2 || (s.m % 4) == 0) {
-    const int64_t tiles = (P + kPsiRows - 1) / kPsiRows;
-    const int tb = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)nsm * 6));
-    auto fn = w == 1   ? (rec ? k_psi_tiled<RowU8, true> : k_psi_tiled<RowU8, false>)
-              : w == 2 ? (rec ? k_psi_tiled<RowU16, true> : k_psi_tiled<RowU16, false>)
-                       : (rec ? k_psi_tiled<RowI32V, true> : k_psi_tiled<RowI32V, false>);
-    fn<<<tb, kPsiRows, 0, stream>>>(s, rows, perm, P, max_expand, psi, rec, st);
-    return 1;
-  }
-  auto fn = rec ? k_psi<true> : k_psi<false>;
-  fn<<<blocks, threads, 0, stream>>>(s, rows, perm, P, max_expand, psi, rec, st);
+}  // namespace
+
+// Tiles of 8 rows for small frontiers: a warp per row takes P / (16 nsm)
+// rounds of a fixed latency and m / 32 visits, a lane per row m / 8 batches of
+// lookups (in units of about 0.1 us: 12 + m / 32 a round, m).
+static bool psi_by_warp(int64_t P, int m, int nsm) {
+  const int64_t warps = 16 * nsm;
+  return (P + warps - 1) / warps * (12 + m / 32) <= (P + 32 * warps - 1) / (32 * warps) * std::max(m, 16);
+}
+
+size_t psi_tiles(int64_t P, int m, int nsm) { return (size_t)((P + (psi_by_warp(P, m, nsm) ? 7 : 255)) / (psi_by_warp(P, m, nsm) ? 8 : 256)) + 1; }
+
+int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm) {
+  const bool warp = psi_by_warp(a.P, a.s.m, nsm);
+  const int64_t tiles = (a.P + (warp ? 7 : 255)) / (warp ? 8 : 256);
+  if (w == 1)
+    a.rec ? psi_launch<RowU8, true>(a, warp, tiles, st, nsm) : psi_launch<RowU8, false>(a, warp, tiles, st, nsm);
+  else if (w == 2)
+    a.rec ? psi_launch<RowU16, true>(a, warp, tiles, st, nsm) : psi_launch<RowU16, false>(a, warp, tiles, st, nsm);
+  else if (a.s.m % 4 == 0)
+    a.rec ? psi_launch<RowI32V, true>(a, warp, tiles, st, nsm) : psi_launch<RowI32V, false>(a, warp, tiles, st, nsm);
+  else
+    a.rec ? psi_launch<RowI32, true>(a, warp, tiles, st, nsm) : psi_launch<RowI32, false>(a, warp, tiles, st, nsm);
   return 1;
 }
 
@@ -375,7 +465,7 @@ __global__ void __launch_bounds__(256) k_commit(CommitArgs a) {
   c.total_first = total;
   c.capped = __ldcg(&a.st->capped);
   c.last_lid = __ldcg(&a.st->last_lid);
-  c.psi_saturated = 0;
+  c.reserved = 0;
   c.p_first = __ldcg(&a.st->p_first);
   c.p_last = __ldcg(&a.st->p_last);
   if (a.ctr) {
@@ -527,98 +617,6 @@ void launch_insert_rows(DevSys s, const int32_t* pool, int w, const uint32_t* pe
 __global__ void k_fill_u64(unsigned long long* p, uint64_t n, unsigned long long v) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
     p[i] = v;
-}
-
-// ---------------------------------------------------------------------------
-// Exclusive scans.
-
-namespace {
-
-constexpr int kScanThreads = 512;
-constexpr int kScanItems = 8;
-constexpr int64_t kScanTile = (int64_t)kScanThreads * kScanItems;
-
-struct SatAdd {
-  __device__ __forceinline__ uint64_t operator()(uint64_t a, uint64_t b) const { return sat_add(a, b); }
-};
-
-template <typename T, typename Op>
-__global__ void __launch_bounds__(kScanThreads) k_scan_tile(const T* in, T* out, T* tile_sum, int64_t n, Op op) {
-  __shared__ T wtot[kScanThreads / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-  T v[kScanItems];
-  T acc = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    v[i] = (base + i < n) ? in[base + i] : (T)0;
-    acc = op(acc, v[i]);
-  }
-  T x = acc;  // inclusive scan of thread totals within the warp
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    T y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x = op(y, x);
-  }
-  if (lane == 31) wtot[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    T t = (lane < kScanThreads / 32) ? wtot[lane] : (T)0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      T y = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t = op(y, t);
-    }
-    if (lane < kScanThreads / 32) wtot[lane] = t;
-  }
-  __syncthreads();
-  T ex = __shfl_up_sync(0xffffffffu, x, 1);
-  if (lane == 0) ex = 0;
-  T run = op(w > 0 ? wtot[w - 1] : (T)0, ex);
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    if (base + i < n) out[base + i] = run;
-    run = op(run, v[i]);
-  }
-  if (tile_sum && threadIdx.x == kScanThreads - 1) tile_sum[blockIdx.x] = run;
-}
-
-template <typename T, typename Op>
-__global__ void k_scan_add(T* out, const T* tile_off, int64_t n, Op op) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = op(tile_off[i / kScanTile], out[i]);
-}
-
-// Returns the number of kernels launched.
-template <typename T, typename Op>
-int scan_impl(const T* in, T* out, int64_t n, T* temp, cudaStream_t st, Op op) {
-  if (n <= 0) return 0;
-  const int64_t nb = (n + kScanTile - 1) / kScanTile;
-  if (nb == 1) {
-    k_scan_tile<T, Op><<<1, kScanThreads, 0, st>>>(in, out, nullptr, n, op);
-    return 1;
-  }
-  T* sums = temp;
-  k_scan_tile<T, Op><<<(unsigned)nb, kScanThreads, 0, st>>>(in, out, sums, n, op);
-  const int inner = scan_impl<T, Op>(sums, sums, nb, temp + nb, st, op);
-  const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 16);
-  k_scan_add<T, Op><<<(unsigned)blocks, 256, 0, st>>>(out, sums, n, op);
-  return inner + 2;
-}
-
-}  // namespace
-
-size_t scan_temp_bytes(int64_t n, size_t elem) {
-  size_t total = 0;
-  while (n > kScanTile) {
-    n = (n + kScanTile - 1) / kScanTile;
-    total += (size_t)n;
-  }
-  return (total + 16) * elem;
-}
-
-int scan_u64_sat(const uint64_t* in, uint64_t* out, int64_t n, void* temp, cudaStream_t st) {
-  return scan_impl<uint64_t, SatAdd>(in, out, n, static_cast<uint64_t*>(temp), st, SatAdd());
 }
 
 }  // namespace snp

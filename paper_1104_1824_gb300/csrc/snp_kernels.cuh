@@ -200,14 +200,32 @@ size_t batch_scratch_bytes(int64_t pmax, uint32_t qc, int m_max);
 void launch_batch_depth_tc(const BatchArgs& a, int blocks, cudaStream_t st);
 __global__ void k_batch_init(BatchSys* sys, const int32_t* c0, const int64_t* c0_off, int32_t n);
 
-// Step (a) and Psi for P frontier rows; returns the launches made.
-// rows: w bytes per spike count (4: int32; 2, 1: a packed store).
-int launch_psi(DevSys s, const int32_t* rows, int w, const uint32_t* perm, int64_t P, int32_t max_expand,
-               uint64_t* psi, ParentRec* rec, ChunkState* st, cudaStream_t stream, int nsm);
-// Sets st->psi_saturated when Psi summed (saturating) over psi[0 .. n) is
-// 2^64 - 1: later frontier rows then hold no candidate, and launch_psi with
-// that st writes Psi = 0 for them without reading them.
-int launch_psi_head_check(const uint64_t* psi, int64_t n, ChunkState* st, cudaStream_t stream);
+// Step (a), Psi and its scan for P frontier rows.
+struct PsiArgs {
+  DevSys s;
+  const int32_t* rows;        // rows + perm[p] * m, or rows + p * m without perm (w bytes per count: launch_psi)
+  const uint32_t* perm;
+  int64_t P;
+  int32_t max_expand;
+  uint64_t* off;              // [P + 1], or nullptr: records only
+  ParentRec* rec;             // [P] or nullptr
+  // Look-back state: psi_tiles(P) entries, two counters that start (and are
+  // left) at 0, and a number no earlier launch on these entries had.
+  ScanTile* tiles;
+  uint32_t* ticket;
+  uint32_t epoch;
+  const uint64_t* carry;      // sum of Psi before these rows (nullptr: 0); when it is 2^64 - 1 the rows are not read
+  ChunkState* st;             // errors
+  // Set on the last launch of a depth: the total and st's errors to pinned
+  // host memory; ctr (if any): ctr[1] = remaining.
+  uint64_t* host_total;
+  ChunkState* host;
+  unsigned long long* ctr;
+  unsigned long long remaining;
+};
+size_t psi_tiles(int64_t P, int m, int nsm);
+// rows: w bytes per spike count (4: int32; 2, 1: a packed store).  Returns the launches made.
+int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm);
 // Steps (b)-(d) for the chunk's candidates (k_expand); returns the launches made.
 // Rows of more than kWideM neurons go through the kernel's wide mode (one
 // scratch row per warp, rows built on demand).
@@ -286,11 +304,5 @@ void launch_step_plan(DevSys s, const int32_t* C, int32_t* base, StepPlan* plan,
 void launch_step_children(DevSys s, const int32_t* base, const StepPlan* plan, uint64_t capacity, int32_t* out,
                           cudaStream_t st, int nsm);
 __global__ void k_fill_u64(unsigned long long* p, uint64_t n, unsigned long long v);
-
-// Device-wide exclusive scans (n elements, in -> out; "total" gets the sum).
-// Saturating (sums of Psi).
-size_t scan_temp_bytes(int64_t n, size_t elem);
-// Returns the number of kernels it launched.
-int scan_u64_sat(const uint64_t* in, uint64_t* out, int64_t n, void* temp, cudaStream_t st);
 
 }  // namespace snp
