@@ -741,6 +741,10 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     const int64_t P = level_hi - level_lo;
     sd.parents = P;
     CK(cudaEventRecord(h->ev[d & 1][0], st));
+    // When the previous depth's Psi sum saturated, the first rows alone may
+    // hold 2^64 - 1 candidates: they go first, and if they do, the rest are
+    // not read (no candidate and no statistic depends on them).
+    const int64_t P0 = psi_saturated_before && P > 2 * kPsiHead ? kPsiHead : P;
     {  // buffers of the frontier: when capped, once for all depths
       const int64_t want = cap > 0 ? std::max<int64_t>(P, std::min<int64_t>(cap, 1 << 22)) : P;
       if (h->psi_cap < P) {
@@ -748,7 +752,9 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         TRY(h->d_off.reserve(sizeof(uint64_t) * (want + 1)));
         h->psi_cap = want;
       }
-      const size_t tiles = sizeof(ScanTile) * (1 + psi_tiles(P, m, nsm));  // two counters, entries
+      // two counters, then the entries of the largest of the depth's launches
+      const size_t tiles =
+          sizeof(ScanTile) * (1 + std::max({psi_tiles(P, m, nsm), psi_tiles(P0, m, nsm), psi_tiles(P - P0, m, nsm)}));
       if (h->d_scan.bytes < tiles) {
         TRY(h->d_scan.reserve(std::max(tiles, sizeof(ScanTile) * 8192)));
         h->scan_epoch = 0x3FFFFFFFu;  // clear it below
@@ -789,10 +795,6 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
       CK(cudaGetLastError());
       return SNP_OK;
     };
-    // When the previous depth's Psi sum saturated, the first rows alone may
-    // hold 2^64 - 1 candidates: they go first, and if they do, the rest are
-    // not read (no candidate and no statistic depends on them).
-    const int64_t P0 = psi_saturated_before && P > 2 * kPsiHead ? kPsiHead : P;
     TRY(psi_rows(0, P0));
     if (P0 < P) TRY(psi_rows(P0, P));
     CK(cudaEventRecord(h->evs[0], st));

@@ -50,3 +50,24 @@ def test_large_frontier_of_short_rows(gpu, m):
     s.explore(5, cap=12000, budget=100000)
     check(s, e)
     assert max(d.parents for d in s.depth_stats()) > 256 * 33
+
+
+@pytest.mark.gpu
+def test_rows_past_the_last_candidate_of_a_wide_frontier(gpu):
+    """A frontier whose first 8192 rows hold 2^64 - 1 candidates: the other
+    rows go in tiles of 8, more of them than the whole frontier has tiles.
+    Against the allocation-free path, which evaluates every row."""
+    import torch
+    system = snp_synth.random_system(5, 512, (4, 4), (32, 32), (0, 16), "dense")
+    depth, cap, budget = 3, 90112, 1 << 20
+    s = gpu.System(system)
+    s.explore(depth, cap=cap, budget=budget)
+    assert s.depth_stats()[2].candidates == gpu.SNP_PSI_SAT and s.depth_stats()[3].parents == cap
+    n = s.count()
+    got = torch.zeros((n, 512), dtype=torch.int32, device="cuda")
+    gpu.snp_reachable(s.h, got, n)
+    o = gpu.snp_explore_opts_init()
+    o.depth, o.frontier_cap, o.candidate_budget = depth, cap, budget
+    out = torch.zeros((1 + depth * cap, 512), dtype=torch.int32, device="cuda")
+    assert gpu.snp_explore_static(s.h, o, out, out.shape[0])[0] == n
+    assert bool((out[:n] == got).all())
