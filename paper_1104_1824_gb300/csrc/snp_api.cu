@@ -100,10 +100,10 @@ int ensure_chunk_buffers(snp_system* h, uint64_t q, cudaStream_t st) {
   TRY(h->d_srow.reserve(sizeof(uint32_t) * q));
   TRY(h->d_bits.reserve(sizeof(uint32_t) * words));
   TRY(h->d_own.reserve(sizeof(uint32_t) * words));
-  const size_t tiles = sizeof(unsigned long long) * (1 + (size_t)commit_tiles((uint32_t)words));  // two counters, words
-  TRY(h->d_tiles.reserve(tiles));
-  CK(cudaMemsetAsync(h->d_tiles.p, 0, h->d_tiles.bytes, st));
-  h->epoch = 0;
+  if (!h->d_counts.p) {
+    TRY(h->d_counts.reserve(sizeof(uint32_t) * (2 + kCommitTiles)));
+    CK(cudaMemsetAsync(h->d_counts.p, 0, h->d_counts.bytes, st));
+  }
   CK(cudaMemsetAsync(h->d_bits.p, 0, sizeof(uint32_t) * words, st));
   CK(cudaMemsetAsync(h->d_own.p, 0, sizeof(uint32_t) * words, st));
   h->q_cap = q;
@@ -752,11 +752,8 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         TRY(h->d_off.reserve(sizeof(uint64_t) * (want + 1)));
         h->psi_cap = want;
       }
-      // two counters, then the entries of the largest of the depth's launches
-      const size_t tiles =
-          sizeof(ScanTile) * (1 + std::max({psi_tiles(P, m, nsm), psi_tiles(P0, m, nsm), psi_tiles(P - P0, m, nsm)}));
-      if (h->d_scan.bytes < tiles) {
-        TRY(h->d_scan.reserve(std::max(tiles, sizeof(ScanTile) * 8192)));
+      if (!h->d_scan.p) {
+        TRY(h->d_scan.reserve(sizeof(ScanTile) * (1 + psi_runs(nsm))));  // two counters, entries
         h->scan_epoch = 0x3FFFFFFFu;  // clear it below
       }
     }
@@ -1022,13 +1019,8 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         c.Q = (uint32_t)Q;
         c.nwords = nwords;
         c.bits = h->d_bits.as<uint32_t>();
-        c.ticket = h->d_tiles.as<uint32_t>();
-        c.tiles = h->d_tiles.as<unsigned long long>() + 1;
-        if (++h->epoch >> 30) {  // numbers used up: start over with clear words
-          CK(cudaMemsetAsync(h->d_tiles.p, 0, h->d_tiles.bytes, st));
-          h->epoch = 1;
-        }
-        c.epoch = h->epoch;
+        c.ticket = h->d_counts.as<uint32_t>();
+        c.counts = c.ticket + 2;
         c.srow = h->d_srow.as<uint32_t>();
         c.slot_of = h->d_slot_of.as<uint32_t>();
         c.staging = nullptr;
@@ -1248,17 +1240,16 @@ struct StaticLayout {
   ChunkState* st;
   unsigned long long* slots;
   uint64_t* off;
-  ScanTile* scan;  // two counters, then scan_n look-back entries
-  int64_t scan_n;
+  ScanTile* scan;  // two counters, then look-back entries
   ParentRec* prec;  // records of frontiers of up to kStaticRecRows rows
   int32_t* staging;
   uint32_t *gmin, *slot_of, *srow, *bits, *own;
-  unsigned long long* tiles;  // two counters, then look-back words
+  uint32_t* counts;  // two words, then the commit tiles' counters
   uint64_t q;  // candidates per pass
 };
 
 // Carves the scratch array; every piece starts on a 256-byte boundary.
-bool static_layout(unsigned char* base, int m, StaticLayout* L) {
+bool static_layout(unsigned char* base, int m, int nsm, StaticLayout* L) {
   size_t at = 0;
   auto take = [&](size_t bytes) {
     unsigned char* p = base + at;
@@ -1272,14 +1263,13 @@ bool static_layout(unsigned char* base, int m, StaticLayout* L) {
   L->slots = reinterpret_cast<unsigned long long*>(take(kStaticSlots * sizeof(unsigned long long)));
   L->off = reinterpret_cast<uint64_t*>(take((kStaticMaxRows + 1) * sizeof(uint64_t)));
   L->prec = reinterpret_cast<ParentRec*>(take(sizeof(ParentRec) * kStaticRecRows));
-  L->scan_n = (int64_t)1 << 17;  // a frontier of kStaticMaxRows rows in tiles of 8 needs no more
-  L->scan = reinterpret_cast<ScanTile*>(take(sizeof(ScanTile) * (2 + L->scan_n)));
+  L->scan = reinterpret_cast<ScanTile*>(take(sizeof(ScanTile) * (1 + psi_runs(nsm))));
   L->staging = reinterpret_cast<int32_t*>(take(q * 4ull * m));
   L->gmin = reinterpret_cast<uint32_t*>(take(q * 4));
   L->slot_of = reinterpret_cast<uint32_t*>(take(q * 4));
   L->srow = reinterpret_cast<uint32_t*>(take(q * 4));
   L->bits = reinterpret_cast<uint32_t*>(take((q / 32 + 1) * 4));
-  L->tiles = reinterpret_cast<unsigned long long*>(take((1 + (size_t)commit_tiles((uint32_t)(q / 32 + 1))) * 8));
+  L->counts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (2 + kCommitTiles)));
   L->own = reinterpret_cast<uint32_t*>(take((q / 32 + 1) * 4));
   return at <= kStaticScratchBytes;
 }
@@ -1313,10 +1303,10 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
   unsigned char* base = nullptr;
   TRY(static_scratch(h->device, &base));
   StaticLayout L;
-  if (!static_layout(base, h->m, &L)) return fail(SNP_E_INTERNAL, "static scratch layout does not fit");
+  const int nsm = sm_count(h->device);
+  if (!static_layout(base, h->m, nsm, &L)) return fail(SNP_E_INTERNAL, "static scratch layout does not fit");
   cudaStream_t st = static_cast<cudaStream_t>(o->stream);
   const int m = h->m;
-  const int nsm = sm_count(h->device);
   const int64_t cap = o->frontier_cap > 0 ? o->frontier_cap : 0;
   const int64_t budget = o->candidate_budget > 0 ? o->candidate_budget : 0;
   const uint64_t qmax = o->chunk > 0 ? std::min<uint64_t>((uint64_t)o->chunk, L.q) : L.q;
@@ -1328,10 +1318,10 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
   CK(cudaMemsetAsync(L.st, 0, sizeof(ChunkState), st));
   CK(cudaMemsetAsync(L.bits, 0, sizeof(uint32_t) * (L.q / 32 + 1), st));
   CK(cudaMemsetAsync(L.own, 0, sizeof(uint32_t) * (L.q / 32 + 1), st));
-  CK(cudaMemsetAsync(L.tiles, 0, 8 * (1 + (size_t)commit_tiles((uint32_t)(L.q / 32 + 1))), st));
-  uint32_t epoch = 0, scan_epoch = 0;
+  CK(cudaMemsetAsync(L.counts, 0, sizeof(uint32_t) * (2 + kCommitTiles), st));
+  uint32_t scan_epoch = 0;
   bool few_before = true;
-  CK(cudaMemsetAsync(L.scan, 0, sizeof(ScanTile) * (1 + L.scan_n), st));
+  CK(cudaMemsetAsync(L.scan, 0, sizeof(ScanTile) * (1 + psi_runs(nsm)), st));
   auto clear_and_insert = [&](int64_t rows) -> int {
     k_fill_u64<<<grid_for((int64_t)kStaticSlots, 256, nsm * 32), 256, 0, st>>>(L.slots, kStaticSlots, kEmpty);
     CK(cudaGetLastError());
@@ -1422,9 +1412,8 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
       c.Q = (uint32_t)Q;
       c.nwords = nwords;
       c.bits = L.bits;
-      c.ticket = reinterpret_cast<uint32_t*>(L.tiles);
-      c.tiles = L.tiles + 1;
-      c.epoch = ++epoch;
+      c.ticket = L.counts;
+      c.counts = L.counts + 2;
       c.host = h->pin.slot[0];
       c.srow = L.srow;
       c.slot_of = L.slot_of;

@@ -632,54 +632,16 @@ static __device__ void block_scan_sat(uint64_t* v, int64_t n, uint64_t* wsum) {
   }
 }
 
-// Decoupled look-back over tiles that are handed out in order: publishes this
-// tile's sum and returns the sum of all tiles before it (one warp, all lanes).
-// A tile's word is {epoch:30 | flag:2 | value:32}, flag 1 = the tile's own sum,
-// 2 = the sum through the tile; words of another epoch are stale.  The wait is
-// bounded by kSpinLimit polls; false when it ran out.
-__device__ __forceinline__ bool lookback_u32(unsigned long long* tiles, uint32_t tile, uint32_t epoch, uint32_t sum,
-                                             uint32_t& prefix, int lane) {
-  volatile unsigned long long* t = tiles;
-  const unsigned long long tag = (unsigned long long)epoch << 34;
-  prefix = 0;
-  if (tile == 0) {
-    if (lane == 0) t[0] = tag | (2ull << 32) | sum;
-    return true;
-  }
-  if (lane == 0) t[tile] = tag | (1ull << 32) | sum;
-  int64_t at = (int64_t)tile - 1 - lane;
-  bool ok = true;
-  for (int polls = 0;;) {
-    unsigned long long v = at >= 0 ? t[at] : tag | (2ull << 32);
-    const bool ready = (uint32_t)(v >> 34) == epoch && ((v >> 32) & 3ull) != 0;
-    if (!__all_sync(0xffffffffu, ready)) {
-      if (++polls >= kSpinLimit) {
-        ok = false;
-        break;
-      }
-      __nanosleep(20);
-      continue;
-    }
-    const uint32_t full = __ballot_sync(0xffffffffu, ((v >> 32) & 3ull) == 2ull);
-    const int last = full ? __ffs(full) - 1 : 31;  // the nearest tile with its inclusive sum
-    uint32_t x = lane <= last ? (uint32_t)v : 0u;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    prefix += x;
-    if (full) break;
-    at -= 32;
-  }
-  if (lane == 0 && ok) t[tile] = tag | (2ull << 32) | (prefix + sum);
-  return ok;
-}
-
 // Look-back state of one tile of a saturating 64-bit scan.
 struct ScanTile {
   unsigned long long sum, through;  // the tile's own sum; the sum through the tile
   uint32_t flag, pad;               // epoch << 2 | (1: sum is set, 2: through is set)
 };
 
-// lookback_u32 for saturating 64-bit sums; base: what comes before tile 0.
+// Decoupled look-back over tiles that are handed out in order: publishes this
+// tile's sum and returns base (what comes before tile 0) plus the sums of all
+// tiles before it, saturating (one warp, all lanes).  Entries of another epoch
+// are stale.  The wait is bounded by kSpinLimit polls; false when it ran out.
 __device__ __forceinline__ bool lookback_sat(ScanTile* tiles, uint32_t tile, uint32_t epoch, uint64_t base,
                                              uint64_t sum, uint64_t& prefix, int lane) {
   volatile ScanTile* t = tiles;

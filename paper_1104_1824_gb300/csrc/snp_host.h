@@ -166,7 +166,7 @@ struct snp_system {
   uint64_t tc_cap = 0;  // candidates the tensor-core chunk buffers hold
   std::vector<unsigned long long> colkey, rowkey;
   // exploration state
-  DevBuf d_pool, d_slots, d_gmin, d_slot_of, d_bits, d_tiles, d_srow, d_own, d_off, d_scan, d_st,
+  DevBuf d_pool, d_slots, d_gmin, d_slot_of, d_bits, d_counts, d_srow, d_own, d_off, d_scan, d_st,
       d_rec_parent, d_rec_index, d_tmp,
       d_prec, d_ctr, d_perm, d_sidx,
       d_bcache;  // wide mode: base children of each pass's largest parents
@@ -176,8 +176,7 @@ struct snp_system {
   int64_t n_store = 0;    // store rows in use
   uint64_t nbuckets = 0;
   uint64_t q_cap = 0;     // staging capacity in rows
-  uint32_t epoch = 0;     // last look-back epoch used in d_tiles
-  uint32_t scan_epoch = 0;  // ... and in d_scan
+  uint32_t scan_epoch = 0;  // last look-back epoch used in d_scan
   int64_t psi_cap = 0;    // parents
   int64_t rec_rows = 0;
   PinnedState pin;

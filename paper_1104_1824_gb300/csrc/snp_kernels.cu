@@ -20,6 +20,8 @@
 //              into the discovery-ordered pool), and their table slots point
 //              at their rows; the rest become tombstones (the cap stops the
 //              depth).
+#include <algorithm>
+
 #include "snp_kernels.cuh"
 
 namespace snp {
@@ -35,8 +37,10 @@ __device__ __forceinline__ void set_error(ChunkState* st, uint32_t bits) { atomi
 // Step (a), Eq. psi and its saturating exclusive scan for every frontier row:
 // off[p] = the sum of Psi over rows before p, off[P] = the total; with REC the
 // rows' ParentRecs.  Rows not to be expanded (max_expand) get Psi = 0, rows
-// whose children could leave int32 raise kErrOverflow.  Tiles of rows are
-// handed out in order and chained by decoupled look-back.
+// whose children could leave int32 raise kErrOverflow.  A CTA takes one run of
+// a.sub consecutive tiles; runs are handed out in order, at most one per
+// resident CTA, and chained by decoupled look-back at their ends (a hop per 32
+// runs; a chain over all tiles of 2^20 rows cost over 100 us).
 //   WARP = false: tiles of 256 rows, a lane per row.  A warp moves its 32 rows
 //     through shared memory 32 columns at a time (16-byte pieces where rows
 //     are whole pieces, else one coalesced 128-byte load per row), unpacked to
@@ -55,7 +59,7 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
   __shared__ int32_t slabs[WARP ? 1 : 8][32][33];
   __shared__ uint64_t s_w[8];
   __shared__ uint64_t s_prefix;
-  __shared__ uint32_t s_tile;
+  __shared__ uint32_t s_run;
   __shared__ int s_ok, s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const DevSys& s = a.s;
@@ -67,17 +71,11 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
     for (int64_t p = (int64_t)blockIdx.x * 256 + tid; p < a.P; p += (int64_t)gridDim.x * 256) a.off[p + 1] = kSat;
   } else {
     bool over = false;
-    for (uint32_t step = 0;; ++step) {
-      uint32_t tile;
-      if (a.off) {
-        __syncthreads();
-        if (tid == 0) s_tile = atomicAdd(a.ticket, 1u);
-        __syncthreads();
-        tile = s_tile;
-      } else {  // records only: no order needed
-        tile = blockIdx.x + step * gridDim.x;
-      }
-      if (tile >= ntiles) break;
+    if (tid == 0) s_run = a.off ? atomicAdd(a.ticket, 1u) : blockIdx.x;
+    __syncthreads();
+    const uint32_t run = s_run, tile0 = run * a.sub, tile1 = min(tile0 + a.sub, ntiles);
+    uint64_t through = 0, before = 0;  // sum of the run's tiles so far; this lane's exclusive sum within the run
+    for (uint32_t tile = tile0; tile < tile1; ++tile) {
       const int64_t p0 = (int64_t)tile * R + (WARP ? warp : warp * 32);  // this warp's first row
       PsiAcc acc;
       uint64_t v = 0;  // Psi of this lane's row (WARP: lane 0's)
@@ -184,12 +182,10 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
         }
       }
       if (!a.off) continue;
-      // this lane's exclusive sum within the tile
-      uint64_t before, sum;
+      uint64_t sum = 0;
       if (WARP) {
         __syncthreads();
         before = 0;
-        sum = 0;
         for (int w = 0; w < 8; ++w) {
           if (w < lane) before = sat_add(before, s_w[w]);  // warp 0: lane l writes row l
           sum = sat_add(sum, s_w[w]);
@@ -205,30 +201,38 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
         before = __shfl_up_sync(0xffffffffu, inc, 1);
         if (lane == 0) before = 0;
         __syncthreads();
-        uint64_t wb = 0;
-        sum = 0;
         for (int w = 0; w < 8; ++w) {
-          if (w < warp) wb = sat_add(wb, s_w[w]);
+          if (w < warp) before = sat_add(before, s_w[w]);
           sum = sat_add(sum, s_w[w]);
         }
-        before = sat_add(wb, before);
       }
+      before = sat_add(before, through);
+      through = sat_add(through, sum);
+      __syncthreads();
+      const int64_t p = WARP ? (int64_t)tile * R + lane : p0 + lane;
+      if (a.sub > 1 && (!WARP || (warp == 0 && lane < 8)) && p < a.P) a.off[p] = before;
+    }
+    if (a.off && tile0 < ntiles) {
       if (warp == 0) {
         uint64_t prefix = 0;
-        const bool ok = lookback_sat(a.tiles, tile, a.epoch, base, sum, prefix, lane);
+        const bool ok = lookback_sat(a.tiles, run, a.epoch, base, through, prefix, lane);
         if (lane == 0) {
           s_prefix = prefix;
           s_ok = ok ? 1 : 0;
+          if (!ok) atomicOr(&a.st->error, kErrTimeout);
         }
       }
       __syncthreads();
-      if (!s_ok) {
-        if (tid == 0) atomicOr(&a.st->error, kErrTimeout);
-        break;
+      if (s_ok) {
+        const uint64_t prefix = s_prefix;
+        if (!WARP || (warp == 0 && lane < 8)) {
+          for (uint32_t tile = tile0; tile < tile1; ++tile) {  // each thread's own rows
+            const int64_t p = (int64_t)tile * R + (WARP ? lane : tid);
+            if (p < a.P) a.off[p] = sat_add(prefix, a.sub > 1 ? a.off[p] : before);
+          }
+        }
+        if (tile1 == ntiles && tid == 0) a.off[a.P] = sat_add(prefix, through);
       }
-      const int64_t p = WARP ? (int64_t)tile * R + lane : p0 + lane;
-      if ((!WARP || (warp == 0 && lane < 8)) && p < a.P) a.off[p] = sat_add(s_prefix, before);
-      if (tile + 1 == ntiles && tid == 0) a.off[a.P] = sat_add(s_prefix, sum);
     }
     if (__any_sync(0xffffffffu, over) && lane == 0) set_error(a.st, kErrOverflow);
   }
@@ -252,8 +256,11 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
 namespace {
 
 template <class RF, bool REC>
-void psi_launch(const PsiArgs& a, bool warp, int64_t tiles, cudaStream_t st, int nsm) {
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)nsm * (warp ? 8 : REC ? 2 : 3)));
+void psi_launch(PsiArgs a, bool warp, cudaStream_t st, int nsm) {
+  const int64_t tiles = (a.P + (warp ? 7 : 255)) / (warp ? 8 : 256);
+  const int64_t resident = (int64_t)nsm * (REC ? 2 : 3);
+  a.sub = (uint32_t)((tiles + resident - 1) / resident);
+  const int blocks = (int)std::max<int64_t>(1, (tiles + a.sub - 1) / a.sub);
   if (warp)
     k_psi<RF, REC, true><<<blocks, 256, 0, st>>>(a);
   else
@@ -270,29 +277,28 @@ static bool psi_by_warp(int64_t P, int m, int nsm) {
   return (P + warps - 1) / warps * (12 + m / 32) <= (P + 32 * warps - 1) / (32 * warps) * std::max(m, 16);
 }
 
-size_t psi_tiles(int64_t P, int m, int nsm) { return (size_t)((P + (psi_by_warp(P, m, nsm) ? 7 : 255)) / (psi_by_warp(P, m, nsm) ? 8 : 256)) + 1; }
+size_t psi_runs(int nsm) { return (size_t)nsm * 3; }
 
 int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm) {
   const bool warp = psi_by_warp(a.P, a.s.m, nsm);
-  const int64_t tiles = (a.P + (warp ? 7 : 255)) / (warp ? 8 : 256);
   if (w == 1)
-    a.rec ? psi_launch<RowU8, true>(a, warp, tiles, st, nsm) : psi_launch<RowU8, false>(a, warp, tiles, st, nsm);
+    a.rec ? psi_launch<RowU8, true>(a, warp, st, nsm) : psi_launch<RowU8, false>(a, warp, st, nsm);
   else if (w == 2)
-    a.rec ? psi_launch<RowU16, true>(a, warp, tiles, st, nsm) : psi_launch<RowU16, false>(a, warp, tiles, st, nsm);
+    a.rec ? psi_launch<RowU16, true>(a, warp, st, nsm) : psi_launch<RowU16, false>(a, warp, st, nsm);
   else if (a.s.m % 4 == 0)
-    a.rec ? psi_launch<RowI32V, true>(a, warp, tiles, st, nsm) : psi_launch<RowI32V, false>(a, warp, tiles, st, nsm);
+    a.rec ? psi_launch<RowI32V, true>(a, warp, st, nsm) : psi_launch<RowI32V, false>(a, warp, st, nsm);
   else
-    a.rec ? psi_launch<RowI32, true>(a, warp, tiles, st, nsm) : psi_launch<RowI32, false>(a, warp, tiles, st, nsm);
+    a.rec ? psi_launch<RowI32, true>(a, warp, st, nsm) : psi_launch<RowI32, false>(a, warp, st, nsm);
   return 1;
 }
 
 // One bit per first occurrence: every candidate lid that claimed a key
-// (ownbits) names the key's first candidate gmin[lid]; clears ownbits.  A warp
-// takes four words, a lane per claim, so that the four words' gmin loads are
+// (ownbits) names the key's first candidate gmin[lid]; clears ownbits and
+// counts the first occurrences of each commit tile.  A warp takes four words, a lane per claim, so that the four words' gmin loads are
 // in flight together (a thread per word walked its claims one after another:
 // 8 us per pass of 2^16, 11 us per pass of 2^20).
 __global__ void __launch_bounds__(256) k_mark(uint32_t* ownbits, const uint32_t* gmin, uint32_t* bits, uint32_t* srow,
-                                              uint32_t nwords, ChunkState* st) {
+                                              uint32_t nwords, uint32_t* counts, int tile_log, ChunkState* st) {
   constexpr int U = kMarkWords;
   const int lane = threadIdx.x & 31;
   const uint32_t limit = nwords * 32u;
@@ -309,13 +315,19 @@ __global__ void __launch_bounds__(256) k_mark(uint32_t* ownbits, const uint32_t*
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (!((word[u] >> lane) & 1u)) continue;
-      if (f[u] >= limit) {  // not a claim of this pass: record and skip
+      bool ok = (word[u] >> lane) & 1u;
+      if (ok && f[u] >= limit) {  // not a claim of this pass: record and skip
         atomicOr(&st->error, kErrInternal);
-        continue;
+        ok = false;
       }
-      atomicOr(bits + (f[u] >> 5), 1u << (f[u] & 31));
-      srow[f[u]] = (w0 + u) * 32u + lane;
+      if (ok) {
+        atomicOr(bits + (f[u] >> 5), 1u << (f[u] & 31));
+        srow[f[u]] = (w0 + u) * 32u + lane;
+      }
+      // one addition per tile the warp's claims fall into (mostly one)
+      const uint32_t tile = ok ? f[u] >> tile_log : 0xFFFFFFFFu;
+      const uint32_t same = __match_any_sync(0xffffffffu, tile);
+      if (ok && lane == __ffs(same) - 1) atomicAdd(counts + tile, (uint32_t)__popc(same));
     }
   }
 }
@@ -335,58 +347,58 @@ __device__ __forceinline__ int nth_bit(uint32_t v, int n) {
   return pos;
 }
 
+// rows staged rows (row r: staging row s of lane r) to consecutive rows at dst,
+// `per` elements each, by the whole warp with eight loads in flight.
+template <typename T>
+__device__ __forceinline__ void copy_staged(const T* staging, T* dst, uint32_t s, uint32_t rows, uint32_t per,
+                                            int lane) {
+  const uint32_t total = rows * per;
+  for (uint32_t i0 = 0; i0 < total; i0 += 32 * 8) {
+    T v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const uint32_t i = i0 + 32u * u + lane, q = min(i / per, 31u);
+      const uint32_t src = __shfl_sync(0xffffffffu, s, (int)q);
+      if (i < total) v[u] = __ldcg(staging + (size_t)src * per + (i - q * per));
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i0 + 32u * u + lane < total) dst[i0 + 32u * u + lane] = v[u];
+  }
+}
+
 // Ranks the chunk's first occurrences in candidate order and commits them: the
 // first `remaining` get their discovery index (store mode: perm[row] = the
 // store row their owner wrote; else the staged row is copied to pool row
 // row_base + rank) and their table slot pointed at it, the others become
-// tombstones.  A CTA takes a tile of kCommitWords bitmap words (2048
-// candidates), gets its first rank by decoupled look-back (tiles are handed
-// out in order, so every tile waited for is running or done) and deals its
-// set bits out one per thread.  The last CTA to finish advances the device
-// counters, hands the chunk's counters to the host and clears them.
-// Bound by the latency of its dependent loads (owner, slot and store row);
-// the popcount, scan, commit, clear and copy launches it replaces were six to
-// eight per pass (3 neurons to depth 10: 1012 us -> 855 us; 64 neurons, 18
-// passes: 11.29 ms -> 10.52 ms).
-__global__ void __launch_bounds__(256) k_commit(CommitArgs a) {
-  __shared__ uint32_t s_word[kCommitWords], s_pre[kCommitWords];
-  __shared__ uint32_t s_tile, s_cnt, s_prefix;
-  __shared__ int s_ok, s_last;
+// tombstones.  A CTA takes a tile of the bitmap; the marks counted every
+// tile's first occurrences, so the CTA adds up the counts before its own (at
+// most kCommitTiles of them) and deals its set bits out one per thread, 64
+// words at a time.  The last CTA to finish advances the device counters,
+// hands the chunk's counters to the host and clears them.  Bound by the
+// latency of its dependent loads (owner, slot and store row).  (Ranks by
+// decoupled look-back cost a hop of about 1 us per 32 tiles: 64 neurons, 18
+// passes of about 2^20: 10.5 ms with 512 tiles a pass, 12.2 ms with 2048.)
+constexpr int kCommitChunk = 64;  // bitmap words a CTA ranks at a time
+__global__ void __launch_bounds__(256) k_commit(CommitArgs a, uint32_t tile_words) {
+  __shared__ uint32_t s_word[kCommitChunk], s_pre[kCommitChunk];
+  __shared__ uint32_t s_part[8], s_cnt, s_prefix;
+  __shared__ int s_last;
   __shared__ int64_t s_p0, s_p1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t row_base = a.ctr ? (int64_t)__ldcg(a.ctr) : a.row_base;
   const uint64_t remaining = a.ctr ? __ldcg(a.ctr + 1) : a.remaining;
-  if (tid == 0) s_tile = atomicAdd(a.ticket, 1u);
-  __syncthreads();
-  const uint32_t tile = s_tile, w0 = tile * kCommitWords;
-  if (warp == 0) {  // two words per lane
-    static_assert(kCommitWords == 64, "two words per lane");
-    const uint32_t i0 = w0 + 2u * lane, i1 = i0 + 1;
-    const uint32_t x0 = i0 < a.nwords ? a.bits[i0] : 0u, x1 = i1 < a.nwords ? a.bits[i1] : 0u;
-    if (x0) a.bits[i0] = 0u;  // clear for the next chunk
-    if (x1) a.bits[i1] = 0u;
-    const uint32_t c0 = __popc(x0), c1 = __popc(x1);
-    uint32_t inc = c0 + c1;
+  const uint32_t tile = blockIdx.x, t0 = tile * tile_words, t1 = min(t0 + tile_words, a.nwords);
+  const uint32_t mine = __ldcg(a.counts + tile);
+  {  // first occurrences of the tiles before this one (the last CTA: of all)
+    uint32_t sum = 0;
+    for (uint32_t i = tid; i < tile; i += 256) sum += __ldcg(a.counts + i);
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    s_word[2 * lane] = x0;
-    s_word[2 * lane + 1] = x1;
-    s_pre[2 * lane] = inc - c0 - c1;
-    s_pre[2 * lane + 1] = inc - c1;
-    const uint32_t cnt = __shfl_sync(0xffffffffu, inc, 31);
-    uint32_t prefix = 0;
-    const bool ok = lookback_u32(a.tiles, tile, a.epoch, cnt, prefix, lane);
-    if (lane == 0) {
-      s_cnt = cnt;
-      s_prefix = prefix;
-      s_ok = ok ? 1 : 0;
-      if (!ok) atomicOr(&a.st->error, kErrTimeout);
-    }
-  } else if (warp == 1 && a.rec_parent) {  // the parents of the tile's candidates
-    const uint64_t gf = a.g0 + (uint64_t)w0 * 32u, gl = min(gf + kCommitWords * 32u, a.g0 + a.Q) - 1;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) s_part[warp] = sum;
+  }
+  if (warp == 1 && a.rec_parent && mine) {  // the parents of the tile's candidates
+    const uint64_t gf = a.g0 + (uint64_t)t0 * 32u, gl = min(a.g0 + (uint64_t)t1 * 32u, a.g0 + a.Q) - 1;
     const int64_t p0 = warp_find_parent(a.off, a.P, gf, lane), p1 = warp_find_parent(a.off, a.P, gl, lane);
     if (lane == 0) {
       s_p0 = p0;
@@ -394,71 +406,95 @@ __global__ void __launch_bounds__(256) k_commit(CommitArgs a) {
     }
   }
   __syncthreads();
-  const uint32_t cnt = s_ok ? s_cnt : 0u;
+  uint32_t prefix = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) prefix += s_part[w];
+  const uint32_t through = prefix + mine;  // the last tile's: all of the chunk's
   const int m = a.sys.m;
-  for (uint32_t r0 = (uint32_t)warp * 32u; r0 < cnt; r0 += blockDim.x) {
-    const uint32_t r = r0 + (uint32_t)lane;
-    const uint64_t rank0 = (uint64_t)s_prefix + r0, rank = rank0 + lane;
-    uint32_t s = 0;
-    if (r < cnt) {
-      int w = 0;  // the word holding rank r of the tile
+  for (uint32_t w0 = t0; mine && w0 < t1; w0 += kCommitChunk) {
+    __syncthreads();
+    if (warp == 0) {  // two words per lane
+      const uint32_t i0 = w0 + 2u * lane, i1 = i0 + 1;
+      const uint32_t x0 = i0 < t1 ? a.bits[i0] : 0u, x1 = i1 < t1 ? a.bits[i1] : 0u;
+      if (x0) a.bits[i0] = 0u;  // clear for the next chunk
+      if (x1) a.bits[i1] = 0u;
+      const uint32_t c0 = __popc(x0), c1 = __popc(x1);
+      uint32_t inc = c0 + c1;
 #pragma unroll
-      for (int step = kCommitWords / 2; step > 0; step >>= 1)
-        if (s_pre[w + step] <= r) w += step;
-      const uint32_t lid = (w0 + (uint32_t)w) * 32u + (uint32_t)nth_bit(s_word[w], (int)(r - s_pre[w]));
-      s = a.srow[lid];
-      // the slot keeps its fingerprint (high half): only the row is written
-      uint32_t* slot = reinterpret_cast<uint32_t*>(a.table.slots + a.slot_of[s]);
-      if (rank < remaining) {
-        const int64_t row = row_base + (int64_t)rank;
-        const uint32_t at = a.perm ? a.sidx_of[s] : (uint32_t)row;
-        if (a.perm) a.perm[row] = at;
-        *slot = at;
-        if (rank + 1 == remaining) {
-          a.st->capped = 1;
-          a.st->last_lid = lid;
-        }
-        if (a.rec_parent) {
-          const uint64_t g = a.g0 + lid;
-          int64_t lo = s_p0, hi = s_p1 + 1;  // largest p with off[p] <= g
-          while (hi - lo > 1) {
-            const int64_t mid = lo + (hi - lo) / 2;
-            if (__ldg(a.off + mid) <= g) lo = mid; else hi = mid;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      s_word[2 * lane] = x0;
+      s_word[2 * lane + 1] = x1;
+      s_pre[2 * lane] = inc - c0 - c1;
+      s_pre[2 * lane + 1] = inc - c1;
+      if (lane == 31) s_cnt = inc;
+    }
+    __syncthreads();
+    const uint32_t cnt = s_cnt;
+    for (uint32_t r0 = (uint32_t)warp * 32u; r0 < cnt; r0 += blockDim.x) {
+      const uint32_t r = r0 + (uint32_t)lane;
+      const uint64_t rank0 = (uint64_t)prefix + r0, rank = rank0 + lane;
+      uint32_t s = 0;
+      if (r < cnt) {
+        int w = 0;  // the word holding rank r of the chunk
+#pragma unroll
+        for (int step = kCommitChunk / 2; step > 0; step >>= 1)
+          if (s_pre[w + step] <= r) w += step;
+        const uint32_t lid = (w0 + (uint32_t)w) * 32u + (uint32_t)nth_bit(s_word[w], (int)(r - s_pre[w]));
+        s = a.srow[lid];
+        // the slot keeps its fingerprint (high half): only the row is written
+        uint32_t* slot = reinterpret_cast<uint32_t*>(a.table.slots + a.slot_of[s]);
+        if (rank < remaining) {
+          const int64_t row = row_base + (int64_t)rank;
+          const uint32_t at = a.perm ? a.sidx_of[s] : (uint32_t)row;
+          if (a.perm) a.perm[row] = at;
+          *slot = at;
+          if (rank + 1 == remaining) {
+            a.st->capped = 1;
+            a.st->last_lid = lid;
           }
-          a.rec_parent[row] = a.parent_base + lo;
-          a.rec_index[row] = g - __ldg(a.off + lo);
+          if (a.rec_parent) {
+            const uint64_t g = a.g0 + lid;
+            int64_t lo = s_p0, hi = s_p1 + 1;  // largest p with off[p] <= g
+            while (hi - lo > 1) {
+              const int64_t mid = lo + (hi - lo) / 2;
+              if (__ldg(a.off + mid) <= g) lo = mid; else hi = mid;
+            }
+            a.rec_parent[row] = a.parent_base + lo;
+            a.rec_index[row] = g - __ldg(a.off + lo);
+          }
+        } else {
+          *slot = kRowTomb;
         }
-      } else {
-        *slot = kRowTomb;
+      }
+      if (!a.perm && rank0 < remaining) {  // staged rows to consecutive pool rows, by the whole warp
+        const uint32_t rows = (uint32_t)min((uint64_t)min(cnt - r0, 32u), remaining - rank0);
+        int32_t* dst = a.pool + (size_t)(row_base + (int64_t)rank0) * m;
+        if ((m & 3) == 0)
+          copy_staged(reinterpret_cast<const int4*>(a.staging), reinterpret_cast<int4*>(dst), s, rows, (uint32_t)m >> 2,
+                      lane);
+        else
+          copy_staged(a.staging, dst, s, rows, (uint32_t)m, lane);
       }
     }
-    if (!a.perm && rank0 < remaining) {  // staged rows to consecutive pool rows, by the whole warp
-      const uint32_t rows = (uint32_t)min((uint64_t)min(cnt - r0, 32u), remaining - rank0);
-      int32_t* dst = a.pool + (size_t)(row_base + (int64_t)rank0) * m;
-      const uint32_t total = rows * (uint32_t)m;
-      for (uint32_t i0 = 0; i0 < total; i0 += 32 * 8) {
-        int32_t v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const uint32_t i = i0 + 32u * u + lane, q = min(i / (uint32_t)m, 31u);
-          const uint32_t src = __shfl_sync(0xffffffffu, s, (int)q);
-          if (i < total) v[u] = __ldcg(a.staging + (size_t)src * m + (i - q * (uint32_t)m));
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (i0 + 32u * u + lane < total) dst[i0 + 32u * u + lane] = v[u];
-      }
-    }
+    prefix += cnt;
   }
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(a.ticket + 1, 1u) + 1 == gridDim.x ? 1 : 0;
+  if (tid == 0) {
+    if (tile + 1 == gridDim.x) a.ticket[1] = through;
+    __threadfence();
+    s_last = atomicAdd(a.ticket, 1u) + 1 == gridDim.x ? 1 : 0;
+  }
   __syncthreads();
-  if (!s_last || tid != 0) return;
+  if (!s_last) return;
+  for (uint32_t i = tid; i < gridDim.x; i += 256) a.counts[i] = 0u;
+  if (tid != 0) return;
   __threadfence();
+  const uint32_t total = __ldcg(a.ticket + 1);
   a.ticket[0] = 0;
-  a.ticket[1] = 0;
-  const uint32_t total = (uint32_t)__ldcg(a.tiles + gridDim.x - 1);  // the last tile's inclusive prefix
   ChunkState c;
   c.n_alloc = total;
   c.error = __ldcg(&a.st->error);
@@ -483,13 +519,20 @@ __global__ void __launch_bounds__(256) k_commit(CommitArgs a) {
   }
 }
 
-uint32_t commit_tiles(uint32_t nwords) { return (nwords + kCommitWords - 1) / kCommitWords; }
+// Bitmap words per commit tile, as a power of two: 8 (256 candidates, so that a
+// pass of 2^16 is 256 CTAs), more when that would make over kCommitTiles tiles.
+static int commit_words_log(uint32_t nwords) {
+  int lg = 3;
+  while (((uint64_t)nwords + (1ull << lg) - 1) >> lg > kCommitTiles) ++lg;
+  return lg;
+}
 
 void launch_mark_commit(const CommitArgs& c, uint32_t* ownbits, const uint32_t* gmin, cudaStream_t st, int nsm) {
   const uint32_t per = 8 * kMarkWords;
   const int blocks = (int)std::min<uint32_t>((c.nwords + per - 1) / per, (uint32_t)nsm * 16);
-  k_mark<<<blocks, 256, 0, st>>>(ownbits, gmin, c.bits, const_cast<uint32_t*>(c.srow), c.nwords, c.st);
-  k_commit<<<commit_tiles(c.nwords), 256, 0, st>>>(c);
+  const int lg = commit_words_log(c.nwords);
+  k_mark<<<blocks, 256, 0, st>>>(ownbits, gmin, c.bits, const_cast<uint32_t*>(c.srow), c.nwords, c.counts, lg + 5, c.st);
+  k_commit<<<(c.nwords + (1u << lg) - 1) >> lg, 256, 0, st>>>(c, 1u << lg);
 }
 
 __global__ void k_iota_u32(uint32_t* out, int64_t n) {

@@ -54,11 +54,10 @@ struct CommitArgs {
   uint32_t Q;                 // candidates in the chunk
   uint32_t nwords;            // ceil(Q / 32)
   uint32_t* bits;             // [nwords] first-occurrence bitmap over chunk-local indices; cleared on the way
-  // Look-back state: a word per tile (commit_tiles), two counters that start
-  // (and are left) at 0, and a number no earlier chunk of these words had.
-  unsigned long long* tiles;
+  // Counters that start (and are left) at 0: first occurrences of each commit
+  // tile (kCommitTiles), and two words (tiles done; all first occurrences).
+  uint32_t* counts;
   uint32_t* ticket;
-  uint32_t epoch;
   const uint32_t* srow;       // [Q] owner (candidate that claimed the key) of each first occurrence
   const uint32_t* slot_of;
   const int32_t* staging;
@@ -81,9 +80,8 @@ struct CommitArgs {
   ChunkState* st;             // the chunk's counters; with host, copied there and cleared at the end
   ChunkState* host;           // pinned host copy, or nullptr
 };
-constexpr int kCommitWords = 64;  // bitmap words per commit tile
 constexpr int kMarkWords = 4;     // bitmap words per warp of the mark kernel
-uint32_t commit_tiles(uint32_t nwords);
+constexpr uint32_t kCommitTiles = 2048;  // most commit tiles of a chunk
 // First-occurrence marks of the chunk (ownbits cleared on the way), ranks and
 // commit: two launches.
 void launch_mark_commit(const CommitArgs& c, uint32_t* ownbits, const uint32_t* gmin, cudaStream_t st, int nsm);
@@ -209,11 +207,12 @@ struct PsiArgs {
   int32_t max_expand;
   uint64_t* off;              // [P + 1], or nullptr: records only
   ParentRec* rec;             // [P] or nullptr
-  // Look-back state: psi_tiles(P) entries, two counters that start (and are
+  // Look-back state: psi_runs() entries, two counters that start (and are
   // left) at 0, and a number no earlier launch on these entries had.
   ScanTile* tiles;
   uint32_t* ticket;
   uint32_t epoch;
+  uint32_t sub;               // tiles per run (set by launch_psi)
   const uint64_t* carry;      // sum of Psi before these rows (nullptr: 0); when it is 2^64 - 1 the rows are not read
   ChunkState* st;             // errors
   // Set on the last launch of a depth: the total and st's errors to pinned
@@ -223,7 +222,7 @@ struct PsiArgs {
   unsigned long long* ctr;
   unsigned long long remaining;
 };
-size_t psi_tiles(int64_t P, int m, int nsm);
+size_t psi_runs(int nsm);
 // rows: w bytes per spike count (4: int32; 2, 1: a packed store).  Returns the launches made.
 int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm);
 // Steps (b)-(d) for the chunk's candidates (k_expand); returns the launches made.
