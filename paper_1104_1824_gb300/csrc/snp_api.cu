@@ -694,8 +694,14 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
   }
   CK(cudaMemsetAsync(h->d_st.p, 0, sizeof(ChunkState), st));
   {
-    const uint64_t want =
-        (uint64_t)((long double)(rows_plan + (int64_t)std::min<uint64_t>(qmax, 1 << 16)) * 4.0L / 3.0L / kBucket) + 1;
+    // rows planned for plus one pass of candidates, all of which might be new
+    // (a table without that room is rebuilt half way: 860 us for 10^6 rows of
+    // 301 counts); a pass never holds more than the budget
+    // (nor, mostly, than eight times the cap: shares of new ones below 1/8)
+    uint64_t pass = std::min<uint64_t>(qmax, 1 << 16);
+    if (cap > 0) pass = std::min<uint64_t>(qmax, std::max<uint64_t>(8ull * (uint64_t)cap, 1 << 16));
+    if (cap > 0 && budget > 0) pass = std::min<uint64_t>(pass, std::max<uint64_t>((uint64_t)budget, 1 << 16));
+    const uint64_t want = (uint64_t)((long double)(rows_plan + (int64_t)pass) * 4.0L / 3.0L / kBucket) + 1;
     TRY(rebuild_table(h, pow2_at_least(want), st));
     if (!rs && g_hold_root_slot.exchange(0)) {  // testing hook: C0's slot stays "being claimed"
       const uint64_t nslots = h->nbuckets * kBucket;
