@@ -78,9 +78,12 @@ __global__ void __launch_bounds__(256, 2) k_expand(ClaimArgs a, int B, int ts) {
   expand_warp<RF, 0>(a, B, ts, w, (uint64_t)blockIdx.x * wpb + wib, (uint64_t)gridDim.x * wpb, lane);
 }
 
-// The wide mode of k_expand (rows of more than kWideM neurons).
-template <class RF>
-__global__ void __launch_bounds__(kWideWarps * 32, 1) k_expand_wide(ClaimArgs a) {
+// The wide mode of k_expand (rows of more than kWideM neurons).  WARPS per CTA,
+// one CTA per SM: 16 (128 registers each) where their shared memory fits, else
+// kWideWarps.  The passes are latency-bound: 301 neurons, cap 2^18: 6874 us with
+// 11 warps, 5510 us with 16.
+template <class RF, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 1) k_expand_wide(ClaimArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (a.ctr && __ldcg(a.ctr + 1) == 0) return;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
@@ -140,7 +143,8 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
   const int m = a.sys.m;
   if (m > kWideM) {
     const size_t per_warp = expand_wide_bytes(m);
-    const int wpb = (int)std::max<size_t>(1, std::min<size_t>(kWideWarps, (226u << 10) / per_warp));
+    const bool many = per_warp * kWideWarpsMany <= (226u << 10);
+    const int wpb = many ? kWideWarpsMany : (int)std::max<size_t>(1, std::min<size_t>(kWideWarps, (226u << 10) / per_warp));
     const size_t smem = per_warp * wpb;
     // one task per warp: a task's first block costs a full decode (C + S . M
     // over every neuron), which wide rows make expensive; at least 16
@@ -156,8 +160,11 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
                 : (m % 4) == 0 ? k_wide_base<RowI32V> : k_wide_base<RowI32>;
       fb<<<kBaseSlots, std::min(1024, (m + 31) / 32 * 32), bs, st>>>(a);
     }
-    auto fn = a.w == 2 ? k_expand_wide<RowU16> : a.w == 1 ? k_expand_wide<RowU8>
-              : (m % 4) == 0 ? k_expand_wide<RowI32V> : k_expand_wide<RowI32>;
+    constexpr int kM = kWideWarpsMany, kF = kWideWarps;
+    auto fn = many ? (a.w == 2 ? k_expand_wide<RowU16, kM> : a.w == 1 ? k_expand_wide<RowU8, kM>
+                      : (m % 4) == 0 ? k_expand_wide<RowI32V, kM> : k_expand_wide<RowI32, kM>)
+                   : (a.w == 2 ? k_expand_wide<RowU16, kF> : a.w == 1 ? k_expand_wide<RowU8, kF>
+                      : (m % 4) == 0 ? k_expand_wide<RowI32V, kF> : k_expand_wide<RowI32, kF>);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     fn<<<blocks > 0 ? blocks : 1, wpb * 32, smem, st>>>(a);
     return a.bcache ? 2 : 1;

@@ -78,6 +78,7 @@ __host__ __device__ inline size_t expand_warp_bytes(int m, int B, int ts) {
 constexpr int kWideB = 32;
 constexpr int kWide = 2;        // KIND of the wide mode
 constexpr int kWideWarps = 11;  // warps per CTA (one CTA per SM: 11 x 20.6 KB of shared memory at m = 1024)
+constexpr int kWideWarpsMany = 16;  // of rows short enough (about 640 neurons): 128 registers a thread
 // words of the low neurons' header: (start, length) per low neuron, then the
 // packed low digits of the block's candidates (5 bits per neuron); then the table
 constexpr int kLowDig = 16, kLowHdr = 48, kLowTab = 1024;
