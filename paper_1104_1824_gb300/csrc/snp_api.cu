@@ -610,7 +610,7 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
   h->row_w = W;
   h->pool_rows = (int64_t)(h->d_pool.bytes / ((size_t)W * m));  // the store's capacity in rows of this width
   // Pool: exact when capped, growing otherwise.
-  int64_t rows_plan = 1 << 12;
+  int64_t rows_plan = 1 << 15;
   if (cap > 0) {
     const long double want = 1.0L + (long double)o->depth * (long double)cap;
     rows_plan = want > 2.0e9L ? (int64_t)2000000000 : (int64_t)want;
@@ -727,6 +727,11 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
   int64_t tombs = 0;
   double rate = 1.0;  // new configurations per candidate, for chunk sizing
   bool few_before = true;  // the last depth had at most 256 candidates per parent
+  // Whatever way this function is left, nothing of it is still running.
+  struct Drain {
+    cudaStream_t st;
+    ~Drain() { cudaStreamSynchronize(st); }
+  } drain{st};
   h->pin.ctr[0] = (unsigned long long)h->n_rows;
   h->pin.ctr[1] = 0;  // set per depth by the Psi kernel
   h->pin.ctr[2] = (unsigned long long)h->n_store;
@@ -737,37 +742,221 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     return SNP_OK;
   };
 
+  // Arguments that every pass of this exploration shares.
+  auto claim_args = [&](int64_t lo) {
+    ClaimArgs a;
+    a.sys = h->dev();
+    a.parents = h->d_pool.as<int32_t>();
+    a.pperm = h->d_perm.as<uint32_t>() + lo;
+    a.off = h->d_off.as<uint64_t>();
+    a.run = 0;
+    a.table = h->table();
+    a.pool = h->d_pool.as<int32_t>();
+    a.staging = nullptr;
+    a.store_ctr = h->d_ctr.as<unsigned long long>() + 2;
+    a.sidx_of = h->d_sidx.as<uint32_t>();
+    a.store_cap = (uint64_t)h->pool_rows;
+    a.gmin = h->d_gmin.as<uint32_t>();
+    a.slot_of = h->d_slot_of.as<uint32_t>();
+    a.ownbits = h->d_own.as<uint32_t>();
+    a.ctr = h->d_ctr.as<unsigned long long>();
+    a.st = h->d_st.as<ChunkState>();
+    a.wait_ns = wait_ns;
+    a.w = W;
+    return a;
+  };
+  auto commit_args = [&](int64_t lo, uint64_t Q) {
+    CommitArgs c;
+    c.sys = h->dev();
+    c.Q = (uint32_t)Q;
+    c.nwords = (uint32_t)((Q + 31) / 32);
+    c.bits = h->d_bits.as<uint32_t>();
+    c.ticket = h->d_counts.as<uint32_t>();
+    c.counts = c.ticket + 2;
+    c.srow = h->d_srow.as<uint32_t>();
+    c.slot_of = h->d_slot_of.as<uint32_t>();
+    c.staging = nullptr;
+    c.table = h->table();
+    c.pool = h->d_pool.as<int32_t>();
+    c.perm = h->d_perm.as<uint32_t>();
+    c.sidx_of = h->d_sidx.as<uint32_t>();
+    c.row_base = 0;
+    c.remaining = 0;
+    c.ctr = h->d_ctr.as<unsigned long long>();
+    c.rec_parent = o->record_parents ? h->d_rec_parent.as<int64_t>() : nullptr;
+    c.rec_index = o->record_parents ? h->d_rec_index.as<uint64_t>() : nullptr;
+    c.off = h->d_off.as<uint64_t>();
+    c.parent_base = lo;
+    c.st = h->d_st.as<ChunkState>();
+    c.host = nullptr;
+    c.dyn = nullptr;
+    c.host_depth = nullptr;
+    return c;
+  };
+  auto next_scan_epoch = [&]() -> int {
+    if (++h->scan_epoch >> 30) {
+      CK(cudaMemsetAsync(h->d_scan.p, 0, h->d_scan.bytes, st));
+      h->scan_epoch = 1;
+    }
+    return SNP_OK;
+  };
+  // Small depths run without the host: Psi, the first pass and its commit are
+  // enqueued together, sized on the device, and the next depth's behind them,
+  // which does nothing unless that pass was all its depth needed.  The host
+  // reads a depth back while the next one runs.  (With a wait after Psi and one
+  // after the pass, a depth of a few candidates took 50 us, half of it idle.)
+  constexpr uint64_t kChainQ = 1 << 17;  // largest pass: beyond it the waits no longer show
+  bool chained = false;                  // depth d is already enqueued
+  bool one_pass = true;                  // the last depth took one pass
+  uint64_t last_T = 1;
+  uint64_t flying_q = 0;                 // candidates of such a pass not read back yet
+  bool chain_rec[2] = {false, false};
+  int64_t chain_launches[2] = {0, 0};
+  auto chain_pass = [&]() -> uint64_t {  // candidates of such a pass; 0: not now
+    if (tc || tc5 || !one_pass) return 0;
+    if (psi_saturated_before && (cap <= 0 || cap > 2 * kPsiHead)) return 0;  // large frontiers whose rows mostly are not read
+    double want = cap > 0 ? (double)cap / std::max(rate, 1.0 / 1024.0) * 1.25 + 4096.0
+                          : std::max(4096.0, 8.0 * (double)last_T);
+    if (want > (double)kChainQ) return 0;
+    uint64_t Q = std::min<uint64_t>((uint64_t)want, qmax);
+    if (budget > 0) Q = std::min<uint64_t>(Q, (uint64_t)budget);
+    // room for this pass behind the one not read back, every candidate of them new
+    auto rows = [&](uint64_t q) { return cap > 0 ? std::min<uint64_t>(q, (uint64_t)cap) : q; };
+    if ((uint64_t)h->n_rows + rows(flying_q) + rows(Q) > (uint64_t)h->perm_rows) return 0;
+    if ((uint64_t)h->n_store + flying_q + Q > (uint64_t)h->pool_rows) return 0;
+    if ((long double)(h->n_rows + tombs) + (long double)(flying_q + Q) > 0.75L * (long double)(h->nbuckets * kBucket))
+      return 0;
+    return Q;
+  };
+  // Depth d: the frontier is [lo, lo + P), or with after_prev what depth d - 1
+  // (enqueued just before) finds from row lo on, up to P rows.
+  auto chain_depth = [&](int d, int64_t lo, int64_t P, uint64_t Q, bool after_prev) -> int {
+    const int x = d & 1;
+    DepthDyn* dyn = h->d_dyn.as<DepthDyn>();
+    CK(cudaEventRecord(h->ev[x][0], st));
+    TRY(next_scan_epoch());
+    PsiArgs pa;
+    std::memset(&pa, 0, sizeof pa);
+    pa.s = h->dev();
+    pa.rows = h->d_pool.as<int32_t>();
+    pa.perm = h->d_perm.as<uint32_t>() + lo;
+    pa.P = P;
+    pa.expect = after_prev ? std::min<int64_t>(P, 4 * std::max<int64_t>(level_hi - level_lo, 64)) : P;
+    pa.max_expand = o->max_expand_value;
+    pa.off = h->d_off.as<uint64_t>();
+    chain_rec[x] = few_before;
+    pa.rec = few_before ? h->d_prec.as<ParentRec>() : nullptr;
+    pa.ticket = h->d_scan.as<uint32_t>();
+    pa.tiles = h->d_scan.as<ScanTile>() + 1;
+    pa.epoch = h->scan_epoch;
+    pa.st = h->d_st.as<ChunkState>();
+    pa.ctr = h->d_ctr.as<unsigned long long>();
+    pa.remaining = cap > 0 ? (uint64_t)cap : ~0ull;
+    pa.dyn = dyn + x;
+    pa.prev = after_prev ? dyn + (x ^ 1) : nullptr;
+    pa.level_lo = lo;
+    pa.budget = (unsigned long long)budget;
+    pa.pass_max = (uint32_t)Q;
+    chain_launches[x] = 2 + launch_psi(pa, W, st, nsm);
+    CK(cudaGetLastError());
+    ClaimArgs a = claim_args(lo);
+    a.P = P;
+    a.g0 = 0;
+    a.Q = (uint32_t)Q;
+    a.prec = pa.rec;
+    a.dyn = dyn + x;
+    if (m > kWideM) {
+      TRY(h->d_bcache.reserve(wide_base_bytes(m)));
+      a.bcache = h->d_bcache.as<int32_t>();
+    }
+    if (o->kernel_timing) CK(cudaEventRecord(h->evk[x][0], st));
+    chain_launches[x] += launch_expand(a, st, nsm);
+    CK(cudaGetLastError());
+    if (o->kernel_timing) CK(cudaEventRecord(h->evk[x][1], st));
+    CommitArgs c = commit_args(lo, Q);
+    c.P = P;
+    c.g0 = 0;
+    c.dyn = dyn + x;
+    c.host_depth = h->pin.depth[x];
+    launch_mark_commit(c, h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(), st, nsm);
+    CK(cudaGetLastError());
+    CK(cudaEventRecord(h->ev[x][1], st));
+    return SNP_OK;
+  };
+
   for (int d = d_start; d <= o->depth; ++d) {
     if (cancelled()) {
       CK(cudaStreamSynchronize(st));
       return fail(SNP_E_CANCELLED, "cancelled before depth %d", d);
     }
+    if (timed_depth >= 0) {  // before its events are used again
+      CK(cudaEventSynchronize(h->ev[timed_depth & 1][1]));
+      TRY(depth_ms(timed_depth));
+      timed_depth = -1;
+    }
     snp_depth_info sd;
     std::memset(&sd, 0, sizeof sd);
     const int64_t P = level_hi - level_lo;
     sd.parents = P;
-    CK(cudaEventRecord(h->ev[d & 1][0], st));
-    // When the previous depth's Psi sum saturated, the first rows alone may
-    // hold 2^64 - 1 candidates: they go first, and if they do, the rest are
-    // not read (no candidate and no statistic depends on them).
-    const int64_t P0 = psi_saturated_before && P > 2 * kPsiHead ? kPsiHead : P;
-    {  // buffers of the frontier: when capped, once for all depths
-      const int64_t want = cap > 0 ? std::max<int64_t>(P, std::min<int64_t>(cap, 1 << 22)) : P;
-      if (h->psi_cap < P) {
+    const uint64_t chain_q = chained ? 0 : chain_pass();
+    // buffers of the frontier: when capped, once for all depths
+    auto frontier_buffers = [&](int64_t need) -> int {
+      if (h->psi_cap < need) {
+        const int64_t want = cap > 0 ? std::max<int64_t>(need, std::min<int64_t>(cap, 1 << 22)) : need;
         TRY(h->d_prec.reserve(sizeof(ParentRec) * want));
         TRY(h->d_off.reserve(sizeof(uint64_t) * (want + 1)));
         h->psi_cap = want;
       }
       if (!h->d_scan.p) {
         TRY(h->d_scan.reserve(sizeof(ScanTile) * (1 + psi_runs(nsm))));  // two counters, entries
-        h->scan_epoch = 0x3FFFFFFFu;  // clear it below
+        h->scan_epoch = 0x3FFFFFFFu;  // clear it on first use
       }
+      if (!h->d_dyn.p) TRY(h->d_dyn.reserve(sizeof(DepthDyn) * 2));
+      return SNP_OK;
+    };
+    HostDepth hd;
+    std::memset(&hd, 0, sizeof hd);
+    bool next_chained = false;
+    if (!chained && chain_q > 0) {
+      TRY(frontier_buffers(std::max<int64_t>(P, (int64_t)chain_q)));
+      TRY(ensure_chunk_buffers(h, chain_q, st));
+      TRY(chain_depth(d, level_lo, P, chain_q, false));
+      flying_q = chain_q;
+      chained = true;
     }
+    if (chained) {
+      const uint64_t q1 = d < o->depth ? chain_pass() : 0;
+      if (q1 > 0 && q1 <= h->q_cap) {
+        TRY(chain_depth(d + 1, level_hi, cap > 0 ? std::min<int64_t>(h->psi_cap, cap) : h->psi_cap, q1, true));
+        next_chained = true;
+      }
+      flying_q = next_chained ? q1 : 0;
+      CK(cudaEventSynchronize(h->ev[d & 1][1]));
+      hd = *h->pin.depth[d & 1];
+      if (const uint32_t e = hd.cs.error) {
+        const char* where = hd.d.go ? "expand/claim/commit" : "applicability scan";
+        if (e & kErrOverflow) return fail(SNP_E_OVERFLOW, "%s: a spike count could leave the int32 range", where);
+        if (e & kErrTimeout) return fail(SNP_E_TIMEOUT, "%s: bounded wait for a hash slot ran out", where);
+        return fail(SNP_E_INTERNAL, "%s: device consistency check failed (bits 0x%x)", where, e);
+      }
+      sd.launches += chain_launches[d & 1];
+      chained = false;
+    }
+    const bool scanned = hd.d.P > 0;  // Psi of this depth is done (and its first pass, if any, too)
+    if (scanned && hd.d.P != P) return fail(SNP_E_INTERNAL, "frontier of %lld rows, %lld expected", (long long)hd.d.P, (long long)P);
+    if (!scanned) {
+      TRY(frontier_buffers(P));
+      CK(cudaEventRecord(h->ev[d & 1][0], st));
+    }
+    // When the previous depth's Psi sum saturated, the first rows alone may
+    // hold 2^64 - 1 candidates: they go first, and if they do, the rest are
+    // not read (no candidate and no statistic depends on them).
+    const int64_t P0 = psi_saturated_before && P > 2 * kPsiHead ? kPsiHead : P;
     const int32_t* parents = h->d_pool.as<int32_t>();            // the store (W bytes per count)
     const uint32_t* pperm = h->d_perm.as<uint32_t>() + level_lo;  // its rows of this frontier
     // Parent records serve the batches that cross parents; they are worth their
     // writing with few candidates per parent, as expected from the last depth.
-    bool with_records = !tc && !tc5 && few_before;
+    bool with_records = scanned ? chain_rec[d & 1] : !tc && !tc5 && few_before;
     uint64_t remaining = cap > 0 ? (uint64_t)cap : ~0ull;  // as of the passes read back so far
     PsiArgs pa;
     std::memset(&pa, 0, sizeof pa);
@@ -778,10 +967,7 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     pa.tiles = h->d_scan.as<ScanTile>() + 1;
     pa.st = h->d_st.as<ChunkState>();
     auto psi_rows = [&](int64_t lo, int64_t hi) -> int {
-      if (++h->scan_epoch >> 30) {
-        CK(cudaMemsetAsync(h->d_scan.p, 0, h->d_scan.bytes, st));
-        h->scan_epoch = 1;
-      }
+      TRY(next_scan_epoch());
       pa.perm = pperm + lo;
       pa.P = hi - lo;
       pa.off = h->d_off.as<uint64_t>() + lo;
@@ -798,22 +984,22 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
       CK(cudaGetLastError());
       return SNP_OK;
     };
-    TRY(psi_rows(0, P0));
-    if (P0 < P) TRY(psi_rows(P0, P));
-    CK(cudaEventRecord(h->evs[0], st));
-    CK(cudaEventSynchronize(h->evs[0]));
-    if (const uint32_t e = h->pin.h->error) {
-      if (e & kErrOverflow) return fail(SNP_E_OVERFLOW, "applicability scan: a spike count could leave the int32 range");
-      if (e & kErrTimeout) return fail(SNP_E_TIMEOUT, "applicability scan: bounded wait ran out");
-      return fail(SNP_E_INTERNAL, "applicability scan: device consistency check failed (bits 0x%x)", e);
+    if (!scanned) {
+      TRY(psi_rows(0, P0));
+      if (P0 < P) TRY(psi_rows(P0, P));
+      CK(cudaEventRecord(h->evs[0], st));
+      CK(cudaEventSynchronize(h->evs[0]));
+      if (const uint32_t e = h->pin.h->error) {
+        if (e & kErrOverflow) return fail(SNP_E_OVERFLOW, "applicability scan: a spike count could leave the int32 range");
+        if (e & kErrTimeout) return fail(SNP_E_TIMEOUT, "applicability scan: bounded wait ran out");
+        return fail(SNP_E_INTERNAL, "applicability scan: device consistency check failed (bits 0x%x)", e);
+      }
     }
-    if (timed_depth >= 0) TRY(depth_ms(timed_depth));  // the last depth's events have passed
-    timed_depth = -1;
-    const uint64_t total = *h->pin.u64;
+    const uint64_t total = scanned ? hd.d.total : *h->pin.u64;
     sd.candidates = total;
     psi_saturated_before = total == ~0ull;
     few_before = total <= 256ull * (uint64_t)P;
-    if (!with_records && few_before && !tc && !tc5 && P > 0) {
+    if (!with_records && few_before && !tc && !tc5 && P > 0 && !hd.d.complete) {
       with_records = true;
       pa.perm = pperm;
       pa.P = P;
@@ -825,6 +1011,7 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
       CK(cudaGetLastError());
     }
     const uint64_t T = budget > 0 ? std::min<uint64_t>(total, (uint64_t)budget) : total;
+    last_T = T;
     uint64_t g0 = 0, examined = 0;  // g0: first candidate of the next pass
     int64_t nnew = 0;
     bool capped = false;
@@ -839,6 +1026,37 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     Flight fl[2];
     int nfl = 0, next_slot = 0;
     uint64_t pend_add = 0, pend_q = 0;  // rows the passes in flight may add; their candidates
+    auto absorb = [&](const ChunkState& cs, uint64_t first, uint64_t Q, int slot) -> int {  // a finished pass
+      if (o->kernel_timing) {
+        float kms = 0.f;
+        CK(cudaEventElapsedTime(&kms, h->evk[slot][0], h->evk[slot][1]));
+        sd.expand_ms += kms;
+      }
+      const uint64_t acc = std::min<uint64_t>(cs.n_alloc, remaining);
+      {
+        // algorithmic bytes of the expand kernel (include/snp.h, snp_depth_info),
+        // over the candidates examined (a pass that reaches the cap examines
+        // its candidates up to the last one accepted)
+        const int64_t row = (int64_t)W * m;
+        const int64_t qx = cs.capped ? (int64_t)cs.last_lid + 1 : (int64_t)Q;
+        const int64_t nparents = (int64_t)(cs.p_last - cs.p_first + 1);
+        sd.expand_bytes += qx * 8 + (qx - (int64_t)acc) * row + (int64_t)acc * (row + 8) + nparents * row;
+      }
+      h->n_store += tc5 ? (int64_t)Q : (int64_t)cs.n_alloc;  // every claim (fp8 form: candidate) took a store row
+      tombs += (int64_t)(cs.n_alloc - acc);
+      nnew += (int64_t)acc;
+      h->n_rows += (int64_t)acc;
+      if (remaining != ~0ull) remaining -= acc;
+      if (cs.capped) {
+        examined = first + cs.last_lid + 1;
+        capped = true;
+      } else {
+        examined = first + Q;
+      }
+      rate = std::max(1e-6, (double)cs.n_alloc / (double)Q);
+      sd.chunks += 1;
+      return SNP_OK;
+    };
     auto retire = [&]() -> int {        // reads back the oldest pass in flight
       const Flight f = fl[0];
       fl[0] = fl[1];
@@ -855,36 +1073,12 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         return fail(SNP_E_INTERNAL, "expand/claim/commit: device consistency check failed (bits 0x%x)", e);
       }
       if (capped) return SNP_OK;  // enqueued before the cap was known: did nothing
-      if (o->kernel_timing) {
-        float kms = 0.f;
-        CK(cudaEventElapsedTime(&kms, h->evk[f.slot][0], h->evk[f.slot][1]));
-        sd.expand_ms += kms;
-      }
-      const uint64_t acc = std::min<uint64_t>(cs.n_alloc, remaining);
-      {
-        // algorithmic bytes of the expand kernel (include/snp.h, snp_depth_info),
-        // over the candidates examined (a pass that reaches the cap examines
-        // its candidates up to the last one accepted)
-        const int64_t row = (int64_t)W * m;
-        const int64_t qx = cs.capped ? (int64_t)cs.last_lid + 1 : (int64_t)f.Q;
-        const int64_t nparents = (int64_t)(cs.p_last - cs.p_first + 1);
-        sd.expand_bytes += qx * 8 + (qx - (int64_t)acc) * row + (int64_t)acc * (row + 8) + nparents * row;
-      }
-      h->n_store += tc5 ? (int64_t)f.Q : (int64_t)cs.n_alloc;  // every claim (fp8 form: candidate) took a store row
-      tombs += (int64_t)(cs.n_alloc - acc);
-      nnew += (int64_t)acc;
-      h->n_rows += (int64_t)acc;
-      if (remaining != ~0ull) remaining -= acc;
-      if (cs.capped) {
-        examined = f.g0 + cs.last_lid + 1;
-        capped = true;
-      } else {
-        examined = f.g0 + f.Q;
-      }
-      rate = std::max(1e-6, (double)cs.n_alloc / (double)f.Q);
-      sd.chunks += 1;
-      return SNP_OK;
+      return absorb(cs, f.g0, f.Q, f.slot);
     };
+    if (hd.d.go) {
+      TRY(absorb(hd.cs, 0, hd.d.Q, d & 1));
+      g0 = hd.d.Q;
+    }
     for (;;) {
       if (cancelled()) {  // the passes in flight finish first
         while (nfl > 0) {
@@ -947,29 +1141,11 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         const int slot = next_slot;
         next_slot ^= 1;
         {
-          ClaimArgs a;
-          a.sys = h->dev();
-          a.parents = parents;
-          a.off = h->d_off.as<uint64_t>();
+          ClaimArgs a = claim_args(level_lo);
           a.P = P;
           a.g0 = g0;
           a.Q = (uint32_t)Q;
-          a.run = 0;
-          a.table = h->table();
-          a.pperm = pperm;
-          a.pool = h->d_pool.as<int32_t>();
-          a.staging = nullptr;
-          a.store_ctr = h->d_ctr.as<unsigned long long>() + 2;
-          a.sidx_of = h->d_sidx.as<uint32_t>();
-          a.store_cap = (uint64_t)h->pool_rows;
-          a.gmin = h->d_gmin.as<uint32_t>();
-          a.slot_of = h->d_slot_of.as<uint32_t>();
-          a.ownbits = h->d_own.as<uint32_t>();
           a.prec = with_records ? h->d_prec.as<ParentRec>() : nullptr;
-          a.ctr = h->d_ctr.as<unsigned long long>();
-          a.st = h->d_st.as<ChunkState>();
-          a.wait_ns = wait_ns;
-          a.w = W;
           if (o->kernel_timing) CK(cudaEventRecord(h->evk[slot][0], st));
           if (tc5) {
             Tc5Args t;
@@ -1019,31 +1195,9 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
           CK(cudaGetLastError());
           if (o->kernel_timing) CK(cudaEventRecord(h->evk[slot][1], st));
         }
-        const uint32_t nwords = (uint32_t)((Q + 31) / 32);
-        CommitArgs c;
-        c.sys = h->dev();
-        c.Q = (uint32_t)Q;
-        c.nwords = nwords;
-        c.bits = h->d_bits.as<uint32_t>();
-        c.ticket = h->d_counts.as<uint32_t>();
-        c.counts = c.ticket + 2;
-        c.srow = h->d_srow.as<uint32_t>();
-        c.slot_of = h->d_slot_of.as<uint32_t>();
-        c.staging = nullptr;
-        c.table = h->table();
-        c.pool = h->d_pool.as<int32_t>();
-        c.perm = h->d_perm.as<uint32_t>();
-        c.sidx_of = h->d_sidx.as<uint32_t>();
-        c.row_base = 0;
-        c.remaining = 0;
-        c.ctr = h->d_ctr.as<unsigned long long>();
-        c.rec_parent = o->record_parents ? h->d_rec_parent.as<int64_t>() : nullptr;
-        c.rec_index = o->record_parents ? h->d_rec_index.as<uint64_t>() : nullptr;
-        c.off = h->d_off.as<uint64_t>();
+        CommitArgs c = commit_args(level_lo, Q);
         c.P = P;
-        c.parent_base = level_lo;
         c.g0 = g0;
-        c.st = h->d_st.as<ChunkState>();
         c.host = h->pin.slot[slot];
         launch_mark_commit(c, h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(), st, nsm);
         CK(cudaGetLastError());
@@ -1058,8 +1212,11 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
       if (nfl == 0) break;
       TRY(retire());
     }
-    CK(cudaEventRecord(h->ev[d & 1][1], st));
+    if (!hd.d.complete) CK(cudaEventRecord(h->ev[d & 1][1], st));  // else recorded behind its only pass
     timed_depth = d;
+    chained = next_chained && hd.d.complete;
+    if (!chained) flying_q = 0;  // what is enqueued for the next depth does nothing
+    one_pass = sd.chunks <= 1;
     sd.new_configs = nnew;
     sd.examined = (int64_t)examined;
     sd.truncated = examined < total ? 1 : 0;
@@ -1421,6 +1578,8 @@ extern "C" int snp_explore_static(snp_handle h, const snp_explore_opts* o, int32
       c.ticket = L.counts;
       c.counts = L.counts + 2;
       c.host = h->pin.slot[0];
+      c.dyn = nullptr;
+      c.host_depth = nullptr;
       c.srow = L.srow;
       c.slot_of = L.slot_of;
       c.staging = L.staging;

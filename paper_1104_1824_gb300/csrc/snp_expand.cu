@@ -15,11 +15,14 @@ __global__ void __launch_bounds__(1024) k_wide_base(ClaimArgs a) {
   __shared__ unsigned long long s_h;
   const DevSys& s = a.sys;
   const int m = s.m;
+  if (a.dyn && !__ldcg(&a.dyn->go)) return;
+  const int64_t P = a.dyn ? __ldcg(&a.dyn->P) : a.P;
+  const uint32_t Q = a.dyn ? __ldcg(&a.dyn->Q) : a.Q;
   BaseSlot* hdr = reinterpret_cast<BaseSlot*>(a.bcache);
   int32_t* out = reinterpret_cast<int32_t*>(reinterpret_cast<unsigned char*>(a.bcache) + base_rows_offset()) +
                  (size_t)blockIdx.x * round4(m);
   if (threadIdx.x == 0) {
-    int64_t lo = 0, hi = a.P;  // largest p with off[p] <= g0 (off is sorted, off[0] = 0)
+    int64_t lo = 0, hi = P;  // largest p with off[p] <= g0 (off is sorted, off[0] = 0)
     while (hi - lo > 1) {
       const int64_t mid = lo + (hi - lo) / 2;
       if (__ldg(a.off + mid) <= a.g0) lo = mid; else hi = mid;
@@ -29,9 +32,9 @@ __global__ void __launch_bounds__(1024) k_wide_base(ClaimArgs a) {
   }
   __syncthreads();
   const int64_t p = s_p0 + blockIdx.x;
-  bool use = !(a.ctr && __ldcg(a.ctr + 1) == 0) && p < a.P;
+  bool use = !(a.ctr && __ldcg(a.ctr + 1) == 0) && p < P;
   if (use) {
-    const uint64_t lo = max(__ldg(a.off + p), a.g0), hi = min(__ldg(a.off + p + 1), a.g0 + a.Q);
+    const uint64_t lo = max(__ldg(a.off + p), a.g0), hi = min(__ldg(a.off + p + 1), a.g0 + Q);
     use = hi > lo && hi - lo >= kBaseMin;
   }
   if (!use) {
@@ -69,26 +72,32 @@ __global__ void __launch_bounds__(1024) k_wide_base(ClaimArgs a) {
   }
 }
 
-template <class RF>
+constexpr uint32_t kMinRun = 32, kMinRunWide = 16;  // least candidates of a task (launch_expand has the figures)
+
+// DYN: a depth without the host (a.dyn).
+template <class RF, bool DYN>
 __global__ void __launch_bounds__(256, 2) k_expand(ClaimArgs a, int B, int ts) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (DYN && !__ldcg(&a.dyn->go)) return;
   if (a.ctr && __ldcg(a.ctr + 1) == 0) return;  // the depth is full: a chunk enqueued ahead has nothing to do
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   ExpandSmem w = expand_smem(smem_raw + (size_t)wib * expand_warp_bytes(a.sys.m, B, ts), a.sys.m, B, ts);
-  expand_warp<RF, 0>(a, B, ts, w, (uint64_t)blockIdx.x * wpb + wib, (uint64_t)gridDim.x * wpb, lane);
+  expand_warp<RF, 0, DYN>(a, B, ts, w, (uint64_t)blockIdx.x * wpb + wib, (uint64_t)gridDim.x * wpb, kMinRun, lane);
 }
 
 // The wide mode of k_expand (rows of more than kWideM neurons).  WARPS per CTA,
 // one CTA per SM: 16 (128 registers each) where their shared memory fits, else
 // kWideWarps.  The passes are latency-bound: 301 neurons, cap 2^18: 6874 us with
 // 11 warps, 5510 us with 16.
-template <class RF, int WARPS>
+template <class RF, int WARPS, bool DYN>
 __global__ void __launch_bounds__(WARPS * 32, 1) k_expand_wide(ClaimArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (DYN && !__ldcg(&a.dyn->go)) return;
   if (a.ctr && __ldcg(a.ctr + 1) == 0) return;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   ExpandSmem w = expand_smem_wide(smem_raw + (size_t)wib * expand_wide_bytes(a.sys.m), a.sys.m);
-  expand_warp<RF, kWide>(a, kWideB, 0, w, (uint64_t)blockIdx.x * wpb + wib, (uint64_t)gridDim.x * wpb, lane);
+  expand_warp<RF, kWide, DYN>(a, kWideB, 0, w, (uint64_t)blockIdx.x * wpb + wib, (uint64_t)gridDim.x * wpb, kMinRunWide,
+                              lane);
 }
 
 // Step (d) for rows already built in global memory (the tensor-core form):
@@ -151,7 +160,7 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
     // candidates (919 neurons, passes of a few thousand: 1031 us per
     // exploration with 256 or more, 552 with 32, 498 with 16, 502 with 8)
     const uint64_t warps = (uint64_t)nsm * wpb;
-    a.run = (uint32_t)std::max<uint64_t>(16, ((uint64_t)a.Q + warps - 1) / warps);
+    a.run = (uint32_t)std::max<uint64_t>(kMinRunWide, ((uint64_t)a.Q + warps - 1) / warps);
     const uint64_t ntasks = ((uint64_t)a.Q + a.run - 1) / a.run;
     const int blocks = (int)std::min<uint64_t>((ntasks + wpb - 1) / wpb, (uint64_t)nsm);
     if (a.bcache) {  // base children of the pass's largest parents
@@ -161,10 +170,12 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
       fb<<<kBaseSlots, std::min(1024, (m + 31) / 32 * 32), bs, st>>>(a);
     }
     constexpr int kM = kWideWarpsMany, kF = kWideWarps;
-    auto fn = many ? (a.w == 2 ? k_expand_wide<RowU16, kM> : a.w == 1 ? k_expand_wide<RowU8, kM>
-                      : (m % 4) == 0 ? k_expand_wide<RowI32V, kM> : k_expand_wide<RowI32, kM>)
-                   : (a.w == 2 ? k_expand_wide<RowU16, kF> : a.w == 1 ? k_expand_wide<RowU8, kF>
-                      : (m % 4) == 0 ? k_expand_wide<RowI32V, kF> : k_expand_wide<RowI32, kF>);
+    auto pick = [&](auto rf) -> void (*)(ClaimArgs) {
+      using RF = decltype(rf);
+      if (a.dyn) return many ? k_expand_wide<RF, kM, true> : k_expand_wide<RF, kF, true>;
+      return many ? k_expand_wide<RF, kM, false> : k_expand_wide<RF, kF, false>;
+    };
+    auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : (m % 4) == 0 ? pick(RowI32V()) : pick(RowI32());
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     fn<<<blocks > 0 ? blocks : 1, wpb * 32, smem, st>>>(a);
     return a.bcache ? 2 : 1;
@@ -182,12 +193,15 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
   // passes of half a million: two tasks of 103 each run 9% slower)
   {
     const uint64_t warps = (uint64_t)nsm * per_sm * wpb, each = ((uint64_t)a.Q + warps - 1) / warps;
-    a.run = (uint32_t)std::max<uint64_t>(32, each <= 256 ? each : std::max<uint64_t>(256, (each + 1) / 2));
+    a.run = (uint32_t)std::max<uint64_t>(kMinRun, each <= 256 ? each : std::max<uint64_t>(256, (each + 1) / 2));
   }
   const uint64_t ntasks = ((uint64_t)a.Q + a.run - 1) / a.run;
   const int blocks = (int)std::min<uint64_t>((ntasks + wpb - 1) / wpb, (uint64_t)nsm * per_sm);
-  auto fn = a.w == 2 ? k_expand<RowU16> : a.w == 1 ? k_expand<RowU8>
-            : (m % 4) == 0 ? k_expand<RowI32V> : k_expand<RowI32>;
+  auto pick = [&](auto rf) -> void (*)(ClaimArgs, int, int) {
+    using RF = decltype(rf);
+    return a.dyn ? k_expand<RF, true> : k_expand<RF, false>;
+  };
+  auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : (m % 4) == 0 ? pick(RowI32V()) : pick(RowI32());
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   fn<<<blocks > 0 ? blocks : 1, wpb * 32, smem, st>>>(a, B, ts);
   return 1;

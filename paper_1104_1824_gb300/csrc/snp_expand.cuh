@@ -551,11 +551,11 @@ struct FlatLane {
 // repeats an earlier applicable rule's row.  Returns nf, which shrinks when
 // parents without candidates push a parent beyond the 32 examined.
 template <class RF>
-__device__ __forceinline__ int flat_decode(const ClaimArgs& a, uint64_t g, int nf, int64_t p, uint64_t p_lo,
-                                           int lane, FlatLane& f, bool& keep) {
+__device__ __forceinline__ int flat_decode(const ClaimArgs& a, int64_t P, uint64_t g, int nf, int64_t p,
+                                           uint64_t p_lo, int lane, FlatLane& f, bool& keep) {
   const DevSys& s = a.sys;
   const int64_t pj = p + 1 + lane;
-  f.o = pj <= a.P ? __ldcg(a.off + pj) : ~0ull;
+  f.o = pj <= P ? __ldcg(a.off + pj) : ~0ull;
   const uint64_t o31 = __shfl_sync(0xffffffffu, f.o, 31);
   if (o31 - g < (uint64_t)nf) nf = (int)(o31 - g);  // o31 > g: parent p holds g
   const uint64_t c = g + lane;
@@ -1313,8 +1313,8 @@ struct WarpTask {
 // while the parent has 32 or more candidates left, else crossing batches.  A
 // warp takes the tasks of a chunk in increasing order.
 template <class RF, int KIND>
-__device__ __forceinline__ void expand_task(const ClaimArgs& a, int B, int ts, ExpandSmem& w, uint64_t la, uint64_t lb,
-                                            WarpTask& k, int lane) {
+__device__ __forceinline__ void expand_task(const ClaimArgs& a, int64_t P, uint32_t Q, int B, int ts, ExpandSmem& w,
+                                            uint64_t la, uint64_t lb, WarpTask& k, int lane) {
   int64_t p = k.p;
   {
     // tasks come in increasing order: look among the 32 parents from the
@@ -1323,9 +1323,9 @@ __device__ __forceinline__ void expand_task(const ClaimArgs& a, int B, int ts, E
     int n = 32;
     if (p >= 0) {
       const int64_t pj = p + 1 + lane;
-      n = __popc(__ballot_sync(0xffffffffu, pj <= a.P && __ldcg(a.off + pj) <= g));
+      n = __popc(__ballot_sync(0xffffffffu, pj <= P && __ldcg(a.off + pj) <= g));
     }
-    p = n < 32 ? p + n : warp_find_parent(a.off, a.P, g, lane);
+    p = n < 32 ? p + n : warp_find_parent(a.off, P, g, lane);
   }
   uint64_t p_lo = __ldcg(a.off + p), p_hi = __ldcg(a.off + p + 1);
   if (la == 0 && lane == 0) a.st->p_first = (unsigned long long)p;
@@ -1357,7 +1357,7 @@ __device__ __forceinline__ void expand_task(const ClaimArgs& a, int B, int ts, E
     // crossing batch
     FlatLane f;
     bool keep = false;
-    const int nb = flat_decode<RF>(a, g, (int)min((uint64_t)B, lb - l), p, p_lo, lane, f, keep);
+    const int nb = flat_decode<RF>(a, P, g, (int)min((uint64_t)B, lb - l), p, p_lo, lane, f, keep);
     const uint32_t kept = __ballot_sync(0xffffffffu, keep);
     if (fill + __popc(kept) > B) {
       flush_any<RF, KIND>(a, w, ts, fill, lane);
@@ -1385,22 +1385,31 @@ __device__ __forceinline__ void expand_task(const ClaimArgs& a, int B, int ts, E
       if (kn > 0) p_lo = lo;
       p += kn;
     } else {
-      p = warp_find_parent(a.off, a.P, gn, lane);
+      p = warp_find_parent(a.off, P, gn, lane);
       p_lo = __ldcg(a.off + p);
       p_hi = __ldcg(a.off + p + 1);
     }
   }
-  if (lb == (uint64_t)a.Q && lane == 0) a.st->p_last = (unsigned long long)p;
+  if (lb == (uint64_t)Q && lane == 0) a.st->p_last = (unsigned long long)p;
   k.p = p;
 }
 
-// The tasks task0, task0 + tstride, ... of chunk a (runs of a.run candidates).
-template <class RF, int KIND>
+// The tasks task0, task0 + tstride, ... of chunk a: runs of a.run of its
+// candidates.  DYN: the chunk's frontier and size come from a.dyn, and a run is
+// a warp's share of it, at least min_run.
+template <class RF, int KIND, bool DYN>
 __device__ __forceinline__ void expand_warp(const ClaimArgs& a, int B, int ts, ExpandSmem& w, uint64_t task0,
-                                            uint64_t tstride, int lane) {
+                                            uint64_t tstride, uint32_t min_run, int lane) {
   WarpTask k;
-  for (uint64_t la = task0 * a.run; la < a.Q; la += tstride * a.run)
-    expand_task<RF, KIND>(a, B, ts, w, la, min(la + a.run, (uint64_t)a.Q), k, lane);
+  if constexpr (DYN) {
+    const int64_t P = __ldcg(&a.dyn->P);
+    const uint32_t Q = __ldcg(&a.dyn->Q), run = max(min_run, (uint32_t)((Q + tstride - 1) / tstride));
+    for (uint64_t la = task0 * run; la < Q; la += tstride * run)
+      expand_task<RF, KIND>(a, P, Q, B, ts, w, la, min(la + run, (uint64_t)Q), k, lane);
+  } else {
+    for (uint64_t la = task0 * a.run; la < a.Q; la += tstride * a.run)
+      expand_task<RF, KIND>(a, a.P, a.Q, B, ts, w, la, min(la + a.run, (uint64_t)a.Q), k, lane);
+  }
 }
 
 }  // namespace

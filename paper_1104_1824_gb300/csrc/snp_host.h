@@ -90,16 +90,19 @@ struct PinnedState {
   ChunkState* h = nullptr;      // counters of the last pass read back
   ChunkState* slot[2] = {nullptr, nullptr};  // counters of passes in flight
   uint64_t* u64 = nullptr;
-  unsigned long long* ctr = nullptr;         // source of the device counters {rows, still acceptable}
+  unsigned long long* ctr = nullptr;         // source of the device counters {rows, still acceptable, store rows}
+  HostDepth* depth[2] = {nullptr, nullptr};  // depths that run without the host, by parity
   PinnedState() {
     void* p = nullptr;
-    if (cudaMallocHost(&p, 512) == cudaSuccess) {
+    if (cudaMallocHost(&p, 1024) == cudaSuccess) {
       char* c = static_cast<char*>(p);
       h = reinterpret_cast<ChunkState*>(c);
       u64 = reinterpret_cast<uint64_t*>(c + 128);
       slot[0] = reinterpret_cast<ChunkState*>(c + 192);
       slot[1] = reinterpret_cast<ChunkState*>(c + 256);
       ctr = reinterpret_cast<unsigned long long*>(c + 320);
+      depth[0] = reinterpret_cast<HostDepth*>(c + 512);
+      depth[1] = reinterpret_cast<HostDepth*>(c + 768);
     }
   }
   ~PinnedState() {
@@ -169,6 +172,7 @@ struct snp_system {
   DevBuf d_pool, d_slots, d_gmin, d_slot_of, d_bits, d_counts, d_srow, d_own, d_off, d_scan, d_st,
       d_rec_parent, d_rec_index, d_tmp,
       d_prec, d_ctr, d_perm, d_sidx,
+      d_dyn,     // depths that run without the host, by parity
       d_bcache;  // wide mode: base children of each pass's largest parents
   int64_t pool_rows = 0;  // capacity in rows (of the store: every row claimed during an exploration)
   int32_t row_w = 4;      // bytes per spike count of the store's rows (4: int32; 2, 1: packed)

@@ -65,23 +65,30 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const DevSys& s = a.s;
   const int m = s.m;
-  const uint32_t ntiles = (uint32_t)((a.P + R - 1) / R);
+  int64_t P = a.P;
+  uint32_t sub = a.sub;
+  if (a.prev) {  // the frontier is what the depth before found, if it is complete
+    P = __ldcg(&a.prev->go) && __ldcg(&a.prev->complete) ? (int64_t)__ldcg(a.ctr) - a.level_lo : 0;
+    if (P > a.P) P = 0;  // more than the buffers hold: the host takes over
+  }
+  const uint32_t ntiles = (uint32_t)((P + R - 1) / R);
+  if (a.prev) sub = max(1u, (ntiles + gridDim.x - 1) / gridDim.x);
   const uint64_t base = a.carry ? __ldcg(a.carry) : 0ull;
   if (a.off && base == kSat) {
     // these rows lie past the last candidate: Psi is not needed
-    for (int64_t p = (int64_t)blockIdx.x * 256 + tid; p < a.P; p += (int64_t)gridDim.x * 256) a.off[p + 1] = kSat;
+    for (int64_t p = (int64_t)blockIdx.x * 256 + tid; p < P; p += (int64_t)gridDim.x * 256) a.off[p + 1] = kSat;
   } else {
     bool over = false;
     if (tid == 0) s_run = a.off ? atomicAdd(a.ticket, 1u) : blockIdx.x;
     __syncthreads();
-    const uint32_t run = s_run, tile0 = run * a.sub, tile1 = min(tile0 + a.sub, ntiles);
+    const uint32_t run = s_run, tile0 = run * sub, tile1 = min(tile0 + sub, ntiles);
     uint64_t through = 0, before = 0;  // sum of the run's tiles so far; this lane's exclusive sum within the run
     for (uint32_t tile = tile0; tile < tile1; ++tile) {
       const int64_t p0 = (int64_t)tile * R + (WARP ? warp : warp * 32);  // this warp's first row
       PsiAcc acc;
       uint64_t v = 0;  // Psi of this lane's row (WARP: lane 0's)
       if (WARP) {
-        if (p0 < a.P) {
+        if (p0 < P) {
           const typename RF::T* row = row_at<RF>(a.rows, a.perm ? __ldg(a.perm + p0) : (uint64_t)p0, m);
           ParentRec* rec = REC ? a.rec + p0 : nullptr;
           for (int n0 = 0; n0 < m; n0 += 32 * kPsiBatch) {
@@ -136,7 +143,7 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
         if (lane == 0) s_w[warp] = v;
       } else {
         int32_t(*slab)[33] = slabs[warp];
-        const int nr = (int)max((int64_t)0, min((int64_t)32, a.P - p0));
+        const int nr = (int)max((int64_t)0, min((int64_t)32, P - p0));
         const uint64_t pr = lane < nr ? (a.perm ? __ldg(a.perm + p0 + lane) : (uint64_t)(p0 + lane)) : 0ull;
         ParentRec* rec = REC ? a.rec + p0 + lane : nullptr;
         for (int n0 = 0; n0 < m && nr > 0; n0 += 32) {
@@ -211,7 +218,7 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
       through = sat_add(through, sum);
       __syncthreads();
       const int64_t p = WARP ? (int64_t)tile * R + lane : p0 + lane;
-      if (a.sub > 1 && (!WARP || (warp == 0 && lane < 8)) && p < a.P) a.off[p] = before;
+      if (sub > 1 && (!WARP || (warp == 0 && lane < 8)) && p < P) a.off[p] = before;
     }
     if (a.off && tile0 < ntiles) {
       if (warp == 0) {
@@ -229,10 +236,10 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
         if (!WARP || (warp == 0 && lane < 8)) {
           for (uint32_t tile = tile0; tile < tile1; ++tile) {  // each thread's own rows
             const int64_t p = (int64_t)tile * R + (WARP ? lane : tid);
-            if (p < a.P) a.off[p] = sat_add(prefix, a.sub > 1 ? a.off[p] : before);
+            if (p < P) a.off[p] = sat_add(prefix, sub > 1 ? a.off[p] : before);
           }
         }
-        if (tile1 == ntiles && tid == 0) a.off[a.P] = sat_add(prefix, through);
+        if (tile1 == ntiles && tid == 0) a.off[P] = sat_add(prefix, through);
       }
     }
     if (__any_sync(0xffffffffu, over) && lane == 0) set_error(a.st, kErrOverflow);
@@ -246,9 +253,21 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
   __threadfence();
   a.ticket[0] = 0;
   a.ticket[1] = 0;
+  if (a.dyn) {
+    DepthDyn y;
+    y.P = P;
+    y.total = P > 0 ? __ldcg(a.off + P) : 0ull;
+    y.T = a.budget ? min(y.total, (uint64_t)a.budget) : y.total;
+    y.Q = (uint32_t)min(y.T, (uint64_t)a.pass_max);
+    y.go = P > 0 && y.T > 0 && __ldcg(&a.st->error) == 0 ? 1u : 0u;
+    y.complete = 0;
+    y.pad = 0;
+    *a.dyn = y;
+    if (P > 0) a.ctr[1] = a.remaining;
+  }
   if (a.host_total) {  // the depth's candidates and errors to the host; the depth's counter starts
     if (a.ctr) a.ctr[1] = a.remaining;
-    *a.host_total = __ldcg(a.off + a.P);
+    *a.host_total = __ldcg(a.off + P);
     a.host->error = __ldcg(&a.st->error);
     __threadfence_system();
   }
@@ -260,7 +279,7 @@ template <class RF, bool REC>
 void psi_launch(PsiArgs a, bool warp, cudaStream_t st, int nsm) {
   const int64_t tiles = (a.P + (warp ? 7 : 255)) / (warp ? 8 : 256);
   const int64_t resident = (int64_t)nsm * (REC ? 2 : 3);
-  a.sub = (uint32_t)((tiles + resident - 1) / resident);
+  a.sub = (uint32_t)std::max<int64_t>(1, (tiles + resident - 1) / resident);
   const int blocks = (int)std::max<int64_t>(1, (tiles + a.sub - 1) / a.sub);
   if (warp)
     k_psi<RF, REC, true><<<blocks, 256, 0, st>>>(a);
@@ -281,7 +300,7 @@ static bool psi_by_warp(int64_t P, int m, int nsm) {
 size_t psi_runs(int nsm) { return (size_t)nsm * 3; }
 
 int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm) {
-  const bool warp = psi_by_warp(a.P, a.s.m, nsm);
+  const bool warp = psi_by_warp(a.expect > 0 ? a.expect : a.P, a.s.m, nsm);
   if (w == 1)
     a.rec ? psi_launch<RowU8, true>(a, warp, st, nsm) : psi_launch<RowU8, false>(a, warp, st, nsm);
   else if (w == 2)
@@ -299,8 +318,10 @@ int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm) {
 // in flight together (a thread per word walked its claims one after another:
 // 8 us per pass of 2^16, 11 us per pass of 2^20).
 __global__ void __launch_bounds__(256) k_mark(uint32_t* ownbits, const uint32_t* gmin, uint32_t* bits, uint32_t* srow,
-                                              uint32_t nwords, uint32_t* counts, int tile_log, ChunkState* st) {
+                                              uint32_t nwords, uint32_t* counts, int tile_log, ChunkState* st,
+                                              const DepthDyn* dyn) {
   constexpr int U = kMarkWords;
+  if (dyn && !__ldcg(&dyn->go)) return;
   const int lane = threadIdx.x & 31;
   const uint32_t limit = nwords * 32u;
   const uint32_t nw = gridDim.x * (blockDim.x >> 5);
@@ -391,6 +412,8 @@ __global__ void __launch_bounds__(256) k_commit(CommitArgs a, uint32_t tile_word
   const uint64_t remaining = a.ctr ? __ldcg(a.ctr + 1) : a.remaining;
   const uint32_t tile = blockIdx.x, t0 = tile * tile_words, t1 = min(t0 + tile_words, a.nwords);
   const uint32_t mine = __ldcg(a.counts + tile);
+  const int64_t P = a.dyn ? __ldcg(&a.dyn->P) : a.P;
+  const uint32_t Q = a.dyn ? __ldcg(&a.dyn->Q) : a.Q;
   {  // first occurrences of the tiles before this one (the last CTA: of all)
     uint32_t sum = 0;
     for (uint32_t i = tid; i < tile; i += 256) sum += __ldcg(a.counts + i);
@@ -399,8 +422,8 @@ __global__ void __launch_bounds__(256) k_commit(CommitArgs a, uint32_t tile_word
     if (lane == 0) s_part[warp] = sum;
   }
   if (warp == 1 && a.rec_parent && mine) {  // the parents of the tile's candidates
-    const uint64_t gf = a.g0 + (uint64_t)t0 * 32u, gl = min(a.g0 + (uint64_t)t1 * 32u, a.g0 + a.Q) - 1;
-    const int64_t p0 = warp_find_parent(a.off, a.P, gf, lane), p1 = warp_find_parent(a.off, a.P, gl, lane);
+    const uint64_t gf = a.g0 + (uint64_t)t0 * 32u, gl = min(a.g0 + (uint64_t)t1 * 32u, a.g0 + Q) - 1;
+    const int64_t p0 = warp_find_parent(a.off, P, gf, lane), p1 = warp_find_parent(a.off, P, gl, lane);
     if (lane == 0) {
       s_p0 = p0;
       s_p1 = p1;
@@ -505,13 +528,21 @@ __global__ void __launch_bounds__(256) k_commit(CommitArgs a, uint32_t tile_word
   c.reserved = 0;
   c.p_first = __ldcg(&a.st->p_first);
   c.p_last = __ldcg(&a.st->p_last);
-  if (a.ctr) {
+  if (a.ctr && !(a.dyn && !__ldcg(&a.dyn->go))) {
     const unsigned long long left = remaining;
     const unsigned long long acc = min((unsigned long long)total, left);
     a.ctr[0] = (unsigned long long)row_base + acc;
     if (left != ~0ull) a.ctr[1] = left - acc;
   }
-  if (a.host) {
+  if (a.dyn) {
+    DepthDyn y = *a.dyn;
+    y.complete = y.go && !c.error && (c.capped || y.Q == y.T) ? 1u : 0u;
+    a.dyn->complete = y.complete;
+    a.host_depth->d = y;
+    a.host_depth->cs = c;
+    __threadfence_system();
+    *a.st = ChunkState{};
+  } else if (a.host) {
     *a.host = c;
     __threadfence_system();
     *a.st = ChunkState{};
@@ -532,7 +563,7 @@ void launch_mark_commit(const CommitArgs& c, uint32_t* ownbits, const uint32_t* 
   const uint32_t per = 8 * kMarkWords;
   const int blocks = (int)std::min<uint32_t>((c.nwords + per - 1) / per, (uint32_t)nsm * 16);
   const int lg = commit_words_log(c.nwords);
-  k_mark<<<blocks, 256, 0, st>>>(ownbits, gmin, c.bits, const_cast<uint32_t*>(c.srow), c.nwords, c.counts, lg + 5, c.st);
+  k_mark<<<blocks, 256, 0, st>>>(ownbits, gmin, c.bits, const_cast<uint32_t*>(c.srow), c.nwords, c.counts, lg + 5, c.st, c.dyn);
   k_commit<<<(c.nwords + (1u << lg) - 1) >> lg, 256, 0, st>>>(c, 1u << lg);
 }
 

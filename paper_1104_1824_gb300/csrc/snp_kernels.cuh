@@ -8,6 +8,22 @@
 
 namespace snp {
 
+// A depth that runs without the host: what its kernels need to know of the
+// depth before it and of one another (device memory).
+struct DepthDyn {
+  int64_t P;                  // frontier rows; 0: the depth does not run (yet)
+  uint64_t total, T;          // candidates, and those within the budget
+  uint32_t Q;                 // candidates of its first pass
+  uint32_t go;                // 1: the pass runs
+  uint32_t complete;          // 1: the pass was all the depth needed
+  uint32_t pad;
+};
+// The same for the host, with the pass's counters (pinned memory).
+struct HostDepth {
+  DepthDyn d;
+  ChunkState cs;
+};
+
 struct ClaimArgs {
   DevSys sys;
   const int32_t* parents;     // frontier rows: parents + pperm[p] * m, or parents + p * m without pperm
@@ -43,6 +59,8 @@ struct ClaimArgs {
   // Wide mode: base children of the pass's largest parents (wide_base_bytes;
   // filled by the launch before each pass), or nullptr.
   int32_t* bcache = nullptr;
+  // A depth without the host: P and Q (at most this Q) come from here.
+  const DepthDyn* dyn = nullptr;
 };
 
 // Wide mode: base children cached per pass (headers, then rows of round4(m)).
@@ -79,6 +97,10 @@ struct CommitArgs {
   uint64_t g0;
   ChunkState* st;             // the chunk's counters; with host, copied there and cleared at the end
   ChunkState* host;           // pinned host copy, or nullptr
+  // A depth without the host: P and Q (at most this Q) come from dyn, whose
+  // `complete` is set at the end; dyn and the counters go to host_depth.
+  DepthDyn* dyn;
+  HostDepth* host_depth;
 };
 constexpr int kMarkWords = 4;     // bitmap words per warp of the mark kernel
 constexpr uint32_t kCommitTiles = 2048;  // most commit tiles of a chunk
@@ -221,6 +243,16 @@ struct PsiArgs {
   ChunkState* host;
   unsigned long long* ctr;
   unsigned long long remaining;
+  // A depth without the host (dyn set): with prev, the frontier is what the
+  // depth before it found, rows level_lo .. ctr[0] - 1, if that depth is
+  // complete and they are at most P; dyn receives the frontier, its candidates
+  // and the first pass (at most pass_max of the budget's candidates).
+  DepthDyn* dyn;
+  const DepthDyn* prev;
+  int64_t level_lo;
+  int64_t expect;             // frontier rows to choose the kernel by (0: P)
+  unsigned long long budget;  // 0: none
+  uint32_t pass_max;
 };
 size_t psi_runs(int nsm);
 // rows: w bytes per spike count (4: int32; 2, 1: a packed store).  Returns the launches made.

@@ -114,7 +114,7 @@ __device__ __noinline__ void expand_item(const ClaimArgs& a, unsigned char* smem
                                          WarpTask& k) {
   const int lane = threadIdx.x & 31, m = a.sys.m, ts = round4(m) + 4;
   ExpandSmem w = KIND == kWide ? expand_smem_wide(smem, m) : expand_smem(smem, m, B, ts);
-  expand_task<RF, KIND>(a, B, ts, w, la, lb, k, lane);
+  expand_task<RF, KIND>(a, a.P, a.Q, B, ts, w, la, lb, k, lane);
 }
 
 }  // namespace
