@@ -325,7 +325,7 @@ def roofline_of(args, system, snp, transition: str, r, packed: bool = False):
         achieved = ops / (r["expand_ms"] * 1e-3) / 1e12 if r["expand_ms"] > 0 else None
         traffic = profiled_traffic(args.workload, "tc_rows")
         return {
-            "kernel": "k_tc_digits + k_tc_rows (mma.sync m16n8k32 s8) + k_resolve_rows, per pass",
+            "kernel": "k_tc_masks + k_tc_rows (mma.sync m16n8k32 s8) + k_resolve_rows, per pass",
             "bound": "tensor", "achieved": round(achieved, 2) if achieved else None, "peak": round(peak, 1),
             "peak_kind": "measured mma.sync m16n8k32 s8 rate on this GPU (snp_tc_peak_tops)", "unit": "TOPS",
             "frac": round(achieved / peak, 4) if achieved else None,
@@ -527,7 +527,7 @@ def bench_batch(args, w, systems, snp, torch, dist, dev, rank, world, local):
             "value": round(vf, 1), "unit": UNIT, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": round(msf / args.steps, 3), "ratio_to_sparse_i32": round(vf / value, 4),
             "dtype": "fp8 e4m3 operands, fp32 accumulation (exact)", "plan": rf["plan"],
-            "roofline": {"kernel": "k_batch_depth<tensor-core form> (tcgen05 tiles of 128 candidates per system, "
+            "roofline": {"kernel": "k_batch_depth_tc (tcgen05 tiles of 128 candidates per system, "
                                    "one launch per depth)", "bound": "hbm",
                          "achieved": round(rf["bytes_step"] * args.steps / (rf["ms"] * 1e-3) / 1e9, 1),
                          "peak": peak, "peak_kind": f"{peak_kind} copy bandwidth", "unit": "GB/s",
@@ -584,7 +584,7 @@ def bench_batch(args, w, systems, snp, torch, dist, dev, rank, world, local):
                        "l2": "inputs larger than L2 (pools of all systems, tens of GB)",
                        "parallelism": f"dp{world}: rank r explores systems of seeds {w['base_seed']} + {w['n']} r ..."
                        if world > 1 else "single GPU"},
-            "roofline": {"kernel": "k_batch_depth (one launch per depth, all systems)", "bound": "hbm",
+            "roofline": {"kernel": "k_many_psi, k_many_expand, k_many_copy and their control kernels (all systems)", "bound": "hbm",
                          "achieved": round(achieved, 1), "peak": peak, "peak_kind": f"{peak_kind} copy bandwidth",
                          "unit": "GB/s", "frac": round(achieved / peak, 4),
                          "algorithmic_bytes_per_launch": int(bytes_step / w["depth"]),

@@ -110,38 +110,20 @@ int ensure_chunk_buffers(snp_system* h, uint64_t q, cudaStream_t st) {
   return SNP_OK;
 }
 
-// Tensor-core form: M_Pi^T in int8 (zero padded) and the rule maps, uploaded
-// on first use; chunk buffers for up to q candidates.
-int tc_prepare(snp_system* h, uint64_t q, cudaStream_t st) {
+// Int8 tensor-core form: M_Pi^T uploaded on first use; chunk buffers for up to
+// q candidates.
+int tc_prepare(snp_system* h, uint64_t q) {
   if (!h->d_MT.p) {
-    const int m = h->m, R = h->R;
-    h->Rp = (R + 31) / 32 * 32;
-    h->mp = (m + 3) / 4 * 4;
-    h->mt_rows = (m + 127) / 128 * 128;
-    std::vector<int8_t> mt((size_t)h->mt_rows * h->Rp, 0);
-    for (int r = 0; r < R; ++r)
-      for (int j = 0; j < m; ++j) mt[(size_t)j * h->Rp + r] = (int8_t)h->M[(size_t)r * m + j];
-    std::vector<int16_t> rn(h->Rp, -1);
-    std::vector<uint8_t> rk(h->Rp, 0);
-    for (int r = 0; r < R; ++r) {
-      rn[r] = (int16_t)h->rule_neuron[r];
-      rk[r] = (uint8_t)(r - h->first_rule[h->rule_neuron[r]]);
-    }
+    h->tc_nb = tc_blocks(h->R);
+    const std::vector<int8_t> mt = tc_pack(h->M.data(), h->R, h->m, h->tc_nb);
     TRY(h->d_MT.reserve(mt.size()));
-    TRY(h->d_rn.reserve(sizeof(int16_t) * h->Rp));
-    TRY(h->d_rk.reserve(h->Rp));
     CK(cudaMemcpy(h->d_MT.p, mt.data(), mt.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->d_rn.p, rn.data(), sizeof(int16_t) * h->Rp, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->d_rk.p, rk.data(), h->Rp, cudaMemcpyHostToDevice));
   }
-  if (h->tc_cap < q) {
-    TRY(h->d_loc.reserve((size_t)q * h->mp));
-    TRY(h->d_pidx.reserve(sizeof(uint32_t) * q));
-    TRY(h->d_rows.reserve(sizeof(int32_t) * (size_t)q * h->m));
-    TRY(h->d_hash.reserve(sizeof(unsigned long long) * q));
-    TRY(h->d_red.reserve(q));
-    h->tc_cap = q;
-  }
+  TRY(h->d_rbits.reserve(sizeof(uint32_t) * q * h->tc_nb));
+  TRY(h->d_pidx.reserve(sizeof(uint32_t) * q));
+  TRY(h->d_rows.reserve(sizeof(int32_t) * (size_t)q * h->m));
+  TRY(h->d_hash.reserve(sizeof(unsigned long long) * q));
+  TRY(h->d_red.reserve(q));
   return SNP_OK;
 }
 
@@ -575,7 +557,7 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
   qmax = std::min<uint64_t>(qmax, 1ull << 30);
   if (tc) {
     qmax = std::min<uint64_t>(qmax, 1ull << 16);
-    TRY(tc_prepare(h, qmax, st));
+    TRY(tc_prepare(h, qmax));
   }
   if (tc5) {  // 2^21 while the in-place store's reserve (two passes per depth) stays within 64 GiB, else 2^20
     const bool big = (long double)(1ull << 21) * 2.0L * std::max(o->depth, 1) * 4.0L * m <= (long double)(64ull << 30);
@@ -1176,12 +1158,11 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
             launch_resolve_rows(a, t.out, t.hash, t.red, st, nsm);
             sd.launches += 2;
           } else if (tc) {
-            launch_tc_digits(a.sys, parents, pperm, a.off, P, g0, (uint32_t)Q, h->d_loc.as<uint8_t>(), h->mp,
-                             h->d_pidx.as<uint32_t>(), h->d_red.as<uint8_t>(), st, nsm);
-            CK(cudaMemsetAsync(h->d_hash.p, 0, sizeof(unsigned long long) * Q, st));
-            launch_tc_rows(a.sys, parents, h->d_loc.as<uint8_t>(), h->mp, h->d_pidx.as<uint32_t>(), (uint32_t)Q,
-                           h->d_MT.as<int8_t>(), h->Rp, h->d_rn.as<int16_t>(), h->d_rk.as<uint8_t>(),
-                           h->d_rows.as<int32_t>(), h->d_hash.as<unsigned long long>(), st);
+            launch_tc_masks(a.sys, parents, pperm, a.off, P, g0, (uint32_t)Q, h->d_rbits.as<uint32_t>(), h->tc_nb,
+                            h->d_pidx.as<uint32_t>(), h->d_hash.as<unsigned long long>(), h->d_red.as<uint8_t>(), a.st,
+                            st, nsm);
+            launch_tc_rows(a.sys, parents, h->d_rbits.as<uint32_t>(), h->tc_nb, h->d_pidx.as<uint32_t>(), (uint32_t)Q,
+                           h->d_MT.as<int8_t>(), h->d_rows.as<int32_t>(), st);
             launch_resolve_rows(a, h->d_rows.as<int32_t>(), h->d_hash.as<unsigned long long>(),
                                 h->d_red.as<uint8_t>(), st, nsm);
             sd.launches += 3;

@@ -160,12 +160,12 @@ struct snp_system {
   std::vector<int32_t> scol, rval;          // neuron supports; rule values on them
   std::vector<int32_t> rterm;               // [R + 1] terms of rule r: [rterm[r], rterm[r + 1])
   std::vector<int2> term;                   // {i, j} of each term a^i (a^j)*
-  // tensor-core form: M_Pi^T as int8 [mt_rows][Rp], per-rule neuron and position
-  DevBuf d_MT, d_rn, d_rk, d_loc, d_pidx, d_rows, d_hash, d_red;
+  // int8 tensor-core form: M_Pi^T (tc_pack); per candidate its rule bits and parent row, and its row
+  DevBuf d_MT, d_rbits, d_pidx, d_rows, d_hash, d_red;
   // fp8 tensor-core form: M_Pi^T in e4m3 (tc5_pack_mt), its column and block counts
   DevBuf d_MB;
   int32_t t5_np = 0, t5_nblocks = 0;
-  int32_t Rp = 0, mp = 0, mt_rows = 0;
+  int32_t tc_nb = 0;  // words of a candidate's rule bits
   uint64_t tc_cap = 0;  // candidates the tensor-core chunk buffers hold
   std::vector<unsigned long long> colkey, rowkey;
   // exploration state

@@ -4,6 +4,8 @@
 
 #include <cuda.h>
 
+#include <vector>
+
 #include "snp_device.cuh"
 
 namespace snp {
@@ -266,14 +268,16 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm);
 // Candidates with redundant[lid] set repeat an earlier candidate and are skipped.
 void launch_resolve_rows(ClaimArgs a, const int32_t* rows, const unsigned long long* hash, const uint8_t* redundant,
                          cudaStream_t st, int nsm);
-// Tensor-core form of step (c) (snp_tc.cu).
-void launch_tc_digits(DevSys s, const int32_t* parents, const uint32_t* perm, const uint64_t* off, int64_t P,
-                      uint64_t g0, uint32_t Q,
-                      uint8_t* loc, int mp, uint32_t* pidx, uint8_t* redundant, cudaStream_t st, int nsm);
-void launch_tc_rows(DevSys s, const int32_t* parents, const uint8_t* loc, int mp, const uint32_t* pidx, uint32_t Q,
-                    const int8_t* MT, int Rp, const int16_t* rn, const uint8_t* rk, int32_t* rows,
-                    unsigned long long* hash, cudaStream_t st);
-size_t tc_rows_smem(int mp);
+// Int8 tensor-core form of step (c) (snp_tc.cu).  nb = tc_blocks(R): words of a
+// spiking vector's bits; M_Pi^T packed by tc_pack (tc_col_tiles(m) tiles).
+int tc_blocks(int R);
+int tc_col_tiles(int m);
+std::vector<int8_t> tc_pack(const int32_t* M, int R, int m, int nb);
+void launch_tc_masks(DevSys s, const int32_t* parents, const uint32_t* perm, const uint64_t* off, int64_t P,
+                     uint64_t g0, uint32_t Q, uint32_t* bits, int nb, uint32_t* pidx, unsigned long long* hash,
+                     uint8_t* redundant, ChunkState* st, cudaStream_t stream, int nsm);
+void launch_tc_rows(DevSys s, const int32_t* parents, const uint32_t* bits, int nb, const uint32_t* pidx, uint32_t Q,
+                    const int8_t* MF, int32_t* rows, cudaStream_t st);
 // fp8 tensor-core form of step (c) on tcgen05 (snp_tc5.cu): candidate rows
 // C' = C + S . M_Pi written to out[lid * m], their linear hashes and repeat flags.
 struct Tc5Args {

@@ -6,23 +6,22 @@
 // entries of M_Pi, each in [-127, 127], far inside int32.
 //
 // Per chunk:
-//   k_tc_digits  one warp per run of candidates: parent, and per neuron the
-//                chosen rule's position among the neuron's rules (0xFF: none);
-//   k_tc_rows    64 candidates x 128 columns per block; each 32-rule slice of
-//                S is generated in shared memory from the digits, M_Pi^T comes
-//                from L2, four warps issue mma.sync; the epilogue adds the
-//                parent row, writes C' and accumulates its linear hash;
+//   k_tc_masks   a warp per run of candidates: parent, the spiking vector as one
+//                bit per rule, its child's linear hash, whether it repeats an
+//                earlier candidate;
+//   k_tc_rows    128 candidates x 256 columns per CTA, 64 x 64 per warp;
 //   then the rows are resolved against the hash table as in the sparse path.
+#include <algorithm>
+
 #include "snp_kernels.cuh"
 
 namespace snp {
 
 namespace {
 
-constexpr int kTcBM = 64;        // candidates per block
-constexpr int kTcBN = 128;       // columns per pass of a block
-constexpr int kTcBK = 32;        // rules per k-step
-constexpr int kTcAStride = 48;   // bytes per A-tile row (conflict-free fragment loads)
+constexpr int kTcWarps = 8;      // per CTA: 2 (candidates) x 4 (columns)
+constexpr int kTcM = 64;         // candidates per warp
+constexpr int kTcN = 64;         // columns per warp
 
 __device__ __forceinline__ void mma_s8(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                        uint32_t b1) {
@@ -32,165 +31,203 @@ __device__ __forceinline__ void mma_s8(int (&c)[4], uint32_t a0, uint32_t a1, ui
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// Bits 4 i .. 4 i + 3 of w as four 0/1 bytes.
+__device__ __forceinline__ uint32_t nibble_bytes(uint32_t w, int i) {
+  return (((w >> (4 * i)) & 0xFu) * 0x00204081u) & 0x01010101u;
+}
+
+// Per-warp shared memory of k_tc_masks.
+struct MaskSmem {
+  uint32_t* msk;   // [m] applicable rules
+  uint32_t* word;  // [nb] the spiking vector's bits
+  uint16_t* ntl;   // [m] neurons with two or more applicable rules, least significant first
+  uint8_t* dig;    // [m] digits over ntl
+};
+__host__ __device__ inline size_t mask_smem_bytes(int m, int nb) {
+  return ((size_t)m * 7 + (size_t)nb * 4 + 15) / 16 * 16;
+}
+
 }  // namespace
 
-// Step (b) for the chunk: per candidate its parent's row (perm[p] when the
-// frontier is reached through a row map, else p) and, per neuron, the
-// position of the chosen rule among the neuron's rules.
-__global__ void __launch_bounds__(128) k_tc_digits(DevSys s, const int32_t* parents, const uint32_t* perm,
-                                                   const uint64_t* off, int64_t P,
-                                                   uint64_t g0, uint32_t Q, uint8_t* loc, int mp, uint32_t* pidx,
-                                                   uint8_t* redundant) {
-  extern __shared__ int32_t smem[];
+// Step (b) for the chunk: per candidate the bits of its chosen rules
+// (bits[lid * nb + r / 32], bit r % 32), its parent's store row (perm[p] when
+// the frontier is reached through a row map, else p), linear hash and repeat
+// flag.  A warp sets the first candidate of its run up from the parent and
+// goes on by the odometer (a digit or two per candidate).  (Decoding every
+// neuron of every candidate took 0.83 ms per 65536 candidates of 1024 neurons.)
+__global__ void __launch_bounds__(256) k_tc_masks(DevSys s, const int32_t* parents, const uint32_t* perm,
+                                                  const uint64_t* off, int64_t P, uint64_t g0, uint32_t Q,
+                                                  uint32_t run, uint32_t* bits, int nb, uint32_t* pidx,
+                                                  unsigned long long* hash, uint8_t* redundant, ChunkState* st) {
+  extern __shared__ __align__(16) unsigned char tc_smem[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int m = s.m;
-  WarpParent w;
-  w.par = smem + (size_t)wib * 2 * m;
-  w.msk = reinterpret_cast<uint32_t*>(w.par + m);
-  w.buf = nullptr;
-  const uint32_t run = 32;
-  const uint64_t ntasks = ((uint64_t)Q + run - 1) / run;
-  const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  for (uint64_t task = (uint64_t)blockIdx.x * (blockDim.x >> 5) + wib; task < ntasks; task += nw) {
-    const uint64_t la = task * run, lb = min(la + run, (uint64_t)Q);
-    int64_t p = warp_find_parent(off, P, g0 + la, lane);
-    uint64_t p_lo = __ldg(off + p), p_hi = __ldg(off + p + 1);
-    uint32_t prow = perm ? __ldg(perm + p) : (uint32_t)p;
-    load_parent(s, parents + (size_t)prow * m, w, lane);
-    for (uint64_t l = la; l < lb; ++l) {
-      const uint64_t g = g0 + l;
-      if (g >= p_hi) {
-        do {
-          ++p;
-          p_lo = p_hi;
-          p_hi = __ldg(off + p + 1);
-        } while (g >= p_hi);
-        prow = perm ? __ldg(perm + p) : (uint32_t)p;
-        load_parent(s, parents + (size_t)prow * m, w, lane);
+  MaskSmem w;
+  w.msk = reinterpret_cast<uint32_t*>(tc_smem + (size_t)wib * mask_smem_bytes(m, nb));
+  w.word = w.msk + m;
+  w.ntl = reinterpret_cast<uint16_t*>(w.word + nb);
+  w.dig = reinterpret_cast<uint8_t*>(w.ntl + m);
+  const uint64_t la = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + wib) * run;
+  if (la >= Q) return;
+  const uint64_t lb = min(la + run, (uint64_t)Q);
+  int64_t p = warp_find_parent(off, P, g0 + la, lane);
+  for (uint64_t l = la; l < lb; ++p) {
+    const uint64_t p_lo = __ldg(off + p), p_hi = __ldg(off + p + 1);
+    if (g0 + l >= p_hi) continue;  // a parent without candidates
+    const uint32_t prow = perm ? __ldg(perm + p) : (uint32_t)p;
+    const int32_t* row = parents + (size_t)prow * m;
+    __syncwarp();
+    for (int i = lane; i < nb; i += 32) w.word[i] = 0u;
+    __syncwarp();
+    // the base child: every firing neuron on its first applicable rule
+    uint64_t h = 0;
+    for (int n = lane; n < m; n += 32) {
+      const int32_t x = __ldg(row + n);
+      const uint32_t mask = appl_mask(s, n, x);
+      w.msk[n] = mask;
+      h += col_hash(s, n, x);
+      if (!mask) continue;
+      const int r = __ldg(s.first_rule + n) + __ffs(mask) - 1;
+      atomicOr(w.word + (r >> 5), 1u << (r & 31));
+      h += __ldg(s.rowkey + r);
+    }
+    h = warp_sum_u64(h);
+    __syncwarp();
+    int len = 0;
+    for (int top = m - 1; top >= 0; top -= 32) {
+      const int n = top - lane;
+      const bool nt = n >= 0 && __popc(w.msk[n]) > 1;
+      const uint32_t b = __ballot_sync(0xffffffffu, nt);
+      const int at = len + __popc(b & ((1u << lane) - 1u));
+      if (nt) {
+        w.ntl[at] = (uint16_t)n;
+        w.dig[at] = 0;
       }
-      const uint64_t t = g - p_lo;
-      const int n0 = lane * s.K, n1 = min(n0 + s.K, m);
-      uint64_t q = (w.after > t) ? 0ull : t / w.after;
-      uint8_t* dst = loc + (size_t)l * mp;
-      bool red = false;
-      for (int n = n1 - 1; n >= n0; --n) {
-        const uint32_t mask = w.msk[n];
-        if (!mask) {
-          dst[n] = 0xFF;
-          continue;
-        }
-        const uint32_t radix = __popc(mask);
-        uint32_t d;
-        if ((q >> 32) == 0) {
-          const uint32_t q32 = (uint32_t)q;
-          d = q32 % radix;
-          q = q32 / radix;
-        } else {
-          d = (uint32_t)(q % radix);
-          q /= radix;
-        }
-        const int k = nth_set_bit(mask, (int)d);
-        dst[n] = (uint8_t)k;
-        red |= redundant_choice(s, mask, __ldg(s.first_rule + n) + k);
+      len += __popc(b);
+    }
+    __syncwarp();
+    int red = 0;
+    // neuron ntl[i] moves from digit d to nd (every lane follows; lane 0 writes)
+    auto move = [&](int i, int d, int nd) {
+      const int n = w.ntl[i];
+      const uint32_t mask = w.msk[n];
+      const int f = __ldg(s.first_rule + n);
+      const int ro = f + nth_set_bit(mask, d), rn = f + nth_set_bit(mask, nd);
+      h += __ldg(s.rowkey + rn) - __ldg(s.rowkey + ro);
+      red += (redundant_choice(s, mask, rn) ? 1 : 0) - (redundant_choice(s, mask, ro) ? 1 : 0);
+      if (lane == 0) {
+        w.word[ro >> 5] &= ~(1u << (ro & 31));
+        w.word[rn >> 5] |= 1u << (rn & 31);
+        w.dig[i] = (uint8_t)nd;
       }
-      red = __any_sync(0xffffffffu, red);
+    };
+    uint64_t q = g0 + l - p_lo;
+#pragma unroll 1
+    for (int i = 0; i < len && q != 0; ++i) {
+      const int d = (int)next_digit(q, __popc(w.msk[w.ntl[i]]));
+      if (d != 0) move(i, 0, d);
+    }
+    if (q != 0 && lane == 0) atomicOr(&st->error, kErrInternal);  // not an index of this parent
+    for (;;) {
+      __syncwarp();
+      for (int i = lane; i < nb; i += 32) bits[l * nb + i] = w.word[i];
       if (lane == 0) {
         pidx[l] = prow;
-        redundant[l] = red ? 1 : 0;
+        hash[l] = h;
+        redundant[l] = red > 0 ? 1 : 0;
       }
       __syncwarp();
+      ++l;
+      if (l >= lb || g0 + l >= p_hi) break;
+#pragma unroll 1
+      for (int i = 0; i < len; ++i) {  // the odometer
+        const int d = w.dig[i], nd = d + 1 == __popc(w.msk[w.ntl[i]]) ? 0 : d + 1;
+        move(i, d, nd);
+        if (nd != 0) break;
+      }
     }
   }
 }
 
-// C' = C + S . M_Pi for 64 candidates per block (all m columns, 128 per pass),
-// its linear hash into hash[lid] (which must start at zero).
-//   MT: M_Pi transposed, int8 [mt_rows >= round_up(m, 128)][Rp = round_up(R, 32)], zero padded.
-//   rn/rk: per rule its neuron and position among the neuron's rules (Rp entries; padding rules: rn = -1).
-__global__ void __launch_bounds__(128) k_tc_rows(DevSys s, const int32_t* parents, const uint8_t* loc, int mp,
-                                                 const uint32_t* pidx, uint32_t Q, const int8_t* MT, int Rp,
-                                                 const int16_t* rn, const uint8_t* rk, int32_t* rows,
-                                                 unsigned long long* hash) {
-  extern __shared__ __align__(16) unsigned char tc_smem[];
+// C' = C + S . M_Pi: 64 candidates x 64 columns per warp, no shared memory and
+// no barriers.  The operands come as the instruction wants them: a lane's
+// bytes of S are two nibbles of its candidates' rule bits, and M_Pi^T is laid
+// out fragment by fragment at load (tc_pack), so that a warp's share of 8
+// columns x 64 rules is one 16-byte load per lane (4 MB in all at 1024
+// neurons: from L2).  Bound by the int8 tensor pipe (one mma.sync in about 66
+// cycles per quarter of an SM); the version before it staged S byte by byte in
+// shared memory and ran at 28% of that rate (11.5 ms per 65536 candidates of
+// 1024 neurons).
+//   MF: [col tiles of 8][nb / 2][32 lanes] 16 bytes.
+__global__ void __launch_bounds__(kTcWarps * 32, 1) k_tc_rows(DevSys s, const int32_t* parents, const uint32_t* bits,
+                                                              int nb, const uint32_t* pidx, uint32_t Q,
+                                                              const uint4* MF, int32_t* rows) {
   const int m = s.m;
-  uint8_t* locs = tc_smem;                                   // [64][mp]
-  uint8_t* At = locs + (size_t)kTcBM * mp;                   // [64][48]
-  int32_t* prow = reinterpret_cast<int32_t*>(At + kTcBM * kTcAStride);  // [64] parent index
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
-  const uint32_t base = blockIdx.x * kTcBM;
-  const int nrows = (int)((Q - base) < (uint32_t)kTcBM ? (Q - base) : (uint32_t)kTcBM);
-  // stage the block's digits and parents
-  for (int i = tid; i < kTcBM * (mp / 4); i += blockDim.x) {
-    const int r = i / (mp / 4), c = i % (mp / 4);
-    const uint32_t v = r < nrows ? reinterpret_cast<const uint32_t*>(loc + (size_t)(base + r) * mp)[c] : 0xFFFFFFFFu;
-    reinterpret_cast<uint32_t*>(locs + (size_t)r * mp)[c] = v;
-  }
-  for (int i = tid; i < kTcBM; i += blockDim.x) prow[i] = i < nrows ? (int32_t)pidx[base + i] : 0;
-  __syncthreads();
-
-  const int row0 = warp * 16 + g, row1 = row0 + 8;
-  for (int c0 = 0; c0 < m; c0 += kTcBN) {
-    int acc[16][4];
+  const uint32_t row0 = (blockIdx.x * 2u + (warp & 1)) * kTcM;
+  const int col0 = ((int)blockIdx.y * 4 + (warp >> 1)) * kTcN;
+  if (row0 >= Q || col0 >= m) return;
+  int acc[4][8][4];
 #pragma unroll
-    for (int nt = 0; nt < 16; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0;
-    for (int r0 = 0; r0 < Rp; r0 += kTcBK) {
-      __syncthreads();
-      {  // S slice: 64 rows x 32 rules, 16 bytes per thread
-        const int i = tid >> 1, cb = (tid & 1) * 16;
-        uint32_t word[4];
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          uint32_t wv = 0;
+    for (int j = 0; j < 8; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0;
+  // rows of this lane: row0 + 16 i + g and + 8
+  const uint32_t* bp[4][2];
 #pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int r = r0 + cb + q * 4 + b;
-            const int n = rn[r];
-            const uint32_t bit = (n >= 0 && locs[(size_t)i * mp + n] == rk[r]) ? 1u : 0u;
-            wv |= bit << (8 * b);
-          }
-          word[q] = wv;
-        }
-        *reinterpret_cast<uint4*>(At + i * kTcAStride + cb) = make_uint4(word[0], word[1], word[2], word[3]);
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) bp[i][k] = bits + (size_t)min(row0 + 16u * i + 8u * k + g, Q - 1) * nb;
+  const uint4* mf = MF + (size_t)(col0 / 8) * (nb / 2) * 32 + lane;
+  for (int k2 = 0; k2 < nb / 2; ++k2) {
+    uint2 aw[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) aw[i][k] = __ldg(reinterpret_cast<const uint2*>(bp[i][k] + 2 * k2));
+    uint4 b[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) b[j] = __ldg(mf + ((size_t)j * (nb / 2) + k2) * 32);
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      uint32_t a[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t lo = ks ? aw[i][0].y : aw[i][0].x, hi = ks ? aw[i][1].y : aw[i][1].x;
+        a[i][0] = nibble_bytes(lo, t4);
+        a[i][1] = nibble_bytes(hi, t4);
+        a[i][2] = nibble_bytes(lo, t4 + 4);
+        a[i][3] = nibble_bytes(hi, t4 + 4);
       }
-      __syncthreads();
-      const uint32_t a0 = *reinterpret_cast<const uint32_t*>(At + row0 * kTcAStride + 4 * t4);
-      const uint32_t a1 = *reinterpret_cast<const uint32_t*>(At + row1 * kTcAStride + 4 * t4);
-      const uint32_t a2 = *reinterpret_cast<const uint32_t*>(At + row0 * kTcAStride + 16 + 4 * t4);
-      const uint32_t a3 = *reinterpret_cast<const uint32_t*>(At + row1 * kTcAStride + 16 + 4 * t4);
 #pragma unroll
-      for (int nt = 0; nt < 16; ++nt) {
-        const int8_t* bcol = MT + (size_t)(c0 + nt * 8 + g) * Rp + r0 + 4 * t4;
-        const uint32_t b0 = __ldg(reinterpret_cast<const uint32_t*>(bcol));
-        const uint32_t b1 = __ldg(reinterpret_cast<const uint32_t*>(bcol + 16));
-        mma_s8(acc[nt], a0, a1, a2, a3, b0, b1);
-      }
-    }
-    // epilogue: add the parent row, store C', accumulate the linear hash
-    uint64_t h0 = 0, h1 = 0;
+      for (int j = 0; j < 8; ++j)
 #pragma unroll
-    for (int nt = 0; nt < 16; ++nt) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int col = c0 + nt * 8 + 2 * t4 + (e & 1);
-        const int i = (e < 2) ? row0 : row1;
-        if (col < m && i < nrows) {
-          const int32_t v = __ldg(parents + (size_t)prow[i] * m + col) + acc[nt][e];
-          rows[(size_t)(base + i) * m + col] = v;
-          const uint64_t hv = (uint64_t)(uint32_t)v * __ldg(s.colkey + col);
-          if (e < 2) h0 += hv; else h1 += hv;
-        }
-      }
-    }
-    h0 += __shfl_xor_sync(0xffffffffu, h0, 1);
-    h0 += __shfl_xor_sync(0xffffffffu, h0, 2);
-    h1 += __shfl_xor_sync(0xffffffffu, h1, 1);
-    h1 += __shfl_xor_sync(0xffffffffu, h1, 2);
-    if (t4 == 0) {
-      if (row0 < nrows) atomicAdd(hash + base + row0, (unsigned long long)h0);
-      if (row1 < nrows) atomicAdd(hash + base + row1, (unsigned long long)h1);
+        for (int i = 0; i < 4; ++i)
+          mma_s8(acc[i][j], a[i][0], a[i][1], a[i][2], a[i][3], ks ? b[j].z : b[j].x, ks ? b[j].w : b[j].y);
     }
   }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint32_t r = row0 + 16u * i + 8u * k + g;
+      if (r >= Q) continue;
+      const int32_t* prow = parents + (size_t)__ldg(pidx + r) * m;
+      int32_t* out = rows + (size_t)r * m;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int col = col0 + 8 * j + 2 * t4;
+        const int v0 = acc[i][j][2 * k], v1 = acc[i][j][2 * k + 1];
+        if ((m & 1) == 0 && col + 1 < m) {
+          const int2 x = __ldg(reinterpret_cast<const int2*>(prow + col));
+          __stcg(reinterpret_cast<int2*>(out + col), make_int2(x.x + v0, x.y + v1));
+        } else {
+          if (col < m) __stcg(out + col, __ldg(prow + col) + v0);
+          if (col + 1 < m) __stcg(out + col + 1, __ldg(prow + col + 1) + v1);
+        }
+      }
+    }
 }
 
 // Peak of mma.sync m16n8k32 s8 on this GPU: each warp issues `iters` rounds of
@@ -210,24 +247,43 @@ __global__ void __launch_bounds__(128) k_tc_peak(int iters, int* out) {
   out[blockIdx.x * blockDim.x + threadIdx.x] = sum;
 }
 
-void launch_tc_digits(DevSys s, const int32_t* parents, const uint32_t* perm, const uint64_t* off, int64_t P,
-                      uint64_t g0, uint32_t Q,
-                      uint8_t* loc, int mp, uint32_t* pidx, uint8_t* redundant, cudaStream_t st, int nsm) {
-  const size_t smem = (size_t)4 * 2 * s.m * sizeof(int32_t);
-  const uint64_t ntasks = ((uint64_t)Q + 31) / 32;
-  const int blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>((ntasks + 3) / 4, (uint64_t)nsm * 16));
-  k_tc_digits<<<blocks, 128, smem, st>>>(s, parents, perm, off, P, g0, Q, loc, mp, pidx, redundant);
+// M_Pi^T in the order k_tc_rows reads it: for each tile of 8 columns and each
+// pair of 32-rule blocks, 16 bytes per lane (column lane / 4; of each block the
+// rules 4 (lane % 4) .. + 3 and 16 + 4 (lane % 4) .. + 3).
+std::vector<int8_t> tc_pack(const int32_t* M, int R, int m, int nb) {
+  const int tiles = tc_col_tiles(m);
+  std::vector<int8_t> out((size_t)tiles * (nb / 2) * 32 * 16, 0);
+  for (int r = 0; r < R; ++r) {
+    const int blk = r >> 5, k = r & 31;
+    const int t4 = (k & 15) >> 2, byte = (blk & 1) * 8 + (k >> 4) * 4 + (k & 3);
+    for (int j = 0; j < m; ++j)
+      out[(((size_t)(j >> 3) * (nb / 2) + (blk >> 1)) * 32 + (j & 7) * 4 + t4) * 16 + byte] = (int8_t)M[(size_t)r * m + j];
+  }
+  return out;
 }
 
-size_t tc_rows_smem(int mp) { return (size_t)kTcBM * mp + kTcBM * kTcAStride + kTcBM * sizeof(int32_t); }
+int tc_blocks(int R) { return ((R + 63) / 64) * 2; }
 
-void launch_tc_rows(DevSys s, const int32_t* parents, const uint8_t* loc, int mp, const uint32_t* pidx, uint32_t Q,
-                    const int8_t* MT, int Rp, const int16_t* rn, const uint8_t* rk, int32_t* rows,
-                    unsigned long long* hash, cudaStream_t st) {
-  const size_t smem = tc_rows_smem(mp);
-  if (smem > (48u << 10)) cudaFuncSetAttribute(k_tc_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const unsigned blocks = (Q + kTcBM - 1) / kTcBM;
-  k_tc_rows<<<blocks, 128, smem, st>>>(s, parents, loc, mp, pidx, Q, MT, Rp, rn, rk, rows, hash);
+int tc_col_tiles(int m) { return (m + kTcN - 1) / kTcN * (kTcN / 8); }
+
+void launch_tc_masks(DevSys s, const int32_t* parents, const uint32_t* perm, const uint64_t* off, int64_t P,
+                     uint64_t g0, uint32_t Q, uint32_t* bits, int nb, uint32_t* pidx, unsigned long long* hash,
+                     uint8_t* redundant, ChunkState* st, cudaStream_t stream, int nsm) {
+  const size_t per = mask_smem_bytes(s.m, nb);
+  int warps = 8;
+  while (warps > 1 && per * warps > (200u << 10)) warps >>= 1;
+  const size_t smem = per * warps;
+  if (smem > (48u << 10)) cudaFuncSetAttribute(k_tc_masks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const uint32_t run = std::max<uint32_t>(8, (uint32_t)(((uint64_t)Q + 16ull * nsm - 1) / (16ull * nsm)));
+  const uint32_t tasks = (Q + run - 1) / run;
+  k_tc_masks<<<(tasks + warps - 1) / warps, warps * 32, smem, stream>>>(s, parents, perm, off, P, g0, Q, run, bits, nb,
+                                                                        pidx, hash, redundant, st);
+}
+
+void launch_tc_rows(DevSys s, const int32_t* parents, const uint32_t* bits, int nb, const uint32_t* pidx, uint32_t Q,
+                    const int8_t* MF, int32_t* rows, cudaStream_t st) {
+  const dim3 grid((Q + 2 * kTcM - 1) / (2 * kTcM), (s.m + 4 * kTcN - 1) / (4 * kTcN));
+  k_tc_rows<<<grid, kTcWarps * 32, 0, st>>>(s, parents, bits, nb, pidx, Q, reinterpret_cast<const uint4*>(MF), rows);
 }
 
 }  // namespace snp
