@@ -64,13 +64,14 @@ int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_
     b.fixed_q = plan.qc > 0 ? 1 : 0;
     items += many_items(b.cap, qc, run);
   }
-  TRY(arena->items.reserve(sizeof(int2) * (2 * kMqForms + 2) * items));
+  TRY(arena->items.reserve(sizeof(int2) * (2 * kMqForms + 3) * items));
   TRY(arena->queue.reserve(sizeof(uint32_t) * kMqCounters));
   ManyQueue q;
   q.expand[0] = arena->items.as<int2>();
   q.expand[1] = q.expand[0] + kMqForms * items;
   q.copy = q.expand[1] + kMqForms * items;
-  q.psi = q.copy + items;
+  q.psi[0] = q.copy + items;
+  q.psi[1] = q.psi[0] + items;
   q.ctr = arena->queue.as<uint32_t>();
   q.cap = items;
   BatchSys* dsys = arena->sys.as<BatchSys>() + lo;

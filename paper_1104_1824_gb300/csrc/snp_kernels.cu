@@ -39,7 +39,7 @@ __device__ __forceinline__ void set_error(ChunkState* st, uint32_t bits) { atomi
 // off[p] = the sum of Psi over rows before p, off[P] = the total; with REC the
 // rows' ParentRecs.  Rows not to be expanded (max_expand) get Psi = 0, rows
 // whose children could leave int32 raise kErrOverflow.  A CTA takes one run of
-// a.sub consecutive tiles; runs are handed out in order, at most one per
+// a.sub consecutive tiles, a warp an eighth of them; runs are handed out in order, at most one per
 // resident CTA, and chained by decoupled look-back at their ends (a hop per 32
 // runs; a chain over all tiles of 2^20 rows cost over 100 us).
 //   WARP = false: tiles of 256 rows, a lane per row.  A warp moves its 32 rows
@@ -82,9 +82,14 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
     if (tid == 0) s_run = a.off ? atomicAdd(a.ticket, 1u) : blockIdx.x;
     __syncthreads();
     const uint32_t run = s_run, tile0 = run * sub, tile1 = min(tile0 + sub, ntiles);
-    uint64_t through = 0, before = 0;  // sum of the run's tiles so far; this lane's exclusive sum within the run
-    for (uint32_t tile = tile0; tile < tile1; ++tile) {
-      const int64_t p0 = (int64_t)tile * R + (WARP ? warp : warp * 32);  // this warp's first row
+    uint64_t through = 0;  // sum of the warp's rows so far
+    // The run's rows: each warp takes a share of consecutive ones, so that the
+    // warps meet only at the run's end (a barrier per tile cost a quarter).
+    constexpr int W = R / 8;  // rows of a warp's step
+    const int64_t wrow0 = (int64_t)tile0 * R + (int64_t)warp * sub * W;
+    for (uint32_t j = 0; j < sub && tile0 < ntiles; ++j) {
+      const int64_t p0 = wrow0 + (int64_t)j * W;  // this step's first row
+      if (p0 >= P) break;
       PsiAcc acc;
       uint64_t v = 0;  // Psi of this lane's row (WARP: lane 0's)
       if (WARP) {
@@ -140,7 +145,6 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
             }
           }
         }
-        if (lane == 0) s_w[warp] = v;
       } else {
         int32_t(*slab)[33] = slabs[warp];
         const int nr = (int)max((int64_t)0, min((int64_t)32, P - p0));
@@ -190,14 +194,10 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
         }
       }
       if (!a.off) continue;
-      uint64_t sum = 0;
+      // sums within the warp's share: exclusive ones to off, to be raised below
       if (WARP) {
-        __syncthreads();
-        before = 0;
-        for (int w = 0; w < 8; ++w) {
-          if (w < lane) before = sat_add(before, s_w[w]);  // warp 0: lane l writes row l
-          sum = sat_add(sum, s_w[w]);
-        }
+        if (lane == 0) a.off[p0] = through;
+        through = sat_add(through, v);
       } else {
         uint64_t inc = v;
 #pragma unroll
@@ -205,25 +205,24 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
           const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
           if (lane >= o) inc = sat_add(y, inc);
         }
-        if (lane == 31) s_w[warp] = inc;
-        before = __shfl_up_sync(0xffffffffu, inc, 1);
+        uint64_t before = __shfl_up_sync(0xffffffffu, inc, 1);
         if (lane == 0) before = 0;
-        __syncthreads();
-        for (int w = 0; w < 8; ++w) {
-          if (w < warp) before = sat_add(before, s_w[w]);
-          sum = sat_add(sum, s_w[w]);
-        }
+        if (p0 + lane < P) a.off[p0 + lane] = sat_add(through, before);
+        through = sat_add(through, __shfl_sync(0xffffffffu, inc, 31));
       }
-      before = sat_add(before, through);
-      through = sat_add(through, sum);
-      __syncthreads();
-      const int64_t p = WARP ? (int64_t)tile * R + lane : p0 + lane;
-      if (sub > 1 && (!WARP || (warp == 0 && lane < 8)) && p < P) a.off[p] = before;
     }
     if (a.off && tile0 < ntiles) {
+      if (lane == 0) s_w[warp] = through;
+      __syncthreads();
+      uint64_t wbase = 0, all = 0;  // what the run's earlier warps hold; the run's sum
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        if (w < warp) wbase = sat_add(wbase, s_w[w]);
+        all = sat_add(all, s_w[w]);
+      }
       if (warp == 0) {
         uint64_t prefix = 0;
-        const bool ok = lookback_sat(a.tiles, run, a.epoch, base, through, prefix, lane);
+        const bool ok = lookback_sat(a.tiles, run, a.epoch, base, all, prefix, lane);
         if (lane == 0) {
           s_prefix = prefix;
           s_ok = ok ? 1 : 0;
@@ -232,14 +231,14 @@ __global__ void __launch_bounds__(256, REC ? 2 : 3) k_psi(PsiArgs a) {
       }
       __syncthreads();
       if (s_ok) {
-        const uint64_t prefix = s_prefix;
-        if (!WARP || (warp == 0 && lane < 8)) {
-          for (uint32_t tile = tile0; tile < tile1; ++tile) {  // each thread's own rows
-            const int64_t p = (int64_t)tile * R + (WARP ? lane : tid);
-            if (p < P) a.off[p] = sat_add(prefix, sub > 1 ? a.off[p] : before);
+        const uint64_t prefix = sat_add(s_prefix, wbase);
+        if (prefix != 0) {  // each lane raises what it wrote
+          for (uint32_t j = 0; j < sub; ++j) {
+            const int64_t p = wrow0 + (int64_t)j * W + (WARP ? 0 : lane);
+            if (p < P && (!WARP || lane == 0)) a.off[p] = sat_add(prefix, a.off[p]);
           }
         }
-        if (tile1 == ntiles && tid == 0) a.off[P] = sat_add(prefix, through);
+        if (tile1 == ntiles && tid == 0) a.off[P] = sat_add(s_prefix, all);
       }
     }
     if (__any_sync(0xffffffffu, over) && lane == 0) set_error(a.st, kErrOverflow);

@@ -154,20 +154,21 @@ struct BatchSys {
   uint64_t remaining, examined, tombs;
   int64_t nnew;
   float rate;                  // first occurrences per candidate of the last pass
+  int32_t few;                 // 1: the last depth had at most 256 candidates per parent (records pay)
 };
 
 // Work items {system, first element} of one iteration of the sparse form.
 struct ManyQueue {
   int2* expand[2];             // runs of a.run candidates: this iteration's and the next one's; kMqForms regions of `cap`
   int2* copy;                  // 32 first occurrences each
-  int2* psi;                   // 32 frontier rows each
+  int2* psi[2];                // 32 frontier rows each: without and with parent records
   uint32_t* ctr;               // counters, kMq*
   int64_t cap;                 // items of one region
 };
 // Systems by the form of the expand code they take (rows within or beyond
 // kWideM neurons, of whole 16-byte units or not): items of one form together.
 constexpr int kMqForms = 4;
-enum { kMqExpand = 0, kMqHead = 2 * kMqForms, kMqCopy = 4 * kMqForms, kMqPsi, kMqActive, kMqCounters = 20 };
+enum { kMqExpand = 0, kMqHead = 2 * kMqForms, kMqCopy = 4 * kMqForms, kMqPsi, kMqActive = kMqPsi + 2, kMqCounters = 20 };
 
 // Shape of the sparse form's expand launch.
 struct ManyPlan {

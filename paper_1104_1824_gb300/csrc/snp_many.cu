@@ -1,9 +1,9 @@
 // Sparse form of the batch engine and the serving loop: many independent
 // systems advance together through work shared by the whole grid.
 //
-// An iteration is five launches over all systems:
-//   k_many_psi      step (a) of new frontiers: Psi and the parents' records,
-//                   a warp per 32 rows;
+// An iteration is six launches over all systems:
+//   k_many_psi      step (a) of new frontiers: Psi, a warp per 32 rows (two
+//                   launches: without and with the parents' records);
 //   k_many_scan     a CTA per system with a new frontier: the saturating scan
 //                   of Psi, the depth's candidates, its first pass;
 //   k_many_expand   steps (b)-(d) of every system's pass: warps take runs of
@@ -104,6 +104,7 @@ __device__ __forceinline__ int64_t finish_depth(BatchSys& b, uint32_t* active) {
   b.phase = kPhasePsi;
   b.a.parents = b.pool + (size_t)b.level_lo * b.sys.m;
   b.a.P = b.nnew;
+  b.a.prec = b.few ? b.rec : nullptr;
   return b.nnew;
 }
 
@@ -141,7 +142,9 @@ __global__ void __launch_bounds__(kManyThreads) k_many_init(BatchSys* sys, const
         b.phase = kPhasePsi;
         b.a.parents = b.pool;
         b.a.P = 1;
-        q.psi[atomicAdd(q.ctr + kMqPsi, 1u)] = make_int2(si, 0);
+        b.few = 1;
+        b.a.prec = b.rec;
+        q.psi[1][atomicAdd(q.ctr + kMqPsi + 1, 1u)] = make_int2(si, 0);
         atomicAdd(q.ctr + kMqActive, 1u);
       } else {
         b.phase = kPhaseIdle;
@@ -154,20 +157,23 @@ __global__ void __launch_bounds__(kManyThreads) k_many_init(BatchSys* sys, const
 // memory 32 columns at a time (a row's slab is one coalesced 128-byte load,
 // the 32 rows' loads in flight together); lane r then visits row r's slab at
 // a stride of 33 words.
-__global__ void __launch_bounds__(kManyThreads) k_many_psi(BatchSys* sys, ManyQueue q) {
+// REC: the rows' parent records too (systems whose last depth had few
+// candidates per parent; the others' rows take fewer registers and lookups).
+template <bool REC>
+__global__ void __launch_bounds__(kManyThreads, REC ? 2 : 3) k_many_psi(BatchSys* sys, ManyQueue q) {
   __shared__ int32_t slabs[kManyThreads / 32][32][33];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   int32_t(*slab)[33] = slabs[wib];
-  const uint32_t count = __ldcg(q.ctr + kMqPsi);
+  const uint32_t count = __ldcg(q.ctr + kMqPsi + (REC ? 1 : 0));
   const uint32_t nw = gridDim.x * (blockDim.x >> 5);
   for (uint32_t it = blockIdx.x * (blockDim.x >> 5) + wib; it < count; it += nw) {
-    const int2 item = __ldcg(q.psi + it);
+    const int2 item = __ldcg(q.psi[REC ? 1 : 0] + it);
     BatchSys& b = sys[item.x];
     const DevSys s = b.sys;
     const int m = s.m;
     const int nr = (int)min((int64_t)32, b.a.P - item.y);
     const int32_t* rows = b.a.parents + (size_t)item.y * m;
-    ParentRec* rec = b.rec ? b.rec + item.y + lane : nullptr;
+    ParentRec* rec = REC ? b.rec + item.y + lane : nullptr;
     const int32_t max_expand = b.max_expand;
     PsiAcc acc;
     for (int n0 = 0; n0 < m; n0 += 32) {
@@ -185,17 +191,12 @@ __global__ void __launch_bounds__(kManyThreads) k_many_psi(BatchSys* sys, ManyQu
         }
       }
       __syncwarp();
-      if (lane < nr) {
-        if (rec)
-          acc.visit_run<true>(s, n0, slab[lane], w, max_expand, rec);
-        else
-          acc.visit_run<false>(s, n0, slab[lane], w, max_expand, nullptr);
-      }
+      if (lane < nr) acc.visit_run<REC>(s, n0, slab[lane], w, max_expand, rec);
     }
     bool over = false;
     if (lane < nr) {
       b.off[item.y + lane] = acc.psi();
-      if (rec) {
+      if (REC) {
         rec->hbase = acc.hb;
         rec->nnt = acc.nnt;
       }
@@ -211,6 +212,7 @@ __global__ void __launch_bounds__(kControlThreads) k_many_scan(BatchSys* sys, Ma
   __shared__ uint64_t s_q;
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // consumed: the psi items of this iteration, the copy items of the last
     q.ctr[kMqPsi] = 0;
+    q.ctr[kMqPsi + 1] = 0;
     q.ctr[kMqCopy] = 0;
   }
   BatchSys& b = sys[blockIdx.x];
@@ -223,6 +225,7 @@ __global__ void __launch_bounds__(kControlThreads) k_many_scan(BatchSys* sys, Ma
   if (threadIdx.x == 0) {
     const uint64_t total = b.off[P];
     b.total = total;
+    b.few = total <= 256ull * (uint64_t)P ? 1 : 0;
     b.T = b.budget > 0 ? min(total, (uint64_t)b.budget) : total;
     b.remaining = (uint64_t)b.cap;
     b.a.g0 = 0;
@@ -384,7 +387,7 @@ __global__ void __launch_bounds__(kControlThreads) k_many_control(BatchSys* sys,
   }
   __syncthreads();
   push_items(q.copy, q.ctr + kMqCopy, (int32_t)blockIdx.x, found, kCopyRows, &s_base);
-  push_items(q.psi, q.ctr + kMqPsi, (int32_t)blockIdx.x, (uint64_t)s_parents, 32u, &s_base);
+  push_items(q.psi[b.few], q.ctr + kMqPsi + b.few, (int32_t)blockIdx.x, (uint64_t)s_parents, 32u, &s_base);
   push_pass(q, par ^ 1, b, s_q, &s_base);
 }
 
@@ -541,7 +544,8 @@ void launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par
                            int nsm) {
   const size_t smem = (p.warp_bytes + kArgsBytes) * p.warps;
   cudaFuncSetAttribute(k_many_expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_many_psi<<<nsm * 4, kManyThreads, 0, st>>>(sys, q);
+  k_many_psi<false><<<nsm * 3, kManyThreads, 0, st>>>(sys, q);
+  k_many_psi<true><<<nsm * 2, kManyThreads, 0, st>>>(sys, q);
   k_many_scan<<<n, kControlThreads, 0, st>>>(sys, q, par);
   k_many_expand<<<nsm * p.ctas_per_sm, p.warps * 32, smem, st>>>(sys, q, par, (uint32_t)p.warp_bytes);
   k_many_control<<<n, kControlThreads, 0, st>>>(sys, q, par);

@@ -163,7 +163,8 @@ ManyQueue queue_of(const snp_server* S) {
   q.expand[0] = S->items.as<int2>();
   q.expand[1] = q.expand[0] + kMqForms * S->item_cap;
   q.copy = q.expand[1] + kMqForms * S->item_cap;
-  q.psi = q.copy + S->item_cap;
+  q.psi[0] = q.copy + S->item_cap;
+  q.psi[1] = q.psi[0] + S->item_cap;
   q.ctr = S->ctr.as<uint32_t>();
   q.cap = S->item_cap;
   return q;
@@ -178,8 +179,8 @@ int ensure_items(snp_server* S, int64_t items) {
   if (items <= S->item_cap) return SNP_OK;
   const int64_t old = S->item_cap, want = std::max<int64_t>(items, 2 * old);
   DevBuf grown;
-  TRY(grown.reserve(sizeof(int2) * (2 * kMqForms + 2) * want));
-  for (int k = 0; old > 0 && k < 2 * kMqForms + 2; ++k)
+  TRY(grown.reserve(sizeof(int2) * (2 * kMqForms + 3) * want));
+  for (int k = 0; old > 0 && k < 2 * kMqForms + 3; ++k)
     CK(cudaMemcpyAsync(grown.as<int2>() + k * want, S->items.as<int2>() + k * old, sizeof(int2) * old,
                        cudaMemcpyDeviceToDevice, S->st));
   CK(cudaStreamSynchronize(S->st));
