@@ -156,9 +156,12 @@ __global__ void __launch_bounds__(kManyThreads) k_many_init(BatchSys* sys, const
 // Step (a): a warp takes 32 frontier rows and moves them through shared
 // memory 32 columns at a time (a row's slab is one coalesced 128-byte load,
 // the 32 rows' loads in flight together); lane r then visits row r's slab at
-// a stride of 33 words.
-// REC: the rows' parent records too (systems whose last depth had few
-// candidates per parent; the others' rows take fewer registers and lookups).
+// a stride of 33 words.  With fewer items than warps, two or four warps share
+// an item's rows and two or four lanes a row's columns: a row of 512 neurons
+// is 64 batches of lookups for one lane, the length of the launch.
+// REC: the rows' parent records too, in neuron order (systems whose last depth
+// had few candidates per parent; the others' rows take fewer registers and
+// lookups).
 template <bool REC>
 __global__ void __launch_bounds__(kManyThreads, REC ? 2 : 3) k_many_psi(BatchSys* sys, ManyQueue q) {
   __shared__ int32_t slabs[kManyThreads / 32][32][33];
@@ -166,43 +169,54 @@ __global__ void __launch_bounds__(kManyThreads, REC ? 2 : 3) k_many_psi(BatchSys
   int32_t(*slab)[33] = slabs[wib];
   const uint32_t count = __ldcg(q.ctr + kMqPsi + (REC ? 1 : 0));
   const uint32_t nw = gridDim.x * (blockDim.x >> 5);
-  for (uint32_t it = blockIdx.x * (blockDim.x >> 5) + wib; it < count; it += nw) {
-    const int2 item = __ldcg(q.psi[REC ? 1 : 0] + it);
+  // log2 of the lanes per row
+  const int sl = REC || count > nw / 2 ? 0 : count > nw / 4 ? 1 : 2;
+  const int rows_per = 32 >> sl;                      // rows of a warp's share = columns of a lane's
+  const int r = lane & (rows_per - 1), part = lane >> (5 - sl);
+  for (uint32_t it = blockIdx.x * (blockDim.x >> 5) + wib; it < count << sl; it += nw) {
+    const int2 item = __ldcg(q.psi[REC ? 1 : 0] + (it >> sl));
     BatchSys& b = sys[item.x];
     const DevSys s = b.sys;
     const int m = s.m;
-    const int nr = (int)min((int64_t)32, b.a.P - item.y);
-    const int32_t* rows = b.a.parents + (size_t)item.y * m;
-    ParentRec* rec = REC ? b.rec + item.y + lane : nullptr;
+    const int64_t p0 = (int64_t)item.y + (int64_t)(it & ((1u << sl) - 1u)) * rows_per;
+    const int nr = (int)max((int64_t)0, min((int64_t)rows_per, b.a.P - p0));
+    const int32_t* rows = b.a.parents + (size_t)p0 * m;
+    ParentRec* rec = REC ? b.rec + p0 + r : nullptr;
     const int32_t max_expand = b.max_expand;
     PsiAcc acc;
-    for (int n0 = 0; n0 < m; n0 += 32) {
+    for (int n0 = 0; n0 < m && nr > 0; n0 += 32) {
       const int w = min(32, m - n0);
       __syncwarp();
       if (lane < w) {
-        for (int r0 = 0; r0 < nr; r0 += 16) {
-          int32_t v[16];
+        for (int r0 = 0; r0 < nr; r0 += 8) {
+          int32_t v[8];
 #pragma unroll
-          for (int u = 0; u < 16; ++u)
+          for (int u = 0; u < 8; ++u)
             if (r0 + u < nr) v[u] = __ldcg(rows + (size_t)(r0 + u) * m + n0 + lane);
 #pragma unroll
-          for (int u = 0; u < 16; ++u)
+          for (int u = 0; u < 8; ++u)
             if (r0 + u < nr) slab[r0 + u][lane] = v[u];
         }
       }
       __syncwarp();
-      if (lane < nr) acc.visit_run<REC>(s, n0, slab[lane], w, max_expand, rec);
+      const int c0 = part * rows_per, cw = min(rows_per, w - c0);
+      if (r < nr && cw > 0) acc.visit_run<REC>(s, n0 + c0, slab[r] + c0, cw, max_expand, rec);
     }
-    bool over = false;
-    if (lane < nr) {
-      b.off[item.y + lane] = acc.psi();
+    uint64_t prod = acc.prod;
+    bool skip = acc.skip, ov = acc.ov;
+    for (int o = rows_per; o < 32; o <<= 1) {  // a row's lanes together
+      prod = sat_mul(prod, __shfl_xor_sync(0xffffffffu, prod, o));
+      skip |= __shfl_xor_sync(0xffffffffu, skip ? 1 : 0, o) != 0;
+      ov |= __shfl_xor_sync(0xffffffffu, ov ? 1 : 0, o) != 0;
+    }
+    if (part == 0 && r < nr) {
+      b.off[p0 + r] = skip ? 0ull : prod;
       if (REC) {
         rec->hbase = acc.hb;
         rec->nnt = acc.nnt;
       }
-      over = acc.overflow();
     }
-    if (__any_sync(0xffffffffu, over) && lane == 0) atomicOr(&b.error, kErrOverflow);
+    if (__any_sync(0xffffffffu, r < nr && ov && !skip) && lane == 0) atomicOr(&b.error, kErrOverflow);
   }
 }
 
