@@ -839,7 +839,7 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     pa.level_lo = lo;
     pa.budget = (unsigned long long)budget;
     pa.pass_max = (uint32_t)Q;
-    chain_launches[x] = 2 + launch_psi(pa, W, st, nsm);
+    chain_launches[x] = launch_psi(pa, W, st, nsm);
     CK(cudaGetLastError());
     ClaimArgs a = claim_args(lo);
     a.P = P;
@@ -860,7 +860,7 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
     c.g0 = 0;
     c.dyn = dyn + x;
     c.host_depth = h->pin.depth[x];
-    launch_mark_commit(c, h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(), st, nsm);
+    chain_launches[x] += launch_mark_commit(c, h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(), st, nsm);
     CK(cudaGetLastError());
     CK(cudaEventRecord(h->ev[x][1], st));
     return SNP_OK;
@@ -1180,9 +1180,8 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
         c.P = P;
         c.g0 = g0;
         c.host = h->pin.slot[slot];
-        launch_mark_commit(c, h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(), st, nsm);
+        sd.launches += launch_mark_commit(c, h->d_own.as<uint32_t>(), h->d_gmin.as<uint32_t>(), st, nsm);
         CK(cudaGetLastError());
-        sd.launches += 2;
         CK(cudaEventRecord(h->evs[slot], st));
         fl[nfl++] = Flight{g0, Q, may_add, slot};
         pend_add += may_add;

@@ -107,8 +107,8 @@ struct CommitArgs {
 constexpr int kMarkWords = 4;     // bitmap words per warp of the mark kernel
 constexpr uint32_t kCommitTiles = 2048;  // most commit tiles of a chunk
 // First-occurrence marks of the chunk (ownbits cleared on the way), ranks and
-// commit: two launches.
-void launch_mark_commit(const CommitArgs& c, uint32_t* ownbits, const uint32_t* gmin, cudaStream_t st, int nsm);
+// commit; returns the launches made.
+int launch_mark_commit(const CommitArgs& c, uint32_t* ownbits, const uint32_t* gmin, cudaStream_t st, int nsm);
 
 // ---------------------------------------------------------------------------
 // Batch engine and serving loop: many independent systems advance together.
