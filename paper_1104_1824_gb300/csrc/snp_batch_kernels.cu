@@ -391,9 +391,9 @@ __global__ void __launch_bounds__(kTcThreads) k_batch_depth_tc(BatchArgs ba) {
         const uint64_t key = todo ? mix64(sc.hash[lid]) : 0ull;
         const int32_t* row = sc.staging + (size_t)(lid < Q ? lid : 0) * m;
         if ((m & 3) == 0)
-          resolve_warp<RowI32V, 1>(a, row, key, lid, todo);
+          resolve_warp_body<RowI32V>(a, row, key, lid, todo);
         else
-          resolve_warp<RowI32, 1>(a, row, key, lid, todo);
+          resolve_warp_body<RowI32>(a, row, key, lid, todo);
       }
       __threadfence();
       __syncthreads();

@@ -368,45 +368,6 @@ __device__ __forceinline__ int64_t warp_find_parent(const uint64_t* off, int64_t
   return lo;
 }
 
-// Per-warp view of one parent configuration: its row in shared memory, the
-// applicable-rule mask of every neuron and, per lane, the product of the
-// choice counts of all neurons after the lane's own (mixed-radix place value).
-struct WarpParent {
-  int32_t* par;    // [m] spikes
-  uint32_t* msk;   // [m] applicable rules of neuron n, bit k = rule first_rule[n] + k
-  int32_t* buf;    // [m] child under construction
-  uint64_t after;  // product of choice counts of neurons owned by later lanes (saturating)
-  uint64_t psi;    // Psi of the parent (saturating)
-};
-
-// Step (a) for one parent: load the row, mark applicable rules, form the
-// per-lane place values (neuron 0 most significant).
-__device__ __forceinline__ void load_parent(const DevSys& s, const int32_t* __restrict__ row, WarpParent& w,
-                                            int lane) {
-  __syncwarp();
-  for (int n = lane; n < s.m; n += 32) w.par[n] = row[n];
-  __syncwarp();
-  uint64_t prod = 1;
-  const int n0 = lane * s.K;
-  const int n1 = min(n0 + s.K, s.m);
-  for (int n = n0; n < n1; ++n) {
-    const uint32_t mask = (uint32_t)appl(s, n, w.par[n]);
-    w.msk[n] = mask;
-    prod = sat_mul(prod, mask ? (uint64_t)__popc(mask) : 1ull);
-  }
-  // inclusive suffix product over lanes
-  uint64_t v = prod;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint64_t u = __shfl_down_sync(0xffffffffu, v, o);
-    if (lane + o < 32) v = sat_mul(v, u);
-  }
-  w.psi = __shfl_sync(0xffffffffu, v, 0);
-  uint64_t a = __shfl_down_sync(0xffffffffu, v, 1);
-  w.after = (lane == 31) ? 1ull : a;
-  __syncwarp();
-}
-
 // q / radix; the remainder is the digit (out of line: indices beyond 32 bits
 // are rare, and the 64-bit division is long).
 static __device__ __noinline__ uint64_t next_digit_wide(uint64_t q, uint32_t radix) { return q / radix; }
@@ -488,12 +449,6 @@ __device__ __forceinline__ void copy_row_cg(const int32_t* src, int32_t* dst, in
 __device__ __forceinline__ uint32_t fp32_of(uint64_t h) {
   uint32_t f = (uint32_t)(h >> 32);
   return f == 0xFFFFFFFFu ? 0xFFFFFFFEu : f;  // keeps (fp, reserved) distinct from an empty slot
-}
-
-__device__ __forceinline__ bool rows_equal(const int32_t* buf, const int32_t* other, int m, int lane) {
-  bool ok = true;
-  for (int n = lane; n < m; n += 32) ok &= (__ldcg(other + n) == buf[n]);
-  return __all_sync(0xffffffffu, ok);
 }
 
 // One neuron's lookup out of line: {applicable mask, a child could leave

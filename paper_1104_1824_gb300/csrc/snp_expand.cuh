@@ -1,6 +1,6 @@
 // Device code of the expand kernels: steps (b), (c) and (d) for one chunk of
 // candidates, by warps.  Shared by the single-system kernels (snp_expand.cu)
-// and the batch engine (snp_batch_kernels.cu).
+// and the batch engine (snp_many.cu, snp_batch_kernels.cu).
 //
 // Candidates are spiking-vector indices in the mixed radix of the per-neuron
 // choice counts (Eq. psi; last neuron least significant).  A warp walks a run
@@ -97,18 +97,9 @@ __device__ __forceinline__ int rule_of(const DevSys& s, const ExpandSmem& w, int
   return __ldg(s.first_rule + n) + nth_set_bit(w.msk[n], d);
 }
 
-// row += sign * (row r of M_Pi); the row is private to the calling lane
-__device__ __forceinline__ void add_row_private(const DevSys& s, int32_t* row, int r, int sign) {
-  const int e0 = __ldg(&s.rule[r].w), e1 = __ldg(&s.rule[r + 1].w);
-  for (int e = e0; e < e1; ++e) {
-    const int2 cv = __ldg(s.csr + e);
-    row[cv.x] += sign * cv.y;
-  }
-}
-
 // row += M[rn] - M[ro] for two rules of one neuron (the row is private to
 // the calling lane): one pass over the neuron's support.
-__device__ __forceinline__ void swap_rule_private(const DevSys& s, int32_t* row, int ro, int rn) {
+__device__ __forceinline__ void swap_rule(const DevSys& s, int32_t* row, int ro, int rn) {
   const int4 dn = __ldg(s.rdesc + rn);
   const int32_t* vn = s.rval + dn.z;
   const int32_t* vo = s.rval + __ldg(&s.rdesc[ro].z);
@@ -117,31 +108,11 @@ __device__ __forceinline__ void swap_rule_private(const DevSys& s, int32_t* row,
 }
 
 // row += M[r] (the row is private to the calling lane).
-__device__ __forceinline__ void add_rule_private(const DevSys& s, int32_t* row, int r) {
+__device__ __forceinline__ void add_rule(const DevSys& s, int32_t* row, int r) {
   const int4 dr = __ldg(s.rdesc + r);
   const int32_t* v = s.rval + dr.z;
   const int32_t* col = s.scol + dr.x;
   for (int i = 0; i < dr.y; ++i) row[__ldg(col + i)] += __ldg(v + i);
-}
-
-// The batch kernel runs at its register limit: it keeps the CSR walk, which
-// needs fewer live values.
-template <int KIND>
-__device__ __forceinline__ void swap_rule(const DevSys& s, int32_t* row, int ro, int rn) {
-  if constexpr (KIND == 0) {
-    swap_rule_private(s, row, ro, rn);
-  } else {
-    add_row_private(s, row, ro, -1);
-    add_row_private(s, row, rn, 1);
-  }
-}
-
-template <int KIND>
-__device__ __forceinline__ void add_rule(const DevSys& s, int32_t* row, int r) {
-  if constexpr (KIND == 0)
-    add_rule_private(s, row, r);
-  else
-    add_row_private(s, row, r, 1);
 }
 
 __device__ __forceinline__ void add_row_shared(const DevSys& s, int32_t* row, int r, int sign) {
@@ -446,9 +417,8 @@ __device__ __forceinline__ void finish_owner_inplace(const ClaimArgs& a, uint64_
 
 // Step (d) for one row per lane (lanes with todo set): passes until every
 // row is resolved; a lane never waits inside a pass, so owners in this warp
-// publish before anyone looks again.  KIND separates the out-of-line copies
-// of the single-system kernel (0) and the batch kernel (1), whose register
-// budgets differ.
+// publish before anyone looks again.  Out of line for the expand kernels, in
+// line for the fp8 batch kernel, whose register budget differs.
 template <class RF>
 __device__ __forceinline__ void resolve_warp_body(const ClaimArgs& a, const int32_t* row, uint64_t key, uint32_t lid,
                                                   bool todo) {
@@ -483,15 +453,6 @@ template <class RF>
 __device__ __noinline__ void resolve_warp_call(const ClaimArgs& a, const int32_t* row, uint64_t key, uint32_t lid,
                                                bool todo) {
   resolve_warp_body<RF>(a, row, key, lid, todo);
-}
-
-template <class RF, int KIND>
-__device__ __forceinline__ void resolve_warp(const ClaimArgs& a, const int32_t* row, uint64_t key, uint32_t lid,
-                                             bool todo) {
-  if constexpr (KIND == 0)
-    resolve_warp_call<RF>(a, row, key, lid, todo);
-  else
-    resolve_warp_body<RF>(a, row, key, lid, todo);
 }
 
 // Four counts of a row in global memory, from count 4 * j on (VEC rows).
@@ -613,7 +574,7 @@ __device__ __forceinline__ int flat_decode(const ClaimArgs& a, int64_t P, uint64
 
 // Step (c) for a candidate of a crossing batch: C' = C + the chosen rules'
 // rows, built in a tile row (one lane).
-template <class RF, int KIND>
+template <class RF>
 __device__ __forceinline__ void flat_build(const ClaimArgs& a, int64_t pc, uint64_t t, int32_t* trow) {
   const DevSys& s = a.sys;
   const typename RF::T* prow = parent_row<RF>(a, pc);
@@ -623,7 +584,7 @@ __device__ __forceinline__ void flat_build(const ClaimArgs& a, int64_t pc, uint6
     const uint32_t mask = appl_mask(s, n, x);
     if (!mask) return;
     const int kb = nth_set_bit(mask, (int)next_digit(q, __popc(mask)));
-    add_rule<KIND>(s, trow, __ldg(s.first_rule + n) + kb);
+    add_rule(s, trow, __ldg(s.first_rule + n) + kb);
   });
 }
 
@@ -1204,20 +1165,20 @@ __device__ __forceinline__ uint64_t block_run_wide(const ClaimArgs& a, ExpandSme
 // line, as flush_queue_wide: the expand loop has two places that flush, and
 // a copy of the row builder in each made the kernel outgrow the instruction
 // cache.
-template <class RF, int KIND>
+template <class RF>
 __device__ __noinline__ void flush_queue(const ClaimArgs& a, int32_t* tile, const unsigned long long* keys,
                                          const long long* dpc, const unsigned long long* dt, const uint32_t* lids,
                                          int ts, int fill) {
   const int lane = threadIdx.x & 31;
   const bool mine = lane < fill;
-  if (mine && dpc[lane] >= 0) flat_build<RF, KIND>(a, dpc[lane], dt[lane], tile + lane * ts);
+  if (mine && dpc[lane] >= 0) flat_build<RF>(a, dpc[lane], dt[lane], tile + lane * ts);
   __syncwarp();
-  resolve_warp<RF, KIND>(a, tile + lane * ts, mine ? keys[lane] : 0ull, mine ? lids[lane] : 0u, mine);
+  resolve_warp_call<RF>(a, tile + lane * ts, mine ? keys[lane] : 0ull, mine ? lids[lane] : 0u, mine);
 }
 
 // Block mode for parent p from candidate a.g0 + l to the end of the parent or
 // of the task; returns the new l.
-template <class RF, int KIND>
+template <class RF>
 __device__ __forceinline__ uint64_t block_run(const ClaimArgs& a, ExpandSmem& w, int B, int ts, int64_t p,
                                               uint64_t p_lo, uint64_t p_hi, uint64_t l, uint64_t lb,
                                               int64_t& cached_p, uint64_t& after, int lane) {
@@ -1249,7 +1210,7 @@ __device__ __forceinline__ uint64_t block_run(const ClaimArgs& a, ExpandSmem& w,
       q /= radix;
       if (d == 0) continue;
       const int r0 = rule_of(s, w, n, 0), rd = rule_of(s, w, n, (int)d);
-      swap_rule<KIND>(s, row, r0, rd);
+      swap_rule(s, row, r0, rd);
       hk += __ldg(s.rowkey + rd) - __ldg(s.rowkey + r0);
       redk |= redundant_choice(s, mask, rd);
     }
@@ -1258,7 +1219,7 @@ __device__ __forceinline__ uint64_t block_run(const ClaimArgs& a, ExpandSmem& w,
   for (;;) {
     const uint64_t c = gb + lane;
     const bool todo = lane < RL && c >= g && c < gend && !redk && w.hdr[kNred] == 0;
-    resolve_warp<RF, KIND>(a, row, mix64(hbase_of(w) + hk), (uint32_t)(c - a.g0), todo);
+    resolve_warp_call<RF>(a, row, mix64(hbase_of(w) + hk), (uint32_t)(c - a.g0), todo);
     gb += (uint64_t)RL;
     if (gb >= gend) break;
     // next block: the high digits move on by one (odometer, least significant first)
@@ -1287,7 +1248,7 @@ __device__ __forceinline__ uint64_t block_run(const ClaimArgs& a, ExpandSmem& w,
       const int nc = w.hdr[kNchg];
       for (int j = 0; j < nc; ++j) {
         const int2 rr = w.chg[j];
-        swap_rule<KIND>(s, row, rr.x, rr.y);
+        swap_rule(s, row, rr.x, rr.y);
       }
     }
   }
@@ -1299,7 +1260,7 @@ __device__ __forceinline__ void flush_any(const ClaimArgs& a, ExpandSmem& w, int
   if constexpr (KIND == kWide)
     flush_queue_wide<RF>(a, w.tile, w.keys, w.dpc, w.dt, w.lids, fill);
   else
-    flush_queue<RF, KIND>(a, w.tile, w.keys, w.dpc, w.dt, w.lids, ts, fill);
+    flush_queue<RF>(a, w.tile, w.keys, w.dpc, w.dt, w.lids, ts, fill);
 }
 
 // What a warp keeps from one task of a chunk to the next.
@@ -1343,7 +1304,7 @@ __device__ __forceinline__ void expand_task(const ClaimArgs& a, int64_t P, uint3
       if constexpr (KIND == kWide)
         l = block_run_wide<RF>(a, w, p, p_lo, p_hi, l, lb, k.cached_p, k.after, lane);
       else
-        l = block_run<RF, KIND>(a, w, B, ts, p, p_lo, p_hi, l, lb, k.cached_p, k.after, lane);
+        l = block_run<RF>(a, w, B, ts, p, p_lo, p_hi, l, lb, k.cached_p, k.after, lane);
       const uint64_t gn = a.g0 + l;
       if (l < lb) {
         do {

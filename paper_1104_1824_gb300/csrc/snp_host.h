@@ -117,7 +117,6 @@ inline uint64_t pow2_at_least(uint64_t x) {
 }
 
 constexpr int kWarpsPerBlock = 4;
-constexpr int kThreads = kWarpsPerBlock * 32;
 
 inline int grid_for(int64_t work_items, int per_block, int max_blocks) {
   int64_t b = (work_items + per_block - 1) / per_block;

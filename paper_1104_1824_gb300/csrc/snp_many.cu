@@ -13,15 +13,15 @@
 //   k_many_control  a CTA per system with a pass: first-occurrence marks,
 //                   ranks, what the cap accepts, the next pass or frontier;
 //   k_many_copy     accepted rows to their pool rows, table slots pointed at
-//                   them, a warp per 32 first occurrences.
+//                   them, a warp per 8 first occurrences.
 // Systems do not wait for one another: each is in its own depth and pass.
 //
 // Why a shared queue: with a CTA per system and depth, a depth lasted as long
 // as its slowest system on one SM (a burst of 48 systems of up to 512 neurons
 // left 104 SMs idle), and the tile of every system was as small as the widest
 // one's.  48 requests of 8 to 512 neurons (depths 4 to 32, cap 2^12, budget
-// 2^16): 625 ms -> 84 ms; 512 systems of 16 to 256 neurons to depth 6: 101 ms
-// -> 58 ms.
+// 2^16): 618 ms -> 67 ms; 512 systems of 16 to 256 neurons to depth 6: 101 ms
+// -> 49 ms.
 #include <algorithm>
 
 #include "snp_expand.cuh"
