@@ -589,7 +589,8 @@ def bench_batch(args, w, systems, snp, torch, dist, dev, rank, world, local):
                          "unit": "GB/s", "frac": round(achieved / peak, 4),
                          "algorithmic_bytes_per_launch": int(bytes_step / w["depth"]),
                          "avg_launch_ms": round(ms / args.steps / w["depth"], 3), "traffic": None},
-            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": (w["depth"] + 2) * args.steps, "clocks": clk,
+            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": (w["depth"] + 2) * args.steps,  # at least: the sparse form launches more per depth
+            "clocks": clk,
         }
         if compare:
             line["compare"] = compare

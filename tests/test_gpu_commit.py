@@ -1,5 +1,5 @@
 """Marks, ranks and commit of a pass around the edges of its tiles (2048
-candidates; more than 32 tiles look back across a window) against the oracle:
+candidates and more; up to and beyond 32 of them) against the oracle:
 rows of any length, with and without a map to discovery order, parent records."""
 import numpy as np
 import pytest
