@@ -1251,17 +1251,19 @@ int snp_reachable(snp_handle h, int32_t* out, int64_t capacity, int64_t* n, int6
     CK(cudaMemcpy(out, h->result_pool, bytes, cudaMemcpyDefault));
     return SNP_OK;
   }
-  // rows in discovery order: gather from the store (into `out` when it is
-  // device memory, else through a device buffer)
+  // rows in discovery order: gather from the store, into `out` when it is
+  // device memory, else through a device buffer (packed rows too where `out`
+  // is off a 16-byte boundary: they are widened to 16-byte pieces only)
   int32_t* dst = out;
-  if (!is_device_ptr(out)) {
+  const bool on_device = is_device_ptr(out);
+  if (!on_device || (h->result_w < 4 && !aligned16(out))) {
     TRY(h->d_tmp.reserve(bytes));
     dst = h->d_tmp.as<int32_t>();
   }
   launch_gather_rows(h->result_pool, h->result_w, h->result_perm, h->n_rows, h->m, dst, nullptr);
   CK(cudaGetLastError());
-  if (dst != out) CK(cudaMemcpy(out, dst, bytes, cudaMemcpyDeviceToHost));
-  else CK(cudaDeviceSynchronize());
+  if (dst != out) CK(cudaMemcpy(out, dst, bytes, cudaMemcpyDefault));
+  if (on_device) CK(cudaDeviceSynchronize());
   return SNP_OK;
 }
 

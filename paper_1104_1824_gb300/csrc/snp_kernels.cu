@@ -755,14 +755,16 @@ __global__ void __launch_bounds__(256) k_gather_rows(const int32_t* pool, const 
 
 void launch_gather_rows(const int32_t* pool, int w, const uint32_t* perm, int64_t n, int m, int32_t* out,
                         cudaStream_t st) {
-  const uint32_t pieces = (m & 3) == 0 ? (uint32_t)m / 4 : (uint32_t)m;
+  // whole 16-byte pieces where the rows are that and the caller's buffer starts on such a boundary
+  const bool vec = (m & 3) == 0 && aligned16(out);
+  const uint32_t pieces = vec ? (uint32_t)m / 4 : (uint32_t)m;
   const int64_t per = pieces <= kGatherPieces ? 64 : 8;  // rows per CTA
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 152 * 64));
   auto fn = pieces <= kGatherPieces
                 ? (w == 1 ? k_gather_short<RowU8> : w == 2 ? k_gather_short<RowU16>
-                   : (m & 3) == 0 ? k_gather_short<RowI32V> : k_gather_short<RowI32>)
+                   : vec ? k_gather_short<RowI32V> : k_gather_short<RowI32>)
                 : (w == 1 ? k_gather_rows<RowU8> : w == 2 ? k_gather_rows<RowU16>
-                   : (m & 3) == 0 ? k_gather_rows<RowI32V> : k_gather_rows<RowI32>);
+                   : vec ? k_gather_rows<RowI32V> : k_gather_rows<RowI32>);
   fn<<<blocks, 256, 0, st>>>(pool, perm, n, m, out);
 }
 

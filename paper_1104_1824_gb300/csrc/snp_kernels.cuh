@@ -10,6 +10,10 @@
 
 namespace snp {
 
+// True for a 16-byte boundary: device buffers of the caller may start off one,
+// and the kernels' vector forms must not be given such rows.
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // A depth that runs without the host: what its kernels need to know of the
 // depth before it and of one another (device memory).
 struct DepthDyn {
@@ -310,7 +314,8 @@ int tc5_slots(int m, int nblocks);
 bool tc5_store_map(CUtensorMap* map, int32_t* pool, int m, uint64_t rows);
 void launch_tc5(const Tc5Args& a, const CUtensorMap& map, cudaStream_t st, int nsm);
 void launch_iota_u32(uint32_t* out, int64_t n, cudaStream_t st);
-// out[k] = row perm[k] (row k without perm) of a pool of w bytes per count, as int32.
+// out[k] = row perm[k] (row k without perm) of a pool of w bytes per count, as
+// int32.  w < 4: out on a 16-byte boundary.
 void launch_gather_rows(const int32_t* pool, int w, const uint32_t* perm, int64_t n, int m, int32_t* out,
                         cudaStream_t st);
 // Testing hook: marks the slot holding store row `row` as being claimed.

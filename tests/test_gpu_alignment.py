@@ -1,0 +1,46 @@
+"""Device buffers of the caller that start off a 16-byte boundary, with rows
+that are whole 16-byte units (so that the vector forms would be chosen by the
+row length alone).  Results are whole numbers and compared exactly."""
+import numpy as np
+import pytest
+
+import oracle
+import snp_synth
+
+pytestmark = pytest.mark.gpu
+
+MARK = -7
+
+
+def shifted(rows: int, m: int, shift: int):
+    """A marked buffer and its part of rows x m counts that starts `shift` counts in."""
+    import torch
+    buf = torch.full((rows * m + 8,), MARK, dtype=torch.int32, device="cuda")
+    assert buf.data_ptr() % 16 == 0
+    return buf, buf[shift:shift + rows * m].view(rows, m)
+
+
+def check(buf, shift: int, want):
+    got = buf.cpu().numpy()
+    n = want.size
+    assert (got[shift:shift + n] == want.reshape(-1)).all()
+    assert (got[:shift] == MARK).all() and (got[shift + n:] == MARK).all()
+
+
+def system_of(m: int, top: int = 6):
+    return snp_synth.random_system(330 + m, m, (1, 3), (min(4, m - 1), min(4, m - 1)), (0, top), "sparse")
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("m,top,packed,width", [(4, 6, False, 4), (64, 6, False, 4), (61, 6, False, 4),
+                                                (388, 6, False, 4), (64, 6, True, 1), (24, 6, True, 2),
+                                                (400, 6, True, 1), (392, 300, True, 2)])
+def test_reachable_into_a_shifted_buffer(gpu, m, top, packed, width, shift):
+    system = system_of(m, top)
+    s = gpu.System(system)
+    s.explore(3, cap=300, budget=3000, packed=packed)
+    assert s.row_width() == width
+    want = oracle.Oracle(system).explore(3, cap=300, budget=3000).configs
+    buf, out = shifted(len(want), m, shift)
+    assert gpu.snp_reachable(s.h, out, len(want)) == len(want)
+    check(buf, shift, want)
