@@ -380,7 +380,8 @@ int snp_server_destroy(void* srv);
  *  opts           as for snp_explore; transition must be SNP_T_SPARSE_I32
  *                 and record_parents 0.  Uses opts->stream.
  *  out            device memory on the handle's device, capacity rows of m
- *                 int32.
+ *                 int32, on any 4-byte boundary (with m a multiple of 4, a
+ *                 16-byte one is faster).
  *  capacity       1 <= capacity <= 2^20 configurations (the array's limit);
  *                 larger values are refused with SNP_E_INVALID.
  *  *n             configurations written (C0 first, discovery order).

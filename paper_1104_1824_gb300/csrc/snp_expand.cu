@@ -162,6 +162,9 @@ size_t wide_base_bytes(int m) { return base_rows_offset() + (size_t)kBaseSlots *
 
 int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
   const int m = a.sys.m;
+  // rows of whole 16-byte pieces on 16-byte boundaries (snp_explore_static's
+  // rows lie in the caller's buffer, which may start off one)
+  const bool vec = m % 4 == 0 && aligned16(a.parents) && aligned16(a.pool) && aligned16(a.staging);
   if (m > kWideM) {
     const size_t per_warp = expand_wide_bytes(m);
     const bool many = per_warp * kWideWarpsMany <= (226u << 10);
@@ -178,7 +181,7 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
     if (a.bcache) {  // base children of the pass's largest parents
       const size_t bs = (size_t)round4(m) * 4;
       auto fb = a.w == 2 ? k_wide_base<RowU16> : a.w == 1 ? k_wide_base<RowU8>
-                : (m % 4) == 0 ? k_wide_base<RowI32V> : k_wide_base<RowI32>;
+                : vec ? k_wide_base<RowI32V> : k_wide_base<RowI32>;
       fb<<<kBaseSlots, std::min(1024, (m + 31) / 32 * 32), bs, st>>>(a);
     }
     constexpr int kM = kWideWarpsMany, kF = kWideWarps;
@@ -187,7 +190,7 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
       if (a.dyn) return many ? k_expand_wide<RF, kM, true> : k_expand_wide<RF, kF, true>;
       return many ? k_expand_wide<RF, kM, false> : k_expand_wide<RF, kF, false>;
     };
-    auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : (m % 4) == 0 ? pick(RowI32V()) : pick(RowI32());
+    auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : vec ? pick(RowI32V()) : pick(RowI32());
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     fn<<<blocks > 0 ? blocks : 1, wpb * 32, smem, st>>>(a);
     return a.bcache ? 2 : 1;
@@ -213,7 +216,7 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
     using RF = decltype(rf);
     return a.dyn ? k_expand<RF, true> : k_expand<RF, false>;
   };
-  auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : (m % 4) == 0 ? pick(RowI32V()) : pick(RowI32());
+  auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : vec ? pick(RowI32V()) : pick(RowI32());
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   fn<<<blocks > 0 ? blocks : 1, wpb * 32, smem, st>>>(a, B, ts);
   return 1;

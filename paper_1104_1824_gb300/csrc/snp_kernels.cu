@@ -304,7 +304,7 @@ int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm) {
     a.rec ? psi_launch<RowU8, true>(a, warp, st, nsm) : psi_launch<RowU8, false>(a, warp, st, nsm);
   else if (w == 2)
     a.rec ? psi_launch<RowU16, true>(a, warp, st, nsm) : psi_launch<RowU16, false>(a, warp, st, nsm);
-  else if (a.s.m % 4 == 0)
+  else if (a.s.m % 4 == 0 && aligned16(a.rows))
     a.rec ? psi_launch<RowI32V, true>(a, warp, st, nsm) : psi_launch<RowI32V, false>(a, warp, st, nsm);
   else
     a.rec ? psi_launch<RowI32, true>(a, warp, st, nsm) : psi_launch<RowI32, false>(a, warp, st, nsm);
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(256) k_commit(CommitArgs a, uint32_t tile_word
       if (!a.perm && rank0 < remaining) {  // staged rows to consecutive pool rows, by the whole warp
         const uint32_t rows = (uint32_t)min((uint64_t)min(cnt - r0, 32u), remaining - rank0);
         int32_t* dst = a.pool + (size_t)(row_base + (int64_t)rank0) * m;
-        if ((m & 3) == 0)
+        if ((m & 3) == 0 && (reinterpret_cast<uintptr_t>(a.pool) & 15) == 0)
           copy_staged(reinterpret_cast<const int4*>(a.staging), reinterpret_cast<int4*>(dst), s, rows, (uint32_t)m >> 2,
                       lane);
         else

@@ -44,3 +44,18 @@ def test_reachable_into_a_shifted_buffer(gpu, m, top, packed, width, shift):
     buf, out = shifted(len(want), m, shift)
     assert gpu.snp_reachable(s.h, out, len(want)) == len(want)
     check(buf, shift, want)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("m,depth,cap,budget", [(4, 4, 60, 0), (64, 3, 300, 3000), (61, 3, 300, 3000),
+                                                (128, 3, 2000, 40000), (132, 3, 500, 9000), (1024, 2, 200, 3000)])
+def test_static_into_a_shifted_buffer(gpu, m, depth, cap, budget, shift):
+    system = system_of(m)
+    e = oracle.Oracle(system).explore(depth, cap=cap, budget=budget)
+    s = gpu.System(system)
+    o = gpu.snp_explore_opts_init()
+    o.depth, o.frontier_cap, o.candidate_budget = depth, cap, budget
+    buf, out = shifted(1 + depth * cap, m, shift)
+    n, reached = gpu.snp_explore_static(s.h, o, out, out.shape[0])
+    assert n == len(e.configs) and reached == e.depth_reached
+    check(buf, shift, e.configs)
