@@ -15,7 +15,8 @@
  *  - Every function returns an int status (SNP_OK = 0 or an SNP_E_* code) and
  *    never throws.  snp_last_error() gives a message for the calling thread.
  *  - Arrays described as "host or device" may be either; the library infers
- *    the direction of each copy from the pointer.  Arrays described as
+ *    the direction of each copy from the pointer.  Device arrays of int32
+ *    may start on any 4-byte boundary.  Arrays described as
  *    "host" must be host memory.  The caller keeps ownership of every array
  *    it passes; the library copies what it needs before returning.
  *  - A handle owns all device memory it allocates and is bound to the CUDA
@@ -261,8 +262,7 @@ int snp_explore_resume(snp_handle h, const int32_t* rows, int64_t n, const snp_d
  * order (depth by depth, each depth in canonical candidate order), into
  * out[capacity * m] (host or device): the set the paper's simulator collects
  * as allGenCk (Section 5; Algorithm 2 adds every new C_k to it), here as
- * int32 rows whatever the store's width; device memory may start on any
- * 4-byte boundary.  *n receives the count.  With
+ * int32 rows whatever the store's width.  *n receives the count.  With
  * capacity < *n nothing is written and SNP_E_BUFFER is returned (out may then
  * be NULL).  per_depth_new (host, may be NULL) receives depth_reached + 1
  * counts, index 0 being C0's level.  Errors: SNP_E_STATE, SNP_E_BUFFER, SNP_E_CUDA. */

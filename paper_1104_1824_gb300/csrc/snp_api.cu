@@ -568,14 +568,14 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
   // for rows of whole 16-byte pieces, and where the bound on every count the
   // exploration can reach allows it (packed_width); int32 otherwise.
   int W = 4;
-  const int32_t* rs_rows = rs ? rs->rows : nullptr;  // a resumed exploration's rows (device copy when packed)
+  const int32_t* rs_rows = rs ? rs->rows : nullptr;  // a resumed exploration's rows (when packed: device, 16-byte boundary)
   if (o->packed && !tc && !tc5 && m % 8 == 0) {
     std::vector<int64_t> cmax(h->c0.begin(), h->c0.end());
     int64_t depths = o->depth;
     if (rs) {  // the checkpoint's largest count, for every column
-      if (!is_device_ptr(rs->rows)) {
+      if (!is_device_ptr(rs->rows) || !aligned16(rs->rows)) {
         TRY(h->d_tmp.reserve(sizeof(int32_t) * (size_t)m * rs->n));
-        CK(cudaMemcpyAsync(h->d_tmp.p, rs->rows, sizeof(int32_t) * (size_t)m * rs->n, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(h->d_tmp.p, rs->rows, sizeof(int32_t) * (size_t)m * rs->n, cudaMemcpyDefault, st));
         rs_rows = h->d_tmp.as<int32_t>();
       }
       TRY(h->d_ctr.reserve(3 * sizeof(unsigned long long)));

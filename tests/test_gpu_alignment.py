@@ -1,6 +1,8 @@
 """Device buffers of the caller that start off a 16-byte boundary, with rows
 that are whole 16-byte units (so that the vector forms would be chosen by the
 row length alone).  Results are whole numbers and compared exactly."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -59,3 +61,27 @@ def test_static_into_a_shifted_buffer(gpu, m, depth, cap, budget, shift):
     n, reached = gpu.snp_explore_static(s.h, o, out, out.shape[0])
     assert n == len(e.configs) and reached == e.depth_reached
     check(buf, shift, e.configs)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("m,top,packed,width", [(64, 6, True, 1), (24, 6, True, 2), (392, 300, True, 2),
+                                                (64, 6, False, 4)])
+def test_resume_from_a_shifted_buffer(gpu, m, top, packed, width, shift):
+    import torch
+    system = system_of(m, top)
+    s = gpu.System(system)
+    s.explore(2, cap=300, budget=3000)
+    rows, raw = s.checkpoint()
+    buf, dev = shifted(len(rows), m, shift)
+    dev.copy_(torch.from_numpy(rows))
+    k = raw.nbytes // ctypes.sizeof(gpu.snp_depth_info)
+    stats = (gpu.snp_depth_info * k).from_buffer_copy(raw.tobytes())
+    o = gpu.snp_explore_opts_init()
+    o.depth, o.frontier_cap, o.candidate_budget, o.packed = 4, 300, 3000, 1 if packed else 0
+    later = gpu.System(system)
+    later.depth_reached = gpu.snp_explore_resume(later.h, dev, stats, o)
+    assert later.row_width() == width
+    e = oracle.Oracle(system).explore(4, cap=300, budget=3000)
+    got = later.reachable()
+    assert got.shape == e.configs.shape and (got == e.configs).all()
+    check(buf, shift, rows)
