@@ -191,7 +191,7 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
       return many ? k_expand_wide<RF, kM, false> : k_expand_wide<RF, kF, false>;
     };
     auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : vec ? pick(RowI32V()) : pick(RowI32());
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(fn);
     fn<<<blocks > 0 ? blocks : 1, wpb * 32, smem, st>>>(a);
     return a.bcache ? 2 : 1;
   }
@@ -217,7 +217,7 @@ int launch_expand(ClaimArgs a, cudaStream_t st, int nsm) {
     return a.dyn ? k_expand<RF, true> : k_expand<RF, false>;
   };
   auto fn = a.w == 2 ? pick(RowU16()) : a.w == 1 ? pick(RowU8()) : vec ? pick(RowI32V()) : pick(RowI32());
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(fn);
   fn<<<blocks > 0 ? blocks : 1, wpb * 32, smem, st>>>(a, B, ts);
   return 1;
 }

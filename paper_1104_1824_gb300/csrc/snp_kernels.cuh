@@ -14,6 +14,16 @@ namespace snp {
 // and the kernels' vector forms must not be given such rows.
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+// Lets a kernel (without static shared memory) launch with as much dynamic
+// shared memory as a block can have.  Always this much, whatever the launch at
+// hand needs: the limit belongs to the function, handles are used from several
+// threads, and one that a thread lowered to its own launch would refuse a
+// larger launch of another.
+template <class F>
+inline void allow_smem(F fn) {
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 << 10);
+}
+
 // A depth that runs without the host: what its kernels need to know of the
 // depth before it and of one another (device memory).
 struct DepthDyn {

@@ -557,7 +557,7 @@ void launch_many_init(BatchSys* sys, const int32_t* idx, const int32_t* c0, cons
 void launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par, const ManyPlan& p, cudaStream_t st,
                            int nsm) {
   const size_t smem = (p.warp_bytes + kArgsBytes) * p.warps;
-  cudaFuncSetAttribute(k_many_expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_many_expand);
   k_many_psi<false><<<nsm * 3, kManyThreads, 0, st>>>(sys, q);
   k_many_psi<true><<<nsm * 2, kManyThreads, 0, st>>>(sys, q);
   k_many_scan<<<n, kControlThreads, 0, st>>>(sys, q, par);

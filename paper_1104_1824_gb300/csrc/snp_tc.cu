@@ -273,7 +273,7 @@ void launch_tc_masks(DevSys s, const int32_t* parents, const uint32_t* perm, con
   int warps = 8;
   while (warps > 1 && per * warps > (200u << 10)) warps >>= 1;
   const size_t smem = per * warps;
-  if (smem > (48u << 10)) cudaFuncSetAttribute(k_tc_masks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > (48u << 10)) allow_smem(k_tc_masks);
   const uint32_t run = std::max<uint32_t>(8, (uint32_t)(((uint64_t)Q + 16ull * nsm - 1) / (16ull * nsm)));
   const uint32_t tasks = (Q + run - 1) / run;
   k_tc_masks<<<(tasks + warps - 1) / warps, warps * 32, smem, stream>>>(s, parents, perm, off, P, g0, Q, run, bits, nb,

@@ -802,7 +802,7 @@ bool tc5_store_map(CUtensorMap* map, int32_t* pool, int m, uint64_t rows) {
 void launch_tc5(const Tc5Args& a, const CUtensorMap& map, cudaStream_t st, int nsm) {
   // more than a third of an SM's shared memory: two CTAs (256 TMEM columns each) per SM
   const size_t smem = std::max<size_t>(tc5_smem_bytes(a.s.m, a.nblocks, a.slots), 80u << 10);
-  cudaFuncSetAttribute(k_tc5_expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_tc5_expand);
   const uint64_t ntiles = ((uint64_t)a.Q + kT5M - 1) / kT5M;
   const int blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>(ntiles, 2ull * nsm));
   k_tc5_expand<<<blocks, kT5Threads, smem, st>>>(a, map);
