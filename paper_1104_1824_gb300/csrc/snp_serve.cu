@@ -303,7 +303,6 @@ int tick(snp_server* S) {
   CK(cudaMemcpyAsync(S->back.data(), dsys, sizeof(BatchSys) * n, cudaMemcpyDeviceToHost, S->st));
   CK(cudaStreamSynchronize(S->st));
   for (Request* r : S->active) r->bs = S->back[r->slot];
-  ++S->ticks;
   return SNP_OK;
 }
 
@@ -368,31 +367,30 @@ void server_loop(snp_server* S) {
     }
     const auto t0 = Clock::now();
     int rc = init_requests(S, fresh);
+    const int ticked = rc == SNP_OK && !S->active.empty() ? 1 : 0;
     if (rc == SNP_OK) rc = tick(S);
     std::vector<Request*> done;
-    if (rc == SNP_OK) {
-      for (size_t i = 0; i < S->active.size();) {
-        Request* r = S->active[i];
-        if (r->bs.done || r->bs.cur_depth >= r->bs.target_depth || r->bs.error) {
-          rc = retire(S, r);
-          if (rc != SNP_OK) break;
-          r->done = Clock::now();
-          return_scratch(S, r->scratch);
-          S->slots[r->slot] = nullptr;
-          done.push_back(r);
-          S->active.erase(S->active.begin() + i);
-        } else {
-          ++i;
-        }
-      }
+    for (Request* r : S->active) {
+      if (rc != SNP_OK) break;
+      if (!(r->bs.done || r->bs.cur_depth >= r->bs.target_depth || r->bs.error)) continue;
+      rc = retire(S, r);
+      if (rc != SNP_OK) break;
+      r->done = Clock::now();
+      return_scratch(S, r->scratch);
+      S->slots[r->slot] = nullptr;
+      done.push_back(r);
     }
-    S->busy_ms += std::chrono::duration<double, std::milli>(Clock::now() - t0).count();
+    const double busy = std::chrono::duration<double, std::milli>(Clock::now() - t0).count();
     std::lock_guard<std::mutex> lk(S->mu);
+    S->busy_ms += busy;
+    S->ticks += ticked;
     if (rc != SNP_OK && S->loop_error == SNP_OK) {
       S->loop_error = rc;
       S->loop_msg = g_err;
     }
+    // from active to finished in one step, as snp_server_wait and _stats look at them
     for (Request* r : done) {
+      S->active.erase(std::find(S->active.begin(), S->active.end(), r));
       S->alloc->release(r->off, r->bytes);
       S->completed += 1;
       S->total_new += r->bs.n_rows - 1;
