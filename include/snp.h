@@ -320,7 +320,8 @@ int snp_batch_autotune(snp_handle* hs, int32_t n, const snp_explore_opts* opts, 
 /* Serving: explorations submitted at any time run together on the device.
  * The paper's simulator runs one system at a time; this loop serves many.  A
  * server thread admits pending requests while its device memory allows (each
- * request needs its pool, 4m (1 + depth * cap) bytes, and its hash table),
+ * request needs its pool, 4m (1 + depth * cap) bytes, its hash table and the
+ * scratch of its passes, of 2048 to 2^16 candidates by the cap and the room),
  * then advances every admitted request by a few passes at a time (a tick)
  * with the batch engine's kernels, so requests that arrive while others run
  * join at the next tick (continuous batching).  A finished request's configurations are copied
@@ -337,13 +338,18 @@ typedef struct {
 
 /* Creates a server on the current device with hbm_budget bytes of device
  * memory for requests and at most max_active requests on the device at once.
+ * Beside them it holds work queues of up to some hundred KB per admitted
+ * request.  A request whose pool and table leave no room for scratch in all of
+ * hbm_budget waits until no other runs and gets scratch for passes of 2048
+ * candidates from outside, given back when it has finished.
  * Errors: SNP_E_INVALID, SNP_E_NOMEM, SNP_E_CUDA. */
 int snp_server_create(size_t hbm_budget, int32_t max_active, void** srv);
 
 /* Queues an exploration of h with opts (depth >= 1, 1 <= frontier_cap <= 2^20,
  * SNP_T_SPARSE_I32, no parent records).  The caller must not use h until the
  * request is reported finished.  *req_id identifies it in snp_server_poll.
- * Errors: SNP_E_INVALID, SNP_E_NOMEM (larger than the server's memory). */
+ * Errors: SNP_E_INVALID, SNP_E_NOMEM (pool and table larger than the server's
+ * memory). */
 int snp_server_submit(void* srv, snp_handle h, const snp_explore_opts* opts, uint64_t* req_id);
 
 /* Takes up to max finished requests: ids, latencies (ms, submit to result

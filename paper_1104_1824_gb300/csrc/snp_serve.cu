@@ -75,11 +75,14 @@ struct Request {
   snp_system* h = nullptr;
   snp_explore_opts o{};
   Clock::time_point arrival, done;
-  size_t off = 0, bytes = 0;  // arena range: pool, table, stats
+  size_t bytes = 0;           // pool, table, stats
+  size_t off = 0, held = 0;   // range of the server's memory: these, then (unless own) the scratch
+  uint32_t qc = 0;            // candidates of a pass
+  bool own = false;           // its scratch is its own allocation
   int64_t rows = 0;
   uint64_t nslots = 0;
   int32_t slot = -1;         // place in the device array of systems
-  std::unique_ptr<DevBuf> scratch;
+  DevBuf scratch;            // own
   int64_t items = 0;         // work items it can have queued
   BatchSys bs{};
   int status = SNP_OK;
@@ -92,7 +95,6 @@ struct snp_server {
   size_t budget = 0;
   int32_t max_active = 0;
   DevBuf arena, sys_dev, items, ctr, idx_dev, c0_dev, c0_off_dev, fill_ptr, fill_cnt;
-  std::vector<std::unique_ptr<DevBuf>> spare;  // scratch of finished requests, for the next ones (at most kSpare)
   std::vector<Request*> slots;   // requests by their place in sys_dev (null: free)
   std::vector<BatchSys> back;    // sys_dev as read back after a tick
   int64_t item_cap = 0;          // items each queue holds
@@ -123,7 +125,6 @@ namespace {
 constexpr uint32_t kServeQc = 2048;    // claims past the cap a request's table has room for, per depth
 constexpr uint32_t kServeRun = 64;     // candidates per work item (48 requests: 96 ms with 192, 80 with 64 or 32)
 constexpr int kTickIterations = 8;
-constexpr size_t kSpare = 64;
 
 size_t request_bytes(const snp_system* h, const snp_explore_opts& o, int64_t* rows, uint64_t* nslots) {
   *rows = 1 + (int64_t)o.depth * o.frontier_cap;
@@ -133,29 +134,26 @@ size_t request_bytes(const snp_system* h, const snp_explore_opts& o, int64_t* ro
   return r((size_t)*rows * h->m * 4) + r(*nslots * 8) + r(sizeof(BatchDepthStat) * (o.depth + 1));
 }
 
-// Scratch for a request: the smallest spare buffer that holds it, else a new one.
-int take_scratch(snp_server* S, size_t bytes, std::unique_ptr<DevBuf>& out) {
-  size_t best = S->spare.size();
-  for (size_t i = 0; i < S->spare.size(); ++i)
-    if (S->spare[i]->bytes >= bytes && (best == S->spare.size() || S->spare[i]->bytes < S->spare[best]->bytes)) best = i;
-  if (best < S->spare.size()) {
-    out = std::move(S->spare[best]);
-    S->spare.erase(S->spare.begin() + best);
-    return SNP_OK;
-  }
-  out.reset(new DevBuf);
-  int rc = out->reserve(bytes);
-  if (rc == SNP_E_NOMEM && !S->spare.empty()) {  // the spare buffers are too small: give them back and try again
-    S->spare.clear();
-    rc = out->reserve(bytes);
-  }
-  if (rc != SNP_OK) out.reset();
-  return rc;
-}
+size_t scratch_bytes(const Request* r, uint32_t qc) { return many_scratch_bytes(r->o.frontier_cap, qc, r->h->m); }
 
-void return_scratch(snp_server* S, std::unique_ptr<DevBuf>& b) {
-  if (b && S->spare.size() < kSpare) S->spare.push_back(std::move(b));
-  b.reset();
+// A place in the server's memory for a request's pool, table and statistics,
+// and behind them the scratch of its passes: of the size the cap asks for, or,
+// where that does not fit beside the requests that run, of 2048 candidates.  A
+// request that leaves no room for scratch in the whole of the memory waits
+// until no other runs and has the scratch of such passes allocated (r->own).
+// false: it has to wait.  (Scratch allocated apart for every request came to
+// up to 0.3 GB each beyond what the caller gave the server.)
+bool place(snp_server* S, Request* r) {
+  const uint32_t full = many_default_qc(r->o.frontier_cap);
+  for (const uint32_t qc : {full, std::min(full, kServeQc)}) {
+    r->qc = qc;
+    r->held = r->bytes + scratch_bytes(r, qc);
+    if (S->alloc->alloc(r->held, &r->off)) return true;
+  }
+  if (!S->active.empty()) return false;
+  r->held = r->bytes;
+  r->own = true;
+  return S->alloc->alloc(r->held, &r->off);
 }
 
 ManyQueue queue_of(const snp_server* S) {
@@ -188,6 +186,36 @@ int ensure_items(snp_server* S, int64_t items) {
   std::swap(S->items.bytes, grown.bytes);
   S->item_cap = want;
   return SNP_OK;
+}
+
+// The system of an admitted request as the kernels see it, and its place among them.
+void set_up(snp_server* S, Request* r) {
+  auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
+  unsigned char* base = S->arena.as<unsigned char>() + r->off;
+  BatchSys& b = r->bs;
+  std::memset(&b, 0, sizeof b);
+  b.sys = r->h->dev();
+  b.pool = reinterpret_cast<int32_t*>(base);
+  b.slots = reinterpret_cast<unsigned long long*>(base + r256((size_t)r->rows * r->h->m * 4));
+  b.bmask = r->nslots / kBucket - 1;
+  b.stats = reinterpret_cast<BatchDepthStat*>(base + r256((size_t)r->rows * r->h->m * 4) + r256(r->nslots * 8));
+  b.pool_rows = r->rows;
+  b.level_lo = 0;
+  b.level_hi = 1;
+  b.n_rows = 1;
+  b.target_depth = r->o.depth;
+  b.max_expand = r->o.max_expand_value;
+  b.cap = r->o.frontier_cap;
+  b.budget = r->o.candidate_budget > 0 ? r->o.candidate_budget : 0;
+  b.overshoot = kServeQc;
+  many_carve(b, r->own ? r->scratch.as<unsigned char>() : base + r->bytes, r->qc, kServeRun);
+  const ManyPlan mine = many_plan(&r->h->m, 1, 0, 0);
+  b.tile = many_tile(mine, r->h->m, 0);
+  r->items = many_items(b.cap, r->qc, kServeRun);
+  r->slot = 0;
+  while (r->slot < (int32_t)S->slots.size() && S->slots[r->slot]) ++r->slot;
+  if (r->slot == (int32_t)S->slots.size()) S->slots.push_back(nullptr);
+  S->slots[r->slot] = r;
 }
 
 // Device state of newly admitted requests: empty tables, C0 in row 0 and in the table.
@@ -242,6 +270,7 @@ int retire(snp_server* S, Request* r) {
   std::vector<BatchDepthStat> st(depth + 1);
   CK(cudaMemcpyAsync(st.data(), b.stats, sizeof(BatchDepthStat) * (depth + 1), cudaMemcpyDeviceToHost, S->st));
   const size_t bytes = sizeof(int32_t) * (size_t)b.n_rows * h->m;
+  r->scratch.release();  // its passes are done
   if (h->d_pool.reserve(bytes) != SNP_OK) {  // this request fails; the server goes on
     r->status = SNP_E_NOMEM;
     h->explored = false;
@@ -306,6 +335,27 @@ int tick(snp_server* S) {
   return SNP_OK;
 }
 
+// Requests that have run or failed, from the active ones to the finished ones
+// in one step, as snp_server_wait and _stats look at them (S->mu held).
+void finish_locked(snp_server* S, const std::vector<Request*>& done) {
+  for (Request* r : done) {
+    S->active.erase(std::find(S->active.begin(), S->active.end(), r));
+    S->alloc->release(r->off, r->held);
+    S->completed += 1;
+    S->total_new += std::max<int64_t>(r->bs.n_rows - 1, 0);
+    S->lat_ms.push_back(std::chrono::duration<double, std::milli>(r->done - r->arrival).count());
+    S->last_done = r->done;
+    S->finished.push_back(r);
+  }
+  if (!done.empty()) S->cv_done.notify_all();
+}
+
+void finish(snp_server* S, const std::vector<Request*>& done) {
+  for (Request* r : done) r->done = Clock::now();
+  std::lock_guard<std::mutex> lk(S->mu);
+  finish_locked(S, done);
+}
+
 void server_loop(snp_server* S) {
   cudaSetDevice(S->device);
   for (;;) {
@@ -319,51 +369,21 @@ void server_loop(snp_server* S) {
       }
       while (!S->pending.empty() && (int32_t)S->active.size() < S->max_active) {
         Request* r = S->pending.front();
-        size_t off = 0;
-        if (!S->alloc->alloc(r->bytes, &off)) break;  // admitted when memory frees up
-        const uint32_t qc = many_default_qc(r->o.frontier_cap);
-        const int rc = take_scratch(S, many_scratch_bytes(r->o.frontier_cap, qc, r->h->m), r->scratch);
-        if (rc != SNP_OK) {
-          S->alloc->release(off, r->bytes);
-          if (!S->active.empty()) break;  // admitted when running requests give theirs back
-          S->pending.pop_front();         // alone and it does not fit: this request fails
-          r->status = rc;
-          r->done = Clock::now();
-          S->finished.push_back(r);
-          S->cv_done.notify_all();
-          continue;
-        }
+        if (!place(S, r)) break;  // admitted when memory frees up
         S->pending.pop_front();
-        r->off = off;
-        auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
-        unsigned char* base = S->arena.as<unsigned char>() + off;
-        BatchSys& b = r->bs;
-        std::memset(&b, 0, sizeof b);
-        b.sys = r->h->dev();
-        b.pool = reinterpret_cast<int32_t*>(base);
-        b.slots = reinterpret_cast<unsigned long long*>(base + r256((size_t)r->rows * r->h->m * 4));
-        b.bmask = r->nslots / kBucket - 1;
-        b.stats = reinterpret_cast<BatchDepthStat*>(base + r256((size_t)r->rows * r->h->m * 4) + r256(r->nslots * 8));
-        b.pool_rows = r->rows;
-        b.level_lo = 0;
-        b.level_hi = 1;
-        b.n_rows = 1;
-        b.target_depth = r->o.depth;
-        b.max_expand = r->o.max_expand_value;
-        b.cap = r->o.frontier_cap;
-        b.budget = r->o.candidate_budget > 0 ? r->o.candidate_budget : 0;
-        b.overshoot = kServeQc;
-        many_carve(b, r->scratch->as<unsigned char>(), qc, kServeRun);
-        const ManyPlan mine = many_plan(&r->h->m, 1, 0, 0);
-        b.tile = many_tile(mine, r->h->m, 0);
-        r->items = many_items(b.cap, qc, kServeRun);
-        r->slot = 0;
-        while (r->slot < (int32_t)S->slots.size() && S->slots[r->slot]) ++r->slot;
-        if (r->slot == (int32_t)S->slots.size()) S->slots.push_back(nullptr);
-        S->slots[r->slot] = r;
         S->active.push_back(r);
         fresh.push_back(r);
       }
+    }
+    for (size_t i = 0; i < fresh.size();) {
+      Request* r = fresh[i];
+      if (r->own && (r->status = r->scratch.reserve(scratch_bytes(r, r->qc))) != SNP_OK) {  // this request fails
+        finish(S, {r});
+        fresh.erase(fresh.begin() + i);
+        continue;
+      }
+      set_up(S, r);
+      ++i;
     }
     const auto t0 = Clock::now();
     int rc = init_requests(S, fresh);
@@ -376,7 +396,6 @@ void server_loop(snp_server* S) {
       rc = retire(S, r);
       if (rc != SNP_OK) break;
       r->done = Clock::now();
-      return_scratch(S, r->scratch);
       S->slots[r->slot] = nullptr;
       done.push_back(r);
     }
@@ -388,17 +407,7 @@ void server_loop(snp_server* S) {
       S->loop_error = rc;
       S->loop_msg = g_err;
     }
-    // from active to finished in one step, as snp_server_wait and _stats look at them
-    for (Request* r : done) {
-      S->active.erase(std::find(S->active.begin(), S->active.end(), r));
-      S->alloc->release(r->off, r->bytes);
-      S->completed += 1;
-      S->total_new += r->bs.n_rows - 1;
-      S->lat_ms.push_back(std::chrono::duration<double, std::milli>(r->done - r->arrival).count());
-      S->last_done = r->done;
-      S->finished.push_back(r);
-    }
-    if (!done.empty() || rc != SNP_OK) S->cv_done.notify_all();
+    finish_locked(S, done);
     if (rc != SNP_OK) {  // a device error ends the loop; waiting callers are released
       for (Request* r : S->active) {
         r->status = rc;
@@ -555,7 +564,6 @@ int snp_server_destroy(void* srv) {
   for (Request* r : S->finished) delete r;
   for (Request* r : S->pending) delete r;
   for (Request* r : S->active) delete r;
-  S->spare.clear();
   if (S->st) cudaStreamDestroy(S->st);
   delete S->alloc;
   delete S;
