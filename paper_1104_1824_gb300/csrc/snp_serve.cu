@@ -218,18 +218,32 @@ void set_up(snp_server* S, Request* r) {
   S->slots[r->slot] = r;
 }
 
+// Memory that newly admitted requests need beside their own: before anything of them is on the device.
+int room_for(snp_server* S, const std::vector<Request*>& fresh) {
+  if (fresh.empty()) return SNP_OK;
+  const size_t n = fresh.size();
+  size_t counts = 0;
+  int64_t items = 0;
+  for (const Request* r : S->active) items += r->items;  // the new ones among them
+  for (const Request* r : fresh) counts += (size_t)r->h->m;
+  TRY(ensure_items(S, items));
+  TRY(S->sys_dev.reserve(sizeof(BatchSys) * std::max<size_t>(64, S->slots.size() * 2), S->st, true));
+  TRY(S->fill_ptr.reserve(sizeof(void*) * n));
+  TRY(S->fill_cnt.reserve(sizeof(uint64_t) * n));
+  TRY(S->idx_dev.reserve(sizeof(int32_t) * n));
+  TRY(S->c0_dev.reserve(sizeof(int32_t) * counts));
+  TRY(S->c0_off_dev.reserve(sizeof(int64_t) * n));
+  return SNP_OK;
+}
+
 // Device state of newly admitted requests: empty tables, C0 in row 0 and in the table.
-int init_requests(snp_server* S, std::vector<Request*>& fresh) {
+int init_requests(snp_server* S, const std::vector<Request*>& fresh) {
   if (fresh.empty()) return SNP_OK;
   const int n = (int)fresh.size();
   std::vector<unsigned long long*> ptr(n);
   std::vector<uint64_t> cnt(n);
   std::vector<int32_t> c0, idx(n);
   std::vector<int64_t> c0_off(n);
-  int64_t items = 0;
-  for (const Request* r : S->active) items += r->items;  // the new ones among them
-  TRY(ensure_items(S, items));
-  TRY(S->sys_dev.reserve(sizeof(BatchSys) * std::max<size_t>(64, S->slots.size() * 2), S->st, true));
   for (int i = 0; i < n; ++i) {
     Request* r = fresh[i];
     ptr[i] = r->bs.slots;
@@ -238,11 +252,6 @@ int init_requests(snp_server* S, std::vector<Request*>& fresh) {
     c0_off[i] = (int64_t)c0.size();
     c0.insert(c0.end(), r->h->c0.begin(), r->h->c0.end());
   }
-  TRY(S->fill_ptr.reserve(sizeof(void*) * n));
-  TRY(S->fill_cnt.reserve(sizeof(uint64_t) * n));
-  TRY(S->idx_dev.reserve(sizeof(int32_t) * n));
-  TRY(S->c0_dev.reserve(sizeof(int32_t) * c0.size()));
-  TRY(S->c0_off_dev.reserve(sizeof(int64_t) * n));
   CK(cudaMemcpyAsync(S->fill_ptr.p, ptr.data(), sizeof(void*) * n, cudaMemcpyHostToDevice, S->st));
   CK(cudaMemcpyAsync(S->fill_cnt.p, cnt.data(), sizeof(uint64_t) * n, cudaMemcpyHostToDevice, S->st));
   CK(cudaMemcpyAsync(S->idx_dev.p, idx.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, S->st));
@@ -386,7 +395,18 @@ void server_loop(snp_server* S) {
       ++i;
     }
     const auto t0 = Clock::now();
-    int rc = init_requests(S, fresh);
+    int rc = room_for(S, fresh);
+    if (rc == SNP_E_NOMEM) {  // the new requests fail; those that run go on
+      for (Request* r : fresh) {
+        r->status = rc;
+        r->scratch.release();
+        S->slots[r->slot] = nullptr;
+      }
+      finish(S, fresh);
+      fresh.clear();
+      rc = SNP_OK;
+    }
+    if (rc == SNP_OK) rc = init_requests(S, fresh);
     const int ticked = rc == SNP_OK && !S->active.empty() ? 1 : 0;
     if (rc == SNP_OK) rc = tick(S);
     std::vector<Request*> done;

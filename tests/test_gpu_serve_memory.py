@@ -119,6 +119,37 @@ def test_scratch_of_its_own_cannot_be_had(gpu):
         gpu.snp_server_destroy(srv)
 
 
+@pytest.mark.parametrize("k", range(1, 12))
+def test_failed_allocation_fails_its_request_alone(gpu, k):
+    """The k-th allocation of a burst fails: that request is reported, every
+    other one is served, the counters account for all of them."""
+    systems = systems_of(4, 64, seed=2)
+    hs = [gpu.System(x) for x in systems]
+    srv = gpu.snp_server_create(256 * MB, 8)
+    try:
+        gpu.snp_debug_fail_allocation(k)
+        ids = []
+        for h in hs:  # one at a time: what is allocated is the request's
+            ids.append(gpu.snp_server_submit(srv, h.h, opts(gpu, 2, 64, 1000)))
+            gpu.snp_server_wait(srv)
+        got_ids, _, st = gpu.snp_server_poll(srv)
+        status = dict(zip([int(i) for i in got_ids], [int(s) for s in st]))
+        assert sorted(status) == sorted(ids)
+        assert [status[i] for i in ids].count(gpu.SNP_E_NOMEM) == 1
+        for i, h, x in zip(ids, hs, systems):
+            if status[i] == gpu.SNP_E_NOMEM:
+                with pytest.raises(gpu.SnpError):
+                    h.reachable()
+            else:
+                assert status[i] == 0
+                same(h, x, 2, 64, 1000)
+        info = gpu.snp_server_stats(srv)
+        assert info.submitted == info.completed == 4 and info.active == 0 and info.pending == 0
+    finally:
+        gpu.snp_debug_fail_allocation(0)
+        gpu.snp_server_destroy(srv)
+
+
 def test_counters_account_for_every_request(gpu):
     """submitted = completed + active + pending whenever one looks, and a
     finished request can be polled once it is counted."""
