@@ -435,8 +435,14 @@ int snp_step(snp_handle h, const int32_t* C, int64_t capacity, int32_t* out, uin
   const int m = h->m;
   // C twice: the second copy becomes the base child on the device
   std::vector<int32_t> c(2 * (size_t)m);
-  if (is_device_ptr(C)) CK(cudaMemcpy(c.data(), C, sizeof(int32_t) * m, cudaMemcpyDefault));
-  else std::memcpy(c.data(), C, sizeof(int32_t) * m);
+  if (is_device_ptr(C)) {
+    CK(cudaMemcpy(c.data(), C, sizeof(int32_t) * m, cudaMemcpyDefault));
+  } else {
+    // what the default stream still writes there (a copy into pinned memory)
+    // comes first; cudaMemcpy would wait for it too, and take 10 us
+    CK(cudaStreamSynchronize(nullptr));
+    std::memcpy(c.data(), C, sizeof(int32_t) * m);
+  }
   for (int j = 0; j < m; ++j) {
     if (c[j] < 0) return fail(SNP_E_INVALID, "C[%d] = %d < 0", j, c[j]);
     if (c[j] > INT32_MAX - h->gain[j]) return fail(SNP_E_OVERFLOW, "C[%d] = %d: a child could leave int32", j, c[j]);
