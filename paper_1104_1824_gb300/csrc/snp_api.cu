@@ -803,8 +803,10 @@ int explore_impl(snp_handle h, const snp_explore_opts* o, int32_t* depth_reached
   auto chain_pass = [&]() -> uint64_t {  // candidates of such a pass; 0: not now
     if (tc || tc5 || !one_pass) return 0;
     if (psi_saturated_before && (cap <= 0 || cap > 2 * kPsiHead)) return 0;  // large frontiers whose rows mostly are not read
-    double want = cap > 0 ? (double)cap / std::max(rate, 1.0 / 1024.0) * 1.25 + 4096.0
-                          : std::max(4096.0, 8.0 * (double)last_T);
+    // the caller's pass size, else as the cap or the last depth suggests
+    double want = o->chunk > 0 ? (double)qmax
+                  : cap > 0    ? (double)cap / std::max(rate, 1.0 / 1024.0) * 1.25 + 4096.0
+                               : std::max(4096.0, 8.0 * (double)last_T);
     if (want > (double)kChainQ) return 0;
     uint64_t Q = std::min<uint64_t>((uint64_t)want, qmax);
     if (budget > 0) Q = std::min<uint64_t>(Q, (uint64_t)budget);
