@@ -295,6 +295,7 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
         limit = std::min(limit, need) / 4;
         q = std::min(q, std::max<uint32_t>(qs, 1));
         rc = SNP_OK;
+        g_err.clear();  // not a failure of the call
         continue;
       }
       if (rc == SNP_OK) rc = many_group(arena.get(), sys, c0_off.data(), lo, hi, plan, q, hs[0]->pin, hs[0]->evs, st, nsm);

@@ -1,0 +1,34 @@
+"""The batch engine where device memory runs short: whichever allocation
+fails, the call either serves every system (in smaller groups and passes) and
+leaves no message, or returns SNP_E_NOMEM and works the next time."""
+import numpy as np
+import pytest
+
+import oracle
+import snp_synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("k", range(1, 10))
+def test_failed_allocation(gpu, k):
+    systems = snp_synth.batch_systems(6)
+    hs = [gpu.System(x) for x in systems]
+    gpu.snp_debug_fail_allocation(k)
+    try:
+        o = gpu.snp_explore_opts_init()
+        o.depth, o.frontier_cap, o.candidate_budget = 3, 300, 5000
+        status = np.full(len(hs), -1, dtype=np.int32)
+        gpu.snp_explore_batch([h.h for h in hs], o, status)
+        assert gpu.snp_last_error() == ""
+        assert (status == 0).all()
+    except gpu.SnpError as e:
+        assert e.code == gpu.SNP_E_NOMEM
+        gpu.snp_debug_fail_allocation(0)
+        assert (gpu.explore_batch(hs, 3, cap=300, budget=5000) == 0).all()
+    finally:
+        gpu.snp_debug_fail_allocation(0)
+    for h, x in zip(hs, systems):
+        e = oracle.Oracle(x).explore(3, cap=300, budget=5000)
+        got = h.reachable()
+        assert got.shape == e.configs.shape and (got == e.configs).all()
