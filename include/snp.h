@@ -310,10 +310,11 @@ int snp_row_width(snp_handle h, int32_t* bytes_per_count);
 int snp_explore_batch(snp_handle* hs, int32_t n, const snp_explore_opts* opts, int32_t* statuses);
 
 /* Chooses the batch engine's pass size, tile and warps per CTA for this batch
- * by timing the first two depths of each candidate setting (on the real
- * systems; their previous results are discarded).  *chunk, *tile and *warps
- * receive the fastest setting, for snp_explore_batch's options.  Errors as
- * snp_explore_batch. */
+ * by timing the first two depths of each candidate setting on the device (on
+ * the real systems; their previous results are discarded).  Pass sizes: 1024,
+ * 2048, 4096 and, in the sparse form, the one the engine takes by itself for
+ * the cap where that is larger.  *chunk, *tile and *warps receive the fastest
+ * setting, for snp_explore_batch's options.  Errors as snp_explore_batch. */
 int snp_batch_autotune(snp_handle* hs, int32_t n, const snp_explore_opts* opts, int32_t* chunk, int32_t* tile,
                        int32_t* warps);
 

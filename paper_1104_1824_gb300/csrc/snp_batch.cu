@@ -43,9 +43,35 @@ struct BatchPlan {
 // Scratch the systems of one group share the device with.
 constexpr size_t kGroupScratch = (size_t)12 << 30;
 
+// Device time of the parts of a batch that count: what lies between start()
+// and stop(), allocations and graph capture left out.
+struct BatchTimer {
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  float ms = 0.f;
+  ~BatchTimer() {
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+  }
+  int start(cudaStream_t st) {
+    if (!e0) CK(cudaEventCreate(&e0));
+    if (!e1) CK(cudaEventCreate(&e1));
+    CK(cudaEventRecord(e0, st));
+    return SNP_OK;
+  }
+  int stop(cudaStream_t st) {
+    CK(cudaEventRecord(e1, st));
+    CK(cudaEventSynchronize(e1));
+    float part = 0.f;
+    CK(cudaEventElapsedTime(&part, e0, e1));
+    ms += part;
+    return SNP_OK;
+  }
+};
+
 // Runs systems [lo, hi) of the arena (sparse form) to their end on st.
 int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_off, int32_t lo, int32_t hi,
-               const BatchPlan& plan, uint32_t qc, PinnedState& pin, cudaEvent_t* evs, cudaStream_t st, int nsm) {
+               const BatchPlan& plan, uint32_t qc, PinnedState& pin, cudaEvent_t* evs, BatchTimer* timer,
+               cudaStream_t st, int nsm) {
   const int32_t n = hi - lo;
   std::vector<int> ms(n);
   for (int32_t i = 0; i < n; ++i) ms[i] = sys[lo + i].sys.m;
@@ -74,6 +100,7 @@ int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_
   q.psi[1] = q.psi[0] + items;
   q.ctr = arena->queue.as<uint32_t>();
   q.cap = items;
+  if (timer) TRY(timer->start(st));
   BatchSys* dsys = arena->sys.as<BatchSys>() + lo;
   CK(cudaMemcpyAsync(dsys, sys.data() + lo, sizeof(BatchSys) * n, cudaMemcpyHostToDevice, st));
   CK(cudaMemsetAsync(q.ctr, 0, sizeof(uint32_t) * kMqCounters, st));
@@ -91,6 +118,7 @@ int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_
     CK(cudaMemcpyAsync(active[it & 1], q.ctr + kMqActive, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     CK(cudaEventRecord(evs[it & 1], st));
   }
+  if (timer) TRY(timer->stop(st));
   CK(cudaStreamSynchronize(st));
   return SNP_OK;
 }
@@ -122,7 +150,7 @@ int batch_setup(snp_handle* hs, int32_t n, const snp_explore_opts* o) {
 
 // Tensor-core form: depth launches, captured once per arena and replayed as one graph.
 int run_tc_depths(BatchArena* arena, const std::vector<BatchSys>& sys, const BatchArgs& args, int blocks, int depth,
-                  bool fresh, size_t scratch_stride, cudaStream_t st, int nsm) {
+                  bool fresh, size_t scratch_stride, BatchTimer* timer, cudaStream_t st, int nsm) {
   const int32_t n = (int32_t)sys.size();
   CK(cudaMemcpyAsync(arena->sys.p, sys.data(), sizeof(BatchSys) * n, cudaMemcpyHostToDevice, st));
   CK(cudaMemsetAsync(arena->queue.p, 0, sizeof(unsigned int) * (depth + 1), st));
@@ -149,16 +177,18 @@ int run_tc_depths(BatchArena* arena, const std::vector<BatchSys>& sys, const Bat
       return fail(SNP_E_CUDA, "batch graph: %s", cudaGetErrorString(ce));
     }
   }
+  if (timer) TRY(timer->start(st));
   cudaError_t ce = cudaGraphLaunch(arena->exec, st);
+  if (timer && ce == cudaSuccess) TRY(timer->stop(st));
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   if (ce != cudaSuccess) return fail(SNP_E_CUDA, "batch run: %s", cudaGetErrorString(ce));
   return SNP_OK;
 }
 
 // Runs depths 1..depth of the batch (all handles) with the given plan; fills
-// the handles' results.  ms (optional) receives the device time of the depths.
+// the handles' results.  timer (optional) receives the device time of the depths.
 int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchPlan& plan, int32_t* statuses,
-              float* ms) {
+              BatchTimer* timer) {
   const int dev = hs[0]->device;
   CK(cudaSetDevice(dev));
   cudaStream_t st = static_cast<cudaStream_t>(o->stream);
@@ -267,15 +297,9 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
   a.scratch_stride = scratch_stride;
   a.pmax = cap;
   a.m_max = m_max;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (ms) {
-    CK(cudaEventCreate(&e0));
-    CK(cudaEventCreate(&e1));
-  }
   int rc = SNP_OK;
-  if (ms) CK(cudaEventRecord(e0, st));
   if (tc) {
-    rc = run_tc_depths(arena.get(), sys, a, blocks, depth, !same, scratch_stride, st, nsm);
+    rc = run_tc_depths(arena.get(), sys, a, blocks, depth, !same, scratch_stride, timer, st, nsm);
   } else {
     // groups of systems whose scratch fits kGroupScratch; with little memory
     // left, smaller groups (down to one system) and passes of 2048
@@ -298,17 +322,11 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
         g_err.clear();  // not a failure of the call
         continue;
       }
-      if (rc == SNP_OK) rc = many_group(arena.get(), sys, c0_off.data(), lo, hi, plan, q, hs[0]->pin, hs[0]->evs, st, nsm);
+      if (rc == SNP_OK)
+        rc = many_group(arena.get(), sys, c0_off.data(), lo, hi, plan, q, hs[0]->pin, hs[0]->evs, timer, st, nsm);
       lo = hi;
     }
   }
-  if (ms && rc == SNP_OK) {
-    CK(cudaEventRecord(e1, st));
-    CK(cudaEventSynchronize(e1));
-    CK(cudaEventElapsedTime(ms, e0, e1));
-  }
-  if (e0) cudaEventDestroy(e0);
-  if (e1) cudaEventDestroy(e1);
   if (rc != SNP_OK) return rc;
   // results
   std::vector<BatchDepthStat> stats((size_t)n * (depth + 1));
@@ -374,7 +392,10 @@ extern "C" int snp_batch_autotune(snp_handle* hs, int32_t n, const snp_explore_o
   if (!chunk || !tile || !warps) return fail(SNP_E_INVALID, "bad arguments");
   snp_explore_opts t = *o;
   t.depth = std::min(o->depth, 2);
-  const uint32_t qcs[] = {1024, 2048, 4096};
+  std::vector<uint32_t> qcs = {1024, 2048, 4096};
+  // what the sparse form takes by itself for a large cap (64 systems, cap 2^14: 24 ms, 60 ms with passes of 4096)
+  if (o->transition == SNP_T_SPARSE_I32 && many_default_qc(o->frontier_cap) > qcs.back())
+    qcs.push_back(many_default_qc(o->frontier_cap));
   const int tiles[] = {8, 16, 32};
   const int ws[] = {4, 8};
   const bool tc = o->transition == SNP_T_TC_F8;  // the tensor-core form: tile and warps are fixed
@@ -388,10 +409,10 @@ extern "C" int snp_batch_autotune(snp_handle* hs, int32_t n, const snp_explore_o
         p.qc = qc;
         p.tile = tl;
         p.warps = w;
-        float ms = 0.f;
-        TRY(batch_run(hs, n, &t, p, nullptr, &ms));
-        if (ms < best) {
-          best = ms;
+        BatchTimer timer;
+        TRY(batch_run(hs, n, &t, p, nullptr, &timer));
+        if (timer.ms < best) {
+          best = timer.ms;
           bestp = p;
         }
       }
