@@ -455,8 +455,8 @@ def bench_ours(args):
 
 
 def time_batch(args, w, systems, handles, snp, torch, dist, dev, world, local, form: str, steps: int, warmup: int):
-    """Times `steps` batch explorations
-    in one transition form; returns the timing, plan and per-step counts."""
+    """Times `steps` batch explorations in one transition form; returns the
+    timing, plan and per-step counts (launches: of one exploration)."""
     import numpy as np
     hs = [h.h for h in handles]
     stream = torch.cuda.Stream(device=dev)
@@ -499,6 +499,7 @@ def time_batch(args, w, systems, handles, snp, torch, dist, dev, world, local, f
             per_depth.setdefault(d, 0)
             per_depth[d] += a.new
     return dict(ms=ms, clocks=clk, new_step=new_step, bytes_step=bytes_step, per_depth=per_depth,
+                launches=handles[0].depth_stats()[0].launches,
                 plan={"chunk": chunk, "tile": tile, "warps": warps, "autotuned": bool(args.autotune),
                       "autotune_s": round(tune_s, 2)})
 
@@ -513,8 +514,9 @@ def bench_batch(args, w, systems, snp, torch, dist, dev, rank, world, local):
     main_form = args.transition or "sparse"
     r = time_batch(args, w, systems, handles, snp, torch, dist, dev, world, local, main_form, args.steps, args.warmup)
     ms, clk, new_step, bytes_step, per_depth = r["ms"], r["clocks"], r["new_step"], r["bytes_step"], r["per_depth"]
-    ms_max, (total_all,) = aggregate_ranks(ms, [new_step * args.steps], dist if world > 1 else None, dev)
-    total_all = int(total_all)
+    ms_max, (total_all, launches_all) = aggregate_ranks(ms, [new_step * args.steps, r["launches"] * args.steps],
+                                                        dist if world > 1 else None, dev)
+    total_all, launches_all = int(total_all), int(launches_all)
     value = total_all / (ms_max * 1e-3)
     peak, peak_kind = measured_peaks()
     achieved = bytes_step * args.steps / (ms * 1e-3) / 1e9
@@ -533,7 +535,7 @@ def bench_batch(args, w, systems, snp, torch, dist, dev, rank, world, local):
                          "peak": peak, "peak_kind": f"{peak_kind} copy bandwidth", "unit": "GB/s",
                          "frac": round(rf["bytes_step"] * args.steps / (rf["ms"] * 1e-3) / 1e9 / peak, 4),
                          "traffic": None},
-            "clocks": rf["clocks"],
+            "gpu_launches": rf["launches"] * args.steps, "clocks": rf["clocks"],
         }
     chunk, tile, warps = r["plan"]["chunk"], r["plan"]["tile"], r["plan"]["warps"]
     tune_s = r["plan"]["autotune_s"]
@@ -584,13 +586,13 @@ def bench_batch(args, w, systems, snp, torch, dist, dev, rank, world, local):
                        "l2": "inputs larger than L2 (pools of all systems, tens of GB)",
                        "parallelism": f"dp{world}: rank r explores systems of seeds {w['base_seed']} + {w['n']} r ..."
                        if world > 1 else "single GPU"},
-            "roofline": {"kernel": "k_many_psi, k_many_expand, k_many_copy and their control kernels (all systems)", "bound": "hbm",
+            "roofline": {"kernel": "k_many_psi, k_many_expand, k_many_copy and their control kernels (all systems)",
+                         "bound": "hbm",
                          "achieved": round(achieved, 1), "peak": peak, "peak_kind": f"{peak_kind} copy bandwidth",
                          "unit": "GB/s", "frac": round(achieved / peak, 4),
-                         "algorithmic_bytes_per_launch": int(bytes_step / w["depth"]),
-                         "avg_launch_ms": round(ms / args.steps / w["depth"], 3), "traffic": None},
-            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": (w["depth"] + 2) * args.steps,  # at least: the sparse form launches more per depth
-            "clocks": clk,
+                         "algorithmic_bytes_per_depth": int(bytes_step / w["depth"]),
+                         "ms_per_depth": round(ms / args.steps / w["depth"], 3), "traffic": None},
+            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches_all, "clocks": clk,
         }
         if compare:
             line["compare"] = compare

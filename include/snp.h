@@ -201,7 +201,9 @@ typedef struct {
                             key compare, per accepted configuration a 4m-byte
                             row write and an 8-byte slot write, per parent a
                             4m-byte row read */
-  int64_t launches;      /* kernels launched for this depth */
+  int64_t launches;      /* kernels launched for this depth (snp_explore_batch:
+                            depth 0 has the launches of the whole call, which
+                            its systems share, the others 0) */
 } snp_depth_info;
 
 /* Fills *opts with defaults: depth 1, sparse int32, no cap, no budget,

@@ -71,7 +71,7 @@ struct BatchTimer {
 // Runs systems [lo, hi) of the arena (sparse form) to their end on st.
 int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_off, int32_t lo, int32_t hi,
                const BatchPlan& plan, uint32_t qc, PinnedState& pin, cudaEvent_t* evs, BatchTimer* timer,
-               cudaStream_t st, int nsm) {
+               int64_t* launches, cudaStream_t st, int nsm) {
   const int32_t n = hi - lo;
   std::vector<int> ms(n);
   for (int32_t i = 0; i < n; ++i) ms[i] = sys[lo + i].sys.m;
@@ -106,6 +106,7 @@ int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_
   CK(cudaMemsetAsync(q.ctr, 0, sizeof(uint32_t) * kMqCounters, st));
   launch_many_init(dsys, nullptr, arena->c0.as<int32_t>(), arena->c0_off.as<int64_t>() + lo, n, q, st);
   CK(cudaGetLastError());
+  *launches += 1;
   // two iterations in flight: the count read back is the one before last
   uint32_t* active[2] = {reinterpret_cast<uint32_t*>(pin.slot[0]), reinterpret_cast<uint32_t*>(pin.slot[1])};
   for (int it = 0;; ++it) {
@@ -113,7 +114,7 @@ int many_group(BatchArena* arena, std::vector<BatchSys>& sys, const int64_t* c0_
       CK(cudaEventSynchronize(evs[it & 1]));
       if (*active[it & 1] == 0) break;
     }
-    launch_many_iteration(dsys, n, q, it & 1, mp, st, nsm);
+    *launches += launch_many_iteration(dsys, n, q, it & 1, mp, st, nsm);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(active[it & 1], q.ctr + kMqActive, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     CK(cudaEventRecord(evs[it & 1], st));
@@ -298,7 +299,9 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
   a.pmax = cap;
   a.m_max = m_max;
   int rc = SNP_OK;
+  int64_t launches = 1;  // the tables' fill above
   if (tc) {
+    launches += 1 + depth;
     rc = run_tc_depths(arena.get(), sys, a, blocks, depth, !same, scratch_stride, timer, st, nsm);
   } else {
     // groups of systems whose scratch fits kGroupScratch; with little memory
@@ -323,7 +326,8 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
         continue;
       }
       if (rc == SNP_OK)
-        rc = many_group(arena.get(), sys, c0_off.data(), lo, hi, plan, q, hs[0]->pin, hs[0]->evs, timer, st, nsm);
+        rc = many_group(arena.get(), sys, c0_off.data(), lo, hi, plan, q, hs[0]->pin, hs[0]->evs, timer, &launches, st,
+                        nsm);
       lo = hi;
     }
   }
@@ -339,6 +343,7 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
     snp_depth_info s0;
     std::memset(&s0, 0, sizeof s0);
     s0.new_configs = 1;
+    s0.launches = launches;
     h->stats.push_back(s0);
     int64_t lo = 0, hi = 1;
     for (int d = 1; d <= depth; ++d) {

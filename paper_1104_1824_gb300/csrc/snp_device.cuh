@@ -202,7 +202,7 @@ struct DevTable {
 
 // Per-chunk device counters (read back by the host after each chunk).
 struct ChunkState {
-  unsigned int n_alloc;       // staging rows handed out
+  unsigned int n_alloc;       // keys claimed in the chunk (its first occurrences)
   unsigned int error;         // kErr* bits
   unsigned int total_first;   // distinct new keys in the chunk
   unsigned int capped;        // the cap was reached inside the chunk

@@ -174,7 +174,7 @@ struct BatchSys {
 // Work items {system, first element} of one iteration of the sparse form.
 struct ManyQueue {
   int2* expand[2];             // runs of a.run candidates: this iteration's and the next one's; kMqForms regions of `cap`
-  int2* copy;                  // 32 first occurrences each
+  int2* copy;                  // kCopyRows first occurrences each
   int2* psi[2];                // 32 frontier rows each: without and with parent records
   uint32_t* ctr;               // counters, kMq*
   int64_t cap;                 // items of one region
@@ -206,9 +206,9 @@ int64_t many_items(int64_t cap, uint32_t qc, uint32_t run);
 void launch_many_init(BatchSys* sys, const int32_t* idx, const int32_t* c0, const int64_t* c0_off, int32_t n,
                       const ManyQueue& q, cudaStream_t st);
 // One iteration over the systems [0, n): each finishes the Psi scan of a new
-// frontier and at most one pass.  par alternates 0, 1.
-void launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par, const ManyPlan& p, cudaStream_t st,
-                           int nsm);
+// frontier and at most one pass.  par alternates 0, 1.  Returns the launches made.
+int launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par, const ManyPlan& p, cudaStream_t st,
+                          int nsm);
 
 struct BatchDepthStat {
   int64_t new_configs;

@@ -554,7 +554,7 @@ void launch_many_init(BatchSys* sys, const int32_t* idx, const int32_t* c0, cons
   k_many_init<<<std::min((n + per - 1) / per, 152 * 16), kManyThreads, 0, st>>>(sys, idx, c0, c0_off, n, q);
 }
 
-void launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par, const ManyPlan& p, cudaStream_t st,
+int launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par, const ManyPlan& p, cudaStream_t st,
                            int nsm) {
   const size_t smem = (p.warp_bytes + kArgsBytes) * p.warps;
   allow_smem(k_many_expand);
@@ -564,6 +564,7 @@ void launch_many_iteration(BatchSys* sys, int32_t n, const ManyQueue& q, int par
   k_many_expand<<<nsm * p.ctas_per_sm, p.warps * 32, smem, st>>>(sys, q, par, (uint32_t)p.warp_bytes);
   k_many_control<<<n, kControlThreads, 0, st>>>(sys, q, par);
   k_many_copy<<<nsm * 8, kManyThreads, 0, st>>>(sys, q, par);
+  return 6;
 }
 
 }  // namespace snp
