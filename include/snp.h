@@ -307,7 +307,9 @@ int snp_row_width(snp_handle h, int32_t* bytes_per_count);
  *  statuses  (host, [n], may be NULL) per system: SNP_OK, SNP_E_OVERFLOW,
  *            SNP_E_TIMEOUT or SNP_E_INTERNAL.
  * The systems' configurations live in one device arena shared by the handles
- * until each is freed or explored again.  Returns SNP_OK when the batch ran
+ * until each is freed or explored again.  While the call runs it takes up to
+ * 12 GiB of scratch besides (less where memory is short), of which at most
+ * 4 GiB stay with the arena.  Returns SNP_OK when the batch ran
  * (check statuses), else SNP_E_INVALID, SNP_E_NOMEM, SNP_E_CUDA. */
 int snp_explore_batch(snp_handle* hs, int32_t n, const snp_explore_opts* opts, int32_t* statuses);
 

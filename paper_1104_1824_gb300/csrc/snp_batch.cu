@@ -42,6 +42,10 @@ struct BatchPlan {
 
 // Scratch the systems of one group share the device with.
 constexpr size_t kGroupScratch = (size_t)12 << 30;
+// Scratch that stays with the results for the next batch of the same handles;
+// more is given back when the call returns.  (Giving back all of it: 512
+// systems with 2.9 GB of scratch, 48.4 -> 51.1 ms.)
+constexpr size_t kKeptScratch = (size_t)4 << 30;
 
 // Device time of the parts of a batch that count: what lies between start()
 // and stop(), allocations and graph capture left out.
@@ -332,6 +336,7 @@ int batch_run(snp_handle* hs, int32_t n, const snp_explore_opts* o, const BatchP
     }
   }
   if (rc != SNP_OK) return rc;
+  if (arena->scratch.bytes > kKeptScratch) arena->scratch.release();
   // results
   std::vector<BatchDepthStat> stats((size_t)n * (depth + 1));
   CK(cudaMemcpy(sys.data(), arena->sys.p, sizeof(BatchSys) * n, cudaMemcpyDeviceToHost));
