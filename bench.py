@@ -465,7 +465,7 @@ def time_batch(args, w, systems, handles, snp, torch, dist, dev, world, local, f
     o.stream = stream.cuda_stream
     o.transition = transition_code(snp, form)
     t0 = time.perf_counter()
-    chunk, tile, warps = snp.snp_batch_autotune(hs, o) if args.autotune else (2048, 0, 8)
+    chunk, tile, warps = snp.snp_batch_autotune(hs, o) if args.autotune else (0, 0, 0)  # 0: the engine's own
     tune_s = time.perf_counter() - t0
     o.chunk, o.tile, o.warps = chunk, tile, warps
     statuses = np.zeros(len(hs), dtype=np.int32)

@@ -15,11 +15,11 @@
 //              staging row lid), and every candidate holding such a pending
 //              key lowers that key's first-occurrence index;
 //     k_mark   one bit per first occurrence;
-//     k_commit ranks of the first occurrences in candidate order; the first `remaining` of them get their discovery index, in
-//              rank order (the row map entry; or a copy of the staged row
-//              into the discovery-ordered pool), and their table slots point
-//              at their rows; the rest become tombstones (the cap stops the
-//              depth).
+//     k_commit ranks of the first occurrences in candidate order; the first
+//              `remaining` of them get their discovery index, in rank order
+//              (the row map entry; or a copy of the staged row into the
+//              discovery-ordered pool), and their table slots point at their
+//              rows; the rest become tombstones (the cap stops the depth).
 #include <algorithm>
 #include <type_traits>
 
@@ -39,9 +39,10 @@ __device__ __forceinline__ void set_error(ChunkState* st, uint32_t bits) { atomi
 // off[p] = the sum of Psi over rows before p, off[P] = the total; with REC the
 // rows' ParentRecs.  Rows not to be expanded (max_expand) get Psi = 0, rows
 // whose children could leave int32 raise kErrOverflow.  A CTA takes one run of
-// a.sub consecutive tiles, a warp an eighth of them; runs are handed out in order, at most one per
-// resident CTA, and chained by decoupled look-back at their ends (a hop per 32
-// runs; a chain over all tiles of 2^20 rows cost over 100 us).
+// a.sub consecutive tiles, a warp an eighth of them; runs are handed out in
+// order, at most one per resident CTA, and chained by decoupled look-back at
+// their ends (a hop per 32 runs; a chain over all tiles of 2^20 rows cost over
+// 100 us).
 //   WARP = false: tiles of 256 rows, a lane per row.  A warp moves its 32 rows
 //     through shared memory 32 columns at a time (16-byte pieces where rows
 //     are whole pieces, else one coalesced 128-byte load per row), unpacked to
@@ -313,9 +314,10 @@ int launch_psi(PsiArgs a, int w, cudaStream_t st, int nsm) {
 
 // One bit per first occurrence: every candidate lid that claimed a key
 // (ownbits) names the key's first candidate gmin[lid]; clears ownbits and
-// counts the first occurrences of each commit tile.  A warp takes four words, a lane per claim, so that the four words' gmin loads are
-// in flight together (a thread per word walked its claims one after another:
-// 8 us per pass of 2^16, 11 us per pass of 2^20).
+// counts the first occurrences of each commit tile.  A warp takes four words, a
+// lane per claim, so that the four words' gmin loads are in flight together (a
+// thread per word walked its claims one after another: 8 us per pass of 2^16,
+// 11 us per pass of 2^20).
 __global__ void __launch_bounds__(256) k_mark(uint32_t* ownbits, const uint32_t* gmin, uint32_t* bits, uint32_t* srow,
                                               uint32_t nwords, uint32_t* counts, int tile_log, ChunkState* st,
                                               const DepthDyn* dyn) {
@@ -576,8 +578,10 @@ static int commit_words_log(uint32_t nwords) {
 
 // Marks, ranks and commit of a small chunk (at most kSmallWords bitmap words,
 // store mode) by one CTA, the bitmap in shared memory: one launch in place of
-// two where the launches are most of the time (3 neurons to depth 10: 492 us ->
-// 442 us; a pass of 6107 candidates by one CTA made 919 neurons 3% slower).
+// two where the launches are most of the time (3 neurons to depth 10: 525 us with
+// up to 2048 candidates, 460 with 4096, 8192 or 16384; 20, 64, 128 and 300 neurons
+// with caps of 1000 to 2500: within 2% for any of these limits; a pass of 6107
+// candidates by one CTA made 919 neurons 3% slower).
 constexpr uint32_t kSmallWords = 128;
 __global__ void __launch_bounds__(1024) k_commit_small(CommitArgs a, uint32_t* ownbits, const uint32_t* gmin,
                                                        uint32_t* srow) {

@@ -123,7 +123,10 @@ struct snp_server {
 namespace {
 
 constexpr uint32_t kServeQc = 2048;    // claims past the cap a request's table has room for, per depth
-constexpr uint32_t kServeRun = 64;     // candidates per work item (48 requests: 96 ms with 192, 80 with 64 or 32)
+// Candidates per work item.  48 requests of 8 to 512 neurons, cap 2^12: 65.8 ms
+// with 64, 65.9 with 32, 72.4 with 128, 80.6 with 192; 16 of 8 to 128 neurons,
+// cap 2^10: 6.1, 5.6, 7.1, 8.1 ms.
+constexpr uint32_t kServeRun = 64;
 constexpr int kTickIterations = 8;
 
 size_t request_bytes(const snp_system* h, const snp_explore_opts& o, int64_t* rows, uint64_t* nslots) {

@@ -36,22 +36,25 @@ def test_step_children_match_the_oracle(gpu, m, rules, deg, mode, capacity, shif
 
 
 @pytest.mark.gpu
-def test_step_waits_for_copies_into_its_pinned_row(gpu):
-    """C in pinned host memory that a copy on the default stream is still
-    writing when snp_step is called: the step is of the copied row."""
+@pytest.mark.parametrize("pin", [True, False])
+def test_step_waits_for_copies_into_its_row(gpu, pin):
+    """C in host memory, pinned or not, that a copy on the default stream is
+    still writing when snp_step is called: the step is of the copied row."""
     import torch
     system = snp_synth.random_system(78, 64, (2, 3), (4, 4), (0, 6), "sparse")
     s = gpu.System(system)
     o = oracle.Oracle(system)
     later = (np.asarray(system.c0) + 1).astype(np.int32)
     want = o.step(later, cap=500)
-    pinned = torch.from_numpy(np.array(system.c0, dtype=np.int32)).pin_memory()
+    host = torch.from_numpy(np.array(system.c0, dtype=np.int32))
+    if pin:
+        host = host.pin_memory()
     dev = torch.from_numpy(later).cuda()
     out = np.zeros((500, 64), dtype=np.int32)
-    gpu.snp_step(s.h, pinned, 500, out)  # loads the kernels
+    gpu.snp_step(s.h, host, 500, out)  # loads the kernels
     torch.cuda.synchronize()
     torch.cuda._sleep(200_000_000)  # about 0.1 s
-    pinned.copy_(dev, non_blocking=True)
-    psi = gpu.snp_step(s.h, pinned, 500, out)
+    host.copy_(dev, non_blocking=True)
+    psi = gpu.snp_step(s.h, host, 500, out)
     assert min(psi, 500) == len(want)
     assert (out[:len(want)] == want).all()
