@@ -94,6 +94,7 @@ int ensure_chunk_buffers(snp_system* h, uint64_t q, cudaStream_t st) {
   if (h->q_cap >= q) return SNP_OK;
   q = std::max<uint64_t>(q, std::min<uint64_t>(h->q_cap * 2, 1ull << 30));
   const uint64_t words = q / 32 + 1;
+  h->q_cap = 0;  // a failure below leaves new bitmaps that are not clear yet: the next call starts over
   TRY(h->d_sidx.reserve(sizeof(uint32_t) * q));
   TRY(h->d_gmin.reserve(sizeof(uint32_t) * q));
   TRY(h->d_slot_of.reserve(sizeof(uint32_t) * q));
