@@ -29,13 +29,18 @@ int fail(int code, const char* fmt, ...) {
   return code;
 }
 
-bool is_device_ptr(const void* p) {
+cudaMemoryType memory_type(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return cudaMemoryTypeUnregistered;
   }
-  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+  return a.type;
+}
+
+bool is_device_ptr(const void* p) {
+  const cudaMemoryType t = memory_type(p);
+  return t == cudaMemoryTypeDevice || t == cudaMemoryTypeManaged;
 }
 
 // e4m3 byte of an integer v with |v| <= 16 (exact: 1 sign, 4 exponent bits
@@ -436,14 +441,11 @@ int snp_step(snp_handle h, const int32_t* C, int64_t capacity, int32_t* out, uin
   const int m = h->m;
   // C twice: the second copy becomes the base child on the device
   std::vector<int32_t> c(2 * (size_t)m);
-  if (is_device_ptr(C)) {
-    CK(cudaMemcpy(c.data(), C, sizeof(int32_t) * m, cudaMemcpyDefault));
-  } else {
-    // what the default stream still writes there (a copy into pinned memory)
-    // comes first; cudaMemcpy would wait for it too, and take 10 us
-    CK(cudaStreamSynchronize(nullptr));
-    std::memcpy(c.data(), C, sizeof(int32_t) * m);
-  }
+  // What the default stream still writes to C comes first.  A copy into
+  // pageable memory has ended when its call returns; one into pinned memory
+  // may be in flight, and cudaMemcpy waits for it (5 to 10 us, so not for all).
+  if (memory_type(C) == cudaMemoryTypeUnregistered) std::memcpy(c.data(), C, sizeof(int32_t) * m);
+  else CK(cudaMemcpy(c.data(), C, sizeof(int32_t) * m, cudaMemcpyDefault));
   for (int j = 0; j < m; ++j) {
     if (c[j] < 0) return fail(SNP_E_INVALID, "C[%d] = %d < 0", j, c[j]);
     if (c[j] > INT32_MAX - h->gain[j]) return fail(SNP_E_OVERFLOW, "C[%d] = %d: a child could leave int32", j, c[j]);

@@ -21,6 +21,8 @@ extern thread_local std::string g_err;
 // Records a message for snp_last_error and returns code.
 int fail(int code, const char* fmt, ...);
 
+// What kind of memory p points to (cudaMemoryTypeUnregistered: pageable host memory).
+cudaMemoryType memory_type(const void* p);
 // True for device or managed memory.
 bool is_device_ptr(const void* p);
 
