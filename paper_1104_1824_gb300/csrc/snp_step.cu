@@ -11,7 +11,7 @@
 //                    odometer (mostly one swap), and writes the row out.
 //
 // Bound by the rows written and, below that, by the latency of a swap.  The
-// whole call for 2^15 children of 1024 neurons (134 MB) takes 75 us; with a
+// whole call for 2^15 children of 1024 neurons (134 MB) takes 74 us; with a
 // child built from C and every firing neuron's row (26 k shared-memory atomics
 // each) it took 4333 us.
 #include <algorithm>
